@@ -254,3 +254,81 @@ def tolerance(case):
     if case.get("out") == "f32":
         return {"rel": 1e-6, "max": 1e-5}
     return {"rel": 1e-4, "max": 1e-2}
+
+
+# ---- the same outputs in 64 bits -------------------------------------------------------------------------
+def _rotate64(x, block, signs=None):
+    """x R in float64: the Walsh-Hadamard butterfly inside every block (0: the whole row), over sqrt(block)."""
+    y = x.double() if signs is None else x.double() * signs.double()
+    rows, K = y.shape
+    B = block or K
+    h = 1
+    while h < B:
+        y = y.view(rows, K // (2 * h), 2, h)
+        y = torch.stack((y[:, :, 0] + y[:, :, 1], y[:, :, 0] - y[:, :, 1]), dim=2).view(rows, K)
+        h *= 2
+    return y / math.sqrt(B)
+
+
+def _to_grid(a, grid):
+    """Magnitudes to the nearest value of the E2M1 grid or of the integers 0..7 (halves to the even code)."""
+    if grid == "int":
+        return torch.round(a).clamp(max=7)
+    step = torch.exp2(torch.floor(torch.log2(a.clamp(1, 6)))) / 2
+    return (torch.round(a / step) * step).clamp(max=6)
+
+
+def _quantised64(y, fmt):
+    """Rotated values -> the values that the 4-bit format stands for, in float64."""
+    rows, K = y.shape
+    if fmt == "int4_row_asym":
+        lo, hi = y.amin(1, True).clamp(max=0), y.amax(1, True).clamp(min=0)
+        s = ((hi - lo) / 15).half().double()
+        z = torch.round(-lo / s).clamp(max=15)
+        return torch.where(s > 0, ((torch.round(y / s) + z).clamp(0, 15) - z) * s, torch.zeros_like(y))
+    g = y.view(rows, K // 32, 32)
+    amax = g.abs().amax(2, True)
+    grid = "int" if fmt in ("mxint4", "bint4") else "e2m1"
+    if fmt in ("mxfp4", "mxint4"):
+        s = torch.exp2((torch.frexp(amax)[1] - 1).double() - 2)
+    else:
+        s = (amax / (7 if grid == "int" else 6)).half().double()
+    q = torch.where(s > 0, _to_grid(g.abs() / s.clamp(min=2.0 ** -140), grid), torch.zeros_like(g))
+    return (torch.sign(g) * q * s).view(rows, K)
+
+
+def _linear64(x, w, block, signs=None):
+    return _quantised64(_rotate64(x, block, signs), "mxfp4") @ _quantised64(_rotate64(w, block, signs), "mxfp4").T
+
+
+def _gated64(gate, up):
+    return (gate.double() * torch.sigmoid(gate.double()) * up.double()).to(torch.bfloat16)
+
+
+def exact(case, seed):
+    """What run returns, in float64; None for bytes, codes and counts, which are compared bit for bit."""
+    gen = torch.Generator(device="cuda").manual_seed(int(seed))
+    kind, M, block = case["kind"], case["M"], case["block"]
+    if kind == "quantize":
+        return None
+    if kind == "stack":
+        d, kv, f = case["d"], case["kv"], case["f"]
+        x_qkv, x_o, x_gu = (_activations(M, d, gen) for _ in range(3))
+        qkv = _linear64(x_qkv, _weights(d + 2 * kv, d, gen), block)
+        o = _linear64(x_o, _weights(d, d, gen), block)
+        gu = _linear64(x_gu, _weights(2 * f, d, gen), block)
+        h = _gated64(gu[:, :f].to(torch.bfloat16), gu[:, f:].to(torch.bfloat16))
+        return [qkv, o, gu, _linear64(h, _weights(d, f, gen), block)]
+    K = case["K"]
+    x = _activations(M, K, gen)
+    if kind == "linear":
+        signs = _signs(K, gen) if case["signs"] else None
+        return _linear64(x, _weights(case["N"], K, gen), block, signs)
+    if kind == "mlp":
+        h = _gated64(x, _activations(M, K, gen))
+        return _linear64(h, _weights(case["N"], K, gen), block)
+    y = _rotate64(x, block)
+    if kind == "formats":
+        return {fmt: _quantised64(y, fmt) for fmt in STUDY_FORMATS}
+    mse = (y - _quantised64(y, "mxfp4")).square().view(M, K // 32, 32).mean(2)
+    return [None, None, None, None, None, None, mse]
