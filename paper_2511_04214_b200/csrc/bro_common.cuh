@@ -183,30 +183,31 @@ __device__ __forceinline__ void griddep_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Forms for a converged warp in which one lane issues: `issue` is non-zero in that lane only.  The
-// loop around them, and every address they take, stays warp-uniform.
-__device__ __forceinline__ void mbar_arrive_expect_tx_if(uint32_t issue, uint32_t bar, uint32_t bytes) {
+// Forms for a converged warp of which one lane issues.  The lane is picked by elect.sync inside each wrapper (the
+// same lane every time, as bulk groups and tcgen05.commit need): the compiler then knows that the instruction is
+// warp-uniform and takes its operands from uniform registers.  With a predicate computed from the lane number instead,
+// every tensor-core or TMA instruction cost its warp 60-160 cycles of issue (a K step of the GEMM with 4 scale copies
+// and 4 MMAs of 16 columns: 670 cycles; elected: 155).
+__device__ __forceinline__ void mbar_arrive_expect_tx_elect(uint32_t bar, uint32_t bytes) {
   asm volatile(
-      "{ .reg .pred q; .reg .b64 st; setp.ne.b32 q, %2, 0;\n\t"
+      "{ .reg .pred q; .reg .b64 st; elect.sync _|q, 0xffffffff;\n\t"
       "@q mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1; }" ::"r"(bar),
-      "r"(bytes), "r"(issue)
+      "r"(bytes)
       : "memory");
 }
-__device__ __forceinline__ void tma_load_2d_if(uint32_t issue, uint32_t dst, const CUtensorMap* m, int x, int y,
-                                               uint32_t bar) {
+__device__ __forceinline__ void tma_load_2d_elect(uint32_t dst, const CUtensorMap* m, int x, int y, uint32_t bar) {
   asm volatile(
-      "{ .reg .pred q; setp.ne.b32 q, %5, 0;\n\t"
+      "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
       "@q cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
       " [%0], [%1, {%2, %3}], [%4]; }" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(bar), "r"(issue)
+      "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
-__device__ __forceinline__ void bulk_load_1d_if(uint32_t issue, uint32_t dst, const void* src, uint32_t bytes,
-                                                uint32_t bar) {
+__device__ __forceinline__ void bulk_load_1d_elect(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile(
-      "{ .reg .pred q; setp.ne.b32 q, %4, 0;\n\t"
+      "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
       "@q cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3]; }" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar), "r"(issue)
+      "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar)
       : "memory");
 }
 // Bounded wait executed by a whole converged warp; the result is the same in every lane.

@@ -85,62 +85,57 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 // ---- issuing tensor-core work --------------------------------------------------------------------
-// The issuing warp runs its loop with all 32 lanes converged, so that addresses, descriptors and
-// loop counters stay warp-uniform: the tensor-core instructions take their operands from uniform
-// registers, and values computed under a divergent branch (or derived from something the compiler
-// cannot prove uniform, such as a raw threadIdx or a shared-memory load) have to cross register
-// files one by one, which makes instruction issue, not the tensor pipe, the limit.  One lane
-// executes the instruction itself: every wrapper below predicates it on `issue` (non-zero in that lane).
+// The issuing warp runs its loop with all 32 lanes converged, so that addresses, descriptors and loop counters
+// stay warp-uniform, and each wrapper elects the lane that executes the instruction (see the elect forms in
+// bro_common.cuh for what that is worth).
 // CG = 1: this CTA alone; CG = 2: the CTA pair (cta_group::2), issued by the leader CTA.
 template <int CG>
-__device__ __forceinline__ void tc_commit(uint32_t issue, uint32_t bar) {
+__device__ __forceinline__ void tc_commit(uint32_t bar) {
   if constexpr (CG == 1)
     asm volatile(
-        "{ .reg .pred q; setp.ne.b32 q, %1, 0;\n\t"
-        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0]; }" ::"r"(bar),
-        "r"(issue)
+        "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0]; }" ::"r"(bar)
         : "memory");
   else   // arrives on the barrier at this offset in both CTAs of the pair
     asm volatile(
-        "{ .reg .pred q; setp.ne.b32 q, %1, 0;\n\t"
-        "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %2; }" ::"r"(bar),
-        "r"(issue), "h"((uint16_t)3)
+        "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1; }" ::"r"(bar),
+        "h"((uint16_t)3)
         : "memory");
 }
 // Descriptors are passed as their two 32-bit halves: the upper half is a constant per descriptor
 // kind, the lower half is base + a small offset, so no 64-bit arithmetic is needed per instruction.
 template <int CG>
-__device__ __forceinline__ void tc_cp_sf(uint32_t issue, uint32_t taddr, uint32_t desc_lo, uint32_t desc_hi) {
+__device__ __forceinline__ void tc_cp_sf(uint32_t taddr, uint32_t desc_lo, uint32_t desc_hi) {
   if constexpr (CG == 1)
     asm volatile(
-        "{ .reg .pred q; .reg .b64 d; setp.ne.b32 q, %3, 0; mov.b64 d, {%1, %2};\n\t"
+        "{ .reg .pred q; .reg .b64 d; elect.sync _|q, 0xffffffff; mov.b64 d, {%1, %2};\n\t"
         "@q tcgen05.cp.cta_group::1.32x128b.warpx4 [%0], d; }" ::"r"(taddr),
-        "r"(desc_lo), "r"(desc_hi), "r"(issue)
+        "r"(desc_lo), "r"(desc_hi)
         : "memory");
   else
     asm volatile(
-        "{ .reg .pred q; .reg .b64 d; setp.ne.b32 q, %3, 0; mov.b64 d, {%1, %2};\n\t"
+        "{ .reg .pred q; .reg .b64 d; elect.sync _|q, 0xffffffff; mov.b64 d, {%1, %2};\n\t"
         "@q tcgen05.cp.cta_group::2.32x128b.warpx4 [%0], d; }" ::"r"(taddr),
-        "r"(desc_lo), "r"(desc_hi), "r"(issue)
+        "r"(desc_lo), "r"(desc_hi)
         : "memory");
 }
 template <int CG>
-__device__ __forceinline__ void tc_mma_mxf4(uint32_t issue, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo,
-                                            uint32_t desc_hi, uint32_t idesc, uint32_t sfa_tmem, uint32_t sfb_tmem,
-                                            uint32_t accumulate) {
+__device__ __forceinline__ void tc_mma_mxf4(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
+                                            uint32_t sfa_tmem, uint32_t sfb_tmem, uint32_t accumulate) {
   if constexpr (CG == 1)
     asm volatile(
-        "{ .reg .pred p, q; .reg .b64 da, db; setp.ne.b32 p, %7, 0; setp.ne.b32 q, %8, 0;\n\t"
+        "{ .reg .pred p, q; .reg .b64 da, db; setp.ne.b32 p, %7, 0; elect.sync _|q, 0xffffffff;\n\t"
         "mov.b64 da, {%1, %3}; mov.b64 db, {%2, %3};\n\t"
         "@q tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %4, [%5], [%6], p; }" ::"r"(d_tmem),
-        "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(sfa_tmem), "r"(sfb_tmem), "r"(accumulate), "r"(issue)
+        "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(sfa_tmem), "r"(sfb_tmem), "r"(accumulate)
         : "memory");
   else
     asm volatile(
-        "{ .reg .pred p, q; .reg .b64 da, db; setp.ne.b32 p, %7, 0; setp.ne.b32 q, %8, 0;\n\t"
+        "{ .reg .pred p, q; .reg .b64 da, db; setp.ne.b32 p, %7, 0; elect.sync _|q, 0xffffffff;\n\t"
         "mov.b64 da, {%1, %3}; mov.b64 db, {%2, %3};\n\t"
         "@q tcgen05.mma.cta_group::2.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %4, [%5], [%6], p; }" ::"r"(d_tmem),
-        "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(sfa_tmem), "r"(sfb_tmem), "r"(accumulate), "r"(issue)
+        "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(sfa_tmem), "r"(sfb_tmem), "r"(accumulate)
         : "memory");
 }
 __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
@@ -191,35 +186,22 @@ __device__ __forceinline__ void named_barrier_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 // TMA store shared -> global of one box; out-of-range parts of the box are clipped.
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* m, uint32_t src, int x, int y) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
-                   reinterpret_cast<uint64_t>(m)),
-               "r"(src), "r"(x), "r"(y)
-               : "memory");
-}
-// One-lane forms for a converged warp (`issue` non-zero in the issuing lane; operands uniform).
-__device__ __forceinline__ void tma_store_2d_if(uint32_t issue, const CUtensorMap* m, uint32_t src, int x, int y) {
+// Forms for a converged warp, executed by the elected lane.
+__device__ __forceinline__ void tma_store_2d_elect(const CUtensorMap* m, uint32_t src, int x, int y) {
   asm volatile(
-      "{ .reg .pred q; setp.ne.b32 q, %4, 0;\n\t"
+      "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
       "@q cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1]; }" ::"l"(
           reinterpret_cast<uint64_t>(m)),
-      "r"(src), "r"(x), "r"(y), "r"(issue)
+      "r"(src), "r"(x), "r"(y)
       : "memory");
 }
-__device__ __forceinline__ void bulk_commit_if(uint32_t issue) {
-  asm volatile("{ .reg .pred q; setp.ne.b32 q, %0, 0;\n\t@q cp.async.bulk.commit_group; }" ::"r"(issue) : "memory");
+__device__ __forceinline__ void bulk_commit_elect() {
+  asm volatile("{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t@q cp.async.bulk.commit_group; }" ::: "memory");
 }
 template <int N>
-__device__ __forceinline__ void bulk_wait_read_if(uint32_t issue) {
-  asm volatile("{ .reg .pred q; setp.ne.b32 q, %0, 0;\n\t@q cp.async.bulk.wait_group.read %1; }" ::"r"(issue), "n"(N)
-               : "memory");
+__device__ __forceinline__ void bulk_wait_read_elect() {
+  asm volatile("{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t@q cp.async.bulk.wait_group.read %0; }" ::"n"(N) : "memory");
 }
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void bulk_wait_read() {
-  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
@@ -266,10 +248,8 @@ template <int CG, int BN, int STAGES, int A_STAGE, int B_STAGE, int SFA_STAGE, i
           bool OVERLAP>
 __device__ __forceinline__ void mma_issue_loop(const IssueRing& r, uint32_t tmem_base, uint32_t tmem_sfa,
                                                uint32_t tmem_sfb, uint32_t idesc_full, int my_tiles, int num_k_steps,
-                                               bool issue_lane, int narrow_from = 0x7FFFFFFF,
-                                               uint32_t idesc_narrow = 0u) {
+                                               int narrow_from = 0x7FFFFFFF, uint32_t idesc_narrow = 0u) {
   // tiles narrow_from.. of this CTA are half-width: same loop, the instruction descriptor says N = BN/2
-  const uint32_t issue = issue_lane ? 1u : 0u;
   const uint32_t a_lo0 = desc_lo_sw128(r.sA), b_lo0 = desc_lo_sw128(r.sB);
   const uint32_t sfa_lo0 = desc_lo_sf(r.sSFA), sfb_lo0 = desc_lo_sf(r.sSFB);
   const uint32_t hi_op = kDescHiSw128, hi_sf = kDescHiSf;
@@ -280,16 +260,16 @@ __device__ __forceinline__ void mma_issue_loop(const IssueRing& r, uint32_t tmem
   auto copy_scales = [&](int stage, int h, bool narrow) {
     const uint32_t lo_a = sfa_lo0 + (uint32_t)stage * (SFA_STAGE >> 4) + (uint32_t)h * 32u;
     const uint32_t lo_b = sfb_lo0 + (uint32_t)stage * (SFB_STAGE >> 4) + (uint32_t)h * 32u;
-    tc_cp_sf<CG>(issue, tmem_sfa + 4 * h, lo_a, hi_sf);
-    tc_cp_sf<CG>(issue, tmem_sfb + (BN / 32) * h, lo_b, hi_sf);
-    if (BN == 256 && !narrow) tc_cp_sf<CG>(issue, tmem_sfb + (BN / 32) * h + 4, lo_b + 64u, hi_sf);
+    tc_cp_sf<CG>(tmem_sfa + 4 * h, lo_a, hi_sf);
+    tc_cp_sf<CG>(tmem_sfb + (BN / 32) * h, lo_b, hi_sf);
+    if (BN == 256 && !narrow) tc_cp_sf<CG>(tmem_sfb + (BN / 32) * h + 4, lo_b + 64u, hi_sf);
   };
   auto mma_half = [&](int stage, int h, uint32_t tmem_acc, uint32_t accumulate_first) {
     const uint32_t a_lo = a_lo0 + (uint32_t)stage * (A_STAGE >> 4) + 4u * h;
     const uint32_t b_lo = b_lo0 + (uint32_t)stage * (B_STAGE >> 4) + 4u * h;
     const uint32_t tsfa = tmem_sfa + 4 * h, tsfb = tmem_sfb + (BN / 32) * h;
-    tc_mma_mxf4<CG>(issue, tmem_acc, a_lo, b_lo, hi_op, idesc0, tsfa, tsfb, accumulate_first);
-    tc_mma_mxf4<CG>(issue, tmem_acc, a_lo + 2u, b_lo + 2u, hi_op, idesc1, tsfa | (2u << 30), tsfb | (2u << 30), 1u);
+    tc_mma_mxf4<CG>(tmem_acc, a_lo, b_lo, hi_op, idesc0, tsfa, tsfb, accumulate_first);
+    tc_mma_mxf4<CG>(tmem_acc, a_lo + 2u, b_lo + 2u, hi_op, idesc1, tsfa | (2u << 30), tsfb | (2u << 30), 1u);
   };
   int stage = 0;
   uint32_t phase = 0;
@@ -332,12 +312,12 @@ __device__ __forceinline__ void mma_issue_loop(const IssueRing& r, uint32_t tmem
         copy_scales(next_stage, 0, next_narrow);   // half 0's columns were last read by the two MMAs above
       }
       mma_half(stage, 1, tmem_acc, 1u);
-      tc_commit<CG>(issue, r.bar_empty + 8 * stage);   // frees the stage when these MMAs have read it
+      tc_commit<CG>(r.bar_empty + 8 * stage);   // frees the stage when these MMAs have read it
       if (has_next) copy_scales(next_stage, 1, next_narrow);
       stage = next_stage;
       phase = next_phase;
     }
-    tc_commit<CG>(issue, r.bar_acc_full + 8 * buf);    // accumulator complete (or abandoned) -> epilogue
+    tc_commit<CG>(r.bar_acc_full + 8 * buf);    // accumulator complete (or abandoned) -> epilogue
   }
 }
 
@@ -364,7 +344,6 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem_acc, int buf, int la
   static_assert(CHUNKS % 2 == 0, "chunks are processed in pairs");
   constexpr int PAIRS = CHUNKS / 2;
   const int64_t row = (int64_t)row0 + lane;
-  const uint32_t issue = lane == 0 ? 1u : 0u;
   auto pair_of = [&](int pi) { return (OVERLAP && buf == 0) ? (pi == 0 ? PAIRS - 1 : pi - 1) : pi; };
   auto released = [&](int pi) {
     if (pi == 0 || pi == PAIRS - 1) {
@@ -402,7 +381,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem_acc, int buf, int la
       }
       const uint32_t sbuf = stage_buf + (uint32_t)pi * stage_stride;
       // the TMA store that last read the staging buffer must be done reading it
-      if (stage_stride == 0u) bulk_wait_read_if<0>(issue);
+      if (stage_stride == 0u) bulk_wait_read_elect<0>();
       __syncwarp();
       // row `lane` of the box: 128 bytes, 16-byte pieces XOR-swizzled with lane & 7
       const uint32_t rowaddr = sbuf + (uint32_t)lane * 128u;
@@ -414,8 +393,8 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem_acc, int buf, int la
       // A TMA store clips at 16-byte granularity: when N is not a multiple of 8 the ragged last
       // pair is written from registers instead, element by element.
       const bool ragged = ((N & 7) != 0) && ((int64_t)col0 + 2 * kChunkCols > N);
-      tma_store_2d_if((col0 < N && row0 < M && !ragged) ? issue : 0u, tmy, sbuf, col0, row0);
-      bulk_commit_if(issue);           // (possibly empty) keeps the group count in step
+      if (col0 < N && row0 < M && !ragged) tma_store_2d_elect(tmy, sbuf, col0, row0);
+      bulk_commit_elect();             // (possibly empty) keeps the group count in step
       if (ragged && row < M) {
         uint16_t* dst = static_cast<uint16_t*>(y) + row * ldy + col0;
 #pragma unroll
@@ -507,66 +486,68 @@ gemm_mxfp4_kernel(const __grid_constant__ CUtensorMap tma, const __grid_constant
 
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------
+    // All 32 lanes walk the loop together (uniform addresses and counters); an elected lane issues.
     if (lane == 0) {
       tma_prefetch_desc(&tma);
       tma_prefetch_desc(&tmw);
       if (p.total_units > p.full_units) tma_prefetch_desc(&tmw_half);
-      int stage = 0;
-      uint32_t phase = 0;
-      int64_t issued = 0;
-      bool ok = true;
-      // loads of one K step of one unit; `part` selects the weight side (1), the activation side (2) or both (3)
-      auto issue_step = [&](int m0, int n0, int bn, int ks, int st, int part) {
-        // 128-row blocks of W scales that exist for this unit (a half-width unit of a ragged last
-        // tile can lie entirely beyond N: no block is read then, its columns are never stored)
-        const int nblk_valid = (int64_t)n0 >= p.N ? 0 : ((bn == 256 && (int64_t)n0 + 128 < p.N) ? 2 : 1);
-        const uint32_t full = bar_full + 8 * st;
-        if (part & 1) {
-          mbar_arrive_expect_tx(full, p.a_box_bytes + bn * 128 + C::kSfaBytes + nblk_valid * 1024);
-          tma_load_2d(sB + st * C::kBTileBytes, bn == BN ? &tmw : &tmw_half, ks * 128, n0, full);
-          const uint8_t* sfb_src = p.wscales + (int64_t)(n0 / 128) * p.kblocks * 512;
-          for (int nb = 0; nb < nblk_valid; ++nb)
-            bulk_load_1d(sSFB + st * C::kSfbBytes + nb * 1024, sfb_src + ((int64_t)nb * p.kblocks + 2 * ks) * 512, 1024,
-                         full);
-        }
-        if (part & 2) {
-          tma_load_2d(sA + st * kATileBytes, &tma, ks * 128, m0, full);
-          bulk_load_1d(sSFA + st * C::kSfaBytes, p.ascales + ((int64_t)(m0 / kBM) * p.kblocks + 2 * ks) * 512, 1024, full);
-        }
-      };
-      int pre = 0;                  // K steps of the first unit whose loads are issued here
-      if (early_w) {
-        if ((int)blockIdx.x < p.total_units) {
-          int m0, n0, bn;
-          decode_unit<BN>(p, (int)blockIdx.x, m0, n0, bn);
-          pre = p.num_k_steps < C::kStages ? p.num_k_steps : C::kStages;
-          for (int ks = 0; ks < pre; ++ks) issue_step(m0, n0, bn, ks, ks, 1);   // weights: before the wait
-          griddep_wait();
-          for (int ks = 0; ks < pre; ++ks) issue_step(m0, n0, bn, ks, ks, 2);   // activations: after it
-          issued = pre;
-          if (pre == C::kStages) phase = 1u; else stage = pre;
-        } else {
-          griddep_wait();
-        }
+    }
+    __syncwarp();
+    int stage = 0;
+    uint32_t phase = 0;
+    int64_t issued = 0;
+    bool ok = true;
+    // loads of one K step of one unit; `part` selects the weight side (1), the activation side (2) or both (3)
+    auto issue_step = [&](int m0, int n0, int bn, int ks, int st, int part) {
+      // 128-row blocks of W scales that exist for this unit (a half-width unit of a ragged last
+      // tile can lie entirely beyond N: no block is read then, its columns are never stored)
+      const int nblk_valid = (int64_t)n0 >= p.N ? 0 : ((bn == 256 && (int64_t)n0 + 128 < p.N) ? 2 : 1);
+      const uint32_t full = bar_full + 8 * st;
+      if (part & 1) {
+        mbar_arrive_expect_tx_elect(full, p.a_box_bytes + bn * 128 + C::kSfaBytes + nblk_valid * 1024);
+        if (bn == BN) tma_load_2d_elect(sB + st * C::kBTileBytes, &tmw, ks * 128, n0, full);
+        else tma_load_2d_elect(sB + st * C::kBTileBytes, &tmw_half, ks * 128, n0, full);
+        const uint8_t* sfb_src = p.wscales + ((int64_t)(n0 / 128) * p.kblocks + 2 * ks) * 512;
+        if (nblk_valid > 0) bulk_load_1d_elect(sSFB + st * C::kSfbBytes, sfb_src, 1024, full);
+        if (nblk_valid > 1) bulk_load_1d_elect(sSFB + st * C::kSfbBytes + 1024, sfb_src + p.kblocks * 512, 1024, full);
       }
-      for (int u = blockIdx.x; u < p.total_units && ok; u += gridDim.x) {
+      if (part & 2) {
+        tma_load_2d_elect(sA + st * kATileBytes, &tma, ks * 128, m0, full);
+        bulk_load_1d_elect(sSFA + st * C::kSfaBytes, p.ascales + ((int64_t)(m0 / kBM) * p.kblocks + 2 * ks) * 512, 1024, full);
+      }
+    };
+    int pre = 0;                  // K steps of the first unit whose loads are issued here
+    if (early_w) {
+      if ((int)blockIdx.x < p.total_units) {
         int m0, n0, bn;
-        decode_unit<BN>(p, u, m0, n0, bn);
-        for (int ks = (u == (int)blockIdx.x ? pre : 0); ks < p.num_k_steps; ++ks) {
-          if (issued >= C::kStages) ok = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, SITE_GEMM_EMPTY);
-          if (!ok) break;
-          issue_step(m0, n0, bn, ks, stage, 3);
-          ++issued;
-          if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
-        }
+        decode_unit<BN>(p, (int)blockIdx.x, m0, n0, bn);
+        pre = p.num_k_steps < C::kStages ? p.num_k_steps : C::kStages;
+        for (int ks = 0; ks < pre; ++ks) issue_step(m0, n0, bn, ks, ks, 1);   // weights: before the wait
+        griddep_wait();
+        for (int ks = 0; ks < pre; ++ks) issue_step(m0, n0, bn, ks, ks, 2);   // activations: after it
+        issued = pre;
+        if (pre == C::kStages) phase = 1u; else stage = pre;
+      } else {
+        griddep_wait();
       }
-      if (!ok) {
-        // Do not leave while copies may still land in this CTA's shared memory: wait (bounded)
-        // for the last load armed on every stage.
-        const int64_t first = issued > C::kStages ? issued - C::kStages : 0;
-        for (int64_t i = first; i < issued; ++i)
-          mbar_wait(bar_full + 8 * (int)(i % C::kStages), (uint32_t)((i / C::kStages) & 1), SITE_GEMM_DRAIN);
+    }
+    for (int u = blockIdx.x; u < p.total_units && ok; u += gridDim.x) {
+      int m0, n0, bn;
+      decode_unit<BN>(p, u, m0, n0, bn);
+      for (int ks = (u == (int)blockIdx.x ? pre : 0); ks < p.num_k_steps; ++ks) {
+        if (issued >= C::kStages) ok = mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1u, SITE_GEMM_EMPTY);
+        if (!ok) break;
+        issue_step(m0, n0, bn, ks, stage, 3);
+        ++issued;
+        if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
       }
+    }
+    if (!ok) {
+      // Do not leave while copies may still land in this CTA's shared memory: wait (bounded)
+      // for the last load armed on every stage.
+      const int64_t first = issued > C::kStages ? issued - C::kStages : 0;
+      for (int64_t i = first; i < issued; ++i)
+        mbar_wait_warp(bar_full + 8 * (int)(i % C::kStages), (uint32_t)((i / C::kStages) & 1), SITE_GEMM_DRAIN);
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
@@ -576,7 +557,7 @@ gemm_mxfp4_kernel(const __grid_constant__ CUtensorMap tma, const __grid_constant
     };
     mma_issue_loop<1, BN, C::kStages, kATileBytes, C::kBTileBytes, C::kSfaBytes, C::kSfbBytes, C::kAccStride,
                    C::kOverlap>(ring, tmem_base, tmem_sfa, tmem_sfb, make_idesc<BN>(), units_below(p.total_units),
-                                p.num_k_steps, lane == 0, units_below(p.full_units), make_idesc<BN / 2>());
+                                p.num_k_steps, units_below(p.full_units), make_idesc<BN / 2>());
   } else {
     // ------------------------------ epilogue ------------------------------
     const int q = warp & 3;                 // TMEM lane quadrant this warp may read
@@ -603,7 +584,7 @@ gemm_mxfp4_kernel(const __grid_constant__ CUtensorMap tma, const __grid_constant
     }
     // the staging buffer must have been read before this CTA's shared memory goes away; the writes
     // themselves complete with the kernel
-    if (!OUT_F32 && lane == 0) bulk_wait_read<0>();
+    if (!OUT_F32) bulk_wait_read_elect<0>();
   }
   tc_fence_before();
   __syncthreads();

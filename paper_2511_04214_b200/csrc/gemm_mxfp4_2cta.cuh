@@ -83,13 +83,13 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
 }
 // 2-D tiled load into THIS CTA's shared memory whose byte count completes on an mbarrier that may
 // live in the partner CTA (shared::cluster address).  No multicast.
-__device__ __forceinline__ void tma_load_2d_pair_if(uint32_t issue, uint32_t dst, const CUtensorMap* m, int x,
-                                                    int y, uint32_t bar_cluster) {
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* m, int x, int y,
+                                                 uint32_t bar_cluster) {
   asm volatile(
-      "{ .reg .pred q; setp.ne.b32 q, %5, 0;\n\t"
+      "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
       "@q cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
       " [%0], [%1, {%2, %3}], [%4]; }" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(bar_cluster), "r"(issue)
+      "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(bar_cluster)
       : "memory");
 }
 // E2M1 x E2M1, K-major, UE8M0 scales, M = 256 (128 rows per CTA), N = BN.
@@ -178,9 +178,8 @@ gemm_mxfp4_pair_kernel(const __grid_constant__ CUtensorMap tma, const __grid_con
 
   if (warp == 0) {
     // ------------------------------ TMA producer (both CTAs) ------------------------------
-    // All 32 lanes walk the loop together (uniform addresses and counters); lane 0 issues.
+    // All 32 lanes walk the loop together (uniform addresses and counters); an elected lane issues.
     {
-      const uint32_t issue = lane == 0 ? 1u : 0u;
       if (lane == 0) {
         tma_prefetch_desc(&tma);
         tma_prefetch_desc(&tmw);
@@ -204,16 +203,16 @@ gemm_mxfp4_pair_kernel(const __grid_constant__ CUtensorMap tma, const __grid_con
         for (int ks = 0; ks < p.num_k_steps; ++ks) {
           if (issued >= kStages) ok = mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1u, SITE_GEMM_EMPTY);
           if (!ok) break;
-          if (rank == 0) mbar_arrive_expect_tx_if(issue, bar_full + 8 * stage, stage_tx);
+          if (rank == 0) mbar_arrive_expect_tx_elect(bar_full + 8 * stage, stage_tx);
           const uint32_t full = full0 + 8 * stage;
-          tma_load_2d_pair_if(issue, sA + stage * kATileBytes, &tma, ks * 128, m0, full);
+          tma_load_2d_pair(sA + stage * kATileBytes, &tma, ks * 128, m0, full);
           if (bn == kBN)
-            tma_load_2d_pair_if(issue, sB + stage * kBTileBytes, &tmw, ks * 128, n0 + (int)rank * (kBN / 2), full);
+            tma_load_2d_pair(sB + stage * kBTileBytes, &tmw, ks * 128, n0 + (int)rank * (kBN / 2), full);
           else
-            tma_load_2d_pair_if(issue, sB + stage * kBTileBytes, &tmw_half, ks * 128, n0 + (int)rank * (kBN / 4), full);
+            tma_load_2d_pair(sB + stage * kBTileBytes, &tmw_half, ks * 128, n0 + (int)rank * (kBN / 4), full);
           // scale maps are in 32-bit elements: one K step = 1024 bytes = 256 elements per row block
-          tma_load_2d_pair_if(issue, sSFA + stage * kSfaBytes, &tmsfa, ks * 256, m0 >> 7, full);
-          tma_load_2d_pair_if(issue, sSFB + stage * kSfbBytes, &tmsfb, ks * 256, n0 >> 7, full);
+          tma_load_2d_pair(sSFA + stage * kSfaBytes, &tmsfa, ks * 256, m0 >> 7, full);
+          tma_load_2d_pair(sSFB + stage * kSfbBytes, &tmsfb, ks * 256, n0 >> 7, full);
           ++issued;
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
@@ -228,7 +227,7 @@ gemm_mxfp4_pair_kernel(const __grid_constant__ CUtensorMap tma, const __grid_con
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer (leader only) ------------------------------
-    // All 32 lanes of the leader's warp walk the loop together; lane 0 issues for the pair.
+    // All 32 lanes of the leader's warp walk the loop together; an elected lane issues for the pair.
     if (rank == 0) {
       const gemm::IssueRing ring = {sA, sB, sSFA, sSFB, bar_full, bar_empty, bar_acc_full, bar_acc_free, bar_ovl_free};
       auto units_below = [&](int limit) {   // how many of this pair's units have an index below `limit`
@@ -236,7 +235,7 @@ gemm_mxfp4_pair_kernel(const __grid_constant__ CUtensorMap tma, const __grid_con
       };
       gemm::mma_issue_loop<2, kBN, kStages, kATileBytes, kBTileBytes, kSfaBytes, kSfbBytes, kAccStride, true>(
           ring, tmem_base, tmem_sfa, tmem_sfb, make_idesc_pair<kBN>(), units_below(p.total_units), p.num_k_steps,
-          lane == 0, units_below(p.full_units), make_idesc_pair<kBN / 2>());
+          units_below(p.full_units), make_idesc_pair<kBN / 2>());
     }
   } else {
     // ------------------------------ epilogue (both CTAs) ------------------------------
@@ -266,7 +265,7 @@ gemm_mxfp4_pair_kernel(const __grid_constant__ CUtensorMap tma, const __grid_con
     }
     // the staging buffer must have been read before this CTA's shared memory goes away; the writes
     // themselves complete with the kernel
-    if (!OUT_F32 && lane == 0) gemm::bulk_wait_read<0>();
+    if (!OUT_F32) gemm::bulk_wait_read_elect<0>();
   }
   gemm::tc_fence_before();
   __syncthreads();
