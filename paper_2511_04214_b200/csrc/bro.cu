@@ -12,6 +12,7 @@
 #include "rotate_quantize_direct.cuh"
 #include "gemm_mxfp4.cuh"
 #include "gemm_mxfp4_2cta.cuh"
+#include "gemm_mxfp4_splitk.cuh"
 #include "scale_stats.cuh"
 #include "fake_quantize.cuh"
 
@@ -604,7 +605,18 @@ static bro_status gemm_impl(const void* acodes, const void* ascales, const void*
   DeviceInfo di;
   bro_status rc = device_info(&di);
   if (rc != BRO_OK) return rc;
-  // Two kernels.  The two-CTA kernel (256 x 256 tiles, cta_group::2) moves a third fewer bytes into
+  // Three kernels.  Problems whose 128-row tiles of W fit the chip in one wave (decoding; a few hundred tokens through a
+  // narrow layer) go to the split-K kernel, see its plan().
+  if (!(flags & (BRO_FLAG_GEMM_PAIR | BRO_FLAG_GEMM_SINGLE | BRO_FLAG_GEMM_TILE_N128 | BRO_FLAG_GEMM_TILE_N256 |
+                 BRO_FLAG_GEMM_NO_SPLIT))) {
+    bro::gemms::Plan plan;
+    rc = bro::gemms::plan(M, N, (int)ceil_div(K, 256), di.sm_count, &plan);
+    if (rc != BRO_OK) return rc;
+    if (plan.row_blocks > 0)
+      return bro::gemms::launch(plan, acodes, ascales, wcodes, wscales, M, N, K, y, ldy, (int)out_dtype, di.sm_count,
+                                static_cast<cudaStream_t>(stream), w_static);
+  }
+  // Else the two-CTA kernel (256 x 256 tiles, cta_group::2) moves a third fewer bytes into
   // shared memory per flop and measures 3-7 % faster once a problem has at least two rounds of
   // 256 x 256 tiles and tiles long enough (K >= 4096) to amortise its costlier tile hand-over; below
   // that the single-CTA kernel wins (half-width units for the last round, 128-row granularity, cheaper

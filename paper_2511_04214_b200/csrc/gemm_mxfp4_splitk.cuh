@@ -1,0 +1,426 @@
+// Kernel 2s: block-scaled MXFP4 x MXFP4 GEMM for problems with too few output tiles to fill the chip
+// (paper Sec. 1 / Sec. 4.2: W4A4, y = Q(xR) Q(WR)^T; fp32 accumulation, bf16 or fp32 output) — decoding
+// above all, where a launch is one pass over the packed weights and nothing else.
+//
+// The operands change sides: 128 (or 256) rows of W are the M side of the instruction and the tokens, padded
+// to 16, 32, 64 or 128, the N side, so that a few tokens cost a few columns of tensor-core work and of
+// shared memory, and the ring that holds the weights in flight is as deep as shared memory allows.
+// One CTA computes one tile over one part of K, all of it in one wave:
+//   * the `split` CTAs of a cluster share a tile, each takes a contiguous range of its 256-element K steps
+//     and sends its fp32 partial sums to the CTAs that own the tokens (distributed shared memory); a token's
+//     owner adds the parts in rank order, converts and stores.  No workspace, no atomics, fixed order.
+//   * with W packed before the previous kernel in the stream started (the whole-layer calls), the whole ring of
+//     weight tiles is requested before griddepcontrol.wait, under the rotate+quantize kernel.
+// Warps: 0 TMA producer, 1 TMEM owner and MMA issuer, 2..9 epilogue.  Every mbarrier wait is bounded, and all
+// threads of a cluster reach both cluster barriers whatever happened before.
+#pragma once
+
+#include "gemm_mxfp4.cuh"
+#include "gemm_mxfp4_2cta.cuh"
+
+namespace bro {
+namespace gemms {
+
+constexpr int kEpilogueWarps = 8;                // two per TMEM lane quadrant
+constexpr int kThreads = (2 + kEpilogueWarps) * 32;
+constexpr int kRowsW = 128;                      // rows of W per MMA
+constexpr int kMaxTokens = 128;                  // tokens per tile
+constexpr int kWTileBytes = kRowsW * 128;        // 16 KiB: one 256-element K step of 128 rows
+constexpr int kScaleBytes = 1024;                // its scales: 2 blocks of 512 B
+constexpr int kMaxStages = 11;
+constexpr int kMaxSplit = 8;                     // portable cluster size
+constexpr int kMaxSmem = 227 * 1024;
+constexpr int kFixedSmem = 1024 /*align*/ + 256 /*barriers*/;
+constexpr int kScaleCols = 32;                   // TMEM columns kept for scales: W 2 x 8, tokens 2 x 4
+
+struct Params {
+  const uint8_t* ascales;
+  const uint8_t* wscales;
+  void* y;
+  int64_t M, N, ldy;
+  int64_t kblocks;          // 512-byte scale blocks per 128-row block
+  int num_k_steps;          // ceil(K / 256)
+  int tiles_n;              // tiles of 128 (or 256, kernel template) columns of y
+  int tokens;               // N of the instruction: 16, 32, 64 or 128
+  int split;                // CTAs of a cluster, K parts of a tile
+  int groups;               // split > 1: groups of 4 tokens that each CTA of a cluster owns
+  int groups_magic;         // ceil(65536 / groups): i / groups == (i * groups_magic) >> 16 for i < 32
+  int stages, stage_bytes;
+  int a_box_bytes;          // bytes one activation box brings (rows beyond M up to the next power of two)
+  int tmem_cols;            // 256 or 512
+  int out_f32;
+  int w_static;             // the weight operand was complete before the previous kernel started
+};
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void st_cluster_128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+
+// One token's value of the row of W (column n of y) that this lane holds.
+__device__ __forceinline__ void store_f32(void* y, int64_t at, uint32_t v) { static_cast<uint32_t*>(y)[at] = v; }
+__device__ __forceinline__ void store_bf16_pair(void* y, int64_t at, int64_t ldy, uint32_t v0, uint32_t v1, bool second) {
+  uint32_t h;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(__uint_as_float(v1)), "f"(__uint_as_float(v0)));
+  static_cast<uint16_t*>(y)[at] = (uint16_t)h;
+  if (second) static_cast<uint16_t*>(y)[at + ldy] = (uint16_t)(h >> 16);
+}
+
+template <int ROW_BLOCKS>
+__global__ void __launch_bounds__(kThreads, 1)
+gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_constant__ CUtensorMap tmw, const Params p) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  // stage: W tiles | token tile | W scales | token scales; behind the ring (split > 1) the parts received, the barriers
+  constexpr uint32_t w_bytes = (uint32_t)ROW_BLOCKS * kWTileBytes;
+  const uint32_t off_sfw = w_bytes + (uint32_t)p.tokens * 128u;
+  const uint32_t off_sfa = off_sfw + (uint32_t)ROW_BLOCKS * kScaleBytes;
+  const uint32_t parts = smem_base + (uint32_t)(p.stages * p.stage_bytes);     // [source rank][group][row][4 tokens] fp32
+  const uint32_t bar_full = parts + (p.split > 1 ? (uint32_t)(p.split * p.groups) * (kRowsW * 16u) : 0u);   // [kMaxStages]
+  const uint32_t bar_empty = bar_full + 8 * kMaxStages;                        // [kMaxStages]
+  const uint32_t bar_acc = bar_empty + 8 * kMaxStages;
+  const uint32_t tmem_slot = bar_acc + 8;
+  uint32_t* tmem_slot_ptr = reinterpret_cast<uint32_t*>(smem_raw + (tmem_slot - smem_u32(smem_raw)));
+
+  const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);
+  const int lane = threadIdx.x & 31;
+  const int unit = (int)blockIdx.x / p.split, rank = (int)blockIdx.x - unit * p.split;
+  const int tm = unit / p.tiles_n, tn = unit - tm * p.tiles_n;
+  const int m0 = tm * kMaxTokens, n0 = tn * kRowsW * ROW_BLOCKS;
+  const int k_each = p.num_k_steps / p.split, k_more = p.num_k_steps - k_each * p.split;
+  const int k_first = rank * k_each + min(rank, k_more), k_count = k_each + (rank < k_more ? 1 : 0);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < p.stages; ++s) {
+      mbar_init(bar_full + 8 * s, 1);
+      mbar_init(bar_empty + 8 * s, 1);
+    }
+    mbar_init(bar_acc, 1);
+    mbar_fence_init();
+    fence_proxy_async_smem();
+  }
+  if (warp == 1) {
+    gemm::tmem_alloc(tmem_slot, (uint32_t)p.tmem_cols);
+    gemm::tmem_relinquish();
+  }
+  if (threadIdx.x == 0) {
+    tma_prefetch_desc(&tma);
+    tma_prefetch_desc(&tmw);
+  }
+  gemm::tc_fence_before();
+  __syncthreads();
+  gemm::tc_fence_after();
+  if (p.split > 1) cluster_arrive();          // (waited for before the first write to another CTA)
+  griddep_launch_dependents();
+  const bool early_w = p.w_static != 0 && warp == 0;
+  if (!early_w) griddep_wait();
+  const uint32_t tmem_base = __shfl_sync(0xFFFFFFFFu, *tmem_slot_ptr, 0);
+  const uint32_t tmem_sfw = tmem_base + (uint32_t)p.tmem_cols - kScaleCols;
+  const uint32_t tmem_sfa = tmem_sfw + 16u;
+
+  if (warp == 0) {
+    // ------------------------------ TMA producer ------------------------------
+    // scale blocks of W that exist (the second half of a ragged last tile may lie beyond N)
+    const int blocks = ROW_BLOCKS == 2 && (int64_t)n0 + kRowsW < p.N ? 2 : 1;
+    // `part`: 1 the weight side, 2 the token side, 3 both
+    auto issue_step = [&](int i, int st, int part) {
+      const uint32_t full = bar_full + 8 * st, base = smem_base + (uint32_t)(st * p.stage_bytes);
+      const int ks = k_first + i;
+      if (part & 1) {
+        mbar_arrive_expect_tx_elect(full, w_bytes + (uint32_t)p.a_box_bytes + (uint32_t)(blocks + 1) * kScaleBytes);
+        tma_load_2d_elect(base, &tmw, ks * 128, n0, full);                               // (rows beyond N arrive as zeros)
+        const uint8_t* src = p.wscales + ((int64_t)(n0 / kRowsW) * p.kblocks + 2 * ks) * 512;
+        bulk_load_1d_elect(base + off_sfw, src, kScaleBytes, full);
+        if (blocks == 2) bulk_load_1d_elect(base + off_sfw + kScaleBytes, src + p.kblocks * 512, kScaleBytes, full);
+      }
+      if (part & 2) {
+        tma_load_2d_elect(base + w_bytes, &tma, ks * 128, m0, full);
+        bulk_load_1d_elect(base + off_sfa, p.ascales + ((int64_t)tm * p.kblocks + 2 * ks) * 512, kScaleBytes, full);
+      }
+    };
+    int i = 0;
+    if (early_w) {
+      const int pre = min(k_count, p.stages);
+      for (int s = 0; s < pre; ++s) issue_step(s, s, 1);       // weights: before the wait
+      griddep_wait();
+      for (int s = 0; s < pre; ++s) issue_step(s, s, 2);       // tokens: after it
+      i = pre;
+    }
+    bool ok = true;
+    int stage = i == p.stages ? 0 : i;
+    uint32_t phase = i == p.stages ? 1u : 0u;
+    for (; i < k_count; ++i) {
+      if (i >= p.stages) ok = mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1u, SITE_GEMM_EMPTY);
+      if (!ok) break;
+      issue_step(i, stage, 3);
+      if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+    }
+    if (!ok) {
+      // do not leave while copies may still land: wait (bounded) for the last load armed on every stage
+      for (int j = i > p.stages ? i - p.stages : 0; j < i; ++j)
+        mbar_wait_warp(bar_full + 8 * (j % p.stages), (uint32_t)(j / p.stages) & 1u, SITE_GEMM_DRAIN);
+    }
+  } else if (warp == 1) {
+    // ------------------------------ MMA issuer ------------------------------
+    // E2M1 x E2M1, K-major, UE8M0 scales, M = 128, N = tokens; scale bytes {0,1} / {2,3} of a scale word
+    const uint32_t idesc0 = (1u << 7) | (1u << 10) | ((uint32_t)(p.tokens >> 3) << 17) | (1u << 23) | ((128u >> 4) << 24);
+    const uint32_t idesc1 = idesc0 | (2u << 4) | (2u << 29);
+    int stage = 0;
+    uint32_t phase = 0;
+    for (int i = 0; i < k_count; ++i) {
+      if (!mbar_wait_warp(bar_full + 8 * stage, phase, SITE_GEMM_FULL)) break;
+      gemm::tc_fence_after();
+      const uint32_t base = smem_base + (uint32_t)(stage * p.stage_bytes);
+      const uint32_t w_lo = gemm::desc_lo_sw128(base), a_lo = gemm::desc_lo_sw128(base + w_bytes);
+      const uint32_t sfw_lo = gemm::desc_lo_sf(base + off_sfw), sfa_lo = gemm::desc_lo_sf(base + off_sfa);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {       // the two 128-element halves of the step own separate scale columns
+        gemm::tc_cp_sf<1>(tmem_sfa + 4 * h, sfa_lo + 32u * h, gemm::kDescHiSf);
+#pragma unroll
+        for (int b = 0; b < ROW_BLOCKS; ++b)
+          gemm::tc_cp_sf<1>(tmem_sfw + 8 * h + 4 * b, sfw_lo + 64u * b + 32u * h, gemm::kDescHiSf);
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int b = 0; b < ROW_BLOCKS; ++b) {
+          const uint32_t d = tmem_base + (uint32_t)(b * p.tokens), w = w_lo + (uint32_t)b * (kWTileBytes >> 4) + 4u * h;
+          const uint32_t sw = tmem_sfw + 8 * h + 4 * b, sa = tmem_sfa + 4 * h, a = a_lo + 4u * h;
+          gemm::tc_mma_mxf4<1>(d, w, a, gemm::kDescHiSw128, idesc0, sw, sa, (h == 0 && i == 0) ? 0u : 1u);
+          gemm::tc_mma_mxf4<1>(d, w + 2u, a + 2u, gemm::kDescHiSw128, idesc1, sw | (2u << 30), sa | (2u << 30), 1u);
+        }
+      }
+      gemm::tc_commit<1>(bar_empty + 8 * stage);
+      if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+    }
+    gemm::tc_commit<1>(bar_acc);              // accumulator complete (or abandoned) -> epilogue
+  }
+
+  // ------------------------------ epilogue ------------------------------
+  // A lane holds one row of W (column of y) and its tokens: a warp's store of one token is 64 (fp32: 128)
+  // contiguous bytes.  Two warps per TMEM lane quadrant share the row blocks or the chunks of 16 tokens.
+  const int live = (int)(p.M - m0 < p.tokens ? p.M - m0 : p.tokens);       // tokens of this tile that exist
+  const int q = warp & 3, half = (warp - 2) >> 2;
+  const uint32_t tmem_acc = tmem_base + ((uint32_t)(q * 32) << 16);
+  bool ok = true;
+  if (warp >= 2) {
+    ok = mbar_wait_warp(bar_acc, 0u, SITE_GEMM_ACC_FULL);
+    gemm::tc_fence_after();
+  }
+  auto store4 = [&](int64_t at, const uint32_t (&v)[4], int exist) {        // 4 tokens of one column
+    if (p.out_f32) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (j < exist) store_f32(p.y, at + j * p.ldy, v[j]);
+    } else {
+      store_bf16_pair(p.y, at, p.ldy, v[0], v[1], exist > 1);
+      if (exist > 2) store_bf16_pair(p.y, at + 2 * p.ldy, p.ldy, v[2], v[3], exist > 3);
+    }
+  };
+  if (p.split == 1) {
+    if (warp >= 2 && ok) {
+      const int b = ROW_BLOCKS == 2 ? half : 0;
+      const int64_t n = (int64_t)n0 + b * kRowsW + q * 32 + lane;
+      for (int c = ROW_BLOCKS == 2 ? 0 : half * 16; c < live; c += ROW_BLOCKS == 2 ? 16 : 32) {
+        uint32_t r[16];
+        tc_ld16(tmem_acc + (uint32_t)(b * p.tokens + c), r);
+        gemm::tc_wait_ld();
+        if (n < p.N) {
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            const uint32_t v[4] = {r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]};
+            if (c + 4 * g < live) store4((int64_t)(m0 + c + 4 * g) * p.ldy + n, v, live - c - 4 * g);
+          }
+        }
+      }
+    }
+  } else {
+    // (16-byte stores straight into the owners' shared memory; staged locally and sent as bulk copies, 128 tokens took
+    // 2 us longer)
+    cluster_wait();                           // every CTA of the cluster runs
+    if (warp >= 2 && ok) {
+      for (int c = half * 16; c < live; c += 32) {
+        uint32_t r[16];
+        tc_ld16(tmem_acc + (uint32_t)c, r);
+        gemm::tc_wait_ld();
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          const int gi = (c >> 2) + g;
+          const int owner = (gi * p.groups_magic) >> 16, slot = gi - owner * p.groups;
+          if (4 * gi < live)
+            st_cluster_128(gemm2::map_to_cta(parts + (uint32_t)(((rank * p.groups + slot) * kRowsW + q * 32 + lane) * 16), (uint32_t)owner),
+                           r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
+        }
+      }
+    }
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();                           // all parts have arrived; nobody writes here any more
+    if (warp >= 2 && ok) {
+      const int row = q * 32 + lane;
+      const int64_t n = (int64_t)n0 + row;
+      for (int s = half; s < p.groups; s += 2) {
+        const int token = (rank * p.groups + s) * 4;
+        if (token >= live) break;
+        const uint32_t src = parts + (uint32_t)((s * kRowsW + row) * 16);
+        uint4 sum = lds128(src);
+        for (int r = 1; r < p.split; ++r) {    // parts in rank order, whichever arrived first
+          const uint4 v = lds128(src + (uint32_t)(r * p.groups * kRowsW * 16));
+          sum.x = __float_as_uint(__fadd_rn(__uint_as_float(sum.x), __uint_as_float(v.x)));
+          sum.y = __float_as_uint(__fadd_rn(__uint_as_float(sum.y), __uint_as_float(v.y)));
+          sum.z = __float_as_uint(__fadd_rn(__uint_as_float(sum.z), __uint_as_float(v.z)));
+          sum.w = __float_as_uint(__fadd_rn(__uint_as_float(sum.w), __uint_as_float(v.w)));
+        }
+        const uint32_t v[4] = {sum.x, sum.y, sum.z, sum.w};
+        if (n < p.N) store4((int64_t)(m0 + token) * p.ldy + n, v, live - token);
+      }
+    }
+  }
+  gemm::tc_fence_before();
+  __syncthreads();
+  if (warp == 1) gemm::tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
+}
+
+// How many clusters of `split` CTAs (one CTA per SM) run at once on this device; 0 if none.
+inline bro_status resident_clusters(int split, int sm_count, int* out) {
+  static DeviceOnce attr, once[kMaxSplit + 1];
+  bro_status rc = device_once(attr, nullptr, [&](int*) {
+    const bool ok = cuda_ok(cudaFuncSetAttribute(gemm_mxfp4_splitk_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem),
+                            "cudaFuncSetAttribute(gemm split-K)") &&
+                    cuda_ok(cudaFuncSetAttribute(gemm_mxfp4_splitk_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem),
+                            "cudaFuncSetAttribute(gemm split-K)");
+    return ok ? BRO_OK : BRO_ERR_CUDA;
+  });
+  if (rc != BRO_OK) return rc;
+  if (split == 1) { *out = sm_count; return BRO_OK; }
+  int plus_one = 1;                           // (device_once remembers positive values only)
+  rc = device_once(once[split], &plus_one, [&](int* n) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(sm_count / split * split), 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = kMaxSmem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)split;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (!cuda_ok(cudaOccupancyMaxActiveClusters(n, gemm_mxfp4_splitk_kernel<1>, &cfg), "occupancy(gemm split-K)"))
+      return BRO_ERR_CUDA;
+    ++*n;
+    return BRO_OK;
+  });
+  *out = plus_one - 1;
+  return rc;
+}
+
+// N of the instruction for M tokens
+inline int token_columns(int64_t M) {
+  int t = 16;
+  while (t < kMaxTokens && t < M) t *= 2;
+  return t;
+}
+
+struct Plan {
+  int row_blocks = 0, tiles_m = 0, tiles_n = 0, split = 0;     // row_blocks = 0: not a problem for this kernel
+};
+
+// One wave of whole tiles, or none of this.  128-row tiles when they fit the chip at once; else, decoding at most 64
+// tokens through a wider layer, 256-row tiles (K = 8192, N = 28672: 1 token 23.5 -> 21.3 us, 64 tokens 24.8 -> 23.3 us
+// against the persistent kernel; 96 tokens no gain, 128 tokens 2 % slower).  Several token tiles need 8 K steps:
+// (512, 14336, 4096) 21.7 -> 15.6 us and (512, 2048, 2048) even, but (640, 1024, 3000) 4.1 -> 4.3 us.
+// Parts: among the cluster sizes whose clusters are all resident, the fewest K steps per CTA.  The exchange between the
+// CTAs costs about 0.5 us with 16 tokens, 1.3 us with 64 and 4.5 us with 128, a K step 0.1 to 0.2 us, hence the line at
+// 4 + tokens / 5 saved steps.  (16, 14336, 4096): 1 part 10.5 us, 2 parts 7.3, 4 parts 6.3, persistent kernel 20.1;
+// (64, 2048, 2048): 1 part 3.7 us, 2 parts 4.3; (128, 14336, 4096): 1 part 14.5 us, 4 parts 10.9, persistent 20.8.
+inline bro_status plan(int64_t M, int64_t N, int num_k_steps, int sm_count, Plan* out) {
+  const int64_t tiles_m = (M + kMaxTokens - 1) / kMaxTokens, n128 = (N + kRowsW - 1) / kRowsW;
+  const int tokens = token_columns(M);
+  Plan pl;
+  if (tiles_m * n128 <= sm_count && (tiles_m == 1 || num_k_steps >= 8)) {
+    pl.row_blocks = 1;
+    pl.tiles_n = (int)n128;
+    pl.split = 1;
+    int best = num_k_steps;
+    for (int s = 2; s <= kMaxSplit && s <= num_k_steps; ++s) {
+      const int steps = (num_k_steps + s - 1) / s;
+      if (steps >= best || num_k_steps - steps <= 4 + tokens / 5 || tiles_m * n128 * s > sm_count) continue;
+      int fit = 0;
+      const bro_status rc = resident_clusters(s, sm_count, &fit);
+      if (rc != BRO_OK) return rc;
+      if (tiles_m * n128 > fit) continue;
+      best = steps;
+      pl.split = s;
+    }
+  } else if (tokens <= 64 && (n128 + 1) / 2 <= sm_count) {
+    pl.row_blocks = 2;
+    pl.tiles_n = (int)((n128 + 1) / 2);
+    pl.split = 1;
+  }
+  pl.tiles_m = (int)tiles_m;
+  *out = pl;
+  return BRO_OK;
+}
+
+inline bro_status launch(const Plan& pl, const void* acodes, const void* ascales, const void* wcodes, const void* wscales,
+                         int64_t M, int64_t N, int64_t K, void* y, int64_t ldy, int out_dtype, int sm_count, cudaStream_t st,
+                         bool w_static) {
+  Params p;
+  p.ascales = static_cast<const uint8_t*>(ascales);
+  p.wscales = static_cast<const uint8_t*>(wscales);
+  p.y = y;
+  p.M = M; p.N = N; p.ldy = ldy;
+  p.num_k_steps = (int)((K + 255) / 256);
+  p.kblocks = 2 * (int64_t)p.num_k_steps;
+  p.tiles_n = pl.tiles_n;
+  p.split = pl.split;
+  p.out_f32 = out_dtype == BRO_OUT_F32 ? 1 : 0;
+  p.w_static = w_static ? 1 : 0;
+  p.tokens = token_columns(M);
+  // the activation box covers only the next power of two of rows (at least 8): rows it does not bring keep what the
+  // stage held, finite fp4 codes under zero-padded scales, and feed columns that are never stored
+  int a_rows = p.tokens;
+  while (a_rows > 8 && a_rows / 2 >= M) a_rows /= 2;
+  p.a_box_bytes = a_rows * 128;
+  const int tile_groups = (int)((M < p.tokens ? M : p.tokens) + 3) / 4;
+  p.groups = (tile_groups + p.split - 1) / p.split;
+  p.groups_magic = (65536 + p.groups - 1) / p.groups;
+  p.stage_bytes = pl.row_blocks * (kWTileBytes + kScaleBytes) + p.tokens * 128 + kScaleBytes;
+  const int parts = p.split > 1 ? p.split * p.groups * kRowsW * 16 : 0;
+  const int steps = (p.num_k_steps + p.split - 1) / p.split;
+  p.stages = (kMaxSmem - kFixedSmem - parts) / p.stage_bytes;
+  if (p.stages > kMaxStages) p.stages = kMaxStages;
+  if (p.stages > steps) p.stages = steps;
+  // At least a third of an SM, so that no third CTA of 256 TMEM columns can be resident and wait for columns that
+  // CTAs of waiting clusters hold.
+  int smem = kFixedSmem + parts + p.stages * p.stage_bytes;
+  if (smem < kMaxSmem / 3 + 1024) smem = kMaxSmem / 3 + 1024;
+  p.tmem_cols = pl.row_blocks * p.tokens + kScaleCols <= 256 ? 256 : 512;
+  CUtensorMap tma, tmw;
+  bro_status rc = gemm::make_codes_map(&tma, acodes, M, K, a_rows);
+  if (rc != BRO_OK) return rc;
+  rc = gemm::make_codes_map(&tmw, wcodes, N, K, kRowsW * pl.row_blocks);
+  if (rc != BRO_OK) return rc;
+  int fit = 0;
+  rc = resident_clusters(p.split, sm_count, &fit);      // (also the opt-in to large shared memory)
+  if (rc != BRO_OK) return rc;
+  const unsigned grid = (unsigned)(pl.tiles_m * pl.tiles_n * p.split);
+  auto kernel = pl.row_blocks == 2 ? gemm_mxfp4_splitk_kernel<2> : gemm_mxfp4_splitk_kernel<1>;
+  return cuda_ok(launch_kernel(kernel, grid, kThreads, (size_t)smem, st, (unsigned)p.split, tma, tmw, p),
+                 "gemm_mxfp4 split-K launch")
+             ? BRO_OK
+             : BRO_ERR_CUDA;
+}
+
+}  // namespace gemms
+}  // namespace bro
