@@ -181,10 +181,10 @@ __global__ void __launch_bounds__(256) swiglu_kernel(const uint16_t* gate, const
 }
 
 // ---- rotate + quantise ---------------------------------------------------------------------------
-bro_status launch_rotate_quantize(const void* x, int64_t M, int64_t K, int64_t ldx, int block,
-                                  const void* signs, void* codes, void* scales, bro_layout layout,
-                                  uint32_t flags, cudaStream_t st, const void* up = nullptr, int64_t ldu = 0) {
-  // (up != nullptr: x is the gate of the fused producer, the rotated tensor is silu(x) * up)
+// Arguments of a rotate+quantize launch; BRO_OK with M == 0 means that there is nothing to do.
+// (up != nullptr: x is the gate of the fused producer, the rotated tensor is silu(x) * up)
+bro_status check_rotate_quantize(const void* x, int64_t M, int64_t K, int64_t ldx, int block, const void* signs,
+                                 const void* codes, const void* scales, bro_layout layout, const void* up, int64_t ldu) {
   if (up && (ldu < K || ldu % 8 != 0)) return ldu < K ? BRO_ERR_SHAPE : BRO_ERR_ALIGN;
   if (up && !aligned(up, 16)) return BRO_ERR_ALIGN;
   if (up && block == 0) return BRO_ERR_UNSUPPORTED;
@@ -200,9 +200,18 @@ bro_status launch_rotate_quantize(const void* x, int64_t M, int64_t K, int64_t l
   if (block == 0 && (!is_pow2(K) || K < 32 || K > 32768)) return BRO_ERR_UNSUPPORTED;
   if (ldx % 8 != 0 || !aligned(x, 16) || !aligned(codes, 16) || !aligned(scales, 16) || !aligned(signs, 16))
     return BRO_ERR_ALIGN;
+  return BRO_OK;
+}
+
+bro_status launch_rotate_quantize(const void* x, int64_t M, int64_t K, int64_t ldx, int block,
+                                  const void* signs, void* codes, void* scales, bro_layout layout,
+                                  uint32_t flags, cudaStream_t st, const void* up = nullptr, int64_t ldu = 0) {
+  bro_status rc = check_rotate_quantize(x, M, K, ldx, block, signs, codes, scales, layout, up, ldu);
+  if (rc != BRO_OK) return rc;
+  const int64_t B = block == 0 ? K : block;
   if (M == 0) return BRO_OK;
   DeviceInfo di;
-  bro_status rc = device_info(&di);
+  rc = device_info(&di);
   if (rc != BRO_OK) return rc;
 
   if (B > 128) {
@@ -587,9 +596,9 @@ bro_status bro_pack_weights(const void* w_bf16, int64_t N, int64_t K, int64_t ld
                                 static_cast<cudaStream_t>(stream));
 }
 
-static bro_status gemm_impl(const void* acodes, const void* ascales, const void* wcodes, const void* wscales,
-                            int64_t M, int64_t N, int64_t K, void* y, int64_t ldy, bro_out_dtype out_dtype,
-                            void* workspace, size_t workspace_bytes, uint32_t flags, void* stream, bool w_static) {
+static bro_status check_gemm(const void* acodes, const void* ascales, const void* wcodes, const void* wscales, int64_t M,
+                             int64_t N, int64_t K, const void* y, int64_t ldy, bro_out_dtype out_dtype, const void* workspace,
+                             size_t workspace_bytes) {
   if (M < 0 || N < 0 || K <= 0 || K % kGroup != 0 || ldy < N) return BRO_ERR_SHAPE;
   if (M > (int64_t)1 << 30 || N > (int64_t)1 << 30 || K > (int64_t)1 << 30) return BRO_ERR_SHAPE;
   if (out_dtype != BRO_OUT_BF16 && out_dtype != BRO_OUT_F32) return BRO_ERR_SHAPE;
@@ -601,19 +610,26 @@ static bro_status gemm_impl(const void* acodes, const void* ascales, const void*
     return BRO_ERR_ALIGN;
   const size_t need = bro_gemm_workspace_bytes(M, N, K);
   if (need > 0 && (!workspace || workspace_bytes < need)) return BRO_ERR_WORKSPACE;
-  if (M == 0 || N == 0) return BRO_OK;
+  return BRO_OK;
+}
+
+static bro_status gemm_impl(const void* acodes, const void* ascales, const void* wcodes, const void* wscales,
+                            int64_t M, int64_t N, int64_t K, void* y, int64_t ldy, bro_out_dtype out_dtype,
+                            void* workspace, size_t workspace_bytes, uint32_t flags, void* stream, bool w_static) {
+  bro_status rc = check_gemm(acodes, ascales, wcodes, wscales, M, N, K, y, ldy, out_dtype, workspace, workspace_bytes);
+  if (rc != BRO_OK || M == 0 || N == 0) return rc;
   DeviceInfo di;
-  bro_status rc = device_info(&di);
+  rc = device_info(&di);
   if (rc != BRO_OK) return rc;
   // Three kernels.  Problems whose 128-row tiles of W fit the chip in one wave (decoding; a few hundred tokens through a
   // narrow layer) go to the split-K kernel, see its plan().
   if (!(flags & (BRO_FLAG_GEMM_PAIR | BRO_FLAG_GEMM_SINGLE | BRO_FLAG_GEMM_TILE_N128 | BRO_FLAG_GEMM_TILE_N256 |
                  BRO_FLAG_GEMM_NO_SPLIT))) {
     bro::gemms::Plan plan;
-    rc = bro::gemms::plan(M, N, (int)ceil_div(K, 256), di.sm_count, &plan);
+    rc = bro::gemms::plan(M, N, (int)ceil_div(K, 256), false, di.sm_count, &plan);
     if (rc != BRO_OK) return rc;
     if (plan.row_blocks > 0)
-      return bro::gemms::launch(plan, acodes, ascales, wcodes, wscales, M, N, K, y, ldy, (int)out_dtype, di.sm_count,
+      return bro::gemms::launch(plan, nullptr, acodes, ascales, wcodes, wscales, M, N, K, y, ldy, (int)out_dtype, di.sm_count,
                                 static_cast<cudaStream_t>(stream), w_static);
   }
   // Else the two-CTA kernel (256 x 256 tiles, cta_group::2) moves a third fewer bytes into
@@ -659,8 +675,26 @@ static bro_status linear_impl(const void* x_bf16, int64_t M, int64_t K, int64_t 
   uint8_t* acodes = ws;
   uint8_t* ascales = acodes + align_up(bro_codes_bytes(M, K), 1024);
   uint8_t* gws = ascales + align_up(bro_scales_bytes(M, K, BRO_LAYOUT_GEMM), 1024);
-  bro_status rc = launch_rotate_quantize(x_bf16, M, K, ldx, block, signs, acodes, ascales, BRO_LAYOUT_GEMM, flags,
-                                         static_cast<cudaStream_t>(stream));
+  bro_status rc;
+  if (flags == 0 && block != 0) {        // few tokens: one kernel for both steps, where its plan says so
+    rc = check_rotate_quantize(x_bf16, M, K, ldx, block, signs, acodes, ascales, BRO_LAYOUT_GEMM, nullptr, 0);
+    if (rc == BRO_OK)
+      rc = check_gemm(acodes, ascales, wcodes, wscales, M, N, K, y_bf16, ldy, BRO_OUT_BF16, gws, bro_gemm_workspace_bytes(M, N, K));
+    if (rc != BRO_OK) return rc;
+    DeviceInfo di;
+    rc = device_info(&di);
+    if (rc != BRO_OK) return rc;
+    bro::gemms::Plan plan;
+    rc = bro::gemms::plan(M, N, (int)ceil_div(K, 256), true, di.sm_count, &plan);
+    if (rc != BRO_OK) return rc;
+    if (plan.row_blocks > 0) {
+      const bro::gemms::Source src = {x_bf16, ldx, signs, log2_of(block)};
+      return bro::gemms::launch(plan, &src, acodes, ascales, wcodes, wscales, M, N, K, y_bf16, ldy, BRO_OUT_BF16, di.sm_count,
+                                static_cast<cudaStream_t>(stream), true);
+    }
+  }
+  rc = launch_rotate_quantize(x_bf16, M, K, ldx, block, signs, acodes, ascales, BRO_LAYOUT_GEMM, flags,
+                              static_cast<cudaStream_t>(stream));
   if (rc != BRO_OK) return rc;
   // The packed weights are older than the rotate+quantize kernel just enqueued, which signals its
   // dependents only after its own wait: the GEMM may fetch its first weight tiles early.

@@ -9,7 +9,12 @@
 //   * the `split` CTAs of a cluster share a tile, each takes a contiguous range of its 256-element K steps
 //     and sends its fp32 partial sums to the CTAs that own the tokens (distributed shared memory); a token's
 //     owner adds the parts in rank order, converts and stores.  No workspace, no atomics, fixed order.
-//   * with W packed before the previous kernel in the stream started (the whole-layer calls), the whole ring of
+//   * FUSED (the whole-layer calls with few tokens): there is no rotate+quantize kernel in front.  Sixteen warps, eight
+//     of them those of the epilogue, rotate and quantise the [tokens, 256] slice of x of every K step straight into the
+//     stage (a lane owns one MX group, the arithmetic is that of the stand-alone kernel, bit for bit) and arrive on
+//     its barrier beside the weight bytes.  Every CTA repeats the work on its K range, hidden behind the weights; the
+//     first tile of columns also leaves codes and scales in the caller's workspace, as the stand-alone kernel would.
+//   * otherwise, with W packed before the previous kernel in the stream started (the whole-layer calls), the whole ring of
 //     weight tiles is requested before griddepcontrol.wait, under the rotate+quantize kernel.
 // Warps: 0 TMA producer, 1 TMEM owner and MMA issuer, 2..9 epilogue.  Every mbarrier wait is bounded, and all
 // threads of a cluster reach both cluster barriers whatever happened before.
@@ -17,12 +22,14 @@
 
 #include "gemm_mxfp4.cuh"
 #include "gemm_mxfp4_2cta.cuh"
+#include "rotate_quantize.cuh"
 
 namespace bro {
 namespace gemms {
 
 constexpr int kEpilogueWarps = 8;                // two per TMEM lane quadrant
-constexpr int kThreads = (2 + kEpilogueWarps) * 32;
+constexpr int kQuantWarps = 16;                  // FUSED: the epilogue warps and as many more rotate and quantise
+constexpr int kThreads = (2 + kEpilogueWarps) * 32, kThreadsFused = (2 + kQuantWarps) * 32;
 constexpr int kRowsW = 128;                      // rows of W per MMA
 constexpr int kMaxTokens = 128;                  // tokens per tile
 constexpr int kWTileBytes = kRowsW * 128;        // 16 KiB: one 256-element K step of 128 rows
@@ -50,6 +57,16 @@ struct Params {
   int tmem_cols;            // 256 or 512
   int out_f32;
   int w_static;             // the weight operand was complete before the previous kernel started
+  // FUSED: x in place of packed activations
+  const uint16_t* x;        // [M, K] bf16, row stride ldx
+  int64_t ldx;
+  const uint16_t* signs;    // [K] bf16 +-1 or nullptr
+  uint8_t* codes;           // the workspace copy of codes and scales
+  uint8_t* scales;
+  int groups_k;             // K / 32
+  int log2b;                // rotation size 2^1 .. 2^7
+  uint32_t cbits;           // fp32 bits of 2^(-log2b / 2)
+  int token_quads;          // ceil(M / 4): warp tasks per K step
 };
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
@@ -75,8 +92,42 @@ __device__ __forceinline__ void store_bf16_pair(void* y, int64_t at, int64_t ldy
   if (second) static_cast<uint16_t*>(y)[at + ldy] = (uint16_t)(h >> 16);
 }
 
-template <int ROW_BLOCKS>
-__global__ void __launch_bounds__(kThreads, 1)
+// L2 prefetch of what a bulk load would bring: no value is read, so it may run while an older kernel still writes there.
+__device__ __forceinline__ void l2_prefetch_2d_elect(const CUtensorMap* m, int x, int y) {
+  asm volatile(
+      "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
+      "@q cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}]; }" ::"l"(reinterpret_cast<uint64_t>(m)),
+      "r"(x), "r"(y)
+      : "memory");
+}
+
+// Rotation of size 2^log2b (a run-time value) and quantisation of one MX group per lane; groups of a block sit in
+// neighbouring lanes.  Same operations in the same order as the stand-alone kernel's.
+__device__ __forceinline__ uint32_t rotate_quantize_lane(const uint4 (&v)[4], int log2b, uint32_t cbits, int lane, uint32_t (&w)[4]) {
+  uint64_t P[16];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) rq::unpack_stage1(v[j], P + 4 * j);
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    if (log2b >= s + 2) {
+      const int hp = 1 << s;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        if ((k & hp) == 0) {
+          const uint64_t a = P[k], b = P[k + hp];
+          P[k] = rq::add2(a, b);
+          P[k + hp] = rq::sub2(a, b);
+        }
+      }
+    }
+  }
+  if (log2b >= 6) rq::cross_lane_stage(P, 1, (lane & 1) != 0);
+  if (log2b >= 7) rq::cross_lane_stage(P, 2, (lane & 2) != 0);
+  return rq::quantize_group(P, cbits, w);
+}
+
+template <int ROW_BLOCKS, bool FUSED>
+__global__ void __launch_bounds__(FUSED ? kThreadsFused : kThreads, 1)
 gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_constant__ CUtensorMap tmw, const Params p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -101,7 +152,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
-      mbar_init(bar_full + 8 * s, 1);
+      mbar_init(bar_full + 8 * s, FUSED ? 1u + kQuantWarps : 1u);
       mbar_init(bar_empty + 8 * s, 1);
     }
     mbar_init(bar_acc, 1);
@@ -121,7 +172,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
   gemm::tc_fence_after();
   if (p.split > 1) cluster_arrive();          // (waited for before the first write to another CTA)
   griddep_launch_dependents();
-  const bool early_w = p.w_static != 0 && warp == 0;
+  const bool early_w = (FUSED || p.w_static != 0) && warp == 0;
   if (!early_w) griddep_wait();
   const uint32_t tmem_base = __shfl_sync(0xFFFFFFFFu, *tmem_slot_ptr, 0);
   const uint32_t tmem_sfw = tmem_base + (uint32_t)p.tmem_cols - kScaleCols;
@@ -136,19 +187,23 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
       const uint32_t full = bar_full + 8 * st, base = smem_base + (uint32_t)(st * p.stage_bytes);
       const int ks = k_first + i;
       if (part & 1) {
-        mbar_arrive_expect_tx_elect(full, w_bytes + (uint32_t)p.a_box_bytes + (uint32_t)(blocks + 1) * kScaleBytes);
+        mbar_arrive_expect_tx_elect(full, w_bytes + (uint32_t)blocks * kScaleBytes + (FUSED ? 0u : (uint32_t)p.a_box_bytes + kScaleBytes));
         tma_load_2d_elect(base, &tmw, ks * 128, n0, full);                               // (rows beyond N arrive as zeros)
         const uint8_t* src = p.wscales + ((int64_t)(n0 / kRowsW) * p.kblocks + 2 * ks) * 512;
         bulk_load_1d_elect(base + off_sfw, src, kScaleBytes, full);
         if (blocks == 2) bulk_load_1d_elect(base + off_sfw + kScaleBytes, src + p.kblocks * 512, kScaleBytes, full);
       }
-      if (part & 2) {
+      if (!FUSED && (part & 2)) {
         tma_load_2d_elect(base + w_bytes, &tma, ks * 128, m0, full);
         bulk_load_1d_elect(base + off_sfa, p.ascales + ((int64_t)tm * p.kblocks + 2 * ks) * 512, kScaleBytes, full);
       }
     };
     int i = 0;
-    if (early_w) {
+    if (FUSED) {
+      // the weights may be what the kernel before is still writing: before the wait they are only drawn into L2
+      for (int s = 0; s < min(k_count, p.stages); ++s) l2_prefetch_2d_elect(&tmw, (k_first + s) * 128, n0);
+      griddep_wait();
+    } else if (early_w) {
       const int pre = min(k_count, p.stages);
       for (int s = 0; s < pre; ++s) issue_step(s, s, 1);       // weights: before the wait
       griddep_wait();
@@ -212,8 +267,80 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
   const int q = warp & 3, half = (warp - 2) >> 2;
   const uint32_t tmem_acc = tmem_base + ((uint32_t)(q * 32) << 16);
   bool ok = true;
-  if (warp >= 2) {
-    ok = mbar_wait_warp(bar_acc, 0u, SITE_GEMM_ACC_FULL);
+  if (FUSED && warp >= 2) {
+    // ------------------------------ rotate + quantise x ------------------------------
+    // One warp task: 4 tokens x the 8 groups of a K step, one group per lane; task t goes to warp t mod 16.
+    const int in_quad = lane >> 3, g = lane & 7;
+    auto load = [&](int step, int quad, uint4 (&v)[4]) {
+      const int token = quad * 4 + in_quad, group = (k_first + step) * 8 + g;
+      const bool in = token < live && group < p.groups_k;
+      const uint4* src = reinterpret_cast<const uint4*>(p.x + (int64_t)(in ? token : 0) * p.ldx + (int64_t)(in ? group : 0) * 32);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = in ? __ldg(src + j) : make_uint4(0u, 0u, 0u, 0u);     // padding quantises to zeros
+      if (p.signs && in) {
+        const uint4* sp = reinterpret_cast<const uint4*>(p.signs + (int64_t)group * 32);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = rq::apply_signs(v[j], __ldg(sp + j));
+      }
+    };
+    auto advance = [&](int& step, int& quad) {
+      quad += kQuantWarps;
+      while (quad >= p.token_quads) { quad -= p.token_quads; ++step; }
+    };
+    int step = 0, quad = warp - 2 - kQuantWarps;      // this warp's next task
+    advance(step, quad);
+    uint4 cur[4];
+    if (step < k_count) load(step, quad, cur);
+    // Every warp arrives for every step, with or without a task in it: a warp that skipped steps could find the ring two
+    // rounds away from what it saw last, and a parity tells a phase from its neighbours only.
+    int stage = 0;
+    uint32_t phase = 1u;                                 // (parity of the phase before the first: passes at once)
+    for (int i = 0; i < k_count; ++i) {
+      const uint32_t base = smem_base + (uint32_t)(stage * p.stage_bytes);
+      bool waited = false;
+      do {
+        const bool has = step == i;
+        const int row = quad * 4 + in_quad;
+        uint32_t w[4], sb = 0u;
+        if (has) {
+          sb = rotate_quantize_lane(cur, p.log2b, p.cbits, lane, w);
+          advance(step, quad);
+          if (step < k_count) load(step, quad, cur);     // in flight while this task's stage is waited for and written
+          // scale bytes of 4 consecutive groups -> one 32-bit word in the lane with g % 4 == 0
+          sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 1) << 8;
+          sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 2) << 16;
+        }
+        if (!waited) ok = mbar_wait_warp(bar_empty + 8 * stage, phase, SITE_GEMM_EMPTY);
+        waited = true;
+        if (!has || !ok) break;
+        const uint32_t sf_at = (uint32_t)((g >> 2) * 512 + (row & 31) * 16 + (row >> 5) * 4);
+        gemm::sts128(base + w_bytes + (uint32_t)row * 128u + (uint32_t)((g ^ (row & 7)) << 4), w[0], w[1], w[2], w[3]);
+        if ((g & 3) == 0) asm volatile("st.shared.b32 [%0], %1;" ::"r"(base + off_sfa + sf_at), "r"(sb) : "memory");
+        if (tn == 0) {
+          const int group = (k_first + i) * 8 + g;
+          if (row < live && group < p.groups_k)
+            *reinterpret_cast<uint4*>(p.codes + ((int64_t)row * p.groups_k + group) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+          if ((g & 3) == 0) *reinterpret_cast<uint32_t*>(p.scales + (int64_t)(k_first + i) * 1024 + sf_at) = sb;
+        }
+      } while (step == i);
+      if (!ok) break;
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_full + 8 * stage);
+      if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+    }
+    if (tn == 0) {                            // the rows that pad the scale buffer to 128 read as zero
+      const int first = p.token_quads * 4;
+      for (int j = (int)threadIdx.x - 64; j < k_count * 2 * kRowsW; j += kQuantWarps * 32) {
+        const int row = j & (kRowsW - 1);
+        if (row >= first)
+          *reinterpret_cast<uint32_t*>(p.scales + ((int64_t)k_first * 2 + j / kRowsW) * 512 + (row & 31) * 16 + (row >> 5) * 4) = 0u;
+      }
+    }
+  }
+  const bool epilogue = warp >= 2 && warp < 2 + kEpilogueWarps;
+  if (epilogue) {
+    ok = mbar_wait_warp(bar_acc, 0u, SITE_GEMM_ACC_FULL) && ok;
     gemm::tc_fence_after();
   }
   auto store4 = [&](int64_t at, const uint32_t (&v)[4], int exist) {        // 4 tokens of one column
@@ -227,7 +354,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
     }
   };
   if (p.split == 1) {
-    if (warp >= 2 && ok) {
+    if (epilogue && ok) {
       const int b = ROW_BLOCKS == 2 ? half : 0;
       const int64_t n = (int64_t)n0 + b * kRowsW + q * 32 + lane;
       for (int c = ROW_BLOCKS == 2 ? 0 : half * 16; c < live; c += ROW_BLOCKS == 2 ? 16 : 32) {
@@ -247,7 +374,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
     // (16-byte stores straight into the owners' shared memory; staged locally and sent as bulk copies, 128 tokens took
     // 2 us longer)
     cluster_wait();                           // every CTA of the cluster runs
-    if (warp >= 2 && ok) {
+    if (epilogue && ok) {
       for (int c = half * 16; c < live; c += 32) {
         uint32_t r[16];
         tc_ld16(tmem_acc + (uint32_t)c, r);
@@ -265,7 +392,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
     __syncwarp();
     cluster_arrive();
     cluster_wait();                           // all parts have arrived; nobody writes here any more
-    if (warp >= 2 && ok) {
+    if (epilogue && ok) {
       const int row = q * 32 + lane;
       const int64_t n = (int64_t)n0 + row;
       for (int s = half; s < p.groups; s += 2) {
@@ -294,11 +421,12 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
 inline bro_status resident_clusters(int split, int sm_count, int* out) {
   static DeviceOnce attr, once[kMaxSplit + 1];
   bro_status rc = device_once(attr, nullptr, [&](int*) {
-    const bool ok = cuda_ok(cudaFuncSetAttribute(gemm_mxfp4_splitk_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem),
-                            "cudaFuncSetAttribute(gemm split-K)") &&
-                    cuda_ok(cudaFuncSetAttribute(gemm_mxfp4_splitk_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem),
-                            "cudaFuncSetAttribute(gemm split-K)");
-    return ok ? BRO_OK : BRO_ERR_CUDA;
+    for (auto kernel : {gemm_mxfp4_splitk_kernel<1, false>, gemm_mxfp4_splitk_kernel<2, false>, gemm_mxfp4_splitk_kernel<1, true>,
+                        gemm_mxfp4_splitk_kernel<2, true>})
+      if (!cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem),
+                   "cudaFuncSetAttribute(gemm split-K)"))
+        return BRO_ERR_CUDA;
+    return BRO_OK;
   });
   if (rc != BRO_OK) return rc;
   if (split == 1) { *out = sm_count; return BRO_OK; }
@@ -315,7 +443,7 @@ inline bro_status resident_clusters(int split, int sm_count, int* out) {
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (!cuda_ok(cudaOccupancyMaxActiveClusters(n, gemm_mxfp4_splitk_kernel<1>, &cfg), "occupancy(gemm split-K)"))
+    if (!cuda_ok(cudaOccupancyMaxActiveClusters(n, gemm_mxfp4_splitk_kernel<1, false>, &cfg), "occupancy(gemm split-K)"))
       return BRO_ERR_CUDA;
     ++*n;
     return BRO_OK;
@@ -335,44 +463,89 @@ struct Plan {
   int row_blocks = 0, tiles_m = 0, tiles_n = 0, split = 0;     // row_blocks = 0: not a problem for this kernel
 };
 
+// Nanoseconds, as measured: one K step of a CTA that does not wait for HBM, the exchange of parts inside a cluster, the
+// warp tasks (4 tokens of one K step each) of the quantising warps.
+inline int64_t step_ns(int tokens) { return 90 + tokens; }
+inline int64_t exchange_ns(int tokens) { return tokens <= 64 ? 100 + 18 * tokens : 4500; }
+inline int64_t quantise_ns(int64_t tasks) { return 300 + 72 * tasks; }
+
+// K parts of a tile: among the cluster sizes whose clusters are all resident at once, the one of least cost.
+template <typename Cost>
+inline bro_status best_split(int64_t tiles, int num_k_steps, int sm_count, Cost&& cost, int* split, int64_t* ns) {
+  *split = 1;
+  *ns = cost(num_k_steps, 1);
+  int best = num_k_steps;
+  for (int s = 2; s <= kMaxSplit && s <= num_k_steps; ++s) {
+    const int steps = (num_k_steps + s - 1) / s;
+    if (steps >= best || cost(steps, s) >= *ns || tiles * s > sm_count) continue;
+    int fit = 0;
+    const bro_status rc = resident_clusters(s, sm_count, &fit);
+    if (rc != BRO_OK) return rc;
+    if (tiles > fit) continue;
+    best = steps;
+    *split = s;
+    *ns = cost(steps, s);
+  }
+  return BRO_OK;
+}
+
 // One wave of whole tiles, or none of this.  128-row tiles when they fit the chip at once; else, decoding at most 64
 // tokens through a wider layer, 256-row tiles (K = 8192, N = 28672: 1 token 23.5 -> 21.3 us, 64 tokens 24.8 -> 23.3 us
 // against the persistent kernel; 96 tokens no gain, 128 tokens 2 % slower).  Several token tiles need 8 K steps:
 // (512, 14336, 4096) 21.7 -> 15.6 us and (512, 2048, 2048) even, but (640, 1024, 3000) 4.1 -> 4.3 us.
-// Parts: among the cluster sizes whose clusters are all resident, the fewest K steps per CTA.  The exchange between the
-// CTAs costs about 0.5 us with 16 tokens, 1.3 us with 64 and 4.5 us with 128, a K step 0.1 to 0.2 us, hence the line at
-// 4 + tokens / 5 saved steps.  (16, 14336, 4096): 1 part 10.5 us, 2 parts 7.3, 4 parts 6.3, persistent kernel 20.1;
-// (64, 2048, 2048): 1 part 3.7 us, 2 parts 4.3; (128, 14336, 4096): 1 part 14.5 us, 4 parts 10.9, persistent 20.8.
-inline bro_status plan(int64_t M, int64_t N, int num_k_steps, int sm_count, Plan* out) {
+// Parts, by the costs above: (16, 14336, 4096) 1 part 10.5 us, 2 parts 7.3, 4 parts 6.3, persistent kernel 20.1;
+// (64, 2048, 2048) 1 part 3.7 us, 2 parts 4.3; (128, 14336, 4096) 1 part 14.5 us, 4 parts 10.9, persistent 20.8.
+//
+// fused = true asks for a plan that quantises inside the GEMM.  It saves the other kernel (2 us on the device, 4 us of
+// the host's time to launch it) and costs the tasks of the quantising warps, of which about half the time that the
+// weights take from HBM hides; the line is at 2.9 us for the rest.  Whole layer in a graph, two kernels -> fused:
+// (1, 8192, 28672) 23.2 -> 21.3 us, (16, 8192, 28672) 24.2 -> 23.3, (3, 1024, 1024) 4.3 -> 3.4, (16, 2048, 2048)
+// 4.9 -> 4.0, (16, 4096, 4096) even, (64, 2048, 2048) 5.9 -> 6.5 and (24, 5120, 5120) 6.4 -> 7.8, where calls that are
+// launched one by one are bound by the host and still gain its 4 us; beyond the line (32, 8192, 28672) 24.8 -> 29.5,
+// (128, 2048, 2048) 6.6 -> 10.3.
+inline bro_status plan(int64_t M, int64_t N, int num_k_steps, bool fused, int sm_count, Plan* out) {
   const int64_t tiles_m = (M + kMaxTokens - 1) / kMaxTokens, n128 = (N + kRowsW - 1) / kRowsW;
   const int tokens = token_columns(M);
+  const int64_t quads = (M + 3) / 4;
   Plan pl;
-  if (tiles_m * n128 <= sm_count && (tiles_m == 1 || num_k_steps >= 8)) {
-    pl.row_blocks = 1;
-    pl.tiles_n = (int)n128;
-    pl.split = 1;
-    int best = num_k_steps;
-    for (int s = 2; s <= kMaxSplit && s <= num_k_steps; ++s) {
-      const int steps = (num_k_steps + s - 1) / s;
-      if (steps >= best || num_k_steps - steps <= 4 + tokens / 5 || tiles_m * n128 * s > sm_count) continue;
-      int fit = 0;
-      const bro_status rc = resident_clusters(s, sm_count, &fit);
-      if (rc != BRO_OK) return rc;
-      if (tiles_m * n128 > fit) continue;
-      best = steps;
-      pl.split = s;
-    }
-  } else if (tokens <= 64 && (n128 + 1) / 2 <= sm_count) {
-    pl.row_blocks = 2;
-    pl.tiles_n = (int)((n128 + 1) / 2);
-    pl.split = 1;
-  }
   pl.tiles_m = (int)tiles_m;
+  *out = Plan();
+  const bool narrow = tiles_m * n128 <= sm_count;
+  if (narrow ? !(tiles_m == 1 || num_k_steps >= 8) : !(tokens <= 64 && (n128 + 1) / 2 <= sm_count)) return BRO_OK;
+  pl.row_blocks = narrow ? 1 : 2;
+  pl.tiles_n = (int)(narrow ? n128 : (n128 + 1) / 2);
+  pl.split = 1;
+  const auto two_kernels = [&](int steps, int s) { return steps * step_ns(tokens) + (s > 1 ? exchange_ns(tokens) : 0); };
+  const auto one_kernel = [&](int steps, int s) { return quantise_ns(steps * quads) + (s > 1 ? exchange_ns(tokens) : 0); };
+  int64_t ns = two_kernels(num_k_steps, 1), fused_ns = one_kernel(num_k_steps, 1);
+  if (narrow) {
+    const bro_status rc = best_split(tiles_m * n128, num_k_steps, sm_count, two_kernels, &pl.split, &ns);
+    if (rc != BRO_OK) return rc;
+  }
+  if (fused) {
+    if (tiles_m > 1) return BRO_OK;
+    const int64_t hidden = (int64_t)((double)N * num_k_steps * 256 * (17.0 / 32) / 6200) / 2;      // half the weights' time
+    const int64_t beside = (pl.split > 1 ? exchange_ns(tokens) : 0) + hidden;
+    if (narrow) {
+      const bro_status rc = best_split(n128, num_k_steps, sm_count, one_kernel, &pl.split, &fused_ns);
+      if (rc != BRO_OK) return rc;
+    }
+    if (fused_ns - (beside > ns ? beside : ns) > 2900) return BRO_OK;
+  }
   *out = pl;
   return BRO_OK;
 }
 
-inline bro_status launch(const Plan& pl, const void* acodes, const void* ascales, const void* wcodes, const void* wscales,
+// What FUSED reads in place of packed activations.
+struct Source {
+  const void* x;
+  int64_t ldx;
+  const void* signs;
+  int log2b;
+};
+
+// `src` set: the fused kernel; acodes / ascales then receive the workspace copy.
+inline bro_status launch(const Plan& pl, const Source* src, const void* acodes, const void* ascales, const void* wcodes, const void* wscales,
                          int64_t M, int64_t N, int64_t K, void* y, int64_t ldy, int out_dtype, int sm_count, cudaStream_t st,
                          bool w_static) {
   Params p;
@@ -406,17 +579,38 @@ inline bro_status launch(const Plan& pl, const void* acodes, const void* ascales
   int smem = kFixedSmem + parts + p.stages * p.stage_bytes;
   if (smem < kMaxSmem / 3 + 1024) smem = kMaxSmem / 3 + 1024;
   p.tmem_cols = pl.row_blocks * p.tokens + kScaleCols <= 256 ? 256 : 512;
+  p.groups_k = (int)(K / 32);
+  p.token_quads = (int)((M + 3) / 4);
+  p.x = nullptr;
+  p.ldx = 0;
+  p.signs = nullptr;
+  p.codes = p.scales = nullptr;
+  p.log2b = 0;
+  p.cbits = 0;
   CUtensorMap tma, tmw;
-  bro_status rc = gemm::make_codes_map(&tma, acodes, M, K, a_rows);
-  if (rc != BRO_OK) return rc;
+  bro_status rc = BRO_OK;
+  if (src) {
+    p.x = static_cast<const uint16_t*>(src->x);
+    p.ldx = src->ldx;
+    p.signs = static_cast<const uint16_t*>(src->signs);
+    p.codes = static_cast<uint8_t*>(const_cast<void*>(acodes));
+    p.scales = static_cast<uint8_t*>(const_cast<void*>(ascales));
+    p.log2b = src->log2b;
+    p.cbits = (src->log2b % 2 == 0) ? (uint32_t)(127 - src->log2b / 2) << 23 : 0x3FB504F3u - ((uint32_t)((src->log2b + 1) / 2) << 23);
+  } else {
+    rc = gemm::make_codes_map(&tma, acodes, M, K, a_rows);
+    if (rc != BRO_OK) return rc;
+  }
   rc = gemm::make_codes_map(&tmw, wcodes, N, K, kRowsW * pl.row_blocks);
   if (rc != BRO_OK) return rc;
+  if (src) tma = tmw;            // (not used by the fused kernel)
   int fit = 0;
   rc = resident_clusters(p.split, sm_count, &fit);      // (also the opt-in to large shared memory)
   if (rc != BRO_OK) return rc;
   const unsigned grid = (unsigned)(pl.tiles_m * pl.tiles_n * p.split);
-  auto kernel = pl.row_blocks == 2 ? gemm_mxfp4_splitk_kernel<2> : gemm_mxfp4_splitk_kernel<1>;
-  return cuda_ok(launch_kernel(kernel, grid, kThreads, (size_t)smem, st, (unsigned)p.split, tma, tmw, p),
+  auto kernel = src ? (pl.row_blocks == 2 ? gemm_mxfp4_splitk_kernel<2, true> : gemm_mxfp4_splitk_kernel<1, true>)
+                    : (pl.row_blocks == 2 ? gemm_mxfp4_splitk_kernel<2, false> : gemm_mxfp4_splitk_kernel<1, false>);
+  return cuda_ok(launch_kernel(kernel, grid, src ? kThreadsFused : kThreads, (size_t)smem, st, (unsigned)p.split, tma, tmw, p),
                  "gemm_mxfp4 split-K launch")
              ? BRO_OK
              : BRO_ERR_CUDA;

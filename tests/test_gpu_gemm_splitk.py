@@ -50,3 +50,45 @@ def test_splitk_same_result_as_persistent_kernel(bro, M, K, N):
     assert torch.equal(out[0], out[1])            # parts are added in rank order: run after run the same bits
     top = out[2].abs().amax(1, keepdim=True)
     assert ((out[0] - out[2]).abs() <= top * 2.0 ** -20).all()
+
+
+@pytest.mark.parametrize("M,K,N,block", [
+    (1, 8192, 19000, 32),     # 256-row tiles: a ring of 6 stages, 32 steps, one task a step
+    (2, 4096, 1000, 64),      # clusters, rotation across lanes
+    (5, 4128, 264, 32),       # K not a multiple of 256: half of the last step is padding
+    (16, 2176, 136, 128),
+    (31, 1024, 392, 2),       # rotations inside the group
+    (64, 512, 264, 16),
+    (128, 1024, 200, 32),
+])
+@pytest.mark.parametrize("signs", [False, True])
+def test_layer_of_few_tokens_same_bytes_as_two_kernels(bro, M, K, N, block, signs):
+    """bro.linear with few tokens quantises inside the GEMM: codes and scales left in the workspace (padding
+    included) are those of rotate_quantize_mxfp4, the output is that of gemm_mxfp4 up to the order of fp32 sums
+    (bf16: one ulp, 2^-8 of the row's largest magnitude at most)."""
+    gen = torch.Generator(device="cuda").manual_seed(M + K)
+    x = torch.randn(M, K + 8, generator=gen, device="cuda").to(torch.bfloat16)[:, :K]
+    w = torch.randn(N, K, generator=gen, device="cuda").to(torch.bfloat16)
+    s = (1 - 2 * torch.randint(0, 2, (K,), generator=gen, device="cuda")).to(torch.bfloat16) if signs else None
+    wc, wsc = bro.alloc_codes(N, K), bro.alloc_scales(N, K, bro.LAYOUT_GEMM)
+    bro.pack_weights_rs(w, block, s, wc, wsc) if signs else bro.pack_weights(w, block, wc, wsc)
+    nbytes = bro.linear_workspace_bytes(M, N, K)
+    ws = Guarded(nbytes + 1024, fill=0x7F)
+    off = (-ws.view.data_ptr()) % 1024
+    work = ws.view[off:off + nbytes]
+    ldy = (N + 7) // 8 * 8
+    out = Guarded(M * ldy * 2, fill=0x7F)
+    y = out.view.view(torch.bfloat16).view(M, ldy)[:, :N]
+    bro.linear_rs(x, block, s, wc, wsc, N, y, work) if signs else bro.linear(x, block, wc, wsc, N, y, work)
+    assert bro.last_device_status() == 0
+    ws.check()
+    out.check()
+    ac, asc = bro.alloc_codes(M, K), bro.alloc_scales(M, K, bro.LAYOUT_GEMM)
+    bro.rotate_quantize_mxfp4(x, block, ac, asc, signs=s)
+    assert torch.equal(work[:ac.numel()], ac.flatten())
+    at = (ac.numel() + 1023) // 1024 * 1024
+    assert torch.equal(work[at:at + asc.numel()], asc)
+    ref = torch.empty(M, N if N % 8 == 0 else ldy, dtype=torch.bfloat16, device="cuda")[:, :N]
+    bro.gemm_mxfp4(ac, asc, wc, wsc, M, N, K, ref, flags=bro.FLAG_GEMM_SINGLE)
+    top = ref.float().abs().amax(1, keepdim=True)
+    assert ((y.float() - ref.float()).abs() <= top * 2.0 ** -8).all()
