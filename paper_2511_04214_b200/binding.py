@@ -154,14 +154,22 @@ def _check(code: int, where: str) -> None:
         raise BroError(code, where)
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
-def _ptr(t) -> ctypes.c_void_p:
-    return ctypes.c_void_p(0 if t is None else t.data_ptr())
+def _stream(stream) -> int:
+    """Handle of ``stream``, or of the current device's current stream.  The current one is read without building
+    the Python object around it: 0.1 us instead of 3.4 us, which was a quarter of a small call."""
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_current_device())
+
+
+def _ptr(t):
+    return None if t is None else t.data_ptr()
 
 
 def codes_bytes(rows: int, K: int) -> int:
