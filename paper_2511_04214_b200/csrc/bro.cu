@@ -511,27 +511,24 @@ bro_status bro_outlier_groups(const void* x_bf16, int64_t M, int64_t K, int64_t 
   if (rc != BRO_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   unsigned long long* hist = static_cast<unsigned long long*>(workspace);
-  if (!bro::cuda_ok(cudaMemsetAsync(hist, 0, (size_t)bro::stats::kMagBins * 8, st), "cudaMemsetAsync(histogram)"))
+  if (!bro::cuda_ok(cudaMemsetAsync(hist, 0, bro::stats::kWorkspaceBytes, st), "cudaMemsetAsync(histogram)"))
     return BRO_ERR_CUDA;
   static bro::DeviceOnce once;
   const int smem = bro::stats::kMagBins * 4;
-  rc = bro::device_once(once, nullptr, [&](int*) { return set_smem(bro::stats::magnitude_histogram, smem); });
+  rc = bro::device_once(once, nullptr, [&](int*) { return set_smem(bro::stats::outlier_scan, smem); });
   if (rc != BRO_OK) return rc;
   const uint16_t* x = static_cast<const uint16_t*>(x_bf16);
-  const unsigned hgrid = bro::stats::grid_for(M * (K / 8), 512, di.sm_count, 1);
-  if (!bro::cuda_ok(bro::launch_kernel(bro::stats::magnitude_histogram, hgrid, 512, (size_t)smem, st, 1, x, M, K, ldx, hist),
-                    "magnitude_histogram launch"))
-    return BRO_ERR_CUDA;
   const unsigned long long n = (unsigned long long)M * (unsigned long long)K;
   unsigned long long k = (n * (unsigned long long)top_ppm + 999999ull) / 1000000ull;
   if (k < 1) k = 1;
-  if (!bro::cuda_ok(bro::launch_kernel(bro::stats::find_threshold, 1u, 1024u, 0, st, 1,
-                                       static_cast<const unsigned long long*>(hist), k, info),
-                    "find_threshold launch"))
+  const unsigned sgrid = bro::stats::grid_for(M * (K / 32), bro::stats::kScanThreads, di.sm_count, 1);
+  if (!bro::cuda_ok(bro::launch_kernel(bro::stats::outlier_scan, sgrid, bro::stats::kScanThreads, (size_t)smem, st, 1, x, M, K, ldx,
+                                       k, hist, info, mask),
+                    "outlier_scan launch"))
     return BRO_ERR_CUDA;
-  const unsigned mgrid = bro::stats::grid_for(M * (K / 32), 256, di.sm_count, 8);
+  const unsigned mgrid = bro::stats::grid_for(M * (K / 32), 256 * 16, di.sm_count, 8);
   return bro::cuda_ok(bro::launch_kernel(bro::stats::outlier_group_mask, mgrid, 256, 0, st, 1, x, M, K, ldx,
-                                         static_cast<const uint32_t*>(info), mask),
+                                         static_cast<const uint32_t*>(info), static_cast<const unsigned long long*>(hist), mask),
                       "outlier_group_mask launch")
              ? BRO_OK
              : BRO_ERR_CUDA;
@@ -547,11 +544,14 @@ bro_status bro_scale_histogram(const uint8_t* scales, const uint8_t* mask, int64
   bro_status rc = device_info(&di);
   if (rc != BRO_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (!bro::cuda_ok(cudaMemsetAsync(hist, 0, 2 * 256 * sizeof(uint64_t), st), "cudaMemsetAsync(scale histogram)"))
+  const bool alone = n_groups > 0 && bro::stats::count_alone(n_groups);
+  if (!alone &&
+      !bro::cuda_ok(cudaMemsetAsync(hist, 0, 2 * 256 * sizeof(uint64_t), st), "cudaMemsetAsync(scale histogram)"))
     return BRO_ERR_CUDA;
   if (n_groups == 0) return BRO_OK;
-  const unsigned grid = bro::stats::grid_for(n_groups, 256 * 16, di.sm_count, 4);
-  return bro::cuda_ok(bro::launch_kernel(bro::stats::scale_histogram, grid, 256, 0, st, 1, scales, mask, n_groups,
+  const unsigned grid = alone ? 1u : bro::stats::grid_for(n_groups, bro::stats::kCountThreads * 16, di.sm_count, 2);
+  return bro::cuda_ok(bro::launch_kernel(bro::stats::scale_histogram, grid, bro::stats::kCountThreads, 0, st, 1, scales, mask, n_groups,
+                                         alone ? 1 : 0,
                                          reinterpret_cast<unsigned long long*>(hist)),
                       "scale_histogram launch")
              ? BRO_OK
@@ -568,12 +568,14 @@ bro_status bro_scale_inflation(const uint8_t* scales_before, const uint8_t* scal
   bro_status rc = device_info(&di);
   if (rc != BRO_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (!bro::cuda_ok(cudaMemsetAsync(counts, 0, 6 * sizeof(uint64_t), st), "cudaMemsetAsync(inflation counts)"))
+  const bool alone = n_groups > 0 && bro::stats::count_alone(n_groups);
+  if (!alone &&
+      !bro::cuda_ok(cudaMemsetAsync(counts, 0, 6 * sizeof(uint64_t), st), "cudaMemsetAsync(inflation counts)"))
     return BRO_ERR_CUDA;
   if (n_groups == 0) return BRO_OK;
-  const unsigned grid = bro::stats::grid_for(n_groups, 256 * 16, di.sm_count, 4);
-  return bro::cuda_ok(bro::launch_kernel(bro::stats::scale_inflation, grid, 256, 0, st, 1, scales_before, scales_after, mask,
-                                         n_groups, reinterpret_cast<unsigned long long*>(counts)),
+  const unsigned grid = alone ? 1u : bro::stats::grid_for(n_groups, bro::stats::kCountThreads * 16, di.sm_count, 2);
+  return bro::cuda_ok(bro::launch_kernel(bro::stats::scale_inflation, grid, bro::stats::kCountThreads, 0, st, 1, scales_before, scales_after, mask,
+                                         n_groups, alone ? 1 : 0, reinterpret_cast<unsigned long long*>(counts)),
                       "scale_inflation launch")
              ? BRO_OK
              : BRO_ERR_CUDA;

@@ -154,3 +154,53 @@ def test_empty_inputs_and_argument_checks(bro):
     ws = torch.empty(16, dtype=torch.uint8, device="cuda")
     with pytest.raises(bro.BroError):
         bro.outlier_groups(x, out, torch.zeros(4, dtype=torch.int32, device="cuda"), ws)
+
+
+@pytest.mark.parametrize("case", ["sampled", "misled", "wide", "all", "ties"])
+def test_outlier_threshold_from_a_sample(bro, case):
+    """Tensors large enough for the sampled lower bound: ordinary, one whose outliers the sample overrates (every
+    sampled position holds a large value, nothing else does: the exact count falls short and everything is counted),
+    outliers many octaves above the bound, every entry an outlier, and a threshold shared by many entries.  Bit for
+    bit against a sort."""
+    M, K, ppm = 700, 1184, 1000
+    x = synth.activations(M, K, seed=5, recipe=synth.HEAVY_RECIPE)
+    if case == "misled":
+        x = torch.full((M, K), 0.5, dtype=torch.bfloat16)
+        i = torch.arange(4096, dtype=torch.int64)
+        h1 = ((i + 1) * 2654435761) & 0xFFFFFFFF
+        h2 = ((h1 ^ (h1 >> 15)) * 2246822519) & 0xFFFFFFFF
+        rows, cols = (h1 * M) >> 32, (h2 * K) >> 32
+        x[rows[:300], cols[:300]] = 100.0
+        ppm = 2000
+    elif case == "wide":
+        x[::7, 5] = 3.0e30
+        x[3] *= 1.0e-20
+    elif case == "all":
+        ppm = 1000000
+    elif case == "ties":
+        x = torch.full((M, K), -2.0, dtype=torch.bfloat16)
+        x[:, ::40] = 1.0
+    mag = (x.view(torch.int16).int() & 0x7FFF).flatten()
+    k = max(1, -(-M * K * ppm // 1000000))
+    t = int(torch.sort(mag, descending=True).values[k - 1])
+    mask, info = gpu_outliers(bro, x.cuda(), ppm)
+    assert int(info[0]) == t and int(info[2]) == k
+    want = (mag.view(M, K // 32, 32).amax(2) >= t).to(torch.uint8).numpy()
+    assert np.array_equal(np.asarray(mask.cpu() if hasattr(mask, "cpu") else mask), want)
+
+
+@pytest.mark.parametrize("n", [1, 15, 65536, 65537, 300001])
+@pytest.mark.parametrize("offset", [0, 3])
+def test_counts_of_bytes_at_any_alignment(bro, n, offset):
+    gen = torch.Generator().manual_seed(n)
+    b, a = (torch.randint(100, 140, (n + offset,), generator=gen, dtype=torch.uint8).cuda()[offset:] for _ in range(2))
+    m = (torch.randint(0, 5, (n + offset,), generator=gen) == 0).to(torch.uint8).cuda()[offset:]
+    counts = torch.full((2, 3), -1, dtype=torch.int64, device="cuda")
+    hist = torch.full((2, 256), -1, dtype=torch.int64, device="cuda")
+    bro.scale_inflation(b, a, m, counts)
+    bro.scale_histogram(a, m, hist)
+    for c in (0, 1):
+        sel = m == c
+        d = a[sel].int() - b[sel].int()
+        assert counts[c].tolist() == [int((d < 0).sum()), int((d == 0).sum()), int((d > 0).sum())]
+        assert torch.equal(hist[c], torch.bincount(a[sel].long(), minlength=256))
