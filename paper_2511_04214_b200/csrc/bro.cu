@@ -166,7 +166,7 @@ __global__ void expire_wait_kernel(uint64_t budget_ns) {
   bro::mbar_wait(b, 0u, bro::SITE_SELF_TEST, budget_ns);
 }
 
-// h = bf16(silu(gate) * up), 8 values per thread (the producer alone; see rqd::silu_mul).
+// h = bf16(silu(gate) * up), 8 values per thread (the producer alone; see rqd::silu_mul2).
 __global__ void __launch_bounds__(256) swiglu_kernel(const uint16_t* gate, const uint16_t* up, int64_t M, int64_t K,
                                                      int64_t ldg, int64_t ldu, uint16_t* h, int64_t ldh) {
   bro::griddep_wait();

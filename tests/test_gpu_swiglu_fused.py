@@ -109,3 +109,24 @@ def test_full_size_tensor_and_argument_checks(bro):
     with pytest.raises(bro.BroError) as e:
         bro.swiglu_rotate_quantize_mxfp4(g.cuda(), u.cuda(), 0, codes, scales, bro.LAYOUT_GEMM)
     assert e.value.code == 4
+
+
+@pytest.mark.parametrize("shift", [0, 1])
+def test_fused_sigmoid_table_over_the_whole_bf16_range(bro, shift):
+    """The fused kernel takes the sigmoid from a table with clamped ends, the producer alone computes it: every gate
+    pattern, infinities and NaN included, must give the codes and scales of the two-step path."""
+    pats = torch.arange(-32768, 32768, dtype=torch.int32).to(torch.int16)
+    g = pats.roll(shift).view(torch.bfloat16).reshape(-1, 64).contiguous().cuda()       # groups of like magnitude
+    u = torch.where(torch.arange(g.numel(), device="cuda").reshape(g.shape) % 3 == 0, -0.75, 1.0).to(torch.bfloat16)
+    M, K = g.shape
+    h = torch.empty_like(g)
+    bro.swiglu_bf16(g, u, h)
+    out = []
+    for fused in (True, False):
+        c, s = bro.alloc_codes(M, K), bro.alloc_scales(M, K, bro.LAYOUT_CANONICAL)
+        if fused:
+            bro.swiglu_rotate_quantize_mxfp4(g, u, 32, c, s, bro.LAYOUT_CANONICAL)
+        else:
+            bro.rotate_quantize_mxfp4(h, 32, c, s, bro.LAYOUT_CANONICAL)
+        out.append((c, s))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
