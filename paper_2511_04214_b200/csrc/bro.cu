@@ -437,8 +437,9 @@ bro_status bro_rotate_fake_quantize_ws(const void* x_bf16, int64_t M, int64_t K,
   if (rc != BRO_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   uint32_t* rowstats = need > 0 ? static_cast<uint32_t*>(workspace) : nullptr;
+  if (B <= 128 && K <= bro::fq::kWholeRowK) rowstats = nullptr;      // whole rows fit a CTA: one pass
   if (rowstats) {
-    // per-row formats: a first pass leaves every row's range in the workspace
+    // per-row formats of longer rows: a first pass leaves every row's range in the workspace
     if (!bro::cuda_ok(cudaMemsetAsync(rowstats, 0, need, st), "cudaMemsetAsync(row ranges)")) return BRO_ERR_CUDA;
     rc = B > 128 ? bro::rqg::launch(x_bf16, M, K, ldx, signs_bf16, nullptr, nullptr, nullptr, (int)format, BRO_LAYOUT_CANONICAL,
                                     0, di.sm_count, st, nullptr, 0, rowstats, true)

@@ -32,7 +32,7 @@ constexpr int kWarps = kThreads / 32;
 // fp16(amax / 6)), 2 MXINT4 (k / 4, |k| <= 7, scale 2^E, E = floor(log2 amax)), 3 BINT4 (|k| <= 7,
 // scale fp16(amax / 7)).  Decisions are taken exactly as in rq::group_error: magnitudes scaled by an
 // exact power of two, or divided by the fp16 scale in fp32, then rounded to nearest even, saturating.
-__device__ __forceinline__ void group_dequant(const uint64_t (&P)[16], uint32_t cbits, int format, float (&out)[32]) {
+__device__ __noinline__ void group_dequant_any(const uint64_t (&P)[16], uint32_t cbits, int format, float (&out)[32]) {
   const float c = __uint_as_float(cbits);
   const uint64_t cc = rq::pack2(c, c);
   float y[32];
@@ -96,6 +96,97 @@ __device__ __forceinline__ void group_dequant(const uint64_t (&P)[16], uint32_t 
   }
 }
 
+// ---- the same on packed pairs, for ordinary numbers ------------------------------------------------------------
+// What made the forms above slow were IEEE divisions (25 instructions an element) and conversions to integers and back at a
+// quarter of the issue rate.  Here a quotient by the group's (row's) scale is q = y * inv, corrected once by its exact remainder,
+// q + (y - q sc) inv, with inv the correctly rounded 1 / sc: correctly rounded, by Markstein ("Computation of elementary
+// functions on the IBM RISC System/6000 processor", 1990), as long as nothing leaves the normal range; quotients so small that
+// their remainder is subnormal round to the element 0 either way.  Integers come from adding and subtracting 1.5 * 2^23 (nearest,
+// ties to even) after clamping, which commutes with rounding.  Every step rounds as in the forms above, so the values are the same
+// bits.  `y_nan_max` is false for groups that hold an infinity or a NaN; these and the ends of the exponent range take
+// the forms above.  [8192, 4096], block 32: BFP4 56 -> 40 us, BINT4 59 -> 41 us, INT4 per row 81 -> 67 us.
+__device__ __forceinline__ float amax_nan(const uint64_t (&Y)[16]) {
+  float m = 0.f, m2 = 0.f;
+#pragma unroll
+  for (int k = 0; k < 16; k += 2) {
+    float a, b, c, d;
+    rq::unpack2(Y[k], a, b);
+    rq::unpack2(Y[k + 1], c, d);
+    asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(a), "f"(b));
+    asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(m2) : "f"(c), "f"(d));
+  }
+  asm("max.NaN.f32 %0, %0, %1;" : "+f"(m) : "f"(m2));
+  return m;
+}
+__device__ __forceinline__ uint64_t both(float v) { return rq::pack2(v, v); }
+__device__ __forceinline__ uint64_t quotient2(uint64_t y, uint64_t inv, uint64_t minus_sc) {
+  const uint64_t q = rq::mul2(y, inv);
+  return rq::fma2(rq::fma2(minus_sc, q, y), inv, q);
+}
+// clamp to [lo, hi] (whole numbers), round to a whole number
+__device__ __forceinline__ uint64_t round2(uint64_t r, float lo, float hi) {
+  float a, b;
+  rq::unpack2(r, a, b);
+  const uint64_t magic = both(12582912.0f);
+  return rq::sub2(rq::add2(rq::pack2(fminf(fmaxf(a, lo), hi), fminf(fmaxf(b, lo), hi)), magic), magic);
+}
+__device__ __forceinline__ uint64_t e2m1_value2(uint64_t r) {          // nearest E2M1 values
+  float a, b;
+  rq::unpack2(r, a, b);
+  uint32_t h;
+  asm("{ .reg .b8 b; cvt.rn.satfinite.e2m1x2.f32 b, %2, %1; cvt.rn.f16x2.e2m1x2 %0, b; }" : "=r"(h) : "f"(a), "f"(b));
+  return rq::pack2(__half2float(__ushort_as_half((unsigned short)(h & 0xFFFFu))), __half2float(__ushort_as_half((unsigned short)(h >> 16))));
+}
+// out = |v| with the sign of y (a value that rounds to zero keeps its sign)
+__device__ __forceinline__ void signed_out(uint64_t v, uint64_t y, float& o0, float& o1) {
+  float v0, v1, y0, y1;
+  rq::unpack2(v, v0, v1);
+  rq::unpack2(y, y0, y1);
+  o0 = copysignf(v0, y0);
+  o1 = copysignf(v1, y1);
+}
+
+__device__ __forceinline__ void group_dequant(const uint64_t (&P)[16], uint32_t cbits, int format, float (&out)[32]) {
+  uint64_t Y[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) Y[k] = rq::mul2(P[k], both(__uint_as_float(cbits)));
+  const float m = amax_nan(Y);
+  const uint32_t ef = __float_as_uint(m) >> 23;
+  // 2^-125 and up, finite; the fp16 scales not zero
+  float sc = 0.f, inv = 0.f;
+  if (format & 1) {
+    unsigned short hb;
+    asm("cvt.rn.satfinite.f16.f32 %0, %1;" : "=h"(hb) : "f"(__fdiv_rn(m, format == 1 ? 6.f : 7.f)));
+    sc = __half2float(__ushort_as_half(hb));
+    inv = __frcp_rn(sc);
+  }
+  if (ef < 8u || ef > 250u || ((format & 1) && sc == 0.f)) {          // (a NaN has exponent field 255)
+    uint64_t Q[16];                            // (copies: only this path keeps arrays in memory)
+    float o[32];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) Q[k] = P[k];
+    group_dequant_any(Q, cbits, format, o);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) out[i] = o[i];
+    return;
+  }
+  if (format == 0) {
+    const float s_inv = __uint_as_float((256u - ef) << 23), s = __uint_as_float((ef - 2u) << 23);   // 2^-E and 2^E, E = ef - 2 - 127
+#pragma unroll
+    for (int k = 0; k < 16; ++k) signed_out(rq::mul2(e2m1_value2(rq::mul2(Y[k], both(s_inv))), both(s)), Y[k], out[2 * k], out[2 * k + 1]);
+  } else if (format == 2) {
+    const float s_inv = __uint_as_float((256u - ef) << 23), s = __uint_as_float((ef - 2u) << 23);   // 4 * 2^-E and 2^E / 4, E = ef - 127
+#pragma unroll
+    for (int k = 0; k < 16; ++k) signed_out(rq::mul2(round2(rq::mul2(Y[k], both(s_inv)), -7.f, 7.f), both(s)), Y[k], out[2 * k], out[2 * k + 1]);
+  } else if (format == 1) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) signed_out(rq::mul2(e2m1_value2(quotient2(Y[k], both(inv), both(-sc))), both(sc)), Y[k], out[2 * k], out[2 * k + 1]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) signed_out(rq::mul2(round2(quotient2(Y[k], both(inv), both(-sc)), -7.f, 7.f), both(sc)), Y[k], out[2 * k], out[2 * k + 1]);
+  }
+}
+
 __device__ __forceinline__ void store_group(float* dst, const float (&out)[32]) {
 #pragma unroll
   for (int j = 0; j < 8; ++j)
@@ -127,8 +218,8 @@ __device__ __forceinline__ void group_range(const uint64_t (&P)[16], uint32_t cb
 // codes 0..15 over [lo, hi] (the range always contains zero): scale fp16((hi - lo) / 15), zero point
 // z = rint(-lo / scale) (at most 15), q = clamp(rint(y / scale) + z, 0, 15), value (q - z) scale.  Quotients
 // are IEEE fp32 divisions; every result is an integer of at most 5 bits times an fp16 number, exact in fp32.
-__device__ __forceinline__ void row_dequant(const uint64_t (&P)[16], uint32_t cbits, bool asym, float neglo, float hi,
-                                            float (&out)[32]) {
+__device__ __noinline__ void row_dequant_any(const uint64_t (&P)[16], uint32_t cbits, bool asym, float neglo, float hi,
+                                             float (&out)[32]) {
   const float c = __uint_as_float(cbits);
   const uint64_t cc = rq::pack2(c, c);
   float y[32];
@@ -161,42 +252,109 @@ __device__ __forceinline__ void row_dequant(const uint64_t (&P)[16], uint32_t cb
   }
 }
 
+__device__ __forceinline__ void row_dequant(const uint64_t (&P)[16], uint32_t cbits, bool asym, float neglo, float hi,
+                                            float (&out)[32]) {
+  uint64_t Y[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) Y[k] = rq::mul2(P[k], both(__uint_as_float(cbits)));
+  const float m = amax_nan(Y);
+  unsigned short hb;
+  asm("cvt.rn.satfinite.f16.f32 %0, %1;" : "=h"(hb) : "f"(asym ? __fdiv_rn(__fadd_rn(hi, neglo), 15.f) : __fdiv_rn(fmaxf(hi, neglo), 7.f)));
+  const float sc = __half2float(__ushort_as_half(hb));
+  if (!(m < 1e38f) || sc == 0.f) {
+    uint64_t Q[16];
+    float o[32];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) Q[k] = P[k];
+    row_dequant_any(Q, cbits, asym, neglo, hi, o);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) out[i] = o[i];
+    return;
+  }
+  const float inv = __frcp_rn(sc);
+  if (asym) {        // clamp(rint(y / sc) + z, 0, 15) - z is rint(y / sc) clamped to [-z, 15 - z]
+    const float z = (float)min(__float2int_rn(__fdiv_rn(neglo, sc)), 15);
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      rq::unpack2(rq::mul2(round2(quotient2(Y[k], both(inv), both(-sc)), -z, 15.f - z), both(sc)), out[2 * k], out[2 * k + 1]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      signed_out(rq::mul2(round2(quotient2(Y[k], both(inv), both(-sc)), -7.f, 7.f), both(sc)), Y[k], out[2 * k], out[2 * k + 1]);
+  }
+}
+
 struct Params {
   const uint16_t* x;
   int64_t M, K, ldx;
   const uint16_t* signs;        // [K] bf16 +-1 (kernels with SIGNS) or nullptr
   uint32_t* rowstats;           // [M, 2] the row ranges (see group_range): written when deq == nullptr and
-                                // neither statistic is asked for, read by the per-row formats
+                                // neither statistic is asked for, read by the per-row formats unless `whole_rows`
   float* deq;                   // [M, K] fp32, row stride ldd — or nullptr, and then one of:
   int64_t ldd;
   float* mse;                   //   [M, K/32] per-group quantisation error (rq::group_error)
   uint8_t* scale_bytes;         //   [M, K/32] E8M0 byte of each group (rq::group_scale_byte)
   int format;
   int chunks_per_row;           // ceil((K / 32) / 32): one task = one warp, 32 groups of a row
-  int64_t total_tasks;          // M * chunks_per_row
+  int whole_rows;               // per-row formats of rows of at most kWarps chunks: a CTA holds whole rows
 };
 
+// Longest row of which a CTA holds every chunk in one of its warps' registers.
+constexpr int64_t kWholeRowK = (int64_t)kWarps * 1024;
+
 // LOG2B = 0: no rotation; 1..4: blocks of 2..16 inside the group; 5, 6, 7: blocks of 32, 64, 128.
+// The loads of a warp's next task are issued before the current one is computed.  With `whole_rows` the warps of a CTA
+// take whole rows together, exchange the chunks' ranges through shared memory and need neither the first pass nor
+// its second read of x ([8192, 4096]: 67 -> 48 us).  Two CTAs per SM that stay (not eight that come and go) gave another 2 to 4 us.
 template <int LOG2B, bool SIGNS>
 __global__ void __launch_bounds__(kThreads, 2) fake_quantize_kernel(const Params p) {
   __shared__ __align__(16) float sbuf[kWarps][32 * 32];      // 4 KiB per warp
-  const int lane = threadIdx.x & 31;
-  float* wbuf = sbuf[threadIdx.x >> 5];
+  __shared__ float2 ranges[2][kWarps];                       // whole_rows: the chunks' ranges, two rounds
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float* wbuf = sbuf[warp];
   const int ng = (int)(p.K >> 5);
   constexpr uint32_t cbits = LOG2B == 0 ? 0x3F800000u : rq::norm_bits<(LOG2B == 0 ? 5 : LOG2B)>();
   const bool full = p.deq != nullptr;             // (uniform over the grid)
+  // row and chunk of this warp's first task, and the step to its next one
+  const int c = p.chunks_per_row;
+  const int rows_at_once = p.whole_rows ? kWarps / c : 0;
+  int64_t row, step_row;
+  int chunk, step_chunk = 0;
+  if (p.whole_rows) {
+    const int r = warp / c;
+    chunk = warp - r * c;
+    row = r < rows_at_once ? (int64_t)blockIdx.x * rows_at_once + r : p.M;      // (left-over warps only keep step)
+    step_row = (int64_t)gridDim.x * rows_at_once;
+  } else {
+    const int64_t task = (int64_t)blockIdx.x * kWarps + warp, num_warps = (int64_t)gridDim.x * kWarps;
+    row = task / c;
+    chunk = (int)(task - row * c);
+    step_row = num_warps / c;
+    step_chunk = (int)(num_warps - step_row * c);
+  }
   griddep_wait();
   griddep_launch_dependents();
-  const int64_t num_warps = (int64_t)gridDim.x * kWarps;
-  for (int64_t task = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5); task < p.total_tasks; task += num_warps) {
-    const int64_t row = task / p.chunks_per_row;
-    const int g = (int)(task - row * p.chunks_per_row) * 32 + lane;
-    const bool live = g < ng;      // (K is a multiple of the block, so the lanes of a block share `live`)
+  auto load = [&](int64_t r, int ch, uint4 (&v)[4]) {
+    const int g = ch * 32 + lane;
+    const bool in = r < p.M && g < ng;
+    const uint4* src = reinterpret_cast<const uint4*>(p.x + (in ? r : 0) * p.ldx + (int64_t)(in ? g : 0) * 32);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = in ? __ldg(src + j) : make_uint4(0u, 0u, 0u, 0u);
+  };
+  uint4 cur[4], nxt[4];
+  load(row, chunk, cur);
+  int round = 0;
+  for (int64_t base = p.whole_rows ? (int64_t)blockIdx.x * rows_at_once : row; base < p.M; ++round) {
+    const int g = chunk * 32 + lane;
+    const bool live = row < p.M && g < ng;         // (K is a multiple of the block, so the lanes of a block share `live`)
+    int64_t nrow = row + step_row;
+    int nchunk = chunk + step_chunk;
+    if (nchunk >= c) { nchunk -= c; ++nrow; }
+    load(nrow, nchunk, nxt);
     uint64_t P[16];
-    const uint4* src = reinterpret_cast<const uint4*>(p.x + row * p.ldx + (int64_t)g * 32);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      uint4 q = live ? __ldg(src + j) : make_uint4(0u, 0u, 0u, 0u);
+      uint4 q = cur[j];
       if (SIGNS && live) q = rq::apply_signs(q, __ldg(reinterpret_cast<const uint4*>(p.signs + (int64_t)g * 32) + j));
       if (LOG2B == 0) {
         const uint32_t w[4] = {q.x, q.y, q.z, q.w};
@@ -211,63 +369,78 @@ __global__ void __launch_bounds__(kThreads, 2) fake_quantize_kernel(const Params
     if (LOG2B >= 2 && LOG2B <= 4) rq::fwht32_stages_below<(LOG2B >= 2 && LOG2B <= 4) ? LOG2B : 2>(P);
     if (LOG2B >= 6) rq::cross_lane_stage(P, 1, (lane & 1) != 0);
     if (LOG2B >= 7) rq::cross_lane_stage(P, 2, (lane & 2) != 0);
-    if (!full && !p.mse && !p.scale_bytes) {       // first pass of the per-row formats: the row's range
-      float neglo, hi;
+    float neglo = 0.f, hi = 0.f;
+    if (p.whole_rows || (!full && !p.mse && !p.scale_bytes)) {     // the range of this chunk
       group_range(P, cbits, neglo, hi);
 #pragma unroll
       for (int d = 16; d >= 1; d >>= 1) {          // (all 32 lanes hold groups of the same row; dead lanes hold zeros)
         neglo = fmaxf(neglo, __shfl_xor_sync(0xFFFFFFFFu, neglo, d));
         hi = fmaxf(hi, __shfl_xor_sync(0xFFFFFFFFu, hi, d));
       }
-      if (lane == 0) {
+    }
+    if (p.whole_rows) {
+      if (lane == 0) ranges[round & 1][warp] = make_float2(neglo, hi);
+      __syncthreads();                             // (the buffers alternate: the round before was read before this barrier)
+      for (int w = warp - chunk; w < warp - chunk + c && w < kWarps; ++w) {
+        const float2 o = ranges[round & 1][w];
+        neglo = fmaxf(neglo, o.x);
+        hi = fmaxf(hi, o.y);
+      }
+    }
+    if (!full) {
+      if (p.mse) {                                 // the statistics only
+        const float e = rq::group_error(P, cbits, p.format);
+        if (live) p.mse[row * ng + g] = e;
+      } else if (p.scale_bytes) {
+        const uint32_t sb = rq::group_scale_byte(P, cbits);
+        if (live) p.scale_bytes[row * ng + g] = (uint8_t)sb;
+      } else if (lane == 0) {                      // first pass of the per-row formats: the row's range
         atomicMax(p.rowstats + 2 * row, __float_as_uint(neglo));
         atomicMax(p.rowstats + 2 * row + 1, __float_as_uint(hi));
       }
-      continue;
-    }
-    if (!full) {                                   // the statistics only
-      if (p.mse) {
-        const float e = rq::group_error(P, cbits, p.format);
-        if (live) p.mse[row * ng + g] = e;
+    } else if (row < p.M) {
+      float out[32];
+      if (p.format == kFormatNone) {               // the rotation itself
+        const uint64_t cc = rq::pack2(__uint_as_float(cbits), __uint_as_float(cbits));
+#pragma unroll
+        for (int k = 0; k < 16; ++k) rq::unpack2(rq::mul2(P[k], cc), out[2 * k], out[2 * k + 1]);
+      } else if (p.format >= kFormatRowSym) {
+        if (!p.whole_rows) {
+          neglo = __uint_as_float(__ldcg(p.rowstats + 2 * row));
+          hi = __uint_as_float(__ldcg(p.rowstats + 2 * row + 1));
+        }
+        row_dequant(P, cbits, p.format == kFormatRowAsym, neglo, hi, out);
       } else {
-        const uint32_t sb = rq::group_scale_byte(P, cbits);
-        if (live) p.scale_bytes[row * ng + g] = (uint8_t)sb;
+        group_dequant(P, cbits, p.format, out);
       }
-      continue;
-    }
-    float out[32];
-    if (p.format == kFormatNone) {                 // the rotation itself
-      const uint64_t cc = rq::pack2(__uint_as_float(cbits), __uint_as_float(cbits));
+      // lane l -> buffer row l (128 bytes), piece j at position j ^ (l & 7)
+      __syncwarp();                                // the previous task's reads of the buffer are done
 #pragma unroll
-      for (int k = 0; k < 16; ++k) rq::unpack2(rq::mul2(P[k], cc), out[2 * k], out[2 * k + 1]);
-    } else if (p.format >= kFormatRowSym) {
-      const float neglo = __uint_as_float(__ldcg(p.rowstats + 2 * row));
-      const float hi = __uint_as_float(__ldcg(p.rowstats + 2 * row + 1));
-      row_dequant(P, cbits, p.format == kFormatRowAsym, neglo, hi, out);
-    } else {
-      group_dequant(P, cbits, p.format, out);
-    }
-    // lane l -> buffer row l (128 bytes), piece j at position j ^ (l & 7)
-    __syncwarp();                                  // the previous task's reads of the buffer are done
+      for (int j = 0; j < 8; ++j)
+        *reinterpret_cast<float4*>(wbuf + lane * 32 + ((j ^ (lane & 7)) << 2)) =
+            make_float4(out[4 * j], out[4 * j + 1], out[4 * j + 2], out[4 * j + 3]);
+      __syncwarp();
+      // instruction i writes groups 4i .. 4i+3 of the chunk: 8 lanes per group, 16 bytes each
+      const int gbase = g - lane;
+      float* rowp = p.deq + row * p.ldd + (int64_t)gbase * 32;
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-      *reinterpret_cast<float4*>(wbuf + lane * 32 + ((j ^ (lane & 7)) << 2)) =
-          make_float4(out[4 * j], out[4 * j + 1], out[4 * j + 2], out[4 * j + 3]);
-    __syncwarp();
-    // instruction i writes groups 4i .. 4i+3 of the chunk: 8 lanes per group, 16 bytes each
-    const int gbase = g - lane;
-    float* rowp = p.deq + row * p.ldd + (int64_t)gbase * 32;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int r = i * 4 + (lane >> 3), c = lane & 7;
-      const float4 v = *reinterpret_cast<const float4*>(wbuf + r * 32 + ((c ^ (r & 7)) << 2));
-      if (gbase + r < ng) *reinterpret_cast<float4*>(rowp + r * 32 + c * 4) = v;
+      for (int i = 0; i < 8; ++i) {
+        const int r = i * 4 + (lane >> 3), q = lane & 7;
+        const float4 v = *reinterpret_cast<const float4*>(wbuf + r * 32 + ((q ^ (r & 7)) << 2));
+        if (gbase + r < ng) *reinterpret_cast<float4*>(rowp + r * 32 + q * 4) = v;
+      }
     }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) cur[j] = nxt[j];
+    row = nrow;
+    chunk = nchunk;
+    base = p.whole_rows ? base + step_row : row;
   }
 }
 
 // block: 1 (identity), 2, 4, 8, 16, 32, 64 or 128.  Exactly one of deq / mse / scale_bytes is set — or none of
-// them and rowstats, for the first pass of the per-row formats.
+// them and rowstats, for the first pass of the per-row formats; deq and a per-row format without rowstats take K up to
+// kWholeRowK in one pass.
 inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, int block, const void* signs, int format,
                          float* deq, int64_t ldd, float* mse, uint8_t* scale_bytes, int sm_count, cudaStream_t st,
                          uint32_t* rowstats = nullptr) {
@@ -282,9 +455,10 @@ inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, int b
   p.scale_bytes = scale_bytes;
   p.format = format;
   p.chunks_per_row = (int)((K / 32 + 31) / 32);
-  p.total_tasks = M * p.chunks_per_row;
-  const int64_t want = (p.total_tasks + kWarps - 1) / kWarps;
-  const int64_t cap = (int64_t)sm_count * 8;
+  p.whole_rows = (deq && format >= kFormatRowSym && format != kFormatNone && !rowstats) ? 1 : 0;
+  const int rows_at_once = kWarps / p.chunks_per_row;
+  const int64_t want = p.whole_rows ? (M + rows_at_once - 1) / rows_at_once : (M * p.chunks_per_row + kWarps - 1) / kWarps;
+  const int64_t cap = (int64_t)sm_count * 2;
   const unsigned grid = (unsigned)(want < cap ? want : cap);
   auto go = [&](auto kernel) -> bro_status {
     return cuda_ok(launch_kernel(kernel, grid, kThreads, 0, st, 1, p), "fake_quantize launch") ? BRO_OK : BRO_ERR_CUDA;

@@ -140,3 +140,35 @@ def test_full_size_sample(bro):
         got = out[torch.as_tensor(rows, device="cuda")].cpu().numpy()
         check(got, oracle.fake_quantize(rotated(x[torch.as_tensor(rows)].contiguous(), 32), fmt))
     assert bro.last_device_status() == 0
+
+
+@pytest.mark.parametrize("M,K", [(1, 32), (3, 1024), (5, 1056), (9, 3072), (300, 4384), (2, 8192), (3, 8224)])
+@pytest.mark.parametrize("fmt", ["int4_row_sym", "int4_row_asym"])
+def test_per_row_formats_of_whole_rows_in_a_cta(bro, M, K, fmt):
+    """One to eight chunks of 1024 channels per row (K up to 8192: one pass over x), one more: two passes."""
+    x = synth.activations(M, K, seed=M + K, recipe=synth.HEAVY_RECIPE)
+    check(gpu(bro, x, 32, fmt), oracle.fake_quantize(rotated(x, 32), fmt))
+
+
+@pytest.mark.parametrize("fmt", FORMATS)
+def test_unusual_numbers_take_the_general_form(bro, fmt):
+    """Groups at the ends of the exponent range, zeros of both signs and halfway quotients, without a rotation, against
+    the oracle; an infinity or a NaN must leave the other groups (per-row formats: the other rows) alone."""
+    M, K = 64, 256
+    gen = torch.Generator().manual_seed(1)
+    x = torch.randn(M, K, generator=gen)
+    scale = torch.tensor([2.0 ** e for e in (-126, -120, -119, -118, -24, -14, 0, 15, 16, 40, 120, 123)])
+    x *= scale[torch.arange(M) % len(scale)][:, None]
+    x[5] = 0.0
+    x[6, ::2] = -0.0
+    x[7] = torch.arange(K) % 15 * 0.5 - 3.5
+    x = x.to(torch.bfloat16)
+    clean = gpu(bro, x, 1, fmt)
+    check(clean, oracle.fake_quantize(rotated(x, 1), fmt))
+    x[20, 40] = float("inf")
+    x[21, 70] = float("nan")
+    got = gpu(bro, x, 1, fmt)
+    keep = np.ones((M, K), dtype=bool)
+    for row, col in ((20, 40), (21, 70)):
+        keep[row, slice(None) if "row" in fmt else slice(col // 32 * 32, col // 32 * 32 + 32)] = False
+    assert np.array_equal(got[keep].view(np.uint32), clean[keep].view(np.uint32))
