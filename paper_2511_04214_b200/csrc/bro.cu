@@ -115,11 +115,15 @@ bro_status bro::gemm::make_codes_map(CUtensorMap* map, const void* base, int64_t
                      (uint64_t)(K / 2), 128, (uint32_t)box_rows, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
-// bf16 output [M, ldy]: box = 64 columns (128 bytes) x 32 rows (what one epilogue warp stores at a
-// time), 128-byte swizzle to match its staging buffer.
-bro_status bro::gemm::make_out_map(CUtensorMap* map, const void* y, int64_t M, int64_t N, int64_t ldy) {
-  return make_map_2d(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, y, (uint64_t)N, (uint64_t)M, (uint64_t)ldy * 2,
-                     2 * bro::gemm::kChunkCols, 32, CU_TENSOR_MAP_SWIZZLE_128B);
+// Output [M, ldy]: box = 128 bytes (64 bf16 or 32 fp32 columns) x 32 rows (what one epilogue warp stores at a
+// time), 128-byte swizzle to match its staging buffer.  The map ends at the last whole 16 bytes of a row: the epilogue
+// writes the rest itself (and stores nothing through the map when a row is shorter than that).
+bro_status bro::gemm::make_out_map(CUtensorMap* map, const void* y, int64_t M, int64_t N, int64_t ldy, int out_dtype) {
+  const bool f32 = out_dtype == BRO_OUT_F32;
+  return make_map_2d(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, f32 ? 4 : 2, y,
+                     (uint64_t)(N >= (f32 ? 4 : 8) ? N & ~(int64_t)(f32 ? 3 : 7) : N),
+                     (uint64_t)M, (uint64_t)ldy * (f32 ? 4 : 2), f32 ? bro::gemm::kChunkCols : 2 * bro::gemm::kChunkCols, 32,
+                     CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
 // Scale tensor in the tensor-core layout viewed as 32-bit words: one row per 128-row block

@@ -17,7 +17,7 @@
 //   warps 2..5  epilogue, each warp on its own for the 32 rows of its TMEM lane quadrant:
 //               tcgen05.ld of 64 columns (the next 64 in flight), convert to bf16, stage in the
 //               warp's shared-memory buffer (128-byte swizzle), one TMA store of a 64 x 32 box
-//               (which also clips the ragged edges); the fp32 output mode stores from registers.
+//               (which also clips the ragged edges); fp32 output: one box of 32 x 32 per 32 columns.
 // TMEM holds 512 columns.  For BN = 256 two full accumulators plus the scale columns do not
 // fit, so the two accumulators overlap by 32 columns ([0,256) and [224,480)): the epilogue drains
 // the shared 32 columns first and releases them early, and the next tile's MMAs start as soon as
@@ -206,6 +206,17 @@ __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, ui
   asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
+__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint16_t lds16(uint32_t addr) {
+  uint16_t v;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr) : "memory");
+  return v;
+}
+
 // Unit index -> first row, first column and width of its output tile.
 template <int BN>
 __device__ __forceinline__ void decode_unit(const Params& p, int u, int& m0, int& n0, int& bn) {
@@ -355,23 +366,31 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem_acc, int buf, int la
       }
     }
   };
-  auto store_f32 = [&](const uint32_t (&r)[32], int col0) {
-    if (row < M && col0 < N) {
-      float* dst = static_cast<float*>(y) + row * ldy + col0;
-      if ((int64_t)col0 + 32 <= N) {
+  // fp32: one box of 32 columns x 32 rows per chunk, 128 bytes a row as the 64 bf16 columns of a pair.  (Stores from
+  // registers, 16 bytes a lane and the lanes a row of y apart, took 20 of a launch's 31 us at (777, 4384, 6004).)
+  auto emit_f32 = [&](const uint32_t (&r)[32], int col0, uint32_t sbuf) {
+    if (stage_stride == 0u) bulk_wait_read_elect<0>();
+    __syncwarp();
+    const uint32_t rowaddr = sbuf + (uint32_t)lane * 128u, sw = (uint32_t)lane & 7u;
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-          reinterpret_cast<uint4*>(dst)[j] = make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
-      } else {
-        for (int j = 0; j < 32 && col0 + j < N; ++j) dst[j] = __uint_as_float(r[j]);
-      }
+    for (int j = 0; j < 8; ++j) sts128(rowaddr + ((j ^ sw) << 4), r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+    fence_proxy_async_smem();
+    __syncwarp();
+    // (the map ends at the last multiple of 4 columns, see make_out_map; the up to 3 behind it come from the buffer)
+    const int64_t n_tma = N & ~(int64_t)3;
+    if (col0 < n_tma && row0 < M) tma_store_2d_elect(tmy, sbuf, col0, row0);
+    bulk_commit_elect();
+    if (n_tma < N && n_tma >= col0 && n_tma < (int64_t)col0 + kChunkCols && row < M) {
+      float* dst = static_cast<float*>(y) + row * ldy + n_tma;
+      const int k0 = (int)(n_tma - col0);
+      for (int k = 0; k < (int)(N - n_tma); ++k) dst[k] = __uint_as_float(lds32(rowaddr + ((((uint32_t)(k0 >> 2)) ^ sw) << 4) + 4u * k));
     }
   };
   auto emit = [&](const uint32_t (&r0)[32], const uint32_t (&r1)[32], int pr, int pi) {
     const int col0 = n0 + pr * 2 * kChunkCols;
     if (OUT_F32) {
-      store_f32(r0, col0);
-      store_f32(r1, col0 + kChunkCols);
+      emit_f32(r0, col0, stage_buf + (uint32_t)(2 * pi) * stage_stride);
+      emit_f32(r1, col0 + kChunkCols, stage_buf + (uint32_t)(2 * pi + 1) * stage_stride);
     } else {
       uint32_t h[32];
 #pragma unroll
@@ -390,16 +409,15 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem_acc, int buf, int la
       for (int j = 0; j < 8; ++j) sts128(rowaddr + ((j ^ sw) << 4), h[4 * j], h[4 * j + 1], h[4 * j + 2], h[4 * j + 3]);
       fence_proxy_async_smem();
       __syncwarp();
-      // A TMA store clips at 16-byte granularity: when N is not a multiple of 8 the ragged last
-      // pair is written from registers instead, element by element.
-      const bool ragged = ((N & 7) != 0) && ((int64_t)col0 + 2 * kChunkCols > N);
-      if (col0 < N && row0 < M && !ragged) tma_store_2d_elect(tmy, sbuf, col0, row0);
+      // A TMA store clips at 16-byte granularity: the map ends at the last multiple of 8 columns, the up to 7 behind it are
+      // copied from the staging buffer (all 64 columns of a ragged pair, element by element, took 5 us of the last tile).
+      const int64_t n_tma = N & ~(int64_t)7;
+      if (col0 < n_tma && row0 < M) tma_store_2d_elect(tmy, sbuf, col0, row0);
       bulk_commit_elect();             // (possibly empty) keeps the group count in step
-      if (ragged && row < M) {
-        uint16_t* dst = static_cast<uint16_t*>(y) + row * ldy + col0;
-#pragma unroll
-        for (int j = 0; j < 64; ++j)
-          if ((int64_t)col0 + j < N) dst[j] = (uint16_t)((j & 1) ? (h[j >> 1] >> 16) : (h[j >> 1] & 0xFFFFu));
+      if (n_tma < N && n_tma >= col0 && n_tma < (int64_t)col0 + 2 * kChunkCols && row < M) {
+        uint16_t* dst = static_cast<uint16_t*>(y) + row * ldy + n_tma;
+        const uint32_t piece = rowaddr + ((((uint32_t)(n_tma - col0) >> 3) ^ sw) << 4);
+        for (int k = 0; k < (int)(N - n_tma); ++k) dst[k] = lds16(piece + 2u * k);
       }
     }
   };
@@ -571,7 +589,8 @@ gemm_mxfp4_kernel(const __grid_constant__ CUtensorMap tma, const __grid_constant
       const uint32_t tmem_acc = tmem_base + buf * C::kAccStride + ((uint32_t)(q * 32) << 16);
       // the final tile of this CTA stages every pair in its own 4 KiB of the (now idle) A stages
       const bool last = u + (int)gridDim.x >= p.total_units;
-      const uint32_t stage_buf = last ? sA + (uint32_t)q * (4u * 4096u) : sOut + (uint32_t)q * (32u * 128u);
+      // (fp32: twice as many buffers, on into the W stages behind)
+      const uint32_t stage_buf = last ? sA + (uint32_t)q * (OUT_F32 ? 8u * 4096u : 4u * 4096u) : sOut + (uint32_t)q * (32u * 128u);
       const uint32_t stage_stride = last ? 4096u : 0u;
       auto release_shared = [&] { mbar_arrive(bar_ovl_free + 8 * buf); };
       auto release_all = [&] { mbar_arrive(bar_acc_free + 8 * buf); };
@@ -584,7 +603,7 @@ gemm_mxfp4_kernel(const __grid_constant__ CUtensorMap tma, const __grid_constant
     }
     // the staging buffer must have been read before this CTA's shared memory goes away; the writes
     // themselves complete with the kernel
-    if (!OUT_F32) bulk_wait_read_elect<0>();
+    bulk_wait_read_elect<0>();
   }
   tc_fence_before();
   __syncthreads();
@@ -594,7 +613,7 @@ gemm_mxfp4_kernel(const __grid_constant__ CUtensorMap tma, const __grid_constant
 inline size_t workspace_bytes(int64_t, int64_t, int64_t) { return 0; }
 
 bro_status make_codes_map(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int box_rows);
-bro_status make_out_map(CUtensorMap* map, const void* y, int64_t M, int64_t N, int64_t ldy);
+bro_status make_out_map(CUtensorMap* map, const void* y, int64_t M, int64_t N, int64_t ldy, int out_dtype);
 
 template <int BN>
 bro_status launch_tile(const CUtensorMap& tma, const CUtensorMap& tmw, const CUtensorMap& tmw_half,
@@ -663,12 +682,8 @@ inline bro_status launch(const void* acodes, const void* ascales, const void* wc
   if (rc != BRO_OK) return rc;
   rc = make_codes_map(&tmw, wcodes, N, K, bn);
   if (rc != BRO_OK) return rc;
-  if (out_dtype == BRO_OUT_BF16) {
-    rc = make_out_map(&tmy, y, M, N, ldy);
-    if (rc != BRO_OK) return rc;
-  } else {
-    tmy = tma;   // unused by the fp32-output kernel
-  }
+  rc = make_out_map(&tmy, y, M, N, ldy, out_dtype);
+  if (rc != BRO_OK) return rc;
   CUtensorMap tmw_half;       // the same weights seen through a box of half as many rows
   rc = make_codes_map(&tmw_half, wcodes, N, K, bn / 2);
   if (rc != BRO_OK) return rc;

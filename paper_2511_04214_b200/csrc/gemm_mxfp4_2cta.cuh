@@ -265,7 +265,7 @@ gemm_mxfp4_pair_kernel(const __grid_constant__ CUtensorMap tma, const __grid_con
     }
     // the staging buffer must have been read before this CTA's shared memory goes away; the writes
     // themselves complete with the kernel
-    if (!OUT_F32) gemm::bulk_wait_read_elect<0>();
+    gemm::bulk_wait_read_elect<0>();
   }
   gemm::tc_fence_before();
   __syncthreads();
@@ -322,12 +322,8 @@ inline bro_status launch(const void* acodes, const void* ascales, const void* wc
   if (rc != BRO_OK) return rc;
   rc = make_scale_map(&tmsfb, wscales, N, kblocks, 2);
   if (rc != BRO_OK) return rc;
-  if (out_dtype == BRO_OUT_BF16) {
-    rc = gemm::make_out_map(&tmy, y, M, N, ldy);
-    if (rc != BRO_OK) return rc;
-  } else {
-    tmy = tma;   // unused by the fp32-output kernel
-  }
+  rc = gemm::make_out_map(&tmy, y, M, N, ldy, out_dtype);
+  if (rc != BRO_OK) return rc;
   auto go = [&](void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, Params),
                 int which) -> bro_status {
     static DeviceOnce once[2];
