@@ -135,24 +135,35 @@ bro_status bro::gemm2::make_scale_map(CUtensorMap* map, const void* scales, int6
                      CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
-// Rows of x as a 3-D tensor {64 bf16, K / 64, M} with strides {128 bytes, ldx * 2 bytes}: a box of
-// whole rows lands in shared memory as 128-byte segments with the 128-byte swizzle.
-bro_status bro::rqg::make_row_map(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx, int box_rows) {
+namespace {
+// 3-D map of x: {inner bf16, K / inner, M} with strides {inner * 2, ldx * 2} bytes.
+bro_status make_map_3d(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx, int inner, uint32_t box_mid,
+                       uint32_t box_rows, CUtensorMapSwizzle swz) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn) {
     snprintf(bro::g_last_cuda_error, sizeof(bro::g_last_cuda_error), "cuTensorMapEncodeTiled unavailable");
     return BRO_ERR_CUDA;
   }
-  cuuint64_t dims[3] = {64, (cuuint64_t)(K / 64), (cuuint64_t)M};
-  cuuint64_t strides[2] = {128, (cuuint64_t)ldx * 2};
-  cuuint32_t box[3] = {64, (cuuint32_t)(K / 64), (cuuint32_t)box_rows};
+  cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)(K / inner), (cuuint64_t)M};
+  cuuint64_t strides[2] = {(cuuint64_t)inner * 2, (cuuint64_t)ldx * 2};
+  cuuint32_t box[3] = {(cuuint32_t)inner, box_mid, box_rows};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(x), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS)
-    snprintf(bro::g_last_cuda_error, sizeof(bro::g_last_cuda_error), "cuTensorMapEncodeTiled (rows): CUresult %d", (int)r);
+    snprintf(bro::g_last_cuda_error, sizeof(bro::g_last_cuda_error), "cuTensorMapEncodeTiled (3-D): CUresult %d", (int)r);
   return r == CUDA_SUCCESS ? BRO_OK : BRO_ERR_CUDA;
+}
+}  // namespace
+
+// Whole rows of x in segments of 64 bf16: a box lands in shared memory as 128-byte segments with the 128-byte swizzle.
+bro_status bro::rqg::make_row_map(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx, int box_rows) {
+  return make_map_3d(map, x, M, K, ldx, 64, (uint32_t)(K / 64), (uint32_t)box_rows, CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
+// 32 groups of one row: 2 KiB in 64-byte segments with the 64-byte swizzle.
+bro_status bro::rqd::make_group_map(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx) {
+  return make_map_3d(map, x, M, K, ldx, 32, 32, 1, CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
 namespace {

@@ -39,14 +39,14 @@ struct Params {
   int groups_padded;            // groups per row it covers (scale padding included)
   int chunks_per_row;           // ceil(groups_padded / 32)
   int total_tasks;              // rows_padded * chunks_per_row; one task = one warp, 32 groups of a row
-  const uint16_t* up;           // PRODUCER kernels: the second operand of h = silu(x) * up, [M, K] with row stride ldu
+  const uint16_t* up;           // the gated kernel: the second operand of h = silu(x) * up, [M, K] with row stride ldu
   int64_t ldu;
   float* mse;                   // STATS kernels: [M, K/32] per-group quantisation error instead of codes/scales
   int format;                   // STATS kernels: which 4-bit format (see rq::group_error), or
                                 // rq::kFormatScaleOnly: write the E8M0 byte to scales[M, K/32] and nothing else
 };
 
-// ---- the producer fused in front of the rotation (PRODUCER = 1) ------------------------------------------
+// ---- the producer fused in front of the rotation ------------------------------------------
 // The online rotation sits before down_proj (paper Sec. 4.3, "Reduced online computing"), whose input in
 // the LLaMA-family models is h = silu(gate) * up.  Computing h inside this kernel saves writing it to HBM
 // and reading it back (4 of 8.5 bytes per element).  The arithmetic is a fixed sequence of IEEE fp32
@@ -161,24 +161,104 @@ __device__ __forceinline__ uint4 swiglu_bf16x8_table(uint4 g, uint4 u, uint32_t 
   return make_uint4(h[0], h[1], h[2], h[3]);
 }
 
+// Rotate and quantise the 32 groups of one task, a lane's 64 bytes in cur (odd lanes of blocks of 64 / 128: halves
+// exchanged, see kSplit), and store codes and scale bytes (STATS: the statistic).
+template <int LOG2B, bool STATS>
+__device__ __forceinline__ void finish_task(const Params& p, const uint4 (&cur)[4], int row, int chunk, int lane) {
+  constexpr bool kSplit = LOG2B >= 6 && !STATS;
+  constexpr uint32_t cbits = rq::norm_bits<LOG2B>();
+  const int ng = (int)(p.K >> 5);
+  uint64_t P[16];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) rq::unpack_stage1(cur[j], P + 4 * j);
+  const int g = chunk * 32 + lane;
+  const bool live = row < p.M && g < ng;
+  if constexpr (kSplit) {
+    rq::fwht32_stages_2_to_8(P);
+    uint32_t wx[2], wy[2], sx, sy;
+    rq::cross_lane_split<LOG2B>(P, lane, cbits, wx, sx, wy, sy);
+    // the lanes of a block share `live` (K is a multiple of the block); this lane's 16 codes of
+    // group X and of group Y are 8 bytes each, at byte (lane & 1) * 8 of the group's 16
+    const int gb = chunk * 32 + (LOG2B == 6 ? (lane & ~1) : (lane & ~3));
+    const int gx = gb + (LOG2B == 6 ? 0 : ((lane >> 1) & 1));
+    const int gy = gx + (LOG2B == 6 ? 1 : 2);
+    if (live) {
+      uint8_t* rowp = p.codes + (int64_t)row * (p.K >> 1) + (lane & 1) * 8;
+      *reinterpret_cast<uint2*>(rowp + (int64_t)gx * 16) = make_uint2(wx[0], wx[1]);
+      *reinterpret_cast<uint2*>(rowp + (int64_t)gy * 16) = make_uint2(wy[0], wy[1]);
+    }
+    // scale bytes of groups 4j..4j+3 -> one 32-bit word in the lane with lane % 4 == 0
+    uint32_t sb;
+    if (LOG2B == 6) {
+      const uint32_t mine = live ? (sx | (sy << 8)) : 0u;          // groups (2i, 2i+1) of this lane pair
+      sb = mine | (__shfl_xor_sync(0xFFFFFFFFu, mine, 2) << 16);
+    } else {
+      const uint32_t mine = live ? (sx | (sy << 16)) : 0u;         // groups (0, 2) or (1, 3) of the block
+      sb = mine | (__shfl_xor_sync(0xFFFFFFFFu, mine, 2) << 8);
+    }
+    if ((lane & 3) == 0 && g < p.groups_padded) {
+      if (p.layout == BRO_LAYOUT_GEMM) {
+        const int64_t off = ((int64_t)(row >> 7) * p.scale_kblocks + (g >> 2)) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4;
+        *reinterpret_cast<uint32_t*>(p.scales + off) = sb;
+      } else if (row < p.M && g < ng) {
+        // (ng is a multiple of 2 or 4 here, so the 4 groups of this word exist whenever g + 4 <= ng)
+        uint8_t* dst = p.scales + (int64_t)row * ng + g;
+        if (g + 4 <= ng && (reinterpret_cast<uintptr_t>(dst) & 3) == 0) {
+          *reinterpret_cast<uint32_t*>(dst) = sb;
+        } else {
+          for (int i = 0; i < 4 && g + i < ng; ++i) dst[i] = (uint8_t)(sb >> (8 * i));
+        }
+      }
+    }
+    return;
+  }
+  if constexpr (LOG2B >= 5) rq::fwht32_stages_2_to_16(P);
+  else rq::fwht32_stages_below<LOG2B>(P);          // a rotation inside the MX group stops early
+  if (LOG2B >= 6) rq::cross_lane_stage(P, 1, (lane & 1) != 0);
+  if (LOG2B >= 7) rq::cross_lane_stage(P, 2, (lane & 2) != 0);
+  if (STATS) {
+    if (p.format == rq::kFormatScaleOnly) {
+      const uint32_t sbyte = rq::group_scale_byte(P, cbits);
+      if (live) p.scales[(int64_t)row * ng + g] = (uint8_t)sbyte;
+    } else {
+      const float e = rq::group_error(P, cbits, p.format);
+      if (live) p.mse[(int64_t)row * ng + g] = e;
+    }
+    return;
+  }
+  uint32_t w[4];
+  const uint32_t s = rq::quantize_group(P, cbits, w);
+  if (live)
+    *reinterpret_cast<uint4*>(p.codes + (int64_t)row * (p.K >> 1) + (int64_t)g * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+  // scale bytes of 4 consecutive groups -> one 32-bit word in the lane with g % 4 == 0
+  uint32_t sb = live ? s : 0u;
+  sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 1) << 8;
+  sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 2) << 16;
+  if ((lane & 3) == 0 && g < p.groups_padded) {
+    if (p.layout == BRO_LAYOUT_GEMM) {
+      // 512-byte block (row / 128, g / 4): byte (r % 32) * 16 + ((r % 128) / 32) * 4 + g % 4
+      const int64_t off = ((int64_t)(row >> 7) * p.scale_kblocks + (g >> 2)) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4;
+      *reinterpret_cast<uint32_t*>(p.scales + off) = sb;
+    } else if (row < p.M) {
+      uint8_t* dst = p.scales + (int64_t)row * ng + g;
+      if (g + 4 <= ng && (reinterpret_cast<uintptr_t>(dst) & 3) == 0) {
+        *reinterpret_cast<uint32_t*>(dst) = sb;
+      } else {
+        for (int i = 0; i < 4 && g + i < ng; ++i) dst[i] = (uint8_t)(sb >> (8 * i));
+      }
+    }
+  }
+}
+
 // STATS: nothing is quantised to memory; the kernel writes the per-group quantisation error
 // (rq::group_error) — the analysis behind the paper's regular-block / outlier-block comparison.
-// PRODUCER: the rotated tensor is h = silu(x) * up, computed here from the two bf16 inputs with the sigmoid table, which
-// every CTA fills before it waits for the kernel in front.
-template <int LOG2B, bool SIGNS, bool STATS, bool PRODUCER = false>
-__global__ void __launch_bounds__(kThreads, PRODUCER ? 2 : 3)      // (three CTAs of PRODUCER: 66 instead of 63 us)
+template <int LOG2B, bool SIGNS, bool STATS>
+__global__ void __launch_bounds__(kThreads, 3)
 rotate_quantize_direct_kernel(const Params p) {
   const int lane = threadIdx.x & 31;
   const int num_warps = (int)gridDim.x * kWarps;
   const int ng = (int)(p.K >> 5);
-  constexpr uint32_t cbits = rq::norm_bits<LOG2B>();
 
-  __shared__ float sigmoid_table[PRODUCER ? 2 * kSigmoidEntries : 1];
-  const uint32_t table = smem_u32(sigmoid_table);
-  if (PRODUCER) {
-    fill_sigmoid_table(sigmoid_table, (int)threadIdx.x, kThreads);
-    __syncthreads();
-  }
   griddep_wait();               // x may be written, codes/scales still read, by the kernel before
   // (only now: a dependent that starts early may then rely on everything older than this kernel)
   griddep_launch_dependents();
@@ -192,18 +272,13 @@ rotate_quantize_direct_kernel(const Params p) {
   constexpr bool kSplit = LOG2B >= 6 && !STATS;
   const int hswz = (kSplit && (lane & 1)) ? 2 : 0;
 
-  auto load = [&](int r, int c, uint4 (&q)[4], uint4 (&qu)[4]) {
+  auto load = [&](int r, int c, uint4 (&q)[4]) {
     const int g = c * 32 + lane;
     if (r < p.M && g < ng) {
       const uint4* src = reinterpret_cast<const uint4*>(p.x + (int64_t)r * p.ldx + (int64_t)g * 32);
 #pragma unroll
       for (int j = 0; j < 4; ++j) q[j] = __ldg(src + (j ^ hswz));
-      if (PRODUCER) {
-        const uint4* usrc = reinterpret_cast<const uint4*>(p.up + (int64_t)r * p.ldu + (int64_t)g * 32);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) qu[j] = __ldg(usrc + (j ^ hswz));
-      }
-      if (SIGNS && !PRODUCER) {
+      if (SIGNS) {
         const uint4* sp = reinterpret_cast<const uint4*>(p.signs + (int64_t)g * 32);
 #pragma unroll
         for (int j = 0; j < 4; ++j) q[j] = rq::apply_signs(q[j], __ldg(sp + (j ^ hswz)));
@@ -211,128 +286,131 @@ rotate_quantize_direct_kernel(const Params p) {
     } else {
 #pragma unroll
       for (int j = 0; j < 4; ++j) q[j] = make_uint4(0u, 0u, 0u, 0u);   // padding quantises to zeros
-      if (PRODUCER) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) qu[j] = make_uint4(0u, 0u, 0u, 0u);   // (silu(0) * 0 = 0)
-      }
     }
   };
 
-  uint4 cur[4], nxt[4], cur_u[4], nxt_u[4];
-  if (task < p.total_tasks) load(row, chunk, cur, cur_u);
+  uint4 cur[4], nxt[4];
+  if (task < p.total_tasks) load(row, chunk, cur);
   while (task < p.total_tasks) {
     // the next task of this warp: issue its loads now, use them in the next iteration
     const int ntask = task + num_warps;
     int nrow = row + step_row, nchunk = chunk + step_chunk;
     if (nchunk >= p.chunks_per_row) { nchunk -= p.chunks_per_row; ++nrow; }
-    if (ntask < p.total_tasks) load(nrow, nchunk, nxt, nxt_u);
+    if (ntask < p.total_tasks) load(nrow, nchunk, nxt);
 
-    if (PRODUCER) {
-      // h = silu(gate) * up, rounded to bf16: from here on the kernel is the plain one on h
+    finish_task<LOG2B, STATS>(p, cur, row, chunk, lane);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) cur[j] = swiglu_bf16x8_table(cur[j], cur_u[j], table);
-      if (SIGNS && row < p.M && chunk * 32 + lane < ng) {
-        const uint4* sp = reinterpret_cast<const uint4*>(p.signs + (int64_t)(chunk * 32 + lane) * 32);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) cur[j] = rq::apply_signs(cur[j], __ldg(sp + (j ^ hswz)));
-      }
-    }
-
-    uint64_t P[16];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) rq::unpack_stage1(cur[j], P + 4 * j);
-    const int g = chunk * 32 + lane;
-    const bool live = row < p.M && g < ng;
-    if constexpr (kSplit) {
-      rq::fwht32_stages_2_to_8(P);
-      uint32_t wx[2], wy[2], sx, sy;
-      rq::cross_lane_split<LOG2B>(P, lane, cbits, wx, sx, wy, sy);
-      // the lanes of a block share `live` (K is a multiple of the block); this lane's 16 codes of
-      // group X and of group Y are 8 bytes each, at byte (lane & 1) * 8 of the group's 16
-      const int gb = chunk * 32 + (LOG2B == 6 ? (lane & ~1) : (lane & ~3));
-      const int gx = gb + (LOG2B == 6 ? 0 : ((lane >> 1) & 1));
-      const int gy = gx + (LOG2B == 6 ? 1 : 2);
-      if (live) {
-        uint8_t* rowp = p.codes + (int64_t)row * (p.K >> 1) + (lane & 1) * 8;
-        *reinterpret_cast<uint2*>(rowp + (int64_t)gx * 16) = make_uint2(wx[0], wx[1]);
-        *reinterpret_cast<uint2*>(rowp + (int64_t)gy * 16) = make_uint2(wy[0], wy[1]);
-      }
-      // scale bytes of groups 4j..4j+3 -> one 32-bit word in the lane with lane % 4 == 0
-      uint32_t sb;
-      if (LOG2B == 6) {
-        const uint32_t mine = live ? (sx | (sy << 8)) : 0u;          // groups (2i, 2i+1) of this lane pair
-        sb = mine | (__shfl_xor_sync(0xFFFFFFFFu, mine, 2) << 16);
-      } else {
-        const uint32_t mine = live ? (sx | (sy << 16)) : 0u;         // groups (0, 2) or (1, 3) of the block
-        sb = mine | (__shfl_xor_sync(0xFFFFFFFFu, mine, 2) << 8);
-      }
-      if ((lane & 3) == 0 && g < p.groups_padded) {
-        if (p.layout == BRO_LAYOUT_GEMM) {
-          const int64_t off = ((int64_t)(row >> 7) * p.scale_kblocks + (g >> 2)) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4;
-          *reinterpret_cast<uint32_t*>(p.scales + off) = sb;
-        } else if (row < p.M && g < ng) {
-          // (ng is a multiple of 2 or 4 here, so the 4 groups of this word exist whenever g + 4 <= ng)
-          uint8_t* dst = p.scales + (int64_t)row * ng + g;
-          if (g + 4 <= ng && (reinterpret_cast<uintptr_t>(dst) & 3) == 0) {
-            *reinterpret_cast<uint32_t*>(dst) = sb;
-          } else {
-            for (int i = 0; i < 4 && g + i < ng; ++i) dst[i] = (uint8_t)(sb >> (8 * i));
-          }
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) { cur[j] = nxt[j]; if (PRODUCER) cur_u[j] = nxt_u[j]; }
-      task = ntask;
-      row = nrow;
-      chunk = nchunk;
-      continue;
-    }
-    if constexpr (LOG2B >= 5) rq::fwht32_stages_2_to_16(P);
-    else rq::fwht32_stages_below<LOG2B>(P);          // a rotation inside the MX group stops early
-    if (LOG2B >= 6) rq::cross_lane_stage(P, 1, (lane & 1) != 0);
-    if (LOG2B >= 7) rq::cross_lane_stage(P, 2, (lane & 2) != 0);
-    if (STATS) {
-      if (p.format == rq::kFormatScaleOnly) {
-        const uint32_t sbyte = rq::group_scale_byte(P, cbits);
-        if (live) p.scales[(int64_t)row * ng + g] = (uint8_t)sbyte;
-      } else {
-        const float e = rq::group_error(P, cbits, p.format);
-        if (live) p.mse[(int64_t)row * ng + g] = e;
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) { cur[j] = nxt[j]; if (PRODUCER) cur_u[j] = nxt_u[j]; }
-      task = ntask;
-      row = nrow;
-      chunk = nchunk;
-      continue;
-    }
-    uint32_t w[4];
-    const uint32_t s = rq::quantize_group(P, cbits, w);
-    if (live)
-      *reinterpret_cast<uint4*>(p.codes + (int64_t)row * (p.K >> 1) + (int64_t)g * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-    // scale bytes of 4 consecutive groups -> one 32-bit word in the lane with g % 4 == 0
-    uint32_t sb = live ? s : 0u;
-    sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 1) << 8;
-    sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 2) << 16;
-    if ((lane & 3) == 0 && g < p.groups_padded) {
-      if (p.layout == BRO_LAYOUT_GEMM) {
-        // 512-byte block (row / 128, g / 4): byte (r % 32) * 16 + ((r % 128) / 32) * 4 + g % 4
-        const int64_t off = ((int64_t)(row >> 7) * p.scale_kblocks + (g >> 2)) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4;
-        *reinterpret_cast<uint32_t*>(p.scales + off) = sb;
-      } else if (row < p.M) {
-        uint8_t* dst = p.scales + (int64_t)row * ng + g;
-        if (g + 4 <= ng && (reinterpret_cast<uintptr_t>(dst) & 3) == 0) {
-          *reinterpret_cast<uint32_t*>(dst) = sb;
-        } else {
-          for (int i = 0; i < 4 && g + i < ng; ++i) dst[i] = (uint8_t)(sb >> (8 * i));
-        }
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) { cur[j] = nxt[j]; if (PRODUCER) cur_u[j] = nxt_u[j]; }
+    for (int j = 0; j < 4; ++j) cur[j] = nxt[j];
     task = ntask;
     row = nrow;
     chunk = nchunk;
+  }
+}
+
+// ---- the fused producer -----------------------------------------------------------------------------------------------
+// The same tasks on h = silu(gate) * up (see sigmoid2).  A warp's 2 x 2 KiB arrive by TMA in a ring of its own in shared memory
+// (one box of 32 groups of a row each, 64-byte swizzle, a barrier per stage, nothing shared with other warps).  What bounds this
+// kernel is the L1 data path, the table's gathers above all: a warp-wide 16-byte global load whose lanes are 64 bytes apart
+// takes 16 passes of it, eight of them a task, the same read of the swizzled ring 4.  [16384, 4096], block 32: loads into
+// registers 63.5 us, ring 54.5; [512, 8192] 6.8 -> 6.2.  (Without a producer the ring is slower, 28 -> 34 us: the plain
+// kernel is bound by issue, and requesting and waiting cost a quarter of its instructions.  128-byte segments: no difference.)
+struct Ring {
+  static constexpr int kStages = 2;
+  static constexpr int kBoxBytes = 2048;
+  static constexpr int kStageBytes = 2 * kBoxBytes;                        // gate and up
+  static constexpr int kTableAt = kWarps * kStages * kStageBytes;
+  static constexpr int kBarAt = kTableAt + 2 * (int)kSigmoidEntries * 4;
+  static constexpr int kSmemBytes = kBarAt + kWarps * kStages * 8 + 1024 /*alignment*/;
+};
+
+__device__ __forceinline__ void tma_load_3d_elect(uint32_t dst, const CUtensorMap* m, int x, int y, int z, uint32_t bar) {
+  asm volatile(
+      "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
+      "@q cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4}], [%5]; }" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(z), "r"(bar)
+      : "memory");
+}
+
+template <int LOG2B, bool SIGNS>
+__global__ void __launch_bounds__(kThreads, 2)
+rotate_quantize_gated_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmu, const Params p) {
+  using R = Ring;
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const int lane = threadIdx.x & 31, warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);
+  const uint32_t ring = base + (uint32_t)(warp * R::kStages * R::kStageBytes), bars = base + R::kBarAt + (uint32_t)(warp * R::kStages * 8);
+  const uint32_t table = base + R::kTableAt;
+  const int ng = (int)(p.K >> 5);
+  if (lane == 0) {
+    for (int s = 0; s < R::kStages; ++s) mbar_init(bars + 8 * s, 1);
+    mbar_fence_init();
+    fence_proxy_async_smem();
+    tma_prefetch_desc(&tmx);
+    tma_prefetch_desc(&tmu);
+  }
+  fill_sigmoid_table(reinterpret_cast<float*>(smem_raw + (table - smem_u32(smem_raw))), (int)threadIdx.x, kThreads);
+  __syncthreads();
+  griddep_wait();               // x may be written, codes/scales still read, by the kernel before
+  griddep_launch_dependents();  // (only now: see the direct form)
+
+  const int num_warps = (int)gridDim.x * kWarps;
+  int task = (int)blockIdx.x * kWarps + warp;
+  int row = task / p.chunks_per_row, chunk = task - row * p.chunks_per_row;
+  const int step_row = num_warps / p.chunks_per_row, step_chunk = num_warps - step_row * p.chunks_per_row;
+  auto advance = [&](int& t, int& r, int& c) {
+    t += num_warps;
+    r += step_row;
+    c += step_chunk;
+    if (c >= p.chunks_per_row) { c -= p.chunks_per_row; ++r; }
+  };
+  auto loads = [&](int r, int c) { return r < p.M && c * 32 < ng; };      // (padding tasks bring nothing)
+  int atask = task, arow = row, achunk = chunk;                           // the next task to request
+  auto request = [&](int stage) {
+    while (atask < p.total_tasks && !loads(arow, achunk)) advance(atask, arow, achunk);
+    if (atask >= p.total_tasks) return false;
+    const uint32_t bar = bars + 8 * stage, dst = ring + (uint32_t)(stage * R::kStageBytes);
+    mbar_arrive_expect_tx_elect(bar, R::kStageBytes);
+    tma_load_3d_elect(dst, &tmx, 0, achunk * 32, arow, bar);
+    tma_load_3d_elect(dst + R::kBoxBytes, &tmu, 0, achunk * 32, arow, bar);
+    advance(atask, arow, achunk);
+    return true;
+  };
+  int in_flight = 0;
+  for (int s = 0; s < R::kStages; ++s) in_flight += request(s) ? 1 : 0;
+
+  const uint32_t hswz = (LOG2B >= 6 && (lane & 1)) ? 2u : 0u;            // (see kSplit)
+  const uint32_t swz = ((uint32_t)lane >> 1) & 3u;                        // 64-byte swizzle: piece ^ (64-byte row / 2) mod 4
+  int stage = 0;
+  uint32_t phase = 0;
+  for (; task < p.total_tasks; advance(task, row, chunk)) {
+    uint4 cur[4];
+    if (loads(row, chunk)) {
+      if (!mbar_wait_warp(bars + 8 * stage, phase, SITE_RQ_FULL)) break;
+      const uint32_t src = ring + (uint32_t)(stage * R::kStageBytes) + (uint32_t)lane * 64u;
+#pragma unroll
+      for (uint32_t j = 0; j < 4; ++j) {                                  // (zeros beyond K: silu(0) * 0 = 0)
+        const uint32_t at = src + (((j ^ hswz) ^ swz) << 4);
+        cur[j] = swiglu_bf16x8_table(lds128(at), lds128(at + R::kBoxBytes), table);
+      }
+      __syncwarp();
+      in_flight += request(stage) ? 0 : -1;
+      if (++stage == R::kStages) { stage = 0; phase ^= 1u; }
+      if (SIGNS && chunk * 32 + lane < ng) {
+        const uint4* sp = reinterpret_cast<const uint4*>(p.signs + (int64_t)(chunk * 32 + lane) * 32);
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) cur[j] = rq::apply_signs(cur[j], __ldg(sp + (j ^ hswz)));
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) cur[j] = make_uint4(0u, 0u, 0u, 0u);    // padding quantises to zeros
+    }
+    finish_task<LOG2B, false>(p, cur, row, chunk, lane);
+  }
+  // (only after a lost wait is anything left: do not leave while copies may still land, wait once more for each stage)
+  for (; in_flight > 0; --in_flight) {
+    mbar_wait_warp(bars + 8 * stage, phase, SITE_RQ_DRAIN);
+    if (++stage == R::kStages) { stage = 0; phase ^= 1u; }
   }
 }
 
@@ -343,9 +421,12 @@ inline bool supports(int64_t M, int64_t K, bro_layout layout, int64_t scale_kblo
   return rows * ((groups + 31) / 32) < ((int64_t)1 << 30);
 }
 
-template <int LOG2B, bool SIGNS, bool STATS, bool PRODUCER = false>
+// x as a 3-D tensor {32 bf16 (one group), K / 32 groups, M rows}, box = 32 groups of a row, 64-byte swizzle.
+bro_status make_group_map(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx);
+
+template <int LOG2B, bool SIGNS, bool STATS>
 inline bro_status launch_one(Params& p, int sm_count, cudaStream_t st) {
-  auto kernel = rotate_quantize_direct_kernel<LOG2B, SIGNS, STATS, PRODUCER>;
+  auto kernel = rotate_quantize_direct_kernel<LOG2B, SIGNS, STATS>;
   static DeviceOnce once;            // (one per template instantiation)
   int blocks_per_sm = 1;
   const bro_status rc = device_once(once, &blocks_per_sm, [&](int* n) {
@@ -361,39 +442,58 @@ inline bro_status launch_one(Params& p, int sm_count, cudaStream_t st) {
                                                                                                        : BRO_ERR_CUDA;
 }
 
-template <bool STATS, bool PRODUCER = false>
-inline bro_status launch_any(Params& p, int log2b, int sm_count, cudaStream_t st) {
+template <int LOG2B, bool SIGNS>
+inline bro_status launch_gated(Params& p, int sm_count, cudaStream_t st) {
+  using R = Ring;
+  auto kernel = rotate_quantize_gated_kernel<LOG2B, SIGNS>;
+  static DeviceOnce once;            // (one per template instantiation)
+  int blocks_per_sm = 1;
+  bro_status rc = device_once(once, &blocks_per_sm, [&](int* n) {
+    return cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, R::kSmemBytes),
+                   "cudaFuncSetAttribute(rotate_quantize_gated)") &&
+                   cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kernel, kThreads, R::kSmemBytes),
+                           "occupancy(rotate_quantize_gated)")
+               ? BRO_OK
+               : BRO_ERR_CUDA;
+  });
+  if (rc != BRO_OK) return rc;
+  CUtensorMap tmx, tmu;
+  rc = make_group_map(&tmx, p.x, p.M, p.K, p.ldx);
+  if (rc != BRO_OK) return rc;
+  rc = make_group_map(&tmu, p.up, p.M, p.K, p.ldu);
+  if (rc != BRO_OK) return rc;
+  const int64_t want = ((int64_t)p.total_tasks + kWarps - 1) / kWarps, cap = (int64_t)sm_count * blocks_per_sm;
+  return cuda_ok(launch_kernel(kernel, (unsigned)(want < cap ? want : cap), kThreads, R::kSmemBytes, st, 1, tmx, tmu, p),
+                 "rotate_quantize_gated launch")
+             ? BRO_OK
+             : BRO_ERR_CUDA;
+}
+
+template <bool SIGNS, bool STATS, bool GATED, int LOG2B>
+inline bro_status launch_of(Params& p, int sm_count, cudaStream_t st) {
+  if constexpr (GATED) return launch_gated<LOG2B, SIGNS>(p, sm_count, st);
+  else return launch_one<LOG2B, SIGNS, STATS>(p, sm_count, st);
+}
+template <bool SIGNS, bool STATS, bool GATED>
+inline bro_status launch_size(Params& p, int log2b, int sm_count, cudaStream_t st) {
   if constexpr (!STATS) {       // rotations inside the MX group (blocks of 2..16): the quantising kernels only
-    if (p.signs) {
-      switch (log2b) {
-        case 1: return launch_one<1, true, false, PRODUCER>(p, sm_count, st);
-        case 2: return launch_one<2, true, false, PRODUCER>(p, sm_count, st);
-        case 3: return launch_one<3, true, false, PRODUCER>(p, sm_count, st);
-        case 4: return launch_one<4, true, false, PRODUCER>(p, sm_count, st);
-        default: break;
-      }
-    } else {
-      switch (log2b) {
-        case 1: return launch_one<1, false, false, PRODUCER>(p, sm_count, st);
-        case 2: return launch_one<2, false, false, PRODUCER>(p, sm_count, st);
-        case 3: return launch_one<3, false, false, PRODUCER>(p, sm_count, st);
-        case 4: return launch_one<4, false, false, PRODUCER>(p, sm_count, st);
-        default: break;
-      }
-    }
-  }
-  if (p.signs) {
     switch (log2b) {
-      case 5: return launch_one<5, true, STATS, PRODUCER>(p, sm_count, st);
-      case 6: return launch_one<6, true, STATS, PRODUCER>(p, sm_count, st);
-      default: return launch_one<7, true, STATS, PRODUCER>(p, sm_count, st);
+      case 1: return launch_of<SIGNS, STATS, GATED, 1>(p, sm_count, st);
+      case 2: return launch_of<SIGNS, STATS, GATED, 2>(p, sm_count, st);
+      case 3: return launch_of<SIGNS, STATS, GATED, 3>(p, sm_count, st);
+      case 4: return launch_of<SIGNS, STATS, GATED, 4>(p, sm_count, st);
+      default: break;
     }
   }
   switch (log2b) {
-    case 5: return launch_one<5, false, STATS, PRODUCER>(p, sm_count, st);
-    case 6: return launch_one<6, false, STATS, PRODUCER>(p, sm_count, st);
-    default: return launch_one<7, false, STATS, PRODUCER>(p, sm_count, st);
+    case 5: return launch_of<SIGNS, STATS, GATED, 5>(p, sm_count, st);
+    case 6: return launch_of<SIGNS, STATS, GATED, 6>(p, sm_count, st);
+    default: return launch_of<SIGNS, STATS, GATED, 7>(p, sm_count, st);
   }
+}
+template <bool STATS, bool GATED = false>
+inline bro_status launch_any(Params& p, int log2b, int sm_count, cudaStream_t st) {
+  return p.signs ? launch_size<true, STATS, GATED>(p, log2b, sm_count, st) : launch_size<false, STATS, GATED>(p, log2b, sm_count, st);
 }
 
 // `up` != nullptr: x is the gate and the rotated tensor is silu(x) * up (the fused producer).
