@@ -166,14 +166,16 @@ __global__ void __launch_bounds__(kScanThreads, 1) outlier_scan(const uint16_t* 
   // keep their place in a row, and a warp that always met them finished a third later than the others.
   const int64_t step = (int64_t)gridDim.x * kScanThreads;
   GroupWalk at((int64_t)blockIdx.x * kScanThreads, step, ng);       // the CTA's first group
-  const uint32_t magic = ng < kScanThreads ? (uint32_t)((0x100000000ull + ng - 1) / ng) : 0u;
+  // (ceil(2^32 / ng) does not fit 32 bits for rows of one group)
+  const uint32_t magic = ng > 1 && ng < kScanThreads ? (uint32_t)((0x100000000ull + ng - 1) / ng) : 0u;
   {
     uint4 nxt[4];                                     // the next group's 64 bytes, in flight while this one is counted
     int place = (int)threadIdx.x;
     auto load = [&] {
-      // (at.g + place) / ng is 0 or 1 for long rows; for short ones the product with ceil(2^32 / ng) is exact
+      // (at.g + place) / ng is 0 or 1 for long rows; for short ones the product with ceil(2^32 / ng) is exact; a row of
+      // one group is its own quotient
       const uint32_t v = (uint32_t)at.g + (uint32_t)place;
-      const uint32_t over = magic ? __umulhi(v, magic) : (v >= (uint32_t)ng ? 1u : 0u);
+      const uint32_t over = magic ? __umulhi(v, magic) : (ng == 1 ? v : (v >= (uint32_t)ng ? 1u : 0u));
       const uint4* src = reinterpret_cast<const uint4*>(x + (at.row + over) * ldx + (int64_t)(v - over * (uint32_t)ng) * 32);
 #pragma unroll
       for (int j = 0; j < 4; ++j) nxt[j] = __ldg(src + j);

@@ -189,6 +189,20 @@ def test_outlier_threshold_from_a_sample(bro, case):
     assert np.array_equal(np.asarray(mask.cpu() if hasattr(mask, "cpu") else mask), want)
 
 
+@pytest.mark.parametrize("M,K,ldx", [(60, 32, 40), (5000, 32, 40), (4100, 32, 64), (3000, 32, 32), (2500, 64, 72), (1500, 96, 136)])
+def test_outlier_groups_of_rows_of_few_groups_with_a_row_stride(bro, M, K, ldx):
+    """Rows of one, two and three groups whose gaps hold the largest values of the buffer: a group read at a wrong row
+    or column shows in the threshold and in the mask.  Bit for bit against a sort."""
+    buf = torch.full((M, ldx), 1.0e20, dtype=torch.bfloat16)
+    buf[:, :K] = synth.activations(M, K, seed=M, recipe=synth.HEAVY_RECIPE)
+    mag = (buf[:, :K].contiguous().view(torch.int16).int() & 0x7FFF)
+    k = -(-M * K // 1000)
+    t = int(torch.sort(mag.flatten(), descending=True).values[k - 1])
+    mask, info = gpu_outliers(bro, buf.cuda()[:, :K], 1000)
+    assert int(info[0]) == t and int(info[2]) == k
+    assert torch.equal(mask.cpu(), (mag.view(M, K // 32, 32).amax(2) >= t).to(torch.uint8))
+
+
 @pytest.mark.parametrize("n", [1, 15, 65536, 65537, 300001])
 @pytest.mark.parametrize("offset", [0, 3])
 def test_counts_of_bytes_at_any_alignment(bro, n, offset):
