@@ -681,6 +681,12 @@ bro_status bro_gemm_mxfp4_ex(const void* acodes, const void* ascales, const void
                    stream, false);
 }
 
+// Whether [a, a + na) and [b, b + nb) share a byte.
+static bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+  const uintptr_t pa = reinterpret_cast<uintptr_t>(a), pb = reinterpret_cast<uintptr_t>(b);
+  return pa < pb + nb && pb < pa + na;
+}
+
 static bro_status linear_impl(const void* x_bf16, int64_t M, int64_t K, int64_t ldx, int block, const void* signs,
                               const void* wcodes, const void* wscales, int64_t N, void* y_bf16, int64_t ldy,
                               void* workspace, size_t workspace_bytes, uint32_t flags, void* stream) {
@@ -694,7 +700,11 @@ static bro_status linear_impl(const void* x_bf16, int64_t M, int64_t K, int64_t 
   uint8_t* ascales = acodes + align_up(bro_codes_bytes(M, K), 1024);
   uint8_t* gws = ascales + align_up(bro_scales_bytes(M, K, BRO_LAYOUT_GEMM), 1024);
   bro_status rc;
-  if (flags == 0 && block != 0) {        // few tokens: one kernel for both steps, where its plan says so
+  // Few tokens: one kernel for both steps, where its plan says so.  Its CTAs read x (and the signs) while others already
+  // store y, so a layer in place keeps the two kernels, of which the first has read all of x when the second writes.
+  const size_t y_bytes = ((size_t)(M - 1) * ldy + N) * 2;
+  if (flags == 0 && block != 0 && !overlap(x_bf16, ((size_t)(M - 1) * ldx + K) * 2, y_bf16, y_bytes) &&
+      !(signs && overlap(signs, (size_t)K * 2, y_bf16, y_bytes))) {
     rc = check_rotate_quantize(x_bf16, M, K, ldx, block, signs, acodes, ascales, BRO_LAYOUT_GEMM, nullptr, 0);
     if (rc == BRO_OK)
       rc = check_gemm(acodes, ascales, wcodes, wscales, M, N, K, y_bf16, ldy, BRO_OUT_BF16, gws, bro_gemm_workspace_bytes(M, N, K));

@@ -92,3 +92,34 @@ def test_layer_of_few_tokens_same_bytes_as_two_kernels(bro, M, K, N, block, sign
     bro.gemm_mxfp4(ac, asc, wc, wsc, M, N, K, ref, flags=bro.FLAG_GEMM_SINGLE)
     top = ref.float().abs().amax(1, keepdim=True)
     assert ((y.float() - ref.float()).abs() <= top * 2.0 ** -8).all()
+
+
+@pytest.mark.parametrize("M,K,N,shift", [
+    (16, 2048, 2048, 0),       # y is x
+    (16, 2048, 2048, 8),       # y starts 8 elements into x, in rows of the same stride
+    (3, 1024, 1000, 0),        # fewer columns than x has
+    (1, 4096, 4096, 0),
+])
+@pytest.mark.parametrize("signs", [False, True])
+def test_layer_of_few_tokens_in_place(bro, M, K, N, shift, signs):
+    """y over x: the layer is rotate + quantise and then the GEMM, so all of x has been read when y is written.  The same
+    bits as the two calls give with an output of its own (the GEMM is the same kernel)."""
+    gen = torch.Generator(device="cuda").manual_seed(M + K + shift)
+    ld = K + 16
+    buf = torch.randn(M, ld, generator=gen, device="cuda").to(torch.bfloat16)
+    x, y = buf[:, :K], buf[:, shift:shift + N]
+    w = torch.randn(N, K, generator=gen, device="cuda").to(torch.bfloat16)
+    s = (1 - 2 * torch.randint(0, 2, (K,), generator=gen, device="cuda")).to(torch.bfloat16) if signs else None
+    wc, wsc = bro.alloc_codes(N, K), bro.alloc_scales(N, K, bro.LAYOUT_GEMM)
+    bro.pack_weights_rs(w, 32, s, wc, wsc) if signs else bro.pack_weights(w, 32, wc, wsc)
+    ac, asc = bro.alloc_codes(M, K), bro.alloc_scales(M, K, bro.LAYOUT_GEMM)
+    bro.rotate_quantize_mxfp4(x, 32, ac, asc, signs=s)
+    want = torch.empty(M, N, dtype=torch.bfloat16, device="cuda")
+    bro.gemm_mxfp4(ac, asc, wc, wsc, M, N, K, want)
+    around = buf.clone()
+    work = bro.alloc_workspace(bro.linear_workspace_bytes(M, N, K))
+    bro.linear_rs(x, 32, s, wc, wsc, N, y, work) if signs else bro.linear(x, 32, wc, wsc, N, y, work)
+    assert bro.last_device_status() == 0
+    assert torch.equal(y, want)
+    around[:, shift:shift + N] = want
+    assert torch.equal(buf, around)
