@@ -273,26 +273,26 @@ bro_status launch_rotate_quantize(const void* x, int64_t M, int64_t K, int64_t l
 
   // (All six instantiations share one function-pointer type, so the opt-in to large dynamic
   // shared memory is kept per instantiation, per device.)
-  auto go = [&](void (*kernel)(CUtensorMap, Params), int threads, int which) -> bro_status {
+  auto go = [&](void (*kernel)(CUtensorMap, Params), int which) -> bro_status {
     static bro::DeviceOnce once[6];
     bro_status r = bro::device_once(once[which], nullptr, [&](int*) { return set_smem(kernel, bro::rq::kSmemBytes); });
     if (r != BRO_OK) return r;
-    return bro::cuda_ok(bro::launch_kernel(kernel, (unsigned)grid, (unsigned)threads, bro::rq::kSmemBytes, st, 1, tmx, p),
+    return bro::cuda_ok(bro::launch_kernel(kernel, (unsigned)grid, bro::rq::kThreads, bro::rq::kSmemBytes, st, 1, tmx, p),
                         "rotate_quantize launch")
                ? BRO_OK
                : BRO_ERR_CUDA;
   };
   if (signs) {
     switch (B) {
-      case 32: return go(bro::rq::rotate_quantize_kernel<5, true>, bro::rq::Teams<5>::kThreads, 3);
-      case 64: return go(bro::rq::rotate_quantize_kernel<6, true>, bro::rq::Teams<6>::kThreads, 4);
-      default: return go(bro::rq::rotate_quantize_kernel<7, true>, bro::rq::Teams<7>::kThreads, 5);
+      case 32: return go(bro::rq::rotate_quantize_kernel<5, true>, 3);
+      case 64: return go(bro::rq::rotate_quantize_kernel<6, true>, 4);
+      default: return go(bro::rq::rotate_quantize_kernel<7, true>, 5);
     }
   }
   switch (B) {
-    case 32: return go(bro::rq::rotate_quantize_kernel<5, false>, bro::rq::Teams<5>::kThreads, 0);
-    case 64: return go(bro::rq::rotate_quantize_kernel<6, false>, bro::rq::Teams<6>::kThreads, 1);
-    default: return go(bro::rq::rotate_quantize_kernel<7, false>, bro::rq::Teams<7>::kThreads, 2);
+    case 32: return go(bro::rq::rotate_quantize_kernel<5, false>, 0);
+    case 64: return go(bro::rq::rotate_quantize_kernel<6, false>, 1);
+    default: return go(bro::rq::rotate_quantize_kernel<7, false>, 2);
   }
 }
 

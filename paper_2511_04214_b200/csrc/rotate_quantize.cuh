@@ -5,20 +5,19 @@
 //  * One persistent CTA per SM.  A producer thread streams 128-row x 128-column bf16 tiles into
 //    a ring of shared-memory stages with TMA (two 128x64 boxes per tile, 128-byte swizzle), so
 //    the loads in flight are bounded by shared memory, not by registers.
-//  * Consumer warps.  Blocks of 32 and 64: 16 warps, a thread owns one whole MX group (32 consecutive channels of one row):
-//    four conflict-free 16-byte shared loads, then the 5 butterfly stages of the 32-point Walsh-Hadamard transform entirely
-//    in registers; blocks of 64 add one stage between the lanes of the two groups.  Blocks of 128: a thread owns the whole
-//    block, four groups of a row of the tile, and all seven stages are register arithmetic; a team of four warps takes a
-//    tile and three teams take turns.  (With two stages across lanes, 32 shuffles and 32 scalar operations each,
-//    [16384, 4096] took 36.0 us and [2048, 8192] 10.6; now B128_US.  Blocks of 64 owned whole: 32.7 -> 35.9 us, not kept.)
+//  * 16 consumer warps.  Each thread owns one whole MX group (32 consecutive channels of one
+//    row): four conflict-free 16-byte shared loads, then the 5 butterfly stages of the 32-point
+//    Walsh-Hadamard transform entirely in registers — no shuffles for block = 32.  Blocks of 64
+//    and 128 add one or two cross-lane stages (the 2 or 4 groups of a block sit in lanes that
+//    differ in bit 0 / bit 3).
 //  * fp32 arithmetic in exactly this order: butterflies (a+b, a-b) with ascending stride, one
 //    multiply by c = fp32(1/sqrt(block)), amax over the group, shared exponent
 //    E = max(expfield(amax) - 2, 0) - 127, r = y * 2^-E, round-to-nearest-even to E2M1 with
 //    saturation.  The multiply by c and the exact scaling by 2^-E are merged into one multiply by
 //    c*2^-E whenever that product is a normal fp32 (bit-identical result); otherwise the two
 //    multiplies are done separately.
-//  * Output: one 16-byte store of 32 packed codes per group; the 4 scale bytes of a row inside
-//    the tile as one 32-bit store (gathered with two shuffles where four threads share them).
+//  * Output: one 16-byte store of 32 packed codes per thread; the 4 scale bytes of a row inside
+//    the tile are gathered with two shuffles and written as one 32-bit store.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -34,15 +33,8 @@ constexpr int kBoxCols = 64;                // one TMA box: 128 rows x 64 bf16 =
 constexpr int kBoxBytes = kTileRows * kBoxCols * 2;   // 16 KiB
 constexpr int kStageBytes = 2 * kBoxBytes;            // 32 KiB
 constexpr int kStages = 6;
-// Consumer warps and the teams they form, by the groups of 32 that a thread owns.
-template <int LOG2B>
-struct Teams {
-  static constexpr int kGroups = LOG2B == 7 ? 4 : 1;
-  static constexpr int kTeamWarps = 16 / kGroups;                 // 128 rows x 4 groups of a tile
-  static constexpr int kTeams = kGroups == 1 ? 1 : 3;
-  static constexpr int kConsumerWarps = kTeams * kTeamWarps;
-  static constexpr int kThreads = (kConsumerWarps + 1) * 32;      // + 1 producer warp
-};
+constexpr int kConsumerWarps = 16;
+constexpr int kThreads = (kConsumerWarps + 1) * 32;   // + 1 producer warp
 constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/;
 
 struct Params {
@@ -483,9 +475,8 @@ __device__ __forceinline__ float group_error(const uint64_t (&P)[16], uint32_t c
 // SIGNS: the randomised rotation R_i = diag(s) H / sqrt(block) (paper Sec. 5.1) — the channel signs
 // are applied to the bf16 inputs as they leave shared memory; everything else is unchanged.
 template <int LOG2B, bool SIGNS>
-__global__ void __launch_bounds__(Teams<LOG2B>::kThreads, 1)
+__global__ void __launch_bounds__(kThreads, 1)
 rotate_quantize_kernel(const __grid_constant__ CUtensorMap tmx, const Params p) {
-  using T = Teams<LOG2B>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;   // swizzle needs 1 KiB
   const uint32_t bar_base = smem_base + kStages * kStageBytes;
@@ -496,7 +487,7 @@ rotate_quantize_kernel(const __grid_constant__ CUtensorMap tmx, const Params p) 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(bar_base + 8 * s, 1);
-      mbar_init(bar_base + 8 * (kStages + s), T::kTeamWarps);
+      mbar_init(bar_base + 8 * (kStages + s), kConsumerWarps);
     }
     mbar_fence_init();
     fence_proxy_async_smem();
@@ -508,7 +499,7 @@ rotate_quantize_kernel(const __grid_constant__ CUtensorMap tmx, const Params p) 
 
   const int64_t total_tiles = p.tiles_m * p.tiles_k;
 
-  if (warp == T::kConsumerWarps) {
+  if (warp == kConsumerWarps) {
     // ---------------- producer ----------------
     if (lane == 0) {
       tma_prefetch_desc(&tmx);
@@ -545,88 +536,73 @@ rotate_quantize_kernel(const __grid_constant__ CUtensorMap tmx, const Params p) 
     }
   } else {
     // ---------------- consumers ----------------
-    const int team = warp / T::kTeamWarps, tw = warp - team * T::kTeamWarps;
-    // this thread's row of the tile and its first group there
-    const int row = T::kGroups == 1 ? tw * 8 + ((lane >> 4) << 2) + ((lane >> 1) & 3) : tw * 32 + lane;
-    const int g = T::kGroups == 1 ? ((lane >> 3) & 1) * 2 + (lane & 1) : 0;
-    // 16-byte chunk j of a group sits at chunk index ((group & 1) * 4 + j) ^ (row & 7) of its 128-B row
-    const uint32_t row_off = (uint32_t)(g >> 1) * kBoxBytes + (uint32_t)row * 128u;
+    const int gg = lane & 1;                 // group within the 64-column box
+    const int box = (lane >> 3) & 1;         // which box of the tile
+    const int row = warp * 8 + ((lane >> 4) << 2) + ((lane >> 1) & 3);   // row within the tile
+    const int g = box * 2 + gg;              // group within the tile (0..3)
+    // 16-byte chunk j of this group sits at chunk index (gg*4 + j) ^ (row & 7) of its 128-B row
+    const uint32_t row_off = (uint32_t)box * kBoxBytes + (uint32_t)row * 128u;
     const uint32_t sw = (uint32_t)(row & 7);
     constexpr uint32_t cbits = norm_bits<LOG2B>();
 
+    int stage = 0;
+    uint32_t phase = 0;
     const int tiles_k = (int)p.tiles_k;
     int tm = (int)(blockIdx.x / (unsigned)tiles_k), tk = (int)(blockIdx.x % (unsigned)tiles_k);
     const int step_m = (int)(gridDim.x / (unsigned)tiles_k), step_k = (int)(gridDim.x % (unsigned)tiles_k);
-    int stage = 0, turn = 0;
-    uint32_t phase = 0;
     for (int64_t t = blockIdx.x; t < total_tiles; t += gridDim.x) {
-      if (turn == team) {
-        if (!mbar_wait(bar_base + 8 * stage, phase, SITE_RQ_FULL)) break;
-        const uint32_t src = smem_base + stage * kStageBytes + row_off;
-        const int64_t grow = (int64_t)tm * kTileRows + row;
-        const int ggrp = tk * (kTileCols / 32) + g;         // group index along K of this thread's first group
-        const bool in_k = ggrp * 32 < (int)p.K;             // (K is a multiple of the block: the same for all of them)
-        uint64_t P[T::kGroups][16];
+      if (!mbar_wait(bar_base + 8 * stage, phase, SITE_RQ_FULL)) break;
+      const uint32_t src = smem_base + stage * kStageBytes + row_off;
+      uint64_t P[16];
+      uint4 sg[4] = {};
+      if (SIGNS && (tk * (kTileCols / 32) + g) * 32 < (int)p.K) {
+        const uint4* sp = reinterpret_cast<const uint4*>(p.signs + (tk * kTileCols + g * 32));
 #pragma unroll
-        for (int i = 0; i < T::kGroups; ++i) {
+        for (int j = 0; j < 4; ++j) sg[j] = __ldg(sp + j);
+      }
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            uint4 q = lds128(src + (uint32_t)(i >> 1) * kBoxBytes + (((((uint32_t)(g + i) & 1u) * 4u + j) ^ sw) << 4));
-            if (SIGNS && in_k) q = apply_signs(q, __ldg(reinterpret_cast<const uint4*>(p.signs + (int64_t)(ggrp + i) * 32) + j));
-            unpack_stage1(q, P[i] + 4 * j);
-          }
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_base + 8 * (kStages + stage));
+      for (int j = 0; j < 4; ++j) {
+        uint4 q = lds128(src + ((((uint32_t)gg * 4u + j) ^ sw) << 4));
+        if (SIGNS) q = apply_signs(q, sg[j]);
+        unpack_stage1(q, P + 4 * j);
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_base + 8 * (kStages + stage));
+      if (++stage == kStages) { stage = 0; phase ^= 1u; }
 
-#pragma unroll
-        for (int i = 0; i < T::kGroups; ++i) fwht32_stages_2_to_16(P[i]);
-#pragma unroll
-        for (int h = 1; h < T::kGroups; h <<= 1) {          // strides 32 and 64: between the thread's own groups
-#pragma unroll
-          for (int i = 0; i < T::kGroups; ++i) {
-            if ((i & h) == 0) {
-#pragma unroll
-              for (int k = 0; k < 16; ++k) {
-                const uint64_t a = P[i][k], b = P[i + h][k];
-                P[i][k] = add2(a, b);
-                P[i + h][k] = sub2(a, b);
-              }
-            }
-          }
-        }
-        if (LOG2B == 6) cross_lane_stage(P[0], 1, (lane & 1) != 0);
-        uint32_t sb = 0;
-#pragma unroll
-        for (int i = 0; i < T::kGroups; ++i) {
-          uint32_t w[4];
-          sb |= quantize_group(P[i], cbits, w) << (8 * i);
-          if (grow < p.M && in_k)
-            *reinterpret_cast<uint4*>(p.codes + grow * (p.K >> 1) + (int64_t)(ggrp + i) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-        if (!in_k) sb = 0u;
-        if (T::kGroups == 1) {                              // the row's 4 bytes into the lane of group 0
-          sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 1) << 8;
-          sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 8) << 16;
-        }
-        if (T::kGroups > 1 || g == 0) {
-          if (p.layout == BRO_LAYOUT_GEMM) {
-            // 512-byte block (tm, tk): byte (r%32)*16 + (r/32)*4 + g ; padding rows included
-            uint8_t* dst = p.scales + ((int64_t)tm * p.scale_kblocks + tk) * 512 + (row & 31) * 16 + (row >> 5) * 4 + g;
+      fwht32_stages_2_to_16(P);
+      if (LOG2B >= 6) cross_lane_stage(P, 1, gg != 0);
+      if (LOG2B >= 7) cross_lane_stage(P, 8, box != 0);
+
+      uint32_t w[4];
+      const uint32_t s = quantize_group(P, cbits, w);
+
+      const int64_t grow = (int64_t)tm * kTileRows + row;
+      const int ggrp = tk * (kTileCols / 32) + g;         // group index along K
+      const bool in_k = ggrp * 32 < (int)p.K;
+      if (grow < p.M && in_k) {
+        uint4* dst = reinterpret_cast<uint4*>(p.codes + grow * (p.K >> 1) + ggrp * 16);
+        *dst = make_uint4(w[0], w[1], w[2], w[3]);
+      }
+      // gather the row's 4 scale bytes of this tile into the lane with gg == 0 && box == 0
+      uint32_t sb = in_k ? s : 0u;
+      sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 1) << 8;
+      sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 8) << 16;
+      if (g == 0) {
+        if (p.layout == BRO_LAYOUT_GEMM) {
+          // 512-byte block (tm, tk): byte (r%32)*16 + (r/32)*4 + g ; padding rows included
+          const int64_t off = ((int64_t)tm * p.scale_kblocks + tk) * 512 + (row & 31) * 16 + (row >> 5) * 4;
+          *reinterpret_cast<uint32_t*>(p.scales + off) = sb;
+        } else if (grow < p.M) {
+          const int ng = (int)(p.K >> 5);
+          uint8_t* dst = p.scales + grow * ng + tk * 4;
+          if (tk * 4 + 4 <= ng && ((reinterpret_cast<uintptr_t>(dst) & 3) == 0)) {
             *reinterpret_cast<uint32_t*>(dst) = sb;
-          } else if (grow < p.M) {
-            const int ng = (int)(p.K >> 5);
-            uint8_t* dst = p.scales + grow * ng + ggrp;
-            if (ggrp + 4 <= ng && (reinterpret_cast<uintptr_t>(dst) & 3) == 0) {
-              *reinterpret_cast<uint32_t*>(dst) = sb;
-            } else {
-              for (int i = 0; i < 4 && ggrp + i < ng; ++i) dst[i] = (uint8_t)(sb >> (8 * i));
-            }
+          } else {
+            for (int i = 0; i < 4 && tk * 4 + i < ng; ++i) dst[i] = (uint8_t)(sb >> (8 * i));
           }
         }
       }
-      if (++turn == T::kTeams) turn = 0;
-      if (++stage == kStages) { stage = 0; phase ^= 1u; }
       tm += step_m;
       tk += step_k;
       if (tk >= tiles_k) { tk -= tiles_k; ++tm; }
