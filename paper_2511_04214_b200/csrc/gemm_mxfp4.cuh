@@ -86,11 +86,15 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 // ---- issuing tensor-core work --------------------------------------------------------------------
 // The issuing warp runs its loop with all 32 lanes converged, so that addresses, descriptors and loop counters
-// stay warp-uniform, and each wrapper elects the lane that executes the instruction (see the elect forms in
+// stay warp-uniform.
+// CG = 1, this CTA alone: each wrapper elects the lane that executes the instruction (see the elect forms in
 // bro_common.cuh for what that is worth).
-// CG = 1: this CTA alone; CG = 2: the CTA pair (cta_group::2), issued by the leader CTA.
+// CG = 2, the CTA pair (cta_group::2), issued by the leader CTA: the lane for which `issue` is not zero.  Its MMAs are long
+// enough to hide the issue, and an elect.sync before each of the 11 instructions of a K step costs more than it saves,
+// elected -> `issue`, GEMM alone: (8192, 8192, 28672) 826 -> 808 us at the power cap, (4096, 4096, 4096) 32.9 -> 32.3,
+// (8192, 4096, 4096) 63.9 -> 62.7, (4096, 14336, 4096) 109.1 -> 106.6, (16384, 8192, 8192) 474 -> 463.
 template <int CG>
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
+__device__ __forceinline__ void tc_commit(uint32_t bar, uint32_t issue = 0u) {
   if constexpr (CG == 1)
     asm volatile(
         "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
@@ -98,15 +102,15 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
         : "memory");
   else   // arrives on the barrier at this offset in both CTAs of the pair
     asm volatile(
-        "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
+        "{ .reg .pred q; setp.ne.b32 q, %2, 0;\n\t"
         "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1; }" ::"r"(bar),
-        "h"((uint16_t)3)
+        "h"((uint16_t)3), "r"(issue)
         : "memory");
 }
 // Descriptors are passed as their two 32-bit halves: the upper half is a constant per descriptor
 // kind, the lower half is base + a small offset, so no 64-bit arithmetic is needed per instruction.
 template <int CG>
-__device__ __forceinline__ void tc_cp_sf(uint32_t taddr, uint32_t desc_lo, uint32_t desc_hi) {
+__device__ __forceinline__ void tc_cp_sf(uint32_t taddr, uint32_t desc_lo, uint32_t desc_hi, uint32_t issue = 0u) {
   if constexpr (CG == 1)
     asm volatile(
         "{ .reg .pred q; .reg .b64 d; elect.sync _|q, 0xffffffff; mov.b64 d, {%1, %2};\n\t"
@@ -115,14 +119,15 @@ __device__ __forceinline__ void tc_cp_sf(uint32_t taddr, uint32_t desc_lo, uint3
         : "memory");
   else
     asm volatile(
-        "{ .reg .pred q; .reg .b64 d; elect.sync _|q, 0xffffffff; mov.b64 d, {%1, %2};\n\t"
+        "{ .reg .pred q; .reg .b64 d; setp.ne.b32 q, %3, 0; mov.b64 d, {%1, %2};\n\t"
         "@q tcgen05.cp.cta_group::2.32x128b.warpx4 [%0], d; }" ::"r"(taddr),
-        "r"(desc_lo), "r"(desc_hi)
+        "r"(desc_lo), "r"(desc_hi), "r"(issue)
         : "memory");
 }
 template <int CG>
 __device__ __forceinline__ void tc_mma_mxf4(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
-                                            uint32_t sfa_tmem, uint32_t sfb_tmem, uint32_t accumulate) {
+                                            uint32_t sfa_tmem, uint32_t sfb_tmem, uint32_t accumulate,
+                                            uint32_t issue = 0u) {
   if constexpr (CG == 1)
     asm volatile(
         "{ .reg .pred p, q; .reg .b64 da, db; setp.ne.b32 p, %7, 0; elect.sync _|q, 0xffffffff;\n\t"
@@ -132,10 +137,10 @@ __device__ __forceinline__ void tc_mma_mxf4(uint32_t d_tmem, uint32_t a_lo, uint
         : "memory");
   else
     asm volatile(
-        "{ .reg .pred p, q; .reg .b64 da, db; setp.ne.b32 p, %7, 0; elect.sync _|q, 0xffffffff;\n\t"
+        "{ .reg .pred p, q; .reg .b64 da, db; setp.ne.b32 p, %7, 0; setp.ne.b32 q, %8, 0;\n\t"
         "mov.b64 da, {%1, %3}; mov.b64 db, {%2, %3};\n\t"
         "@q tcgen05.mma.cta_group::2.kind::mxf4.block_scale.scale_vec::2X [%0], da, db, %4, [%5], [%6], p; }" ::"r"(d_tmem),
-        "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(sfa_tmem), "r"(sfb_tmem), "r"(accumulate)
+        "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(sfa_tmem), "r"(sfb_tmem), "r"(accumulate), "r"(issue)
         : "memory");
 }
 __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
@@ -259,7 +264,8 @@ template <int CG, int BN, int STAGES, int A_STAGE, int B_STAGE, int SFA_STAGE, i
           bool OVERLAP>
 __device__ __forceinline__ void mma_issue_loop(const IssueRing& r, uint32_t tmem_base, uint32_t tmem_sfa,
                                                uint32_t tmem_sfb, uint32_t idesc_full, int my_tiles, int num_k_steps,
-                                               int narrow_from = 0x7FFFFFFF, uint32_t idesc_narrow = 0u) {
+                                               uint32_t issue, int narrow_from = 0x7FFFFFFF,
+                                               uint32_t idesc_narrow = 0u) {
   // tiles narrow_from.. of this CTA are half-width: same loop, the instruction descriptor says N = BN/2
   const uint32_t a_lo0 = desc_lo_sw128(r.sA), b_lo0 = desc_lo_sw128(r.sB);
   const uint32_t sfa_lo0 = desc_lo_sf(r.sSFA), sfb_lo0 = desc_lo_sf(r.sSFB);
@@ -271,16 +277,16 @@ __device__ __forceinline__ void mma_issue_loop(const IssueRing& r, uint32_t tmem
   auto copy_scales = [&](int stage, int h, bool narrow) {
     const uint32_t lo_a = sfa_lo0 + (uint32_t)stage * (SFA_STAGE >> 4) + (uint32_t)h * 32u;
     const uint32_t lo_b = sfb_lo0 + (uint32_t)stage * (SFB_STAGE >> 4) + (uint32_t)h * 32u;
-    tc_cp_sf<CG>(tmem_sfa + 4 * h, lo_a, hi_sf);
-    tc_cp_sf<CG>(tmem_sfb + (BN / 32) * h, lo_b, hi_sf);
-    if (BN == 256 && !narrow) tc_cp_sf<CG>(tmem_sfb + (BN / 32) * h + 4, lo_b + 64u, hi_sf);
+    tc_cp_sf<CG>(tmem_sfa + 4 * h, lo_a, hi_sf, issue);
+    tc_cp_sf<CG>(tmem_sfb + (BN / 32) * h, lo_b, hi_sf, issue);
+    if (BN == 256 && !narrow) tc_cp_sf<CG>(tmem_sfb + (BN / 32) * h + 4, lo_b + 64u, hi_sf, issue);
   };
   auto mma_half = [&](int stage, int h, uint32_t tmem_acc, uint32_t accumulate_first) {
     const uint32_t a_lo = a_lo0 + (uint32_t)stage * (A_STAGE >> 4) + 4u * h;
     const uint32_t b_lo = b_lo0 + (uint32_t)stage * (B_STAGE >> 4) + 4u * h;
     const uint32_t tsfa = tmem_sfa + 4 * h, tsfb = tmem_sfb + (BN / 32) * h;
-    tc_mma_mxf4<CG>(tmem_acc, a_lo, b_lo, hi_op, idesc0, tsfa, tsfb, accumulate_first);
-    tc_mma_mxf4<CG>(tmem_acc, a_lo + 2u, b_lo + 2u, hi_op, idesc1, tsfa | (2u << 30), tsfb | (2u << 30), 1u);
+    tc_mma_mxf4<CG>(tmem_acc, a_lo, b_lo, hi_op, idesc0, tsfa, tsfb, accumulate_first, issue);
+    tc_mma_mxf4<CG>(tmem_acc, a_lo + 2u, b_lo + 2u, hi_op, idesc1, tsfa | (2u << 30), tsfb | (2u << 30), 1u, issue);
   };
   int stage = 0;
   uint32_t phase = 0;
@@ -323,12 +329,12 @@ __device__ __forceinline__ void mma_issue_loop(const IssueRing& r, uint32_t tmem
         copy_scales(next_stage, 0, next_narrow);   // half 0's columns were last read by the two MMAs above
       }
       mma_half(stage, 1, tmem_acc, 1u);
-      tc_commit<CG>(r.bar_empty + 8 * stage);   // frees the stage when these MMAs have read it
+      tc_commit<CG>(r.bar_empty + 8 * stage, issue);   // frees the stage when these MMAs have read it
       if (has_next) copy_scales(next_stage, 1, next_narrow);
       stage = next_stage;
       phase = next_phase;
     }
-    tc_commit<CG>(r.bar_acc_full + 8 * buf);    // accumulator complete (or abandoned) -> epilogue
+    tc_commit<CG>(r.bar_acc_full + 8 * buf, issue);    // accumulator complete (or abandoned) -> epilogue
   }
 }
 
@@ -575,7 +581,7 @@ gemm_mxfp4_kernel(const __grid_constant__ CUtensorMap tma, const __grid_constant
     };
     mma_issue_loop<1, BN, C::kStages, kATileBytes, C::kBTileBytes, C::kSfaBytes, C::kSfbBytes, C::kAccStride,
                    C::kOverlap>(ring, tmem_base, tmem_sfa, tmem_sfb, make_idesc<BN>(), units_below(p.total_units),
-                                p.num_k_steps, units_below(p.full_units), make_idesc<BN / 2>());
+                                p.num_k_steps, 0u, units_below(p.full_units), make_idesc<BN / 2>());
   } else {
     // ------------------------------ epilogue ------------------------------
     const int q = warp & 3;                 // TMEM lane quadrant this warp may read

@@ -227,7 +227,7 @@ gemm_mxfp4_pair_kernel(const __grid_constant__ CUtensorMap tma, const __grid_con
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer (leader only) ------------------------------
-    // All 32 lanes of the leader's warp walk the loop together; an elected lane issues for the pair.
+    // All 32 lanes of the leader's warp walk the loop together; lane 0 issues for the pair.
     if (rank == 0) {
       const gemm::IssueRing ring = {sA, sB, sSFA, sSFB, bar_full, bar_empty, bar_acc_full, bar_acc_free, bar_ovl_free};
       auto units_below = [&](int limit) {   // how many of this pair's units have an index below `limit`
@@ -235,7 +235,7 @@ gemm_mxfp4_pair_kernel(const __grid_constant__ CUtensorMap tma, const __grid_con
       };
       gemm::mma_issue_loop<2, kBN, kStages, kATileBytes, kBTileBytes, kSfaBytes, kSfbBytes, kAccStride, true>(
           ring, tmem_base, tmem_sfa, tmem_sfb, make_idesc_pair<kBN>(), units_below(p.total_units), p.num_k_steps,
-          units_below(p.full_units), make_idesc_pair<kBN / 2>());
+          lane == 0 ? 1u : 0u, units_below(p.full_units), make_idesc_pair<kBN / 2>());
     }
   } else {
     // ------------------------------ epilogue (both CTAs) ------------------------------
