@@ -32,7 +32,7 @@ constexpr int kWarps = kThreads / 32;
 // fp16(amax / 6)), 2 MXINT4 (k / 4, |k| <= 7, scale 2^E, E = floor(log2 amax)), 3 BINT4 (|k| <= 7,
 // scale fp16(amax / 7)).  Decisions are taken exactly as in rq::group_error: magnitudes scaled by an
 // exact power of two, or divided by the fp16 scale in fp32, then rounded to nearest even, saturating.
-__device__ __noinline__ void group_dequant_any(const uint64_t (&P)[16], uint32_t cbits, int format, float (&out)[32]) {
+__device__ __forceinline__ void group_dequant_any(const uint64_t (&P)[16], uint32_t cbits, int format, float (&out)[32]) {
   const float c = __uint_as_float(cbits);
   const uint64_t cc = rq::pack2(c, c);
   float y[32];
@@ -146,6 +146,13 @@ __device__ __forceinline__ void signed_out(uint64_t v, uint64_t y, float& o0, fl
   o1 = copysignf(v1, y1);
 }
 
+// The rare path as a call, so that the ordinary one keeps its registers.  (Not for the full-dimension rotation, which has
+// no registers to spare around a call: there the short forms and their call made every mode of its kernel 15 to 50 %
+// slower, quantisation to codes included, and it keeps the forms above.)
+__device__ __noinline__ void group_dequant_rare(const uint64_t (&P)[16], uint32_t cbits, int format, float (&out)[32]) {
+  group_dequant_any(P, cbits, format, out);
+}
+
 __device__ __forceinline__ void group_dequant(const uint64_t (&P)[16], uint32_t cbits, int format, float (&out)[32]) {
   uint64_t Y[16];
 #pragma unroll
@@ -165,7 +172,7 @@ __device__ __forceinline__ void group_dequant(const uint64_t (&P)[16], uint32_t 
     float o[32];
 #pragma unroll
     for (int k = 0; k < 16; ++k) Q[k] = P[k];
-    group_dequant_any(Q, cbits, format, o);
+    group_dequant_rare(Q, cbits, format, o);
 #pragma unroll
     for (int i = 0; i < 32; ++i) out[i] = o[i];
     return;
@@ -218,8 +225,8 @@ __device__ __forceinline__ void group_range(const uint64_t (&P)[16], uint32_t cb
 // codes 0..15 over [lo, hi] (the range always contains zero): scale fp16((hi - lo) / 15), zero point
 // z = rint(-lo / scale) (at most 15), q = clamp(rint(y / scale) + z, 0, 15), value (q - z) scale.  Quotients
 // are IEEE fp32 divisions; every result is an integer of at most 5 bits times an fp16 number, exact in fp32.
-__device__ __noinline__ void row_dequant_any(const uint64_t (&P)[16], uint32_t cbits, bool asym, float neglo, float hi,
-                                             float (&out)[32]) {
+__device__ __forceinline__ void row_dequant_any(const uint64_t (&P)[16], uint32_t cbits, bool asym, float neglo, float hi,
+                                                float (&out)[32]) {
   const float c = __uint_as_float(cbits);
   const uint64_t cc = rq::pack2(c, c);
   float y[32];
@@ -252,6 +259,10 @@ __device__ __noinline__ void row_dequant_any(const uint64_t (&P)[16], uint32_t c
   }
 }
 
+__device__ __noinline__ void row_dequant_rare(const uint64_t (&P)[16], uint32_t cbits, bool asym, float neglo, float hi,
+                                              float (&out)[32]) {
+  row_dequant_any(P, cbits, asym, neglo, hi, out);
+}
 __device__ __forceinline__ void row_dequant(const uint64_t (&P)[16], uint32_t cbits, bool asym, float neglo, float hi,
                                             float (&out)[32]) {
   uint64_t Y[16];
@@ -266,7 +277,7 @@ __device__ __forceinline__ void row_dequant(const uint64_t (&P)[16], uint32_t cb
     float o[32];
 #pragma unroll
     for (int k = 0; k < 16; ++k) Q[k] = P[k];
-    row_dequant_any(Q, cbits, asym, neglo, hi, o);
+    row_dequant_rare(Q, cbits, asym, neglo, hi, o);
 #pragma unroll
     for (int i = 0; i < 32; ++i) out[i] = o[i];
     return;

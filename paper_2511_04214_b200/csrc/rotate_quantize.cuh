@@ -371,41 +371,8 @@ __device__ __forceinline__ uint32_t group_scale_byte(const uint64_t (&P)[16], ui
 // E2M1 codes come from the same conversion instruction as in quantize_group and are decoded again
 // in hardware (e2m1x2 -> f16x2).  With a power-of-two scale the difference is exact in the scaled
 // domain; with an fp16 scale it is one fused multiply-add.  Squares and their sum are fp32.
-__device__ __forceinline__ float group_error(const uint64_t (&P)[16], uint32_t cbits, int format) {
+__device__ __forceinline__ float group_error_any(const uint64_t (&P)[16], uint32_t cbits, int format) {
   const float c = __uint_as_float(cbits);
-  if (format == 0) {
-    // MXFP4 away from the ends of the exponent range, on packed pairs: c * 2^-E in one multiply as in quantize_group, squares
-    // added by fused multiply-adds in four chains.  ([16384, 4096], block 32: 37 -> 31 us.)
-    float m = 0.f, m2 = 0.f;
-#pragma unroll
-    for (int k = 0; k < 16; k += 2) {
-      float a, b, a2, b2;
-      unpack2(P[k], a, b);
-      unpack2(P[k + 1], a2, b2);
-      asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(a), "f"(b));
-      asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m2) : "f"(a2), "f"(b2));
-    }
-    const uint32_t ef = __float_as_uint(__fmul_rn(fmaxf(m, m2), c)) >> 23;
-    if (ef >= 27u && ef <= 250u) {
-      const float c2 = __uint_as_float(cbits + ((129u - ef) << 23)), pe = __uint_as_float((ef - 2u) << 23);
-      const uint64_t cc = pack2(c2, c2);
-      uint64_t acc[2] = {0ull, 0ull};
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const uint64_t r = mul2(P[k], cc);
-        float r0, r1;
-        unpack2(r, r0, r1);
-        uint32_t h;
-        asm("{ .reg .b8 b; cvt.rn.satfinite.e2m1x2.f32 b, %2, %1; cvt.rn.f16x2.e2m1x2 %0, b; }" : "=r"(h) : "f"(r0), "f"(r1));
-        const uint64_t d = sub2(r, pack2(__half2float(__ushort_as_half((unsigned short)(h & 0xFFFFu))),
-                                         __half2float(__ushort_as_half((unsigned short)(h >> 16)))));
-        acc[k & 1] = fma2(d, d, acc[k & 1]);
-      }
-      float s0, s1;
-      unpack2(add2(acc[0], acc[1]), s0, s1);
-      return __fmul_rn(__fmul_rn(__fmul_rn(__fadd_rn(s0, s1), 0.03125f), pe), pe);
-    }
-  }
   const uint64_t cc = pack2(c, c);
   float y[32];
 #pragma unroll
@@ -470,6 +437,44 @@ __device__ __forceinline__ float group_error(const uint64_t (&P)[16], uint32_t c
     acc = __fadd_rn(acc, __fmul_rn(d1, d1));
   }
   return __fmul_rn(acc, 0.03125f);
+}
+
+// The same with a short form for MXFP4 away from the ends of the exponent range, on packed pairs: c * 2^-E in one multiply
+// as in quantize_group, squares added by fused multiply-adds in two chains of pairs.  ([16384, 4096], block 32: 37 -> 31 us.)
+__device__ __forceinline__ float group_error(const uint64_t (&P)[16], uint32_t cbits, int format) {
+  const float c = __uint_as_float(cbits);
+  if (format == 0) {
+    float m = 0.f, m2 = 0.f;
+#pragma unroll
+    for (int k = 0; k < 16; k += 2) {
+      float a, b, a2, b2;
+      unpack2(P[k], a, b);
+      unpack2(P[k + 1], a2, b2);
+      asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(a), "f"(b));
+      asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m2) : "f"(a2), "f"(b2));
+    }
+    const uint32_t ef = __float_as_uint(__fmul_rn(fmaxf(m, m2), c)) >> 23;
+    if (ef >= 27u && ef <= 250u) {
+      const float c2 = __uint_as_float(cbits + ((129u - ef) << 23)), pe = __uint_as_float((ef - 2u) << 23);
+      const uint64_t cc = pack2(c2, c2);
+      uint64_t acc[2] = {0ull, 0ull};
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        const uint64_t r = mul2(P[k], cc);
+        float r0, r1;
+        unpack2(r, r0, r1);
+        uint32_t h;
+        asm("{ .reg .b8 b; cvt.rn.satfinite.e2m1x2.f32 b, %2, %1; cvt.rn.f16x2.e2m1x2 %0, b; }" : "=r"(h) : "f"(r0), "f"(r1));
+        const uint64_t d = sub2(r, pack2(__half2float(__ushort_as_half((unsigned short)(h & 0xFFFFu))),
+                                         __half2float(__ushort_as_half((unsigned short)(h >> 16)))));
+        acc[k & 1] = fma2(d, d, acc[k & 1]);
+      }
+      float s0, s1;
+      unpack2(add2(acc[0], acc[1]), s0, s1);
+      return __fmul_rn(__fmul_rn(__fmul_rn(__fadd_rn(s0, s1), 0.03125f), pe), pe);
+    }
+  }
+  return group_error_any(P, cbits, format);
 }
 
 // SIGNS: the randomised rotation R_i = diag(s) H / sqrt(block) (paper Sec. 5.1) — the channel signs

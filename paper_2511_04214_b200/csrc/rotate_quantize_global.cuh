@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rotate_quantize_global_kernel(
       continue;
     }
     if (p.mse) {                 // analysis mode (uniform over the grid)
-      const float e = rq::group_error(P, cbits, p.format);
+      const float e = rq::group_error_any(P, cbits, p.format);
       if (live) p.mse[row * (p.K >> 5) + gi] = e;
       continue;
     }
@@ -126,10 +126,10 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rotate_quantize_global_kernel(
         for (int k = 0; k < 16; ++k) rq::unpack2(rq::mul2(P[k], cc), out[2 * k], out[2 * k + 1]);
       } else if (p.format >= fq::kFormatRowSym) {
         const int64_t r = live ? row : 0;
-        fq::row_dequant(P, cbits, p.format == fq::kFormatRowAsym, __uint_as_float(__ldcg(p.rowstats + 2 * r)),
-                        __uint_as_float(__ldcg(p.rowstats + 2 * r + 1)), out);
+        fq::row_dequant_any(P, cbits, p.format == fq::kFormatRowAsym, __uint_as_float(__ldcg(p.rowstats + 2 * r)),
+                            __uint_as_float(__ldcg(p.rowstats + 2 * r + 1)), out);
       } else
-      fq::group_dequant(P, cbits, p.format, out);
+      fq::group_dequant_any(P, cbits, p.format, out);
       if (live) fq::store_group(p.deq + row * p.ldd + (int64_t)gi * 32, out);
       continue;
     }
