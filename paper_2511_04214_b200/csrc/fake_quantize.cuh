@@ -103,8 +103,10 @@ __device__ __forceinline__ void group_dequant_any(const uint64_t (&P)[16], uint3
 // functions on the IBM RISC System/6000 processor", 1990), as long as nothing leaves the normal range; quotients so small that
 // their remainder is subnormal round to the element 0 either way.  Integers come from adding and subtracting 1.5 * 2^23 (nearest,
 // ties to even) after clamping, which commutes with rounding.  Every step rounds as in the forms above, so the values are the same
-// bits.  `y_nan_max` is false for groups that hold an infinity or a NaN; these and the ends of the exponent range take
-// the forms above.  [8192, 4096], block 32: BFP4 56 -> 40 us, BINT4 59 -> 41 us, INT4 per row 81 -> 67 us.
+// bits.  Groups that hold an infinity or a NaN (amax_nan then is one too) and the ends of the exponent range take the forms
+// above.  They are rare, but a warp that holds one waits for both forms; so groups of zeros have an answer of their own,
+// and the lanes beyond the end of a row compute nothing.
+// [8192, 4096], block 32: BFP4 56 -> 40 us, BINT4 59 -> 41 us, INT4 per row 81 -> 67 us.
 __device__ __forceinline__ float amax_nan(const uint64_t (&Y)[16]) {
   float m = 0.f, m2 = 0.f;
 #pragma unroll
@@ -158,6 +160,14 @@ __device__ __forceinline__ void group_dequant(const uint64_t (&P)[16], uint32_t 
 #pragma unroll
   for (int k = 0; k < 16; ++k) Y[k] = rq::mul2(P[k], both(__uint_as_float(cbits)));
   const float m = amax_nan(Y);
+  if (m == 0.f) {              // zeros, which keep their signs under a power-of-two scale
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      rq::unpack2(Y[k], out[2 * k], out[2 * k + 1]);
+      if (format & 1) out[2 * k] = out[2 * k + 1] = 0.f;
+    }
+    return;
+  }
   const uint32_t ef = __float_as_uint(m) >> 23;
   // 2^-125 and up, finite; the fp16 scales not zero
   float sc = 0.f, inv = 0.f;
@@ -400,8 +410,7 @@ __global__ void __launch_bounds__(kThreads, 2) fake_quantize_kernel(const Params
     }
     if (!full) {
       if (p.mse) {                                 // the statistics only
-        const float e = rq::group_error(P, cbits, p.format);
-        if (live) p.mse[row * ng + g] = e;
+        if (live) p.mse[row * ng + g] = rq::group_error(P, cbits, p.format);
       } else if (p.scale_bytes) {
         const uint32_t sb = rq::group_scale_byte(P, cbits);
         if (live) p.scale_bytes[row * ng + g] = (uint8_t)sb;
@@ -411,7 +420,10 @@ __global__ void __launch_bounds__(kThreads, 2) fake_quantize_kernel(const Params
       }
     } else if (row < p.M) {
       float out[32];
-      if (p.format == kFormatNone) {               // the rotation itself
+      if (!live) {                                 // (beyond the row's end: these lanes must not take the rare path)
+#pragma unroll
+        for (int i = 0; i < 32; ++i) out[i] = 0.f;
+      } else if (p.format == kFormatNone) {        // the rotation itself
         const uint64_t cc = rq::pack2(__uint_as_float(cbits), __uint_as_float(cbits));
 #pragma unroll
         for (int k = 0; k < 16; ++k) rq::unpack2(rq::mul2(P[k], cc), out[2 * k], out[2 * k + 1]);

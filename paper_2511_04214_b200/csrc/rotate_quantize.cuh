@@ -450,10 +450,12 @@ __device__ __forceinline__ float group_error(const uint64_t (&P)[16], uint32_t c
       float a, b, a2, b2;
       unpack2(P[k], a, b);
       unpack2(P[k + 1], a2, b2);
-      asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(a), "f"(b));
-      asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m2) : "f"(a2), "f"(b2));
+      asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(a), "f"(b));
+      asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(m2) : "f"(a2), "f"(b2));
     }
-    const uint32_t ef = __float_as_uint(__fmul_rn(fmaxf(m, m2), c)) >> 23;
+    asm("max.NaN.f32 %0, %0, %1;" : "+f"(m) : "f"(m2));
+    if (m == 0.f) return 0.f;             // (zeros need not wait for the general form)
+    const uint32_t ef = __float_as_uint(__fmul_rn(m, c)) >> 23;
     if (ef >= 27u && ef <= 250u) {
       const float c2 = __uint_as_float(cbits + ((129u - ef) << 23)), pe = __uint_as_float((ef - 2u) << 23);
       const uint64_t cc = pack2(c2, c2);

@@ -221,8 +221,8 @@ __device__ __forceinline__ void finish_task(const Params& p, const uint4 (&cur)[
       const uint32_t sbyte = rq::group_scale_byte(P, cbits);
       if (live) p.scales[(int64_t)row * ng + g] = (uint8_t)sbyte;
     } else {
-      const float e = rq::group_error(P, cbits, p.format);
-      if (live) p.mse[(int64_t)row * ng + g] = e;
+      // (lanes beyond the end of a row hold zeros, which take the general form: not computed beside the short one)
+      if (live) p.mse[(int64_t)row * ng + g] = rq::group_error(P, cbits, p.format);
     }
     return;
   }
