@@ -347,11 +347,11 @@ __global__ void __launch_bounds__(kThreads, 2) fake_quantize_kernel(const Params
     row = r < rows_at_once ? (int64_t)blockIdx.x * rows_at_once + r : p.M;      // (left-over warps only keep step)
     step_row = (int64_t)gridDim.x * rows_at_once;
   } else {
-    const int64_t task = (int64_t)blockIdx.x * kWarps + warp, num_warps = (int64_t)gridDim.x * kWarps;
-    row = task / c;
-    chunk = (int)(task - row * c);
-    step_row = num_warps / c;
-    step_chunk = (int)(num_warps - step_row * c);
+    const uint32_t task = blockIdx.x * kWarps + (uint32_t)warp, num_warps = gridDim.x * kWarps;      // (of the grid: 32 bits)
+    row = task / (uint32_t)c;
+    chunk = (int)(task % (uint32_t)c);
+    step_row = num_warps / (uint32_t)c;
+    step_chunk = (int)(num_warps % (uint32_t)c);
   }
   griddep_wait();
   griddep_launch_dependents();

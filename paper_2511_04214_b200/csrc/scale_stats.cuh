@@ -22,14 +22,16 @@ constexpr size_t kWorkspaceBytes = (size_t)kMagBins * 8 + 64;
 // Behind the histogram: word 0 counts the CTAs that have merged theirs, word 1 is the smallest pattern counted.
 constexpr int kTicketWord = 0, kLowestWord = 1;
 
-// Row and group of a thread's first item and of its stride, so that the loop over a matrix divides once.
+// Row and group of a thread's first item and of its stride, so that the loop over a matrix divides once.  (First item and
+// stride are numbers of threads and fit 32 bits, as K / 32 does: divisions in 64 bits took 0.2 us of a small launch.)
 struct GroupWalk {
   int64_t row, g, step_row, step_g, ng;
-  __device__ GroupWalk(int64_t first, int64_t step, int64_t ng_) : ng(ng_) {
-    row = first / ng;
-    g = first - row * ng;
-    step_row = step / ng;
-    step_g = step - step_row * ng;
+  __device__ GroupWalk(uint32_t first, uint32_t step, int64_t ng_) : ng(ng_) {
+    const uint32_t n = (uint32_t)ng_;
+    row = first / n;
+    g = first % n;
+    step_row = step / n;
+    step_g = step % n;
   }
   __device__ void next() {
     row += step_row;
@@ -59,7 +61,7 @@ __global__ void __launch_bounds__(256) group_scale_bytes_identity(const uint16_t
                                                                   uint8_t* scales) {
   griddep_wait();
   const int64_t ng = K >> 5, total = M * ng;
-  const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  const uint32_t first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
   GroupWalk at(first, step, ng);
   for (int64_t i = first; i < total; i += step, at.next()) {
     const uint32_t ef = group_max_mag(x, at.row, ldx, at.g) >> 7;
@@ -165,7 +167,7 @@ __global__ void __launch_bounds__(kScanThreads, 1) outlier_scan(const uint16_t* 
   // A CTA takes 1024 consecutive groups at a time and its warps change places from one time to the next: outlier channels
   // keep their place in a row, and a warp that always met them finished a third later than the others.
   const int64_t step = (int64_t)gridDim.x * kScanThreads;
-  GroupWalk at((int64_t)blockIdx.x * kScanThreads, step, ng);       // the CTA's first group
+  GroupWalk at(blockIdx.x * (uint32_t)kScanThreads, (uint32_t)step, ng);       // the CTA's first group
   // (ceil(2^32 / ng) does not fit 32 bits for rows of one group)
   const uint32_t magic = ng > 1 && ng < kScanThreads ? (uint32_t)((0x100000000ull + ng - 1) / ng) : 0u;
   {
