@@ -61,10 +61,11 @@ __global__ void __launch_bounds__(256) group_scale_bytes_identity(const uint16_t
                                                                   uint8_t* scales) {
   griddep_wait();
   const int64_t ng = K >> 5, total = M * ng;
-  const uint32_t first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
-  GroupWalk at(first, step, ng);
-  for (int64_t i = first; i < total; i += step, at.next()) {
-    const uint32_t ef = group_max_mag(x, at.row, ldx, at.g) >> 7;
+  // (divided per group, not walked: the walk's two divisions before the loop and its carry in it cost 0.2 us of a small
+  // launch and 24.3 -> 27.2 us at [16384, 4096])
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t row = i / ng, g = i - row * ng;
+    const uint32_t ef = group_max_mag(x, row, ldx, g) >> 7;
     scales[i] = (uint8_t)(ef > 2u ? ef - 2u : 0u);
   }
 }
