@@ -191,21 +191,23 @@ __device__ __forceinline__ void named_barrier_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 // TMA store shared -> global of one box; out-of-range parts of the box are clipped.
-// Forms for a converged warp, executed by the elected lane.
-__device__ __forceinline__ void tma_store_2d_elect(const CUtensorMap* m, uint32_t src, int x, int y) {
+// Forms for a converged warp, executed by the lane for which `issue` is not zero.  (Not elected per instruction as the loads
+// are: that made launches that the epilogue bounds slower.  Elected -> `issue`, (512, 256, 28672) 10.0 -> 8.9 us,
+// (1024, 512, 28672) 17.1 -> 15.4, (8192, 512, 8192) 31.8 -> 29.7; in fp32 15.7 -> 13.8, 26.3 -> 24.8, 48.9 -> 47.1.)
+__device__ __forceinline__ void tma_store_2d_if(uint32_t issue, const CUtensorMap* m, uint32_t src, int x, int y) {
   asm volatile(
-      "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
+      "{ .reg .pred q; setp.ne.b32 q, %4, 0;\n\t"
       "@q cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1]; }" ::"l"(
           reinterpret_cast<uint64_t>(m)),
-      "r"(src), "r"(x), "r"(y)
+      "r"(src), "r"(x), "r"(y), "r"(issue)
       : "memory");
 }
-__device__ __forceinline__ void bulk_commit_elect() {
-  asm volatile("{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t@q cp.async.bulk.commit_group; }" ::: "memory");
+__device__ __forceinline__ void bulk_commit_if(uint32_t issue) {
+  asm volatile("{ .reg .pred q; setp.ne.b32 q, %0, 0;\n\t@q cp.async.bulk.commit_group; }" ::"r"(issue) : "memory");
 }
 template <int N>
-__device__ __forceinline__ void bulk_wait_read_elect() {
-  asm volatile("{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t@q cp.async.bulk.wait_group.read %0; }" ::"n"(N) : "memory");
+__device__ __forceinline__ void bulk_wait_read_if(uint32_t issue) {
+  asm volatile("{ .reg .pred q; setp.ne.b32 q, %0, 0;\n\t@q cp.async.bulk.wait_group.read %1; }" ::"r"(issue), "n"(N) : "memory");
 }
 __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -361,6 +363,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem_acc, int buf, int la
   static_assert(CHUNKS % 2 == 0, "chunks are processed in pairs");
   constexpr int PAIRS = CHUNKS / 2;
   const int64_t row = (int64_t)row0 + lane;
+  const uint32_t issue = lane == 0 ? 1u : 0u;
   auto pair_of = [&](int pi) { return (OVERLAP && buf == 0) ? (pi == 0 ? PAIRS - 1 : pi - 1) : pi; };
   auto released = [&](int pi) {
     if (pi == 0 || pi == PAIRS - 1) {
@@ -375,7 +378,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem_acc, int buf, int la
   // fp32: one box of 32 columns x 32 rows per chunk, 128 bytes a row as the 64 bf16 columns of a pair.  (Stores from
   // registers, 16 bytes a lane and the lanes a row of y apart, took 20 of a launch's 31 us at (777, 4384, 6004).)
   auto emit_f32 = [&](const uint32_t (&r)[32], int col0, uint32_t sbuf) {
-    if (stage_stride == 0u) bulk_wait_read_elect<0>();
+    if (stage_stride == 0u) bulk_wait_read_if<0>(issue);
     __syncwarp();
     const uint32_t rowaddr = sbuf + (uint32_t)lane * 128u, sw = (uint32_t)lane & 7u;
 #pragma unroll
@@ -384,8 +387,8 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem_acc, int buf, int la
     __syncwarp();
     // (the map ends at the last multiple of 4 columns, see make_out_map; the up to 3 behind it come from the buffer)
     const int64_t n_tma = N & ~(int64_t)3;
-    if (col0 < n_tma && row0 < M) tma_store_2d_elect(tmy, sbuf, col0, row0);
-    bulk_commit_elect();
+    if (col0 < n_tma && row0 < M) tma_store_2d_if(issue, tmy, sbuf, col0, row0);
+    bulk_commit_if(issue);
     if (n_tma < N && n_tma >= col0 && n_tma < (int64_t)col0 + kChunkCols && row < M) {
       float* dst = static_cast<float*>(y) + row * ldy + n_tma;
       const int k0 = (int)(n_tma - col0);
@@ -406,7 +409,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem_acc, int buf, int la
       }
       const uint32_t sbuf = stage_buf + (uint32_t)pi * stage_stride;
       // the TMA store that last read the staging buffer must be done reading it
-      if (stage_stride == 0u) bulk_wait_read_elect<0>();
+      if (stage_stride == 0u) bulk_wait_read_if<0>(issue);
       __syncwarp();
       // row `lane` of the box: 128 bytes, 16-byte pieces XOR-swizzled with lane & 7
       const uint32_t rowaddr = sbuf + (uint32_t)lane * 128u;
@@ -418,8 +421,8 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem_acc, int buf, int la
       // A TMA store clips at 16-byte granularity: the map ends at the last multiple of 8 columns, the up to 7 behind it are
       // copied from the staging buffer (all 64 columns of a ragged pair, element by element, took 5 us of the last tile).
       const int64_t n_tma = N & ~(int64_t)7;
-      if (col0 < n_tma && row0 < M) tma_store_2d_elect(tmy, sbuf, col0, row0);
-      bulk_commit_elect();             // (possibly empty) keeps the group count in step
+      if (col0 < n_tma && row0 < M) tma_store_2d_if(issue, tmy, sbuf, col0, row0);
+      bulk_commit_if(issue);             // (possibly empty) keeps the group count in step
       if (n_tma < N && n_tma >= col0 && n_tma < (int64_t)col0 + 2 * kChunkCols && row < M) {
         uint16_t* dst = static_cast<uint16_t*>(y) + row * ldy + n_tma;
         const uint32_t piece = rowaddr + ((((uint32_t)(n_tma - col0) >> 3) ^ sw) << 4);
@@ -609,7 +612,7 @@ gemm_mxfp4_kernel(const __grid_constant__ CUtensorMap tma, const __grid_constant
     }
     // the staging buffer must have been read before this CTA's shared memory goes away; the writes
     // themselves complete with the kernel
-    bulk_wait_read_elect<0>();
+    bulk_wait_read_if<0>(lane == 0 ? 1u : 0u);
   }
   tc_fence_before();
   __syncthreads();
