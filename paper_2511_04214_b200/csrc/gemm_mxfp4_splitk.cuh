@@ -32,6 +32,7 @@ constexpr int kQuantWarps = 16;                  // FUSED: the epilogue warps an
 constexpr int kThreads = (2 + kEpilogueWarps) * 32, kThreadsFused = (2 + kQuantWarps) * 32;
 constexpr int kRowsW = 128;                      // rows of W per MMA
 constexpr int kMaxTokens = 128;                  // tokens per tile
+constexpr int kMaxTokensFused = 4 * kQuantWarps; // FUSED: a warp quantises 4 tokens of a K step
 constexpr int kWTileBytes = kRowsW * 128;        // 16 KiB: one 256-element K step of 128 rows
 constexpr int kScaleBytes = 1024;                // its scales: 2 blocks of 512 B
 constexpr int kMaxStages = 11;
@@ -269,7 +270,8 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
   bool ok = true;
   if (FUSED && warp >= 2) {
     // ------------------------------ rotate + quantise x ------------------------------
-    // One warp task: 4 tokens x the 8 groups of a K step, one group per lane; task t goes to warp t mod 16.
+    // One warp task: 4 tokens x the 8 groups of a K step, one group per lane; task t goes to warp t mod 16.  At most 64
+    // tokens, so a warp has one task of a step or none.
     const int in_quad = lane >> 3, g = lane & 7;
     auto load = [&](int step, int quad, uint4 (&v)[4]) {
       const int token = quad * 4 + in_quad, group = (k_first + step) * 8 + g;
@@ -297,22 +299,20 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
     uint32_t phase = 1u;                                 // (parity of the phase before the first: passes at once)
     for (int i = 0; i < k_count; ++i) {
       const uint32_t base = smem_base + (uint32_t)(stage * p.stage_bytes);
-      bool waited = false;
-      do {
-        const bool has = step == i;
-        const int row = quad * 4 + in_quad;
-        uint32_t w[4], sb = 0u;
-        if (has) {
-          sb = rotate_quantize_lane(cur, p.log2b, p.cbits, lane, w);
-          advance(step, quad);
-          if (step < k_count) load(step, quad, cur);     // in flight while this task's stage is waited for and written
-          // scale bytes of 4 consecutive groups -> one 32-bit word in the lane with g % 4 == 0
-          sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 1) << 8;
-          sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 2) << 16;
-        }
-        if (!waited) ok = mbar_wait_warp(bar_empty + 8 * stage, phase, SITE_GEMM_EMPTY);
-        waited = true;
-        if (!has || !ok) break;
+      const bool has = step == i;
+      const int row = quad * 4 + in_quad;
+      uint32_t w[4], sb = 0u;
+      if (has) {
+        sb = rotate_quantize_lane(cur, p.log2b, p.cbits, lane, w);
+        advance(step, quad);
+        if (step < k_count) load(step, quad, cur);       // in flight while this task's stage is waited for and written
+        // scale bytes of 4 consecutive groups -> one 32-bit word in the lane with g % 4 == 0
+        sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 1) << 8;
+        sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 2) << 16;
+      }
+      ok = mbar_wait_warp(bar_empty + 8 * stage, phase, SITE_GEMM_EMPTY);
+      if (!ok) break;
+      if (has) {
         const uint32_t sf_at = (uint32_t)((g >> 2) * 512 + (row & 31) * 16 + (row >> 5) * 4);
         gemm::sts128(base + w_bytes + (uint32_t)row * 128u + (uint32_t)((g ^ (row & 7)) << 4), w[0], w[1], w[2], w[3]);
         if ((g & 3) == 0) asm volatile("st.shared.b32 [%0], %1;" ::"r"(base + off_sfa + sf_at), "r"(sb) : "memory");
@@ -322,8 +322,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
             *reinterpret_cast<uint4*>(p.codes + ((int64_t)row * p.groups_k + group) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
           if ((g & 3) == 0) *reinterpret_cast<uint32_t*>(p.scales + (int64_t)(k_first + i) * 1024 + sf_at) = sb;
         }
-      } while (step == i);
-      if (!ok) break;
+      }
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_full + 8 * stage);
@@ -496,13 +495,21 @@ inline bro_status best_split(int64_t tiles, int num_k_steps, int sm_count, Cost&
 // Parts, by the costs above: (16, 14336, 4096) 1 part 10.5 us, 2 parts 7.3, 4 parts 6.3, persistent kernel 20.1;
 // (64, 2048, 2048) 1 part 3.7 us, 2 parts 4.3; (128, 14336, 4096) 1 part 14.5 us, 4 parts 10.9, persistent 20.8.
 //
-// fused = true asks for a plan that quantises inside the GEMM.  It saves the other kernel (2 us on the device, 4 us of
+// More than 64 tokens fill 128 columns of the instruction and of the epilogue, whose stores are narrower than the
+// persistent kernel's boxes; with fewer than 4 K steps that shows at both ends.  M = 128, persistent -> this kernel: one
+// tile, K = 256, N = 64 2.93 -> 3.17 us, 128 tiles, K = 768, N = 16384 5.3 -> 5.7, but K = 256, N = 1000 3.6 -> 3.4 and
+// K = 768, N = 8192 4.5 -> 4.0; 4 steps gain throughout (K = 1024, N = 16384 5.9 -> 5.3, N = 64 3.9 -> 3.7).
+//
+// fused = true asks for a plan that quantises inside the GEMM.  It saves the other kernel (2 us on the device, 3 us of
 // the host's time to launch it) and costs the tasks of the quantising warps, of which about half the time that the
-// weights take from HBM hides; the line is at 2.9 us for the rest.  Whole layer in a graph, two kernels -> fused:
-// (1, 8192, 28672) 23.2 -> 21.3 us, (16, 8192, 28672) 24.2 -> 23.3, (3, 1024, 1024) 4.3 -> 3.4, (16, 2048, 2048)
-// 4.9 -> 4.0, (16, 4096, 4096) even, (64, 2048, 2048) 5.9 -> 6.5 and (24, 5120, 5120) 6.4 -> 7.8, where calls that are
-// launched one by one are bound by the host and still gain its 4 us; beyond the line (32, 8192, 28672) 24.8 -> 29.5,
-// (128, 2048, 2048) 6.6 -> 10.3.
+// weights take from HBM hides; what is left may cost up to 2.9 us.  Whole layer in a graph, two kernels -> fused:
+// (1, 8192, 28672) 24.3 -> 22.6 us, (3, 1024, 1024) 4.2 -> 3.3, (16, 2048, 2048) 5.1 -> 3.9, (16, 4096, 4096) 6.8 -> 5.6,
+// (16, 8192, 28672) and (24, 5120, 5120) even, (64, 2048, 2048) 6.0 -> 6.4 and (16, 14336, 4096) 10.5 -> 11.9; called
+// one by one, where the host binds, (64, 2048, 2048) 9.0 -> 6.9.  Beyond the line (32, 8192, 28672) 24.8 -> 29.5.
+// With few K steps the line is lower, 1.25 us and 0.2 us a step: there the persistent kernel is quick, and no layer may be
+// slower in a graph than with it: (64, 512, 4096) persistent 5.1, two kernels 4.4, fused 5.4 us, (48, 1024, 8192) 6.3, 5.3
+// and 6.5, but (48, 1536, 4096) 6.6, 5.4 and 6.2.  More than 64 tokens are two tasks a warp and step and 128 columns:
+// (80, 256, 4096) 4.7, 4.7 and 5.0, (128, 256, 1000) 5.1, 5.1 and 5.8; never fused.
 inline bro_status plan(int64_t M, int64_t N, int num_k_steps, bool fused, int sm_count, Plan* out) {
   const int64_t tiles_m = (M + kMaxTokens - 1) / kMaxTokens, n128 = (N + kRowsW - 1) / kRowsW;
   const int tokens = token_columns(M);
@@ -512,6 +519,7 @@ inline bro_status plan(int64_t M, int64_t N, int num_k_steps, bool fused, int sm
   *out = Plan();
   const bool narrow = tiles_m * n128 <= sm_count;
   if (narrow ? !(tiles_m == 1 || num_k_steps >= 8) : !(tokens <= 64 && (n128 + 1) / 2 <= sm_count)) return BRO_OK;
+  if (tokens > 64 && num_k_steps < 4 && (n128 < 8 || n128 > 64)) return BRO_OK;
   pl.row_blocks = narrow ? 1 : 2;
   pl.tiles_n = (int)(narrow ? n128 : (n128 + 1) / 2);
   pl.split = 1;
@@ -523,14 +531,15 @@ inline bro_status plan(int64_t M, int64_t N, int num_k_steps, bool fused, int sm
     if (rc != BRO_OK) return rc;
   }
   if (fused) {
-    if (tiles_m > 1) return BRO_OK;
+    if (tokens > kMaxTokensFused) return BRO_OK;
     const int64_t hidden = (int64_t)((double)N * num_k_steps * 256 * (17.0 / 32) / 6200) / 2;      // half the weights' time
     const int64_t beside = (pl.split > 1 ? exchange_ns(tokens) : 0) + hidden;
     if (narrow) {
       const bro_status rc = best_split(n128, num_k_steps, sm_count, one_kernel, &pl.split, &fused_ns);
       if (rc != BRO_OK) return rc;
     }
-    if (fused_ns - (beside > ns ? beside : ns) > 2900) return BRO_OK;
+    const int64_t line = 1250 + 200 * (int64_t)num_k_steps;
+    if (fused_ns - (beside > ns ? beside : ns) > (line < 2900 ? line : 2900)) return BRO_OK;
   }
   *out = pl;
   return BRO_OK;

@@ -1,5 +1,7 @@
 """GPU parity of the GEMM for problems of few output tiles (one wave of 128- or 256-row weight tiles, K split over
 the CTAs of a cluster): the edges of its tiles and of its plan, against the CPU oracle and the persistent kernel."""
+import ctypes
+
 import pytest
 import torch
 
@@ -13,6 +15,18 @@ pytestmark = pytest.mark.gpu
 def bro():
     from paper_2511_04214_b200 import binding
     return binding
+
+
+def launches(call):
+    """How many graph nodes a call becomes: 1 for the layer in one kernel, 2 for rotate + quantise and the GEMM."""
+    call()                                            # (loads the kernels outside the capture)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    n = ctypes.c_size_t(0)
+    assert ctypes.CDLL("libcuda.so.1").cuGraphGetNodes(ctypes.c_void_p(graph.raw_cuda_graph()), None, ctypes.byref(n)) == 0
+    return n.value
 
 
 @pytest.mark.parametrize("M,K,N", [
@@ -58,8 +72,9 @@ def test_splitk_same_result_as_persistent_kernel(bro, M, K, N):
     (5, 4128, 264, 32),       # K not a multiple of 256: half of the last step is padding
     (16, 2176, 136, 128),
     (31, 1024, 392, 2),       # rotations inside the group
-    (64, 512, 264, 16),
-    (128, 1024, 200, 32),
+    (33, 2048, 392, 32),      # 9 warp tasks a step for 16 warps, clusters
+    (64, 256, 264, 16),       # as many tasks as warps, one step
+    (64, 2048, 264, 128),
 ])
 @pytest.mark.parametrize("signs", [False, True])
 def test_layer_of_few_tokens_same_bytes_as_two_kernels(bro, M, K, N, block, signs):
@@ -79,7 +94,11 @@ def test_layer_of_few_tokens_same_bytes_as_two_kernels(bro, M, K, N, block, sign
     ldy = (N + 7) // 8 * 8
     out = Guarded(M * ldy * 2, fill=0x7F)
     y = out.view.view(torch.bfloat16).view(M, ldy)[:, :N]
-    bro.linear_rs(x, block, s, wc, wsc, N, y, work) if signs else bro.linear(x, block, wc, wsc, N, y, work)
+    layer = (lambda: bro.linear_rs(x, block, s, wc, wsc, N, y, work)) if signs else (lambda: bro.linear(x, block, wc, wsc, N, y, work))
+    assert launches(layer) == 1
+    out.view.fill_(0x7F)
+    ws.view.fill_(0x7F)
+    layer()
     assert bro.last_device_status() == 0
     ws.check()
     out.check()
@@ -123,3 +142,46 @@ def test_layer_of_few_tokens_in_place(bro, M, K, N, shift, signs):
     assert torch.equal(y, want)
     around[:, shift:shift + N] = want
     assert torch.equal(buf, around)
+
+
+@pytest.mark.parametrize("M,K,N", [(65, 2048, 264), (128, 256, 1000), (64, 512, 4096), (130, 2048, 264), (64, 8192, 19000)])
+def test_layer_of_more_tokens_keeps_two_kernels(bro, M, K, N):
+    x = torch.randn(M, K, device="cuda").to(torch.bfloat16)
+    wc, wsc = bro.alloc_codes(N, K), bro.alloc_scales(N, K, bro.LAYOUT_GEMM)
+    bro.pack_weights(torch.randn(N, K, device="cuda").to(torch.bfloat16), 32, wc, wsc)
+    y, work = torch.empty(M, N, dtype=torch.bfloat16, device="cuda"), bro.alloc_workspace(bro.linear_workspace_bytes(M, N, K))
+    assert launches(lambda: bro.linear(x, 32, wc, wsc, N, y, work)) == 2
+
+
+@pytest.mark.parametrize("M,K,N", [(2, 4096, 4096), (16, 2048, 19000)])
+def test_layer_right_behind_the_packing_of_its_weights(bro, M, K, N):
+    """The one-kernel layer draws its first weight tiles into L2 while the kernel before it may still be writing them: new
+    weights packed into the same buffers just before every call, on two streams with buffers of their own, must be
+    the ones that the layer multiplies."""
+    gen = torch.Generator(device="cuda").manual_seed(K)
+    x = torch.randn(M, K, generator=gen, device="cuda").to(torch.bfloat16)
+    ws = [torch.randn(N, K, generator=gen, device="cuda").to(torch.bfloat16) for _ in range(3)]
+    want = []
+    for w in ws:
+        wc, wsc = bro.alloc_codes(N, K), bro.alloc_scales(N, K, bro.LAYOUT_GEMM)
+        bro.pack_weights(w, 32, wc, wsc)
+        torch.cuda.synchronize()
+        y, work = torch.empty(M, N, dtype=torch.bfloat16, device="cuda"), bro.alloc_workspace(bro.linear_workspace_bytes(M, N, K))
+        bro.linear(x, 32, wc, wsc, N, y, work)
+        want.append(y)
+    torch.cuda.synchronize()
+    lanes = []
+    for _ in range(2):
+        lanes.append((torch.cuda.Stream(), bro.alloc_codes(N, K), bro.alloc_scales(N, K, bro.LAYOUT_GEMM),
+                      bro.alloc_workspace(bro.linear_workspace_bytes(M, N, K)),
+                      [torch.empty(M, N, dtype=torch.bfloat16, device="cuda") for _ in range(12)]))
+    torch.cuda.synchronize()
+    for i in range(12):
+        for stream, wc, wsc, work, ys in lanes:
+            bro.pack_weights(ws[i % 3], 32, wc, wsc, stream=stream)
+            bro.linear(x, 32, wc, wsc, N, ys[i], work, stream=stream)
+    torch.cuda.synchronize()
+    assert bro.last_device_status() == 0
+    for _, _, _, _, ys in lanes:
+        for i, y in enumerate(ys):
+            assert torch.equal(y, want[i % 3]), i
