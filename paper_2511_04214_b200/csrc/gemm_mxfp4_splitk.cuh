@@ -336,6 +336,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
           *reinterpret_cast<uint32_t*>(p.scales + ((int64_t)k_first * 2 + j / kRowsW) * 512 + (row & 31) * 16 + (row >> 5) * 4) = 0u;
       }
     }
+    __syncwarp();                             // (the loops above diverge; the barriers and loads below are .aligned)
   }
   const bool epilogue = warp >= 2 && warp < 2 + kEpilogueWarps;
   if (epilogue) {
@@ -358,6 +359,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
       const int64_t n = (int64_t)n0 + b * kRowsW + q * 32 + lane;
       for (int c = ROW_BLOCKS == 2 ? 0 : half * 16; c < live; c += ROW_BLOCKS == 2 ? 16 : 32) {
         uint32_t r[16];
+        __syncwarp();                         // (the stores of the round before diverge at a ragged N)
         tc_ld16(tmem_acc + (uint32_t)(b * p.tokens + c), r);
         gemm::tc_wait_ld();
         if (n < p.N) {
