@@ -40,6 +40,8 @@ constexpr int kMaxSplit = 8;                     // portable cluster size
 constexpr int kMaxSmem = 227 * 1024;
 constexpr int kFixedSmem = 1024 /*align*/ + 256 /*barriers*/;
 constexpr int kScaleCols = 32;                   // TMEM columns kept for scales: W 2 x 8, tokens 2 x 4
+constexpr int kTmemCols = 256;                   // accumulators below them: 128 tokens, or 2 row blocks of at most 64
+static_assert(kMaxTokens + kScaleCols <= kTmemCols && 2 * 64 + kScaleCols <= kTmemCols, "accumulators and scales share the columns");
 
 struct Params {
   const uint8_t* ascales;
@@ -55,7 +57,6 @@ struct Params {
   int groups_magic;         // ceil(65536 / groups): i / groups == (i * groups_magic) >> 16 for i < 32
   int stages, stage_bytes;
   int a_box_bytes;          // bytes one activation box brings (rows beyond M up to the next power of two)
-  int tmem_cols;            // 256 or 512
   int out_f32;
   int w_static;             // the weight operand was complete before the previous kernel started
   // FUSED: x in place of packed activations
@@ -161,7 +162,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
     fence_proxy_async_smem();
   }
   if (warp == 1) {
-    gemm::tmem_alloc(tmem_slot, (uint32_t)p.tmem_cols);
+    gemm::tmem_alloc(tmem_slot, (uint32_t)kTmemCols);
     gemm::tmem_relinquish();
   }
   if (threadIdx.x == 0) {
@@ -176,7 +177,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
   const bool early_w = (FUSED || p.w_static != 0) && warp == 0;
   if (!early_w) griddep_wait();
   const uint32_t tmem_base = __shfl_sync(0xFFFFFFFFu, *tmem_slot_ptr, 0);
-  const uint32_t tmem_sfw = tmem_base + (uint32_t)p.tmem_cols - kScaleCols;
+  const uint32_t tmem_sfw = tmem_base + (uint32_t)(kTmemCols - kScaleCols);
   const uint32_t tmem_sfa = tmem_sfw + 16u;
 
   if (warp == 0) {
@@ -415,7 +416,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
   }
   gemm::tc_fence_before();
   __syncthreads();
-  if (warp == 1) gemm::tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
+  if (warp == 1) gemm::tmem_dealloc(tmem_base, (uint32_t)kTmemCols);
 }
 
 // How many clusters of `split` CTAs (one CTA per SM) run at once on this device; 0 if none.
@@ -589,7 +590,6 @@ inline bro_status launch(const Plan& pl, const Source* src, const void* acodes, 
   // CTAs of waiting clusters hold.
   int smem = kFixedSmem + parts + p.stages * p.stage_bytes;
   if (smem < kMaxSmem / 3 + 1024) smem = kMaxSmem / 3 + 1024;
-  p.tmem_cols = pl.row_blocks * p.tokens + kScaleCols <= 256 ? 256 : 512;
   p.groups_k = (int)(K / 32);
   p.token_quads = (int)((M + 3) / 4);
   p.x = nullptr;
