@@ -499,9 +499,10 @@ inline bro_status best_split(int64_t tiles, int num_k_steps, int sm_count, Cost&
 // (64, 2048, 2048) 1 part 3.7 us, 2 parts 4.3; (128, 14336, 4096) 1 part 14.5 us, 4 parts 10.9, persistent 20.8.
 //
 // More than 64 tokens fill 128 columns of the instruction and of the epilogue, whose stores are narrower than the
-// persistent kernel's boxes; with fewer than 4 K steps that shows at both ends.  M = 128, persistent -> this kernel: one
-// tile, K = 256, N = 64 2.93 -> 3.17 us, 128 tiles, K = 768, N = 16384 5.3 -> 5.7, but K = 256, N = 1000 3.6 -> 3.4 and
-// K = 768, N = 8192 4.5 -> 4.0; 4 steps gain throughout (K = 1024, N = 16384 5.9 -> 5.3, N = 64 3.9 -> 3.7).
+// persistent kernel's boxes; with fewer than 4 K steps that shows at both ends, with one step throughout.  M = 128,
+// persistent -> this kernel: one tile, K = 512, N = 64 3.2 -> 3.4 us, 128 tiles, K = 768, N = 16384 5.3 -> 5.7, a layer of
+// K = 256, N = 8192 4.85 -> 5.1; but K = 512, N = 1000 4.0 -> 3.6 and K = 768, N = 8192 4.5 -> 4.0; 4 steps gain throughout
+// (K = 1024, N = 16384 5.9 -> 5.3, N = 64 3.9 -> 3.7).
 //
 // fused = true asks for a plan that quantises inside the GEMM.  It saves the other kernel (2 us on the device, 3 us of
 // the host's time to launch it) and costs the tasks of the quantising warps, of which about half the time that the
@@ -522,7 +523,7 @@ inline bro_status plan(int64_t M, int64_t N, int num_k_steps, bool fused, int sm
   *out = Plan();
   const bool narrow = tiles_m * n128 <= sm_count;
   if (narrow ? !(tiles_m == 1 || num_k_steps >= 8) : !(tokens <= 64 && (n128 + 1) / 2 <= sm_count)) return BRO_OK;
-  if (tokens > 64 && num_k_steps < 4 && (n128 < 8 || n128 > 64)) return BRO_OK;
+  if (tokens > 64 && (num_k_steps < 2 || (num_k_steps < 4 && (n128 < 8 || n128 > 64)))) return BRO_OK;
   pl.row_blocks = narrow ? 1 : 2;
   pl.tiles_n = (int)(narrow ? n128 : (n128 + 1) / 2);
   pl.split = 1;

@@ -130,3 +130,22 @@ def test_fused_sigmoid_table_over_the_whole_bf16_range(bro, shift):
             bro.rotate_quantize_mxfp4(h, 32, c, s, bro.LAYOUT_CANONICAL)
         out.append((c, s))
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("block", [2, 4, 8, 16, 32, 64, 128])
+@pytest.mark.parametrize("M,K", [(2, 128), (131, 1152)])
+def test_fused_with_row_strides_of_any_multiple_of_8(bro, block, M, K):
+    """gate and up each with a stride of its own that is no multiple of a group; the gaps hold NaN.  Every rotation size,
+    those inside the MX group included, against the oracle."""
+    g, u = gate_up(M, K, 70 + M)
+    rc, rs = oracle.swiglu_rotate_quantize_mxfp4(synth.bf16_bits(g), synth.bf16_bits(u), block)
+    gd = torch.full((M, K + 8), float("nan"), dtype=torch.bfloat16, device="cuda")
+    ud = torch.full((M, K + 24), float("nan"), dtype=torch.bfloat16, device="cuda")
+    gd[:, :K] = g.cuda()
+    ud[:, :K] = u.cuda()
+    codes = Guarded(bro.codes_bytes(M, K)); scales = Guarded(bro.scales_bytes(M, K, bro.LAYOUT_GEMM))
+    bro.swiglu_rotate_quantize_mxfp4(gd[:, :K], ud[:, :K], block, codes.view, scales.view, bro.LAYOUT_GEMM)
+    assert bro.last_device_status() == 0
+    codes.check(); scales.check()
+    assert np.array_equal(to_canonical(scales.numpy(), M, K), rs)
+    assert np.array_equal(codes.numpy().reshape(M, K // 2), rc)
