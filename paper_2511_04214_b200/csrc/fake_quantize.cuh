@@ -18,6 +18,8 @@
 // that every store instruction of the warp writes 512 contiguous bytes of the row.
 #pragma once
 
+#include <type_traits>
+
 #include "bro_common.cuh"
 #include "rotate_quantize.cuh"
 
@@ -327,7 +329,10 @@ constexpr int64_t kWholeRowK = (int64_t)kWarps * 1024;
 // The loads of a warp's next task are issued before the current one is computed.  With `whole_rows` the warps of a CTA
 // take whole rows together, exchange the chunks' ranges through shared memory and need neither the first pass nor
 // its second read of x ([8192, 4096]: 67 -> 48 us).  Two CTAs per SM that stay (not eight that come and go) gave another 2 to 4 us.
-template <int LOG2B, bool SIGNS>
+// MODE: what the kernel writes, one of the three below.  (One kernel for all: the plain rotation paid for the registers and
+// the length of the formats' code, [1000, 2176], block 32, 3.9 -> 4.4 us, now 3.6; MXFP4 there 5.4 -> 4.9.)
+enum : int { kStatistics, kRotation, kFormats };
+template <int LOG2B, bool SIGNS, int MODE>
 __global__ void __launch_bounds__(kThreads, 2) fake_quantize_kernel(const Params p) {
   __shared__ __align__(16) float sbuf[kWarps][32 * 32];      // 4 KiB per warp
   __shared__ float2 ranges[2][kWarps];                       // whole_rows: the chunks' ranges, two rounds
@@ -335,13 +340,13 @@ __global__ void __launch_bounds__(kThreads, 2) fake_quantize_kernel(const Params
   float* wbuf = sbuf[warp];
   const int ng = (int)(p.K >> 5);
   constexpr uint32_t cbits = LOG2B == 0 ? 0x3F800000u : rq::norm_bits<(LOG2B == 0 ? 5 : LOG2B)>();
-  const bool full = p.deq != nullptr;             // (uniform over the grid)
+  const bool whole_rows = MODE == kFormats && p.whole_rows != 0;
   // row and chunk of this warp's first task, and the step to its next one
   const int c = p.chunks_per_row;
-  const int rows_at_once = p.whole_rows ? kWarps / c : 0;
+  const int rows_at_once = whole_rows ? kWarps / c : 0;
   int64_t row, step_row;
   int chunk, step_chunk = 0;
-  if (p.whole_rows) {
+  if (whole_rows) {
     const int r = warp / c;
     chunk = warp - r * c;
     row = r < rows_at_once ? (int64_t)blockIdx.x * rows_at_once + r : p.M;      // (left-over warps only keep step)
@@ -365,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, 2) fake_quantize_kernel(const Params
   uint4 cur[4], nxt[4];
   load(row, chunk, cur);
   int round = 0;
-  for (int64_t base = p.whole_rows ? (int64_t)blockIdx.x * rows_at_once : row; base < p.M; ++round) {
+  for (int64_t base = whole_rows ? (int64_t)blockIdx.x * rows_at_once : row; base < p.M; ++round) {
     const int g = chunk * 32 + lane;
     const bool live = row < p.M && g < ng;         // (K is a multiple of the block, so the lanes of a block share `live`)
     int64_t nrow = row + step_row;
@@ -391,7 +396,7 @@ __global__ void __launch_bounds__(kThreads, 2) fake_quantize_kernel(const Params
     if (LOG2B >= 6) rq::cross_lane_stage(P, 1, (lane & 1) != 0);
     if (LOG2B >= 7) rq::cross_lane_stage(P, 2, (lane & 2) != 0);
     float neglo = 0.f, hi = 0.f;
-    if (p.whole_rows || (!full && !p.mse && !p.scale_bytes)) {     // the range of this chunk
+    if (whole_rows || (MODE == kStatistics && !p.mse && !p.scale_bytes)) {     // the range of this chunk
       group_range(P, cbits, neglo, hi);
 #pragma unroll
       for (int d = 16; d >= 1; d >>= 1) {          // (all 32 lanes hold groups of the same row; dead lanes hold zeros)
@@ -399,7 +404,7 @@ __global__ void __launch_bounds__(kThreads, 2) fake_quantize_kernel(const Params
         hi = fmaxf(hi, __shfl_xor_sync(0xFFFFFFFFu, hi, d));
       }
     }
-    if (p.whole_rows) {
+    if (whole_rows) {
       if (lane == 0) ranges[round & 1][warp] = make_float2(neglo, hi);
       __syncthreads();                             // (the buffers alternate: the round before was read before this barrier)
       for (int w = warp - chunk; w < warp - chunk + c && w < kWarps; ++w) {
@@ -408,7 +413,7 @@ __global__ void __launch_bounds__(kThreads, 2) fake_quantize_kernel(const Params
         hi = fmaxf(hi, o.y);
       }
     }
-    if (!full) {
+    if (MODE == kStatistics) {
       if (p.mse) {                                 // the statistics only
         if (live) p.mse[row * ng + g] = rq::group_error(P, cbits, p.format);
       } else if (p.scale_bytes) {
@@ -423,12 +428,12 @@ __global__ void __launch_bounds__(kThreads, 2) fake_quantize_kernel(const Params
       if (!live) {                                 // (beyond the row's end: these lanes must not take the rare path)
 #pragma unroll
         for (int i = 0; i < 32; ++i) out[i] = 0.f;
-      } else if (p.format == kFormatNone) {        // the rotation itself
+      } else if (MODE == kRotation) {              // the rotation itself
         const uint64_t cc = rq::pack2(__uint_as_float(cbits), __uint_as_float(cbits));
 #pragma unroll
         for (int k = 0; k < 16; ++k) rq::unpack2(rq::mul2(P[k], cc), out[2 * k], out[2 * k + 1]);
       } else if (p.format >= kFormatRowSym) {
-        if (!p.whole_rows) {
+        if (!whole_rows) {
           neglo = __uint_as_float(__ldcg(p.rowstats + 2 * row));
           hi = __uint_as_float(__ldcg(p.rowstats + 2 * row + 1));
         }
@@ -457,7 +462,7 @@ __global__ void __launch_bounds__(kThreads, 2) fake_quantize_kernel(const Params
     for (int j = 0; j < 4; ++j) cur[j] = nxt[j];
     row = nrow;
     chunk = nchunk;
-    base = p.whole_rows ? base + step_row : row;
+    base = whole_rows ? base + step_row : row;
   }
 }
 
@@ -481,7 +486,9 @@ inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, int b
   p.whole_rows = (deq && format >= kFormatRowSym && format != kFormatNone && !rowstats) ? 1 : 0;
   const int rows_at_once = kWarps / p.chunks_per_row;
   const int64_t want = p.whole_rows ? (M + rows_at_once - 1) / rows_at_once : (M * p.chunks_per_row + kWarps - 1) / kWarps;
-  const int64_t cap = (int64_t)sm_count * 2;
+  // (two CTAs an SM that stay; the plain rotation, which the memory alone bounds, runs steadier in more and shorter ones:
+  // [16384, 4096], block 1, 72 us with two, 65 with eight, 63 with sixteen, and [4096, 4096] 14.6, 16.6 and 17.7)
+  const int64_t cap = (int64_t)sm_count * (deq && format == kFormatNone ? 8 : 2);
   const unsigned grid = (unsigned)(want < cap ? want : cap);
   auto go = [&](auto kernel) -> bro_status {
     return cuda_ok(launch_kernel(kernel, grid, kThreads, 0, st, 1, p), "fake_quantize launch") ? BRO_OK : BRO_ERR_CUDA;
@@ -489,28 +496,23 @@ inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, int b
   int lg = 0;
   while ((1 << lg) < block) ++lg;
   // (with the identity the signs only flip the output signs; they are applied all the same)
-  if (signs) {
+  auto size = [&](auto with_signs, auto mode) -> bro_status {
+    constexpr bool S = decltype(with_signs)::value;
+    constexpr int MODE = decltype(mode)::value;
     switch (lg) {
-      case 0: return go(fake_quantize_kernel<0, true>);
-      case 1: return go(fake_quantize_kernel<1, true>);
-      case 2: return go(fake_quantize_kernel<2, true>);
-      case 3: return go(fake_quantize_kernel<3, true>);
-      case 4: return go(fake_quantize_kernel<4, true>);
-      case 5: return go(fake_quantize_kernel<5, true>);
-      case 6: return go(fake_quantize_kernel<6, true>);
-      default: return go(fake_quantize_kernel<7, true>);
+      case 0: return go(fake_quantize_kernel<0, S, MODE>);
+      case 1: return go(fake_quantize_kernel<1, S, MODE>);
+      case 2: return go(fake_quantize_kernel<2, S, MODE>);
+      case 3: return go(fake_quantize_kernel<3, S, MODE>);
+      case 4: return go(fake_quantize_kernel<4, S, MODE>);
+      case 5: return go(fake_quantize_kernel<5, S, MODE>);
+      case 6: return go(fake_quantize_kernel<6, S, MODE>);
+      default: return go(fake_quantize_kernel<7, S, MODE>);
     }
-  }
-  switch (lg) {
-    case 0: return go(fake_quantize_kernel<0, false>);
-    case 1: return go(fake_quantize_kernel<1, false>);
-    case 2: return go(fake_quantize_kernel<2, false>);
-    case 3: return go(fake_quantize_kernel<3, false>);
-    case 4: return go(fake_quantize_kernel<4, false>);
-    case 5: return go(fake_quantize_kernel<5, false>);
-    case 6: return go(fake_quantize_kernel<6, false>);
-    default: return go(fake_quantize_kernel<7, false>);
-  }
+  };
+  auto any = [&](auto mode) { return signs ? size(std::true_type(), mode) : size(std::false_type(), mode); };
+  if (!deq) return any(std::integral_constant<int, kStatistics>());
+  return format == kFormatNone ? any(std::integral_constant<int, kRotation>()) : any(std::integral_constant<int, kFormats>());
 }
 
 }  // namespace fq
