@@ -486,9 +486,12 @@ inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, int b
   p.whole_rows = (deq && format >= kFormatRowSym && format != kFormatNone && !rowstats) ? 1 : 0;
   const int rows_at_once = kWarps / p.chunks_per_row;
   const int64_t want = p.whole_rows ? (M + rows_at_once - 1) / rows_at_once : (M * p.chunks_per_row + kWarps - 1) / kWarps;
-  // (two CTAs an SM that stay; the plain rotation, which the memory alone bounds, runs steadier in more and shorter ones:
-  // [16384, 4096], block 1, 72 us with two, 65 with eight, 63 with sixteen, and [4096, 4096] 14.6, 16.6 and 17.7)
-  const int64_t cap = (int64_t)sm_count * (deq && format == kFormatNone ? 8 : 2);
+  // (the formats: two CTAs an SM that stay.  The statistics need fewer registers and fit three: BFP4 error of [8192, 4096],
+  // block 1, 44 us with two and 32 with three, MXFP4 of [1000, 2176] 3.3 and 2.7.  The plain rotation, which the memory alone
+  // bounds, runs steadier in more and shorter ones: [16384, 4096], block 1, 72 us with two, 65 with eight, 63 with
+  // sixteen, and [4096, 4096] 14.6, 16.6 and 17.7)
+  const int per_sm = !deq ? 3 : (format == kFormatNone ? 8 : 2);
+  const int64_t cap = (int64_t)sm_count * per_sm;
   const unsigned grid = (unsigned)(want < cap ? want : cap);
   auto go = [&](auto kernel) -> bro_status {
     return cuda_ok(launch_kernel(kernel, grid, kThreads, 0, st, 1, p), "fake_quantize launch") ? BRO_OK : BRO_ERR_CUDA;
