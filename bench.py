@@ -70,8 +70,8 @@ def select_shapes(args):
 # regex:rotate_quantize_direct -s 6 -c 2` under `--workload cfg4 --only-block --block 32`.
 # The figures belong to one exact version of the kernels: every entry names the kernel source files it was
 # captured on and their SHA-256 at capture time, and the benchmark reports null once they have changed.
-# (Which GEMM kernel runs for a shape is decided in bro.cu; gemm_kernel_name() below restates that rule
-# and the launch list under profiles/ shows it in effect at capture time.)
+# (Which GEMM kernel runs for a shape is decided in bro.cu and in the split-K kernel's plan; gemm_kernel_name() below
+# restates the rules.)
 GEMM_SOURCES = ("bro_common.cuh", "gemm_mxfp4.cuh", "gemm_mxfp4_2cta.cuh")
 RQ_SOURCES = ("bro_common.cuh", "rotate_quantize.cuh", "rotate_quantize_direct.cuh")
 NCU_TRAFFIC = {
@@ -391,6 +391,30 @@ def time_steps(layers, steps, warmup, use_graph, barrier, sampler=None):
     return e0.elapsed_time(e1), steps
 
 
+def kernels_per_step(layers):
+    """How many kernels one step launches, counted from a captured step (a layer of few tokens is one kernel, others
+    are rotate+quantize and the GEMM)."""
+    import ctypes
+
+    import torch
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        layers.step(0)
+    cuda, raw, n = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(0)
+    if cuda.cuGraphGetNodes(raw, None, ctypes.byref(n)) != 0:
+        raise RuntimeError("cuGraphGetNodes")
+    nodes = (ctypes.c_void_p * n.value)()
+    if cuda.cuGraphGetNodes(raw, nodes, ctypes.byref(n)) != 0:
+        raise RuntimeError("cuGraphGetNodes")
+    count = 0
+    for node in nodes:
+        kind = ctypes.c_int(-1)
+        if cuda.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) != 0:
+            raise RuntimeError("cuGraphNodeGetType")
+        count += kind.value == 0                # CU_GRAPH_NODE_TYPE_KERNEL
+    return count
+
+
 def time_kernels(layers, groups):
     """Per-kernel device times: the two C-ABI calls bro_linear makes, each timed with CUDA events
     around a group of `ring` back-to-back launches (one per ring set, so no launch finds its operands
@@ -480,8 +504,13 @@ def operand_data_effect(layers, i, groups=6, sampler=None):
 
 
 def gemm_kernel_name(M, K, N, sm_count=148):
-    """Which GEMM kernel the library picks for this problem (the rule of bro.cu, restated for the record's
-    label; the ncu launch list under profiles/ shows the kernels that actually ran)."""
+    """Which GEMM kernel the library picks for this problem (the rules of bro.cu and of the split-K kernel's plan,
+    restated for the record's label)."""
+    steps, tiles_m, n128 = -(-K // 256), -(-M // 128), -(-N // 128)
+    narrow = tiles_m * n128 <= sm_count
+    one_wave = (tiles_m == 1 or steps >= 8) if narrow else (M <= 64 and -(-n128 // 2) <= sm_count)
+    if one_wave and not (M > 64 and (steps < 2 or (steps < 4 and not 8 <= n128 <= 64))):
+        return "gemm_mxfp4_splitk_kernel"
     pair = K >= 4096 and (-(-M // 256)) * (-(-N // 256)) >= 2 * (sm_count // 2)
     return "gemm_mxfp4_pair_kernel" if pair else "gemm_mxfp4_kernel"
 
@@ -524,7 +553,7 @@ def kernel_records(shapes, rq_t, gemm_t, peaks, ring, groups):
     if small:
         b = sum(gemm_bytes(*shapes[i]) for i in small)
         ts = sum(gemm_t[i] for i in small) * 1e-3
-        decode = {"bound": "hbm", "kernel": "gemm_mxfp4_kernel", "achieved": b / ts / 1e9, "peak": peaks["hbm_gbs"],
+        decode = {"bound": "hbm", "kernel": "/".join(sorted({gemm_kernel_name(*shapes[i]) for i in small})), "achieved": b / ts / 1e9, "peak": peaks["hbm_gbs"],
                   "unit": "GB/s", "frac": b / ts / 1e9 / peaks["hbm_gbs"], "peak_source": peaks["source"] + " copy bandwidth",
                   "frac_of_nominal_hbm": b / ts / 1e9 / NOMINAL_HBM_GBS,
                   "shapes": [list(shapes[i]) for i in small], "algorithmic_bytes": b,
@@ -608,11 +637,12 @@ def block_sweep(bro, synth, peaks, blocks, groups):
     producer["speedup"] = round(producer["two_step"]["us"] / producer["fused"]["us"], 3)
     del gates, ups, h
     # Simulated quantisation (Sec. 3.1: how the paper evaluates the formats): rotate, quantise, dequantise
-    # to fp32 in one launch — 2 B read and 4 B written per element (2 + 2 read for the per-row formats).
+    # to fp32 in one launch — 2 B read and 4 B written per element (the per-row formats read rows of more than 8192
+    # channels twice).
     deq = torch.empty((M, K), dtype=torch.float32, device="cuda")
     fws = torch.empty(bro.fake_quantize_workspace_bytes(M, "int4_row_asym"), dtype=torch.uint8, device="cuda")
     fake = {}
-    for fmt in ("mxfp4", "bfp4", "mxint4", "bint4", "int4_row_sym", "int4_row_asym"):     # (the last two: two passes over x)
+    for fmt in ("mxfp4", "bfp4", "mxint4", "bint4", "int4_row_sym", "int4_row_asym"):
         for i in range(2):
             bro.rotate_fake_quantize(xs[i % ring], 32, deq, fmt, workspace=fws)
         ts = []
@@ -625,7 +655,7 @@ def block_sweep(bro, synth, peaks, blocks, groups):
             torch.cuda.synchronize()
             ts.append(a.elapsed_time(c) / ring)
         ms = statistics.mean(ts)
-        nbytes = 8.0 if fmt.startswith("int4_row") else 6.0      # (the per-row formats read x twice)
+        nbytes = 8.0 if fmt.startswith("int4_row") and K > 8192 else 6.0
         fake[fmt] = {"us": round(ms * 1e3, 2), "gbs": round(M * K * nbytes / (ms * 1e-3) / 1e9, 1),
                      "frac_of_measured_copy": round(M * K * nbytes / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"], 4)}
     del deq, fws
@@ -674,6 +704,7 @@ def run_ours(args):
     if status != 0:
         raise SystemExit(f"device status {bro.status_string(status)} after the timed region")
     value = aggregate_throughput(flops_per_step, steps, world, ms_total) / 1e12
+    launches_per_step = kernels_per_step(layers)
 
     groups = max(3, min(steps // ring, 16))
     rq_t, gemm_t = time_kernels(layers, groups)
@@ -824,7 +855,7 @@ def run_ours(args):
                        "rotation": "randomised block Hadamard (diag(s) H)" if args.randomised else "block Hadamard"},
             "clocks": clocks,
             "e2e": e2e,
-            "gpu_launches": steps * len(shapes) * 2,
+            "gpu_launches": steps * launches_per_step,
             "roofline": roofline,
             "decode": decode,
             "rotate_quantize": rq_rec,

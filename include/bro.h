@@ -149,9 +149,11 @@ bro_status bro_gemm_mxfp4(const void* acodes, const void* ascales, const void* w
 
 /*
  * The whole layer on one stream: bro_rotate_quantize_mxfp4(x) into the workspace, then
- * bro_gemm_mxfp4 against weights packed by bro_pack_weights with the same `block`.
+ * bro_gemm_mxfp4 against weights packed by bro_pack_weights with the same `block`.  For at most 64 tokens
+ * and sizes where it pays, one kernel does both: the workspace receives the same codes and scales, the
+ * result the same sums up to the order of fp32 additions.
  *   workspace   bro_linear_workspace_bytes(M, N, K) bytes, 1024-byte aligned.
- *   y_bf16      [M, ldy] bf16.
+ *   y_bf16      [M, ldy] bf16.  May overlap x (a layer in place): all of x is read before y is written.
  */
 bro_status bro_linear(const void* x_bf16, int64_t M, int64_t K, int64_t ldx, int block,
                       const void* wcodes, const void* wscales, int64_t N, void* y_bf16,
@@ -296,7 +298,8 @@ bro_status bro_rotate_fake_quantize(const void* x_bf16, int64_t M, int64_t K, in
  * The first two are the fifth format of the paper's study (Sec. 3.2 / Fig. 2: "INT4" = per-channel
  * symmetric weights — a row of W is an output channel — and per-token asymmetric activations — a row
  * of X is a token); the paper gives no formulas, the rules above are this library's reading.  They
- * take two passes over x (the first leaves each row's range in the workspace) and need
+ * take one pass over x for K <= 8192 and blocks up to 128, else two (the first leaves each row's range in the
+ * workspace), and at any size need
  *   workspace   device, bro_fake_quantize_workspace_bytes(M, format) bytes (8 per row; 0 for the other
  *               formats, which ignore it), 8-byte aligned; contents undefined afterwards.
  * BRO_ERR_WORKSPACE if it is missing or too small.  bro_rotate_fake_quantize is this call without a
@@ -327,8 +330,8 @@ bro_status bro_group_scale_bytes(const void* x_bf16, int64_t M, int64_t K, int64
  *   paper's 0.1 %), t = the k-th largest |x|; an entry is an outlier iff |x| >= t (ties at t all count).
  *   mask[m, g] (uint8 [M, K/32]) = 1 iff group g of row m holds an outlier, else 0.
  *   info       device, 4 x uint32, 16-byte aligned: [0] = the bf16 pattern of t, [1] = 0, [2..3] = k.
- *   workspace  device, bro_outlier_workspace_bytes() bytes, 16-byte aligned (a histogram of the 32768
- *              bf16 magnitudes; overwritten).
+ *   workspace  device, bro_outlier_workspace_bytes() bytes, 16-byte aligned (a histogram of bf16
+ *              magnitudes; overwritten).  The mask also holds an intermediate code per group meanwhile.
  *   Inputs must be finite.
  */
 size_t bro_outlier_workspace_bytes(void);
@@ -351,7 +354,8 @@ bro_status bro_scale_inflation(const uint8_t* scales_before, const uint8_t* scal
 /*
  * ---- tuning and testing -------------------------------------------------------------------------
  * The *_ex entry points are the plain ones plus a `flags` word that forces a kernel variant the
- * library would not pick by itself for this problem (the plain entry points pass 0).  Every variant
+ * library would not pick by itself for this problem (the plain entry points pass 0).  Any GEMM flag
+ * excludes the split-K kernel for few output tiles, any flag of bro_linear_ex the one-kernel layer.  Every variant
  * computes the same function: codes and scales are bit-identical, GEMM results agree within the
  * accumulation-order tolerance.  They exist so that each variant can be tested and timed on any
  * shape; `signs_bf16` may be NULL (plain rotation) or the +-1 vector of the randomised rotation.
@@ -361,7 +365,7 @@ bro_status bro_scale_inflation(const uint8_t* scales_before, const uint8_t* scal
 #define BRO_FLAG_GEMM_PAIR 0x10u      /* GEMM: two CTAs per 256 x 256 tile (cta_group::2) */
 #define BRO_FLAG_GEMM_TILE_N128 0x20u /* GEMM: 128 x 128 tiles */
 #define BRO_FLAG_GEMM_TILE_N256 0x40u /* GEMM: 128 x 256 tiles even when N <= 128 */
-#define BRO_FLAG_GEMM_NO_SPLIT 0x80u  /* GEMM: no half-width units in the last round of the grid */
+#define BRO_FLAG_GEMM_NO_SPLIT 0x80u  /* GEMM: no half-width units in the last round of the grid, no split-K kernel */
 #define BRO_FLAG_GEMM_SINGLE 0x100u   /* GEMM: one CTA per 128 x 256 (or 128 x 128) tile, whatever the size */
 bro_status bro_rotate_quantize_mxfp4_ex(const void* x_bf16, int64_t M, int64_t K, int64_t ldx, int block,
                                         const void* signs_bf16, void* codes, void* scales,

@@ -1,4 +1,4 @@
-// libbro: C ABI over the two sm_100a kernels (see include/bro.h for the contract).
+// libbro: C ABI over the sm_100a kernels of this folder (see include/bro.h for the contract).
 // Host-side work only: argument validation, TMA tensor-map encoding, launches.
 #include <cuda.h>
 #include <cuda_runtime.h>

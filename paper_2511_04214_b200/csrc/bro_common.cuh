@@ -177,7 +177,10 @@ __device__ __forceinline__ void bulk_load_1d(uint32_t dst, const void* src, uint
 // so the next kernel in the stream may be scheduled while this one still runs: its CTAs start on
 // SMs as they become free and run their prologue (barrier set-up, TMEM allocation, descriptor
 // prefetch) early.  griddep_wait() blocks until all earlier grids in the stream have completed
-// and their writes are visible; every thread calls it before its first access to global memory.
+// and their writes are visible; every thread calls it before its first access to global memory, with two
+// exceptions, both of the weights in the GEMMs: inside the whole-layer calls, where the weights are older than the kernel
+// in front (whose own wait precedes its launch_dependents), the first weight tiles are loaded before it, and the
+// one-kernel layer, which has no such kernel in front, only draws them into L2.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

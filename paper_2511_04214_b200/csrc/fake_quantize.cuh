@@ -108,7 +108,7 @@ __device__ __forceinline__ void group_dequant_any(const uint64_t (&P)[16], uint3
 // bits.  Groups that hold an infinity or a NaN (amax_nan then is one too) and the ends of the exponent range take the forms
 // above.  They are rare, but a warp that holds one waits for both forms; so groups of zeros have an answer of their own,
 // and the lanes beyond the end of a row compute nothing.
-// [8192, 4096], block 32: BFP4 56 -> 40 us, BINT4 59 -> 41 us, INT4 per row 81 -> 67 us.
+// [8192, 4096], block 32, general forms -> these: BFP4 56 -> 36 us, BINT4 58 -> 36, MXFP4 39 -> 36, MXINT4 41 -> 36.
 __device__ __forceinline__ float amax_nan(const uint64_t (&Y)[16]) {
   float m = 0.f, m2 = 0.f;
 #pragma unroll
@@ -328,7 +328,8 @@ constexpr int64_t kWholeRowK = (int64_t)kWarps * 1024;
 // LOG2B = 0: no rotation; 1..4: blocks of 2..16 inside the group; 5, 6, 7: blocks of 32, 64, 128.
 // The loads of a warp's next task are issued before the current one is computed.  With `whole_rows` the warps of a CTA
 // take whole rows together, exchange the chunks' ranges through shared memory and need neither the first pass nor
-// its second read of x ([8192, 4096]: 67 -> 48 us).  Two CTAs per SM that stay (not eight that come and go) gave another 2 to 4 us.
+// its second read of x ([8192, 4096], block 32, both formats: 78 us in two passes, now 45).  Without the early loads the
+// formats take 43 instead of 36 us there, with eight CTAs an SM that come and go 44.
 // MODE: what the kernel writes, one of the three below.  (One kernel for all: the plain rotation paid for the registers and
 // the length of the formats' code, [1000, 2176], block 32, 3.9 -> 4.4 us, now 3.6; MXFP4 there 5.4 -> 4.9.)
 enum : int { kStatistics, kRotation, kFormats };

@@ -9,14 +9,14 @@
 //   * the `split` CTAs of a cluster share a tile, each takes a contiguous range of its 256-element K steps
 //     and sends its fp32 partial sums to the CTAs that own the tokens (distributed shared memory); a token's
 //     owner adds the parts in rank order, converts and stores.  No workspace, no atomics, fixed order.
-//   * FUSED (the whole-layer calls with few tokens): there is no rotate+quantize kernel in front.  Sixteen warps, eight
-//     of them those of the epilogue, rotate and quantise the [tokens, 256] slice of x of every K step straight into the
-//     stage (a lane owns one MX group, the arithmetic is that of the stand-alone kernel, bit for bit) and arrive on
-//     its barrier beside the weight bytes.  Every CTA repeats the work on its K range, hidden behind the weights; the
+//   * FUSED (the whole-layer calls with at most 64 tokens, see plan()): there is no rotate+quantize kernel in front.
+//     Sixteen warps, eight of them those of the epilogue, rotate and quantise the [tokens, 256] slice of x of every K
+//     step straight into the stage (a lane owns one MX group, the arithmetic is that of the stand-alone kernel, bit for
+//     bit) and arrive on its barrier beside the weight bytes.  Every CTA repeats the work on its K range, hidden behind the weights; the
 //     first tile of columns also leaves codes and scales in the caller's workspace, as the stand-alone kernel would.
 //   * otherwise, with W packed before the previous kernel in the stream started (the whole-layer calls), the whole ring of
 //     weight tiles is requested before griddepcontrol.wait, under the rotate+quantize kernel.
-// Warps: 0 TMA producer, 1 TMEM owner and MMA issuer, 2..9 epilogue.  Every mbarrier wait is bounded, and all
+// Warps: 0 TMA producer, 1 TMEM owner and MMA issuer, 2..9 epilogue (FUSED: 2..17 quantise).  Every mbarrier wait is bounded, and all
 // threads of a cluster reach both cluster barriers whatever happened before.
 #pragma once
 

@@ -137,7 +137,8 @@ __device__ __forceinline__ bool find_threshold(Count&& count, unsigned long long
 
 // The outliers are the top 0.1 % (top k of n) of the magnitudes, found exactly from a histogram of bf16 patterns; one pass
 // over x.  A shared-memory atomic per value bounded it before (75 us for 67 M values and 20 us for the search in a
-// launch of its own; now 42 us, of which 30 us are the pass, issue-bound, and 12 us merging and search), so only values of at least `lowest` are counted, a pattern that every CTA derives from the same 4096 sampled
+// launch of its own; now 42 us, of which 30 us are the pass, issue-bound, and 12 us merging and search), so only values of
+// at least `lowest` are counted, a pattern that every CTA derives from the same 4096 sampled
 // values such that about 4 k values (and 12 of the sample) lie at or above it: the loop reduces a group to its maximum and
 // touches the histogram for the few groups that reach `lowest`.  The last CTA to merge its histogram searches the
 // threshold, without a launch of its own.  Should the sample have misled (fewer than k counted), that CTA counts everything

@@ -29,6 +29,10 @@ def test_kernel_label_follows_the_dispatch_rule():
     assert bench.gemm_kernel_name(1024, 8192, 28672) == "gemm_mxfp4_pair_kernel"
     assert bench.gemm_kernel_name(2048, 2048, 8192) == "gemm_mxfp4_kernel"           # K < 4096
     assert bench.gemm_kernel_name(4096, 4096, 1024) == "gemm_mxfp4_kernel"           # fewer than two rounds of pairs
+    assert bench.gemm_kernel_name(16, 8192, 28672) == "gemm_mxfp4_splitk_kernel"     # one wave of 256-row tiles of W
+    assert bench.gemm_kernel_name(512, 2048, 2048) == "gemm_mxfp4_splitk_kernel"     # four token tiles, 8 K steps
+    assert bench.gemm_kernel_name(512, 1024, 2048) == "gemm_mxfp4_kernel"            # 4 K steps
+    assert bench.gemm_kernel_name(100, 512, 640) == "gemm_mxfp4_kernel"              # many tokens, few steps, few tiles
 
 
 def test_digest_covers_the_kernel_sources():
