@@ -191,9 +191,11 @@ __device__ __forceinline__ void named_barrier_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 // TMA store shared -> global of one box; out-of-range parts of the box are clipped.
-// Forms for a converged warp, executed by the lane for which `issue` is not zero.  (Not elected per instruction as the loads
-// are: that made launches that the epilogue bounds slower.  Elected -> `issue`, (512, 256, 28672) 10.0 -> 8.9 us,
-// (1024, 512, 28672) 17.1 -> 15.4, (8192, 512, 8192) 31.8 -> 29.7; in fp32 15.7 -> 13.8, 26.3 -> 24.8, 48.9 -> 47.1.)
+// Forms for a converged warp.  The fp32 epilogue elects the lane per instruction, the bf16 one names it by a flag (`issue`,
+// not zero in that lane): electing made launches that the bf16 epilogue bounds slower, flag -> elected (512, 256, 28672)
+// 8.9 -> 10.0 us, (1024, 512, 28672) 15.4 -> 17.1, (8192, 512, 8192) 29.7 -> 31.8.  In fp32 it depends on K: elected
+// (777, 4384, 6004) 24.0 -> 23.8 and (2048, 4096, 4096) 19.1 -> 18.9, but (2048, 512, 8192) 14.0 -> 16.8.  The store, its
+// commit and its wait belong to one lane: an epilogue uses one of the two forms throughout.
 __device__ __forceinline__ void tma_store_2d_if(uint32_t issue, const CUtensorMap* m, uint32_t src, int x, int y) {
   asm volatile(
       "{ .reg .pred q; setp.ne.b32 q, %4, 0;\n\t"
@@ -208,6 +210,21 @@ __device__ __forceinline__ void bulk_commit_if(uint32_t issue) {
 template <int N>
 __device__ __forceinline__ void bulk_wait_read_if(uint32_t issue) {
   asm volatile("{ .reg .pred q; setp.ne.b32 q, %0, 0;\n\t@q cp.async.bulk.wait_group.read %1; }" ::"r"(issue), "n"(N) : "memory");
+}
+__device__ __forceinline__ void tma_store_2d_elect(const CUtensorMap* m, uint32_t src, int x, int y) {
+  asm volatile(
+      "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
+      "@q cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1]; }" ::"l"(
+          reinterpret_cast<uint64_t>(m)),
+      "r"(src), "r"(x), "r"(y)
+      : "memory");
+}
+__device__ __forceinline__ void bulk_commit_elect() {
+  asm volatile("{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t@q cp.async.bulk.commit_group; }" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void bulk_wait_read_elect() {
+  asm volatile("{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t@q cp.async.bulk.wait_group.read %0; }" ::"n"(N) : "memory");
 }
 __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -378,7 +395,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem_acc, int buf, int la
   // fp32: one box of 32 columns x 32 rows per chunk, 128 bytes a row as the 64 bf16 columns of a pair.  (Stores from
   // registers, 16 bytes a lane and the lanes a row of y apart, took 20 of a launch's 31 us at (777, 4384, 6004).)
   auto emit_f32 = [&](const uint32_t (&r)[32], int col0, uint32_t sbuf) {
-    if (stage_stride == 0u) bulk_wait_read_if<0>(issue);
+    if (stage_stride == 0u) bulk_wait_read_elect<0>();
     __syncwarp();
     const uint32_t rowaddr = sbuf + (uint32_t)lane * 128u, sw = (uint32_t)lane & 7u;
 #pragma unroll
@@ -387,8 +404,8 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem_acc, int buf, int la
     __syncwarp();
     // (the map ends at the last multiple of 4 columns, see make_out_map; the up to 3 behind it come from the buffer)
     const int64_t n_tma = N & ~(int64_t)3;
-    if (col0 < n_tma && row0 < M) tma_store_2d_if(issue, tmy, sbuf, col0, row0);
-    bulk_commit_if(issue);
+    if (col0 < n_tma && row0 < M) tma_store_2d_elect(tmy, sbuf, col0, row0);
+    bulk_commit_elect();
     if (n_tma < N && n_tma >= col0 && n_tma < (int64_t)col0 + kChunkCols) {
       if (row < M) {
         float* dst = static_cast<float*>(y) + row * ldy + n_tma;
@@ -616,7 +633,8 @@ gemm_mxfp4_kernel(const __grid_constant__ CUtensorMap tma, const __grid_constant
     }
     // the staging buffer must have been read before this CTA's shared memory goes away; the writes
     // themselves complete with the kernel
-    bulk_wait_read_if<0>(lane == 0 ? 1u : 0u);
+    if (OUT_F32) bulk_wait_read_elect<0>();
+    else bulk_wait_read_if<0>(lane == 0 ? 1u : 0u);
   }
   tc_fence_before();
   __syncthreads();

@@ -265,7 +265,8 @@ gemm_mxfp4_pair_kernel(const __grid_constant__ CUtensorMap tma, const __grid_con
     }
     // the staging buffer must have been read before this CTA's shared memory goes away; the writes
     // themselves complete with the kernel
-    gemm::bulk_wait_read_if<0>(lane == 0 ? 1u : 0u);
+    if (OUT_F32) gemm::bulk_wait_read_elect<0>();
+    else gemm::bulk_wait_read_if<0>(lane == 0 ? 1u : 0u);
   }
   gemm::tc_fence_before();
   __syncthreads();
