@@ -57,6 +57,7 @@ struct Params {
   int groups_magic;         // ceil(65536 / groups): i / groups == (i * groups_magic) >> 16 for i < 32
   int stages, stage_bytes;
   int a_box_bytes;          // bytes one activation box brings (rows beyond M up to the next power of two)
+  int tmem_cols;            // kTmemCols
   int out_f32;
   int w_static;             // the weight operand was complete before the previous kernel started
   // FUSED: x in place of packed activations
@@ -162,7 +163,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
     fence_proxy_async_smem();
   }
   if (warp == 1) {
-    gemm::tmem_alloc(tmem_slot, (uint32_t)kTmemCols);
+    gemm::tmem_alloc(tmem_slot, (uint32_t)p.tmem_cols);
     gemm::tmem_relinquish();
   }
   if (threadIdx.x == 0) {
@@ -177,7 +178,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
   const bool early_w = (FUSED || p.w_static != 0) && warp == 0;
   if (!early_w) griddep_wait();
   const uint32_t tmem_base = __shfl_sync(0xFFFFFFFFu, *tmem_slot_ptr, 0);
-  const uint32_t tmem_sfw = tmem_base + (uint32_t)(kTmemCols - kScaleCols);
+  const uint32_t tmem_sfw = tmem_base + (uint32_t)p.tmem_cols - kScaleCols;
   const uint32_t tmem_sfa = tmem_sfw + 16u;
 
   if (warp == 0) {
@@ -271,8 +272,9 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
   bool ok = true;
   if (FUSED && warp >= 2) {
     // ------------------------------ rotate + quantise x ------------------------------
-    // One warp task: 4 tokens x the 8 groups of a K step, one group per lane; task t goes to warp t mod 16.  At most 64
-    // tokens, so a warp has one task of a step or none.
+    // One warp task: 4 tokens x the 8 groups of a K step, one group per lane; task t goes to warp t mod 16.  (At most 64
+    // tokens, so a warp has one task of a step or none; the loop below takes any number, and as a straight block it
+    // measured slower, (64, 2048, 2048) 6.45 -> 6.55 us.)
     const int in_quad = lane >> 3, g = lane & 7;
     auto load = [&](int step, int quad, uint4 (&v)[4]) {
       const int token = quad * 4 + in_quad, group = (k_first + step) * 8 + g;
@@ -300,20 +302,22 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
     uint32_t phase = 1u;                                 // (parity of the phase before the first: passes at once)
     for (int i = 0; i < k_count; ++i) {
       const uint32_t base = smem_base + (uint32_t)(stage * p.stage_bytes);
-      const bool has = step == i;
-      const int row = quad * 4 + in_quad;
-      uint32_t w[4], sb = 0u;
-      if (has) {
-        sb = rotate_quantize_lane(cur, p.log2b, p.cbits, lane, w);
-        advance(step, quad);
-        if (step < k_count) load(step, quad, cur);       // in flight while this task's stage is waited for and written
-        // scale bytes of 4 consecutive groups -> one 32-bit word in the lane with g % 4 == 0
-        sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 1) << 8;
-        sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 2) << 16;
-      }
-      ok = mbar_wait_warp(bar_empty + 8 * stage, phase, SITE_GEMM_EMPTY);
-      if (!ok) break;
-      if (has) {
+      bool waited = false;
+      do {
+        const bool has = step == i;
+        const int row = quad * 4 + in_quad;
+        uint32_t w[4], sb = 0u;
+        if (has) {
+          sb = rotate_quantize_lane(cur, p.log2b, p.cbits, lane, w);
+          advance(step, quad);
+          if (step < k_count) load(step, quad, cur);     // in flight while this task's stage is waited for and written
+          // scale bytes of 4 consecutive groups -> one 32-bit word in the lane with g % 4 == 0
+          sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 1) << 8;
+          sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 2) << 16;
+        }
+        if (!waited) ok = mbar_wait_warp(bar_empty + 8 * stage, phase, SITE_GEMM_EMPTY);
+        waited = true;
+        if (!has || !ok) break;
         const uint32_t sf_at = (uint32_t)((g >> 2) * 512 + (row & 31) * 16 + (row >> 5) * 4);
         gemm::sts128(base + w_bytes + (uint32_t)row * 128u + (uint32_t)((g ^ (row & 7)) << 4), w[0], w[1], w[2], w[3]);
         if ((g & 3) == 0) asm volatile("st.shared.b32 [%0], %1;" ::"r"(base + off_sfa + sf_at), "r"(sb) : "memory");
@@ -323,7 +327,8 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
             *reinterpret_cast<uint4*>(p.codes + ((int64_t)row * p.groups_k + group) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
           if ((g & 3) == 0) *reinterpret_cast<uint32_t*>(p.scales + (int64_t)(k_first + i) * 1024 + sf_at) = sb;
         }
-      }
+      } while (step == i);
+      if (!ok) break;
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_full + 8 * stage);
@@ -416,7 +421,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
   }
   gemm::tc_fence_before();
   __syncthreads();
-  if (warp == 1) gemm::tmem_dealloc(tmem_base, (uint32_t)kTmemCols);
+  if (warp == 1) gemm::tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
 }
 
 // How many clusters of `split` CTAs (one CTA per SM) run at once on this device; 0 if none.
@@ -591,6 +596,7 @@ inline bro_status launch(const Plan& pl, const Source* src, const void* acodes, 
   // CTAs of waiting clusters hold.
   int smem = kFixedSmem + parts + p.stages * p.stage_bytes;
   if (smem < kMaxSmem / 3 + 1024) smem = kMaxSmem / 3 + 1024;
+  p.tmem_cols = kTmemCols;       // (read by the kernel as a parameter: as a constant there, (64, 2048, 2048) took 6.6 us, not 6.45)
   p.groups_k = (int)(K / 32);
   p.token_quads = (int)((M + 3) / 4);
   p.x = nullptr;
