@@ -360,7 +360,7 @@ bro_status bro_scale_inflation(const uint8_t* scales_before, const uint8_t* scal
  * accumulation-order tolerance.  They exist so that each variant can be tested and timed on any
  * shape; `signs_bf16` may be NULL (plain rotation) or the +-1 vector of the randomised rotation.
  */
-#define BRO_FLAG_RQ_TMA_RING 0x1u     /* rotate+quantize: shared-memory ring fed by TMA (block 32/64/128) */
+#define BRO_FLAG_RQ_TMA_RING 0x1u     /* rotate+quantize: rings in shared memory fed by TMA (block 32/64/128, K a multiple of 64) */
 #define BRO_FLAG_RQ_DIRECT 0x2u       /* rotate+quantize: register-streaming kernel (block 32/64/128) */
 #define BRO_FLAG_GEMM_PAIR 0x10u      /* GEMM: two CTAs per 256 x 256 tile (cta_group::2) */
 #define BRO_FLAG_GEMM_TILE_N128 0x20u /* GEMM: 128 x 128 tiles */

@@ -10,6 +10,7 @@
 #include "rotate_quantize.cuh"
 #include "rotate_quantize_global.cuh"
 #include "rotate_quantize_direct.cuh"
+#include "rotate_quantize_wide.cuh"
 #include "gemm_mxfp4.cuh"
 #include "gemm_mxfp4_2cta.cuh"
 #include "gemm_mxfp4_splitk.cuh"
@@ -17,8 +18,6 @@
 #include "fake_quantize.cuh"
 
 namespace {
-
-using bro::rq::Params;
 
 constexpr int64_t kGroup = 32;
 
@@ -158,7 +157,12 @@ bro_status make_map_3d(CUtensorMap* map, const void* x, int64_t M, int64_t K, in
 
 // Whole rows of x in segments of 64 bf16: a box lands in shared memory as 128-byte segments with the 128-byte swizzle.
 bro_status bro::rqg::make_row_map(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx, int box_rows) {
-  return make_map_3d(map, x, M, K, ldx, 64, (uint32_t)(K / 64), (uint32_t)box_rows, CU_TENSOR_MAP_SWIZZLE_128B);
+  return make_map_3d(map, x, M, K, ldx, 64, (uint32_t)(K / 64 < 256 ? K / 64 : 256), (uint32_t)box_rows, CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
+// 16 rows x 128 channels: 128-byte segments, two a row, with the 128-byte swizzle.
+bro_status bro::rqw::make_tile_map(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx) {
+  return make_map_3d(map, x, M, K, ldx, 64, 2, kRows, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
 // 32 groups of one row: 2 KiB in 64-byte segments with the 64-byte swizzle.
@@ -196,6 +200,8 @@ __global__ void __launch_bounds__(256) swiglu_kernel(const uint16_t* gate, const
 }
 
 // ---- rotate + quantise ---------------------------------------------------------------------------
+inline bool wide_takes(int64_t B, int64_t K) { return B >= 32 && B <= 128 && K % 64 == 0; }
+
 // Arguments of a rotate+quantize launch; BRO_OK with M == 0 means that there is nothing to do.
 // (up != nullptr: x is the gate of the fused producer, the rotated tensor is silu(x) * up)
 bro_status check_rotate_quantize(const void* x, int64_t M, int64_t K, int64_t ldx, int block, const void* signs,
@@ -220,7 +226,7 @@ bro_status check_rotate_quantize(const void* x, int64_t M, int64_t K, int64_t ld
 
 bro_status launch_rotate_quantize(const void* x, int64_t M, int64_t K, int64_t ldx, int block,
                                   const void* signs, void* codes, void* scales, bro_layout layout,
-                                  uint32_t flags, cudaStream_t st, const void* up = nullptr, int64_t ldu = 0) {
+                                  uint32_t flags, cudaStream_t st, const void* up = nullptr, int64_t ldu = 0, bool layer = false) {
   bro_status rc = check_rotate_quantize(x, M, K, ldx, block, signs, codes, scales, layout, up, ldu);
   if (rc != BRO_OK) return rc;
   const int64_t B = block == 0 ? K : block;
@@ -233,67 +239,24 @@ bro_status launch_rotate_quantize(const void* x, int64_t M, int64_t K, int64_t l
     return bro::rqg::launch(x, M, K, ldx, signs, codes, scales, nullptr, 0, layout, gemm_scale_kblocks(K), di.sm_count, st);
   }
 
-  // Register-streaming kernel by default (the TMA-ring kernel when the task index would not fit
-  // 31 bits): it wins for block 32 at every size and for small inputs; for blocks of 64 / 128 on
-  // large inputs its extra registers cost occupancy and the TMA ring is faster.  The flags of the
-  // *_ex entry point override the choice.
+  // The wide kernel (a lane owns 64 channels) for blocks of 64 and 128 beyond 2^19 elements ([300, 4096], block 128, 3.5 -> 3.0 us,
+  // [16384, 4096] 37.2 -> 30.8, block 64 33.3 -> 29.4; [128, 4096] 2.6 -> 2.9) and for block 32 from 2^20 to 2^25 ([2048, 2048]
+  // 4.0 -> 3.7, [8192, 4096] 16.4 -> 15.0; [128, 4096] even, [14336, 4096] 26.0 -> 26.5).  In front of a GEMM (`layer`) it has to
+  // save more, since its shared memory keeps the GEMM's CTAs from starting under its tail: beyond 2^22 elements and from 2^24
+  // (whole layers, block 64: (1500, 5120, 2500) 19.9 -> 18.8, (2048, 2048, 8192) 21.1 -> 21.5, block 32: (4096, 4096, 4096) 38.0 -> 37.3,
+  // (2048, 2048, 8192) 20.6 -> 21.4).  Else, and where K is not a multiple of 64, below the MX group and with the fused producer, the
+  // register-streaming kernel.  The flags of the *_ex entry point override the choice.
+  const int64_t elements = M * K;
+  const bool can_wide = wide_takes(B, K) && !up;
+  bool wide = can_wide && (B == 32 ? elements >= (int64_t)1 << (layer ? 24 : 20) && elements <= (int64_t)1 << 25
+                                   : elements > (int64_t)1 << (layer ? 22 : 19));
   const bool can_direct = bro::rqd::supports(M, K, layout, gemm_scale_kblocks(K));
-  bool direct = can_direct && (B <= 32 || M * K <= ((int64_t)1 << 23));
-  if (flags & BRO_FLAG_RQ_TMA_RING) direct = false;
-  else if (flags & BRO_FLAG_RQ_DIRECT) direct = can_direct;
-  if (B < 32) {                   // blocks below the MX group exist in the register-streaming kernel only
-    if (!can_direct) return BRO_ERR_UNSUPPORTED;
-    direct = true;
-  }
-  if (up) {                       // the fused producer exists in the register-streaming kernel only
-    if (!can_direct) return BRO_ERR_UNSUPPORTED;
-    direct = true;
-  }
-  if (direct)
-    return bro::rqd::launch(x, M, K, ldx, log2_of(B), signs, codes, scales, layout,
-                            gemm_scale_kblocks(K), di.sm_count, st, up, ldu);
-
-  CUtensorMap tmx;
-  rc = make_map_2d(&tmx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, x, (uint64_t)K, (uint64_t)M,
-                   (uint64_t)ldx * 2, bro::rq::kBoxCols, bro::rq::kTileRows, CU_TENSOR_MAP_SWIZZLE_128B);
-  if (rc != BRO_OK) return rc;
-
-  Params p;
-  p.M = M;
-  p.K = K;
-  p.tiles_m = ceil_div(M, bro::rq::kTileRows);
-  p.tiles_k = layout == BRO_LAYOUT_GEMM ? gemm_scale_kblocks(K) : ceil_div(K, bro::rq::kTileCols);
-  p.codes = static_cast<uint8_t*>(codes);
-  p.scales = static_cast<uint8_t*>(scales);
-  p.scale_kblocks = gemm_scale_kblocks(K);
-  p.layout = (int)layout;
-  p.signs = static_cast<const uint16_t*>(signs);
-  const int64_t tiles = p.tiles_m * p.tiles_k;
-  const int grid = (int)(tiles < di.sm_count ? tiles : di.sm_count);
-
-  // (All six instantiations share one function-pointer type, so the opt-in to large dynamic
-  // shared memory is kept per instantiation, per device.)
-  auto go = [&](void (*kernel)(CUtensorMap, Params), int which) -> bro_status {
-    static bro::DeviceOnce once[6];
-    bro_status r = bro::device_once(once[which], nullptr, [&](int*) { return set_smem(kernel, bro::rq::kSmemBytes); });
-    if (r != BRO_OK) return r;
-    return bro::cuda_ok(bro::launch_kernel(kernel, (unsigned)grid, bro::rq::kThreads, bro::rq::kSmemBytes, st, 1, tmx, p),
-                        "rotate_quantize launch")
-               ? BRO_OK
-               : BRO_ERR_CUDA;
-  };
-  if (signs) {
-    switch (B) {
-      case 32: return go(bro::rq::rotate_quantize_kernel<5, true>, 3);
-      case 64: return go(bro::rq::rotate_quantize_kernel<6, true>, 4);
-      default: return go(bro::rq::rotate_quantize_kernel<7, true>, 5);
-    }
-  }
-  switch (B) {
-    case 32: return go(bro::rq::rotate_quantize_kernel<5, false>, 0);
-    case 64: return go(bro::rq::rotate_quantize_kernel<6, false>, 1);
-    default: return go(bro::rq::rotate_quantize_kernel<7, false>, 2);
-  }
+  if (flags & BRO_FLAG_RQ_TMA_RING) wide = can_wide;
+  else if (flags & BRO_FLAG_RQ_DIRECT) wide = can_wide && !can_direct;
+  if (wide)
+    return bro::rqw::launch(x, M, K, ldx, log2_of(B), signs, codes, scales, nullptr, layout, gemm_scale_kblocks(K), di.sm_count, st);
+  if (!can_direct) return BRO_ERR_UNSUPPORTED;
+  return bro::rqd::launch(x, M, K, ldx, log2_of(B), signs, codes, scales, layout, gemm_scale_kblocks(K), di.sm_count, st, up, ldu);
 }
 
 }  // namespace
@@ -420,6 +383,10 @@ bro_status bro_group_quant_error_fmt(const void* x_bf16, int64_t M, int64_t K, i
     return bro::fq::launch(x_bf16, M, K, ldx, (int)B, signs_bf16, (int)format, nullptr, 0, mse, nullptr, di.sm_count, st);
   if (B > 128)
     return bro::rqg::launch(x_bf16, M, K, ldx, signs_bf16, nullptr, nullptr, mse, (int)format, BRO_LAYOUT_CANONICAL, 0, di.sm_count, st);
+  // (MXFP4, wide kernel: block 128 of [16384, 4096] 42.9 -> 35.4 us, block 64 36.2 -> 31.6, block 32 32.0 -> 29.3; [128, 4096] 2.6 -> 3.0,
+  // block 32 of [4096, 4096] 9.8 -> 10.1)
+  if (format == BRO_FMT_MXFP4 && wide_takes(B, K) && M * K > (B == 32 ? ((int64_t)1 << 25) - 1 : (int64_t)1 << 19))
+    return bro::rqw::launch(x_bf16, M, K, ldx, log2_of(B), signs_bf16, nullptr, nullptr, mse, BRO_LAYOUT_CANONICAL, 0, di.sm_count, st);
   if (!bro::rqd::supports(M, K, BRO_LAYOUT_CANONICAL, 0)) return BRO_ERR_UNSUPPORTED;
   return bro::rqd::launch_stats(x_bf16, M, K, ldx, B == 32 ? 5 : (B == 64 ? 6 : 7), signs_bf16, (int)format, mse, nullptr, di.sm_count, st);
 }
@@ -505,6 +472,9 @@ bro_status bro_group_scale_bytes(const void* x_bf16, int64_t M, int64_t K, int64
   if (B > 128)
     return bro::rqg::launch(x_bf16, M, K, ldx, signs_bf16, nullptr, scales, nullptr, bro::rq::kFormatScaleOnly,
                             BRO_LAYOUT_CANONICAL, 0, di.sm_count, st);
+  // (wide kernel: block 128 of [16384, 4096] 38.1 -> 25.9 us, block 64 30.3 -> 24.3; block 32 23.6 -> 24.2, [128, 4096] 2.4 -> 2.5)
+  if (B > 32 && wide_takes(B, K) && M * K > (int64_t)1 << 19)
+    return bro::rqw::launch(x_bf16, M, K, ldx, log2_of(B), signs_bf16, nullptr, scales, nullptr, BRO_LAYOUT_CANONICAL, 0, di.sm_count, st);
   if (!bro::rqd::supports(M, K, BRO_LAYOUT_CANONICAL, 0)) return BRO_ERR_UNSUPPORTED;
   return bro::rqd::launch_stats(x_bf16, M, K, ldx, B == 32 ? 5 : (B == 64 ? 6 : 7), signs_bf16,
                                 bro::rq::kFormatScaleOnly, nullptr, scales, di.sm_count, st);
@@ -722,7 +692,7 @@ static bro_status linear_impl(const void* x_bf16, int64_t M, int64_t K, int64_t 
     }
   }
   rc = launch_rotate_quantize(x_bf16, M, K, ldx, block, signs, acodes, ascales, BRO_LAYOUT_GEMM, flags,
-                              static_cast<cudaStream_t>(stream));
+                              static_cast<cudaStream_t>(stream), nullptr, 0, true);
   if (rc != BRO_OK) return rc;
   // The packed weights are older than the rotate+quantize kernel just enqueued, which signals its
   // dependents only after its own wait: the GEMM may fetch its first weight tiles early.

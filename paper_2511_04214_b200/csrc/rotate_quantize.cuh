@@ -1,23 +1,15 @@
-// Kernel 1: fused block-Hadamard rotation + MXFP4 quantisation (paper Sec. 4.3 Eq. 1, Sec. 4.1).
+// Kernel 1, the arithmetic: block-Hadamard rotation + MXFP4 quantisation of one MX group (paper Sec. 4.3 Eq. 1, Sec. 4.1),
+// shared by the kernels that move the bytes (rotate_quantize_direct.cuh, rotate_quantize_wide.cuh, rotate_quantize_global.cuh
+// and the split-K GEMM).
 //
-// HBM-bound streaming kernel: 2 bytes in and 0.53125 bytes out per element, one pass.
-//
-//  * One persistent CTA per SM.  A producer thread streams 128-row x 128-column bf16 tiles into
-//    a ring of shared-memory stages with TMA (two 128x64 boxes per tile, 128-byte swizzle), so
-//    the loads in flight are bounded by shared memory, not by registers.
-//  * 16 consumer warps.  Each thread owns one whole MX group (32 consecutive channels of one
-//    row): four conflict-free 16-byte shared loads, then the 5 butterfly stages of the 32-point
-//    Walsh-Hadamard transform entirely in registers — no shuffles for block = 32.  Blocks of 64
-//    and 128 add one or two cross-lane stages (the 2 or 4 groups of a block sit in lanes that
-//    differ in bit 0 / bit 3).
+//  * A thread owns whole MX groups (32 consecutive channels of one row): the 5 butterfly stages of the 32-point
+//    Walsh-Hadamard transform run entirely in registers.
 //  * fp32 arithmetic in exactly this order: butterflies (a+b, a-b) with ascending stride, one
 //    multiply by c = fp32(1/sqrt(block)), amax over the group, shared exponent
 //    E = max(expfield(amax) - 2, 0) - 127, r = y * 2^-E, round-to-nearest-even to E2M1 with
 //    saturation.  The multiply by c and the exact scaling by 2^-E are merged into one multiply by
 //    c*2^-E whenever that product is a normal fp32 (bit-identical result); otherwise the two
 //    multiplies are done separately.
-//  * Output: one 16-byte store of 32 packed codes per thread; the 4 scale bytes of a row inside
-//    the tile are gathered with two shuffles and written as one 32-bit store.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -26,26 +18,6 @@
 
 namespace bro {
 namespace rq {
-
-constexpr int kTileRows = 128;
-constexpr int kTileCols = 128;              // 4 MX groups
-constexpr int kBoxCols = 64;                // one TMA box: 128 rows x 64 bf16 = 128 B per row
-constexpr int kBoxBytes = kTileRows * kBoxCols * 2;   // 16 KiB
-constexpr int kStageBytes = 2 * kBoxBytes;            // 32 KiB
-constexpr int kStages = 6;
-constexpr int kConsumerWarps = 16;
-constexpr int kThreads = (kConsumerWarps + 1) * 32;   // + 1 producer warp
-constexpr int kSmemBytes = kStages * kStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/;
-
-struct Params {
-  int64_t M, K;
-  int64_t tiles_m, tiles_k;     // tiles_k covers the scale padding when layout == GEMM
-  uint8_t* codes;               // [M, K/2]
-  uint8_t* scales;
-  int64_t scale_kblocks;        // GEMM layout: 512-byte blocks per 128-row block
-  int layout;                   // bro_layout
-  const uint16_t* signs;        // [K] bf16 +-1 (randomised rotation, kernels with SIGNS) or nullptr
-};
 
 // x diag(s): flip the bf16 sign bits of a 16-byte chunk of x where the sign vector is negative.
 // One three-input logic operation per 32-bit word (x ^ (s & 0x80008000)); exact.
@@ -477,144 +449,6 @@ __device__ __forceinline__ float group_error(const uint64_t (&P)[16], uint32_t c
     }
   }
   return group_error_any(P, cbits, format);
-}
-
-// SIGNS: the randomised rotation R_i = diag(s) H / sqrt(block) (paper Sec. 5.1) — the channel signs
-// are applied to the bf16 inputs as they leave shared memory; everything else is unchanged.
-template <int LOG2B, bool SIGNS>
-__global__ void __launch_bounds__(kThreads, 1)
-rotate_quantize_kernel(const __grid_constant__ CUtensorMap tmx, const Params p) {
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;   // swizzle needs 1 KiB
-  const uint32_t bar_base = smem_base + kStages * kStageBytes;
-  // full[s] at bar_base + 8*s ; empty[s] at bar_base + 8*(kStages + s)
-  const int warp = threadIdx.x >> 5;
-  const int lane = threadIdx.x & 31;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(bar_base + 8 * s, 1);
-      mbar_init(bar_base + 8 * (kStages + s), kConsumerWarps);
-    }
-    mbar_fence_init();
-    fence_proxy_async_smem();
-  }
-  __syncthreads();
-  griddep_wait();               // x may be written, codes/scales still read, by the kernel before
-  // (only now: a dependent that starts early may then rely on everything older than this kernel)
-  griddep_launch_dependents();
-
-  const int64_t total_tiles = p.tiles_m * p.tiles_k;
-
-  if (warp == kConsumerWarps) {
-    // ---------------- producer ----------------
-    if (lane == 0) {
-      tma_prefetch_desc(&tmx);
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      int64_t issued = 0;
-      const int tiles_k = (int)p.tiles_k;
-      int tm = (int)(blockIdx.x / (unsigned)tiles_k), tk = (int)(blockIdx.x % (unsigned)tiles_k);
-      const int step_m = (int)(gridDim.x / (unsigned)tiles_k), step_k = (int)(gridDim.x % (unsigned)tiles_k);
-      for (int64_t t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
-        if (issued >= kStages)
-          ok = mbar_wait(bar_base + 8 * (kStages + stage), phase ^ 1u, SITE_RQ_EMPTY);
-        if (!ok) break;
-        const uint32_t full = bar_base + 8 * stage;
-        const uint32_t dst = smem_base + stage * kStageBytes;
-        mbar_arrive_expect_tx(full, kStageBytes);
-        tma_load_2d(dst, &tmx, tk * kTileCols, tm * kTileRows, full);
-        tma_load_2d(dst + kBoxBytes, &tmx, tk * kTileCols + kBoxCols, tm * kTileRows, full);
-        ++issued;
-        if (++stage == kStages) { stage = 0; phase ^= 1u; }
-        tm += step_m;
-        tk += step_k;
-        if (tk >= tiles_k) { tk -= tiles_k; ++tm; }
-      }
-      if (!ok) {
-        // A consumer gave up.  Do not leave the CTA while copies may still land in its shared
-        // memory: wait (bounded) for the last load armed on every stage.  Issue i used stage
-        // i % kStages in phase (i / kStages) & 1.
-        const int64_t first = issued > kStages ? issued - kStages : 0;
-        for (int64_t i = first; i < issued; ++i)
-          mbar_wait(bar_base + 8 * (int)(i % kStages), (uint32_t)((i / kStages) & 1), SITE_RQ_DRAIN);
-      }
-    }
-  } else {
-    // ---------------- consumers ----------------
-    const int gg = lane & 1;                 // group within the 64-column box
-    const int box = (lane >> 3) & 1;         // which box of the tile
-    const int row = warp * 8 + ((lane >> 4) << 2) + ((lane >> 1) & 3);   // row within the tile
-    const int g = box * 2 + gg;              // group within the tile (0..3)
-    // 16-byte chunk j of this group sits at chunk index (gg*4 + j) ^ (row & 7) of its 128-B row
-    const uint32_t row_off = (uint32_t)box * kBoxBytes + (uint32_t)row * 128u;
-    const uint32_t sw = (uint32_t)(row & 7);
-    constexpr uint32_t cbits = norm_bits<LOG2B>();
-
-    int stage = 0;
-    uint32_t phase = 0;
-    const int tiles_k = (int)p.tiles_k;
-    int tm = (int)(blockIdx.x / (unsigned)tiles_k), tk = (int)(blockIdx.x % (unsigned)tiles_k);
-    const int step_m = (int)(gridDim.x / (unsigned)tiles_k), step_k = (int)(gridDim.x % (unsigned)tiles_k);
-    for (int64_t t = blockIdx.x; t < total_tiles; t += gridDim.x) {
-      if (!mbar_wait(bar_base + 8 * stage, phase, SITE_RQ_FULL)) break;
-      const uint32_t src = smem_base + stage * kStageBytes + row_off;
-      uint64_t P[16];
-      uint4 sg[4] = {};
-      if (SIGNS && (tk * (kTileCols / 32) + g) * 32 < (int)p.K) {
-        const uint4* sp = reinterpret_cast<const uint4*>(p.signs + (tk * kTileCols + g * 32));
-#pragma unroll
-        for (int j = 0; j < 4; ++j) sg[j] = __ldg(sp + j);
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        uint4 q = lds128(src + ((((uint32_t)gg * 4u + j) ^ sw) << 4));
-        if (SIGNS) q = apply_signs(q, sg[j]);
-        unpack_stage1(q, P + 4 * j);
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar_base + 8 * (kStages + stage));
-      if (++stage == kStages) { stage = 0; phase ^= 1u; }
-
-      fwht32_stages_2_to_16(P);
-      if (LOG2B >= 6) cross_lane_stage(P, 1, gg != 0);
-      if (LOG2B >= 7) cross_lane_stage(P, 8, box != 0);
-
-      uint32_t w[4];
-      const uint32_t s = quantize_group(P, cbits, w);
-
-      const int64_t grow = (int64_t)tm * kTileRows + row;
-      const int ggrp = tk * (kTileCols / 32) + g;         // group index along K
-      const bool in_k = ggrp * 32 < (int)p.K;
-      if (grow < p.M && in_k) {
-        uint4* dst = reinterpret_cast<uint4*>(p.codes + grow * (p.K >> 1) + ggrp * 16);
-        *dst = make_uint4(w[0], w[1], w[2], w[3]);
-      }
-      // gather the row's 4 scale bytes of this tile into the lane with gg == 0 && box == 0
-      uint32_t sb = in_k ? s : 0u;
-      sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 1) << 8;
-      sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 8) << 16;
-      if (g == 0) {
-        if (p.layout == BRO_LAYOUT_GEMM) {
-          // 512-byte block (tm, tk): byte (r%32)*16 + (r/32)*4 + g ; padding rows included
-          const int64_t off = ((int64_t)tm * p.scale_kblocks + tk) * 512 + (row & 31) * 16 + (row >> 5) * 4;
-          *reinterpret_cast<uint32_t*>(p.scales + off) = sb;
-        } else if (grow < p.M) {
-          const int ng = (int)(p.K >> 5);
-          uint8_t* dst = p.scales + grow * ng + tk * 4;
-          if (tk * 4 + 4 <= ng && ((reinterpret_cast<uintptr_t>(dst) & 3) == 0)) {
-            *reinterpret_cast<uint32_t*>(dst) = sb;
-          } else {
-            for (int i = 0; i < 4 && tk * 4 + i < ng; ++i) dst[i] = (uint8_t)(sb >> (8 * i));
-          }
-        }
-      }
-      tm += step_m;
-      tk += step_k;
-      if (tk >= tiles_k) { tk -= tiles_k; ++tm; }
-    }
-  }
 }
 
 }  // namespace rq
