@@ -425,7 +425,7 @@ bro_status bro_linear_host(const void* x_host_bf16, int64_t M, int64_t K, int bl
  * this library, the first launch of each kernel variant on a device (one per block size, per
  * size class of the input, per GEMM tile width and output type) loads that kernel and opts it in
  * to its shared-memory size: run one call of every (block, shape class) you will use before
- * capturing.  With block = 0 the call also enqueues a memset of the scale buffer's padding.
+ * capturing.
  *
  * Sharing: every call on a device uses the same array and finds in it whatever the previous
  * call left.  Each call rewrites everything it later reads (padding included), so stale contents

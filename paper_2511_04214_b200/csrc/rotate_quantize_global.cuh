@@ -2,10 +2,12 @@
 // Sec. 5.2) fused with MXFP4 quantisation.  K = 2^p, 32 <= K <= 32768.
 //
 // Same arithmetic contract as the block kernel: butterflies with ascending stride in fp32, one
-// multiply by fp32(1/sqrt(K)), then per-32 quantisation.  A thread owns one MX group:
-//   strides 1..16      in registers,
-//   strides 32..512    between lanes (one shuffle per element per stage),
-//   strides >= 1024    between warps through shared memory (swizzled, conflict-free float4).
+// multiply by fp32(1/sqrt(K)), then per-32 quantisation.  Two kernels:
+//   rotate_quantize_global_wide_kernel   codes, scale bytes, MXFP4 error: every stage in registers, two transposes through shared
+//                                        memory
+//   rotate_quantize_global_kernel        everything else (simulated quantisation, the error in the other formats, the statistics of few
+//                                        short rows): a thread owns one MX group; strides 1..16 in registers, 32..512 between
+//                                        lanes (one shuffle per element per stage), >= 1024 between warps through shared memory.
 // The global rotation costs log2(K) stages instead of 5; it is expected to run below the HBM
 // roofline — that cost difference is the paper's point (Sec. 4.3 "Reduced online computing").
 #pragma once
@@ -13,6 +15,7 @@
 #include "bro_common.cuh"
 #include "rotate_quantize.cuh"
 #include "fake_quantize.cuh"
+#include "gemm_mxfp4.cuh"
 
 namespace bro {
 namespace rqg {
@@ -118,252 +121,399 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rotate_quantize_global_kernel(
       }
       continue;
     }
-    if (p.deq) {                 // simulated quantisation (uniform over the grid)
-      float out[32];
-      if (p.format == fq::kFormatNone) {
-        const uint64_t cc = rq::pack2(__uint_as_float(cbits), __uint_as_float(cbits));
+    // simulated quantisation
+    float out[32];
+    if (p.format == fq::kFormatNone) {
+      const uint64_t cc = rq::pack2(__uint_as_float(cbits), __uint_as_float(cbits));
 #pragma unroll
-        for (int k = 0; k < 16; ++k) rq::unpack2(rq::mul2(P[k], cc), out[2 * k], out[2 * k + 1]);
-      } else if (p.format >= fq::kFormatRowSym) {
-        const int64_t r = live ? row : 0;
-        fq::row_dequant_any(P, cbits, p.format == fq::kFormatRowAsym, __uint_as_float(__ldcg(p.rowstats + 2 * r)),
-                            __uint_as_float(__ldcg(p.rowstats + 2 * r + 1)), out);
-      } else
+      for (int k = 0; k < 16; ++k) rq::unpack2(rq::mul2(P[k], cc), out[2 * k], out[2 * k + 1]);
+    } else if (p.format >= fq::kFormatRowSym) {
+      const int64_t r = live ? row : 0;
+      fq::row_dequant_any(P, cbits, p.format == fq::kFormatRowAsym, __uint_as_float(__ldcg(p.rowstats + 2 * r)),
+                          __uint_as_float(__ldcg(p.rowstats + 2 * r + 1)), out);
+    } else {
       fq::group_dequant_any(P, cbits, p.format, out);
-      if (live) fq::store_group(p.deq + row * p.ldd + (int64_t)gi * 32, out);
-      continue;
     }
-    uint32_t w[4];
-    const uint32_t s = rq::quantize_group(P, cbits, w);
-    if (live) {
-      *reinterpret_cast<uint4*>(p.codes + row * (p.K >> 1) + (int64_t)gi * 16) =
-          make_uint4(w[0], w[1], w[2], w[3]);
-      if (p.layout == BRO_LAYOUT_GEMM) {
-        const int64_t off = ((row >> 7) * p.scale_kblocks + (gi >> 2)) * 512 + (row & 31) * 16 +
-                            ((row & 127) >> 5) * 4 + (gi & 3);
-        p.scales[off] = (uint8_t)s;
-      } else {
-        p.scales[row * (p.K >> 5) + gi] = (uint8_t)s;
-      }
-    }
+    if (live) fq::store_group(p.deq + row * p.ldd + (int64_t)gi * 32, out);
   }
 }
 
-// ---- K = 2048 / 4096, codes path: the stages above stride 16 through two shared-memory transposes ----
-// A thread always works on 32 values in registers, but on a different set in each of three phases, so
-// that every butterfly stage is register arithmetic (no shuffle in the transform):
-//   phase 1   element bits 0..4  : the thread's 32 consecutive channels (as loaded)
-//   phase 2   element bits 5..9  : 32 channels 32 apart (one column of a 32 x 32 block)
-//   phase 3   element bits 10..  : 2 (K = 2048) or 4 (K = 4096) runs of 16 / 8 consecutive channels, 1024 apart
-// Stage order is still ascending stride with one fp32 rounding per add / subtract, so the result is the
-// same bit for bit.  Between the phases the row passes through shared memory (fp32, K values per row,
-// two buffers so that one barrier per transpose suffices); all accesses are bank-conflict free:
-//   transpose 1  writes 8 x 16 bytes per thread, 16-byte pieces XOR-swizzled with the thread index, and
-//                reads 32 scalars per thread (a warp reads one 128-byte line per instruction);
-//   transpose 2  writes 32 scalars per thread (a warp writes one line per instruction) and reads 8 x 16
-//                bytes, pieces swizzled with bits 3..4 of the piece index.
-// After phase 3 a thread holds 8 (16) consecutive values of 4 (2) MX groups; the group maximum takes two
-// (one) shuffles per group, codes go out as one 32-bit (64-bit) store per group.
-// The bf16 rows arrive by TMA (one 8 KiB box per pass: ROWS rows x K/64 segments of 128 bytes, 128-byte
-// swizzle), issued by thread 0 for the NEXT pass as soon as every thread has taken its 64 bytes of the
-// current one: the load/store unit's data path, which bounds this kernel, then carries only the
-// conflict-free shared-memory reads instead of one 128-byte line per two lanes of a global load.
-template <int LOG2K, bool SIGNS>
-__global__ void __launch_bounds__(128, 5) rotate_quantize_global_smem_kernel(const __grid_constant__ CUtensorMap tmx,
-                                                                              const Params p) {
-  static_assert(LOG2K == 11 || LOG2K == 12, "K = 2048 or 4096");
-  constexpr int K = 1 << LOG2K;
-  constexpr int T = K / 32;                   // threads per row
-  constexpr int ROWS = 128 / T;               // rows per pass of the CTA
-  constexpr int HB = LOG2K - 10;              // element bits handled in phase 3
-  constexpr int NJ = 1 << HB;                 // runs per thread in phase 3
-  constexpr int RUN = 32 / NJ;                // consecutive values per run
-  constexpr uint32_t kRawBytes = (uint32_t)ROWS * K * 2;          // 8 KiB
-  extern __shared__ uint8_t smem_raw[];       // [raw bf16 box | barrier | fp32 [2][ROWS][K]], 1 KiB aligned
-  const uint32_t raw = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t bar = raw + kRawBytes;
-  float* xbuf = reinterpret_cast<float*>(smem_raw + (raw - smem_u32(smem_raw)) + kRawBytes + 1024);
-  constexpr uint32_t cbits = (LOG2K % 2 == 0) ? (uint32_t)(127 - LOG2K / 2) << 23
-                                              : 0x3FB504F3u - ((uint32_t)((LOG2K + 1) / 2) << 23);
-  const int t = threadIdx.x % T;              // thread within the row
-  const int rs = threadIdx.x / T;             // row slot
-  const int lo5 = t & 31, hi = t >> 5;
-  float* bufA = xbuf + (size_t)rs * K;
-  float* bufB = xbuf + (size_t)(ROWS + rs) * K;
-  const int64_t row_iters = (p.M + ROWS - 1) / ROWS;
+// ---- codes, scale bytes and the MXFP4 error: the stages above stride 32 through two shared-memory transposes ----
+// A thread works on 64 values in registers, a different set in each of three phases, so that every butterfly stage is
+// register arithmetic on packed pairs (no shuffle in the transform):
+//   phase 1   element bits 0..5       : the thread's 64 consecutive channels (as loaded)
+//   phase 2   element bits 0, 6..10   : 32 pairs of channels 64 apart
+//   phase 3   element bits 11..       : NJ runs of 64 / NJ consecutive channels, NJ = V / 2048
+// Stage order is ascending stride with one fp32 rounding per add / subtract, so the result is that of the shuffle form
+// bit for bit.  A unit of V = max(K, 4096) elements (several rows where K < 4096, and then the stages of stride K and more
+// are left out) is worked on by V / 64 threads of their own, which meet at a named barrier; no barrier spans the CTA.
+// Between the phases the unit passes through ONE shared-memory buffer of fp32: phase 2 writes back where it read.  128-byte
+// lines of 32 values, 16-byte piece q of line L at q ^ g(L), g(L) = (L ^ (L >> 3)) & 7; all accesses are free of bank
+// conflicts: 16 bytes a thread and threads 2 lines apart (phase 1) or one line or less apart (phase 3), 8 bytes a
+// thread and a warp on two lines (phase 2).
+// What bounds it is the L1 data path (two fp32 round trips through shared memory are 16 bytes an element, the bf16 rows 4 more) and
+// instruction issue.  64 values a thread rather than 32: the strided side of both transposes moves 8 bytes an instruction instead of
+// 4, its five stages are all packed, and from K = 4096 down a thread ends with whole MX groups (no shuffle for their maximum).
+// [16384, 4096] codes 66.5 -> 52.7 us, scale bytes 98 -> 49, error 113 -> 55; K = 2048 60 -> 52, 1024 71 -> 51, 8192 124 -> 61, 16384 152 -> 78,
+// 32768 (one CTA an SM) 174 -> 105 us for as many elements; [300, 4096] 5.5 -> 4.1.
+// The bf16 rows arrive by TMA (128-byte segments, 128-byte swizzle: a thread's 64 channels are a segment), requested for the
+// unit's NEXT pass as soon as its threads have taken the current one.
+enum Mode { kCodes = 0, kBytes = 1, kError = 2 };
 
-  if (threadIdx.x == 0) {
+template <int LOG2V>
+struct Shape {
+  static constexpr int V = 1 << LOG2V;
+  static constexpr int T = V / 64;                          // threads of a unit
+  static constexpr int kThreads = T < 128 ? 128 : T;
+  static constexpr int kUnits = kThreads / T;
+  static constexpr int NJ = V / 2048;                       // runs of a thread in phase 3
+  static constexpr int RUN = 64 / NJ;
+  static constexpr int G = 32 / RUN;                        // lanes that share an MX group
+  static constexpr int kRawBytes = V * 2;
+  static constexpr int kBufBytes = V * 4;
+  static constexpr int kBarAt = kUnits * (kRawBytes + kBufBytes);
+  static constexpr int kSmemBytes = kBarAt + 128 + 1024 /*alignment*/;
+  static constexpr int kMinBlocks = kThreads == 128 ? 4 : (kThreads == 256 ? 2 : 1);
+};
+
+__device__ __forceinline__ uint64_t lds64(uint32_t addr) {
+  uint64_t v;
+  asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts64(uint32_t addr, uint64_t v) {
+  asm volatile("st.shared.b64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+__device__ __forceinline__ void lds_pairs(uint32_t addr, uint64_t& a, uint64_t& b) {
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void sts_pairs(uint32_t addr, uint64_t a, uint64_t b) {
+  asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(addr), "l"(a), "l"(b) : "memory");
+}
+
+// All threads of a unit; the result is true if it was true in each of them.
+template <int T>
+__device__ __forceinline__ bool unit_sync_and(int unit, bool ok) {
+  return gemm::named_barrier_and(unit + 1, T, ok);
+}
+template <int T>
+__device__ __forceinline__ void unit_sync(int unit) {
+  gemm::named_barrier_sync(unit + 1, T);
+}
+
+// Maximum of the magnitudes of a group whose values lie in G neighbouring lanes, RUN of them in E; NaN-preserving on demand.
+template <int RUN, int G, bool NAN_TOO>
+__device__ __forceinline__ float run_amax(const uint64_t* E) {
+  float m = 0.f, m2 = 0.f;
+#pragma unroll
+  for (int i = 0; i < RUN / 2; i += 2) {
+    float a, b, a2, b2;
+    rq::unpack2(E[i], a, b);
+    rq::unpack2(E[i + 1], a2, b2);
+    if (NAN_TOO) {
+      asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(a), "f"(b));
+      asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(m2) : "f"(a2), "f"(b2));
+    } else {
+      asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(a), "f"(b));
+      asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m2) : "f"(a2), "f"(b2));
+    }
+  }
+  if (NAN_TOO) asm("max.NaN.f32 %0, %0, %1;" : "+f"(m) : "f"(m2));
+  else m = fmaxf(m, m2);
+#pragma unroll
+  for (int d = 1; d < G; d <<= 1) {
+    const float o = __shfl_xor_sync(0xFFFFFFFFu, m, d);
+    if (NAN_TOO) asm("max.NaN.f32 %0, %0, %1;" : "+f"(m) : "f"(o));
+    else m = fmaxf(m, o);
+  }
+  return m;
+}
+
+// Scale byte and codes (RUN / 2 bytes) of a run, the arithmetic of rq::quantize_group.
+template <int RUN, int G>
+__device__ __forceinline__ uint32_t quantize_run(const uint64_t* E, uint32_t cbits, uint32_t* w) {
+  const float c = __uint_as_float(cbits);
+  const uint32_t ef = __float_as_uint(__fmul_rn(run_amax<RUN, G, false>(E), c)) >> 23;
+  const uint32_t s = ef > 2u ? ef - 2u : 0u;
+  float r[RUN];
+  if (ef >= 27u && ef <= 250u) {
+    const float c2 = __uint_as_float(cbits + ((127u - s) << 23));
+    const uint64_t cc = rq::pack2(c2, c2);
+#pragma unroll
+    for (int k = 0; k < RUN / 2; ++k) rq::unpack2(rq::mul2(E[k], cc), r[2 * k], r[2 * k + 1]);
+  } else {
+    const float p2 = __uint_as_float((254u - s) << 23);
+    const uint64_t cc = rq::pack2(c, c), pp = rq::pack2(p2, p2);
+#pragma unroll
+    for (int k = 0; k < RUN / 2; ++k) rq::unpack2(rq::mul2(rq::mul2(E[k], cc), pp), r[2 * k], r[2 * k + 1]);
+  }
+  if constexpr (RUN >= 8) {
+#pragma unroll
+    for (int j = 0; j < RUN / 8; ++j)
+      w[j] = rq::pack_e2m1x8(r[8 * j], r[8 * j + 1], r[8 * j + 2], r[8 * j + 3], r[8 * j + 4], r[8 * j + 5], r[8 * j + 6], r[8 * j + 7]);
+  } else {
+    w[0] = rq::pack_e2m1x8(r[0], r[1], r[2], r[3], 0.f, 0.f, 0.f, 0.f);
+  }
+  return s;
+}
+
+// MXFP4 error of a group (rq::group_error with format 0) whose values lie in G neighbouring lanes; the same in all of them.
+template <int RUN, int G>
+__device__ __forceinline__ float run_error(const uint64_t* E, uint32_t cbits) {
+  const float c = __uint_as_float(cbits);
+  const float m = run_amax<RUN, G, true>(E);
+  const uint32_t ef = __float_as_uint(__fmul_rn(m, c)) >> 23;
+  const bool usual = ef >= 27u && ef <= 250u;
+  // 2^-E and 2^E; away from the ends of the exponent range c * 2^-E is a normal number and one multiply does
+  const uint32_t s = ef > 2u ? ef - 2u : 0u;
+  const float inv = usual ? __uint_as_float(cbits + ((127u - s) << 23)) : __uint_as_float(s <= 253u ? ((254u - s) << 23) : 0x00400000u);
+  const float pe = __uint_as_float(s >= 1u ? (s << 23) : 0x00400000u);
+  const uint64_t cc = rq::pack2(c, c), ii = rq::pack2(inv, inv);
+  uint64_t acc[2] = {0ull, 0ull};
+#pragma unroll
+  for (int k = 0; k < RUN / 2; ++k) {
+    const uint64_t r = rq::mul2(usual ? E[k] : rq::mul2(E[k], cc), ii);
+    float r0, r1;
+    rq::unpack2(r, r0, r1);
+    uint32_t h;
+    asm("{ .reg .b8 b; cvt.rn.satfinite.e2m1x2.f32 b, %2, %1; cvt.rn.f16x2.e2m1x2 %0, b; }" : "=r"(h) : "f"(r0), "f"(r1));
+    const uint64_t d = rq::sub2(r, rq::pack2(__half2float(__ushort_as_half((unsigned short)(h & 0xFFFFu))),
+                                             __half2float(__ushort_as_half((unsigned short)(h >> 16)))));
+    acc[k & 1] = rq::fma2(d, d, acc[k & 1]);
+  }
+  float s0, s1;
+  rq::unpack2(rq::add2(acc[0], acc[1]), s0, s1);
+  float sum = __fadd_rn(s0, s1);
+#pragma unroll
+  for (int d = 1; d < G; d <<= 1) sum = __fadd_rn(sum, __shfl_xor_sync(0xFFFFFFFFu, sum, d));
+  return __fmul_rn(__fmul_rn(__fmul_rn(sum, 0.03125f), pe), pe);
+}
+
+// K = 2^LOG2K; 0: p.log2k.  K < V: units of several rows.
+template <int LOG2V, int LOG2K, int MODE>
+__global__ void __launch_bounds__(Shape<LOG2V>::kThreads, Shape<LOG2V>::kMinBlocks)
+rotate_quantize_global_wide_kernel(const __grid_constant__ CUtensorMap tmx, const Params p) {
+  using S = Shape<LOG2V>;
+  constexpr int V = S::V, T = S::T, NJ = S::NJ, RUN = S::RUN, G = S::G;
+  extern __shared__ uint8_t smem_raw[];      // [units: bf16 | units: fp32 | barriers], 1 KiB aligned
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const int unit = (int)threadIdx.x / T, t = (int)threadIdx.x % T;
+  const uint32_t raw = base + (uint32_t)(unit * S::kRawBytes), buf = base + (uint32_t)(S::kUnits * S::kRawBytes + unit * S::kBufBytes);
+  const uint32_t bar = base + (uint32_t)(S::kBarAt + 8 * unit);
+  constexpr bool ROWS = LOG2K != LOG2V;
+  const int log2k = LOG2K == 0 ? p.log2k : LOG2K;
+  const int segs = 1 << (log2k - 6);          // 128-byte segments of a row
+  const int rows = V >> log2k;                // rows of a unit
+  const uint32_t cbits = (log2k % 2 == 0) ? (uint32_t)(127 - log2k / 2) << 23 : 0x3FB504F3u - ((uint32_t)((log2k + 1) / 2) << 23);
+  if (t == 0) {
     mbar_init(bar, 1);
     mbar_fence_init();
     fence_proxy_async_smem();
+    if (unit == 0) tma_prefetch_desc(&tmx);
   }
   __syncthreads();
-  griddep_wait();
+  griddep_wait();               // x may be written, the outputs still read, by the kernel before
   griddep_launch_dependents();
-  // this thread's 64 bytes inside the box: segment (t >> 1) of row slot rs, 16-byte pieces 4 (t & 1) + i,
-  // stored at piece index ^ (segment & 7)
-  const uint32_t seg = (uint32_t)rs * (K / 64) + (uint32_t)(t >> 1);
-  const uint32_t raw_mine = raw + seg * 128u;
-  const uint32_t raw_swz = seg & 7u;
-  if (threadIdx.x == 0) {
-    tma_prefetch_desc(&tmx);
-    if ((int64_t)blockIdx.x < row_iters) {
-      mbar_arrive_expect_tx(bar, kRawBytes);
-      tma_load_3d(raw, &tmx, 0, 0, (int)((int64_t)blockIdx.x * ROWS), bar);
+  constexpr int kBoxSegs = V / 64 > 256 ? 256 : V / 64;
+  auto request = [&](int it) {
+    mbar_arrive_expect_tx(bar, S::kRawBytes);
+#pragma unroll
+    for (int b = 0; b < V / 64 / kBoxSegs; ++b)
+      tma_load_3d(raw + (uint32_t)(b * kBoxSegs * 128), &tmx, 0, b * kBoxSegs, it * rows, bar);
+  };
+  const int M = (int)p.M, iters = (M + rows - 1) / rows, stride = (int)gridDim.x * S::kUnits;      // (M is at most 2^30)
+  int it = (int)blockIdx.x * S::kUnits + unit;
+  if (t == 0 && it < iters) request(it);
+  // A thread's 64 channels are the same in every pass, so the signs are two registers: bits 31 - k and 15 - k of sg[h] are those of
+  // the two channels of word 16 h + k.
+  uint32_t sg[2] = {0u, 0u};
+  if (p.signs) {
+    const uint4* sp = reinterpret_cast<const uint4*>(p.signs) + (t & (segs - 1)) * 8;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const uint4 q = __ldg(sp + j);
+      const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) sg[j >> 2] |= (w[c] & 0x80008000u) >> ((4 * j + c) & 15);
+    }
+  }
+  if (MODE == kCodes && p.layout == BRO_LAYOUT_GEMM) {        // the rows that pad the scale buffer to 128 read as zero
+    const int pad = (int)((128 - (p.M & 127)) & 127), words = pad << (log2k - 7);
+    for (int i = (int)(blockIdx.x * S::kThreads + threadIdx.x); i < words; i += (int)gridDim.x * S::kThreads) {
+      const int r = (int)(p.M & 127) + (i >> (log2k - 7)), kb = i & ((1 << (log2k - 7)) - 1);
+      *reinterpret_cast<uint32_t*>(p.scales + ((p.M >> 7) * p.scale_kblocks + kb) * 512 + (r & 31) * 16 + (r >> 5) * 4) = 0u;
     }
   }
 
-  uint4 sg[4] = {};
-  if (SIGNS) {
-    const uint4* sp = reinterpret_cast<const uint4*>(p.signs + (int64_t)t * 32);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) sg[j] = __ldg(sp + j);
-  }
-  // shared-memory addresses that do not change from row to row
-  const uint32_t a_w = smem_u32(bufA) + (uint32_t)t * 128u;                     // transpose 1, writes
-  uint32_t a_r[8];                                                               // transpose 1, reads: row j + 32 hi
-#pragma unroll
-  for (int m = 0; m < 8; ++m)
-    a_r[m] = smem_u32(bufA) + (uint32_t)hi * 4096u + (uint32_t)(((lo5 >> 2) ^ m) << 4) + (uint32_t)((lo5 & 3) << 2);
-  uint32_t b_w[4];                                                               // transpose 2, writes
-#pragma unroll
-  for (int m = 0; m < 4; ++m)
-    b_w[m] = smem_u32(bufB) + (uint32_t)hi * 4096u + (uint32_t)(((lo5 >> 2) ^ m) << 4) + (uint32_t)((lo5 & 3) << 2);
-  const uint32_t b_r = smem_u32(bufB);                                           // transpose 2, reads
+  // shared-memory addresses that do not change from pass to pass
+  // (every swizzle is an XOR into bits 4..6 of an address whose base has them free: one instruction, no register kept for it)
+  const uint32_t raw_mine = raw + (uint32_t)t * 128u + (((uint32_t)t & 7u) << 4);
+  const uint32_t g1 = (uint32_t)((2 * t) ^ ((2 * t) >> 3)) & 7u;                    // g of the thread's even line
+  const uint32_t w1 = buf + (uint32_t)t * 256u + (g1 << 4);
+  // phase 2: pair t & 31 of line pair j
+  const uint32_t l2 = (uint32_t)t & 31u;
+  const uint32_t w2 = buf + (uint32_t)(t >> 5) * 8192u + (l2 >> 4) * 128u + ((((l2 >> 1) & 7u) ^ (l2 >> 4)) << 4) + (l2 & 1u) * 8u;
+  const uint32_t l3 = (uint32_t)t / G, q3 = ((uint32_t)t % G) * (RUN / 4);           // phase 3: line and first piece of run 0
+  const uint32_t g3 = (l3 ^ (l3 >> 3)) & 7u;
+  const uint32_t r3 = buf + l3 * 128u + ((q3 ^ g3) << 4);
 
   uint32_t parity = 0;
-  for (int64_t it = blockIdx.x; it < row_iters; it += gridDim.x) {
-    const int64_t row = it * ROWS + rs;
-    const bool live = row < p.M;                      // (rows beyond M arrive as zeros)
+  for (; it < iters; it += stride) {
     const bool ok = mbar_wait(bar, parity, SITE_RQ_FULL);
     parity ^= 1u;
-    uint64_t P[16];
+    uint64_t P[32];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint4 q = lds128(raw_mine + ((((uint32_t)(t & 1) * 4u + (uint32_t)j) ^ raw_swz) << 4));
-      rq::unpack_stage1(SIGNS ? rq::apply_signs(q, sg[j]) : q, P + 4 * j);
-    }
-    rq::fwht32_stages_2_to_16(P);                                   // strides 1..16
-    // ---- transpose 1
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      float a0, a1, a2, a3;
-      rq::unpack2(P[2 * c], a0, a1);
-      rq::unpack2(P[2 * c + 1], a2, a3);
-      asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a_w + (uint32_t)((c ^ (t & 7)) << 4)), "f"(a0), "f"(a1),
-                   "f"(a2), "f"(a3)
-                   : "memory");
-    }
-    // (also: every thread has taken its bytes of the bf16 box; a lost load ends the loop for all)
-    if (!__syncthreads_and(ok)) break;
-    if (threadIdx.x == 0 && it + gridDim.x < row_iters) {
-      mbar_arrive_expect_tx(bar, kRawBytes);
-      tma_load_3d(raw, &tmx, 0, 0, (int)((it + gridDim.x) * ROWS), bar);
-    }
-    {
-      float v[32];
-#pragma unroll
-      for (int j = 0; j < 32; ++j)
-        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[j]) : "r"(a_r[j & 7] + (uint32_t)(j * 128)) : "memory");
-      // strides 32..256 on pairs (v[k], v[k + 16]); stride 512 inside the pairs
-#pragma unroll
-      for (int k = 0; k < 16; ++k) P[k] = rq::pack2(v[k], v[k + 16]);
-      rq::fwht32_stages_2_to_16(P);
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        float lo, hi2;
-        rq::unpack2(P[k], lo, hi2);
-        v[k] = __fadd_rn(lo, hi2);
-        v[k + 16] = __fsub_rn(lo, hi2);
+    for (uint32_t j = 0; j < 8; ++j) {
+      uint4 q = lds128(raw_mine ^ (j << 4));
+      if (p.signs) {
+        const int k = 4 * ((int)j & 3);
+        q = rq::apply_signs(q, make_uint4(sg[j >> 2] << k, sg[j >> 2] << (k + 1), sg[j >> 2] << (k + 2), sg[j >> 2] << (k + 3)));
       }
-      // ---- transpose 2: value j is element lo5 + 32 j + 1024 hi of the row
-#pragma unroll
-      for (int j = 0; j < 32; ++j)
-        asm volatile("st.shared.f32 [%0], %1;" ::"r"(b_w[j & 3] + (uint32_t)(j * 128)), "f"(v[j]) : "memory");
+      rq::unpack_stage1(q, P + 4 * j);
     }
-    __syncthreads();
-    // ---- phase 3: runs of RUN consecutive values at RUN * t + 1024 * j2
-    uint64_t E[NJ][RUN / 2];
 #pragma unroll
-    for (int j2 = 0; j2 < NJ; ++j2) {
+    for (int hp = 1; hp < 32; hp <<= 1) {                       // strides 2..32
 #pragma unroll
-      for (int h = 0; h < RUN / 4; ++h) {
-        const uint32_t ci = (uint32_t)(j2 * 256 + t * (RUN / 4) + h);              // 16-byte piece of the row
-        float a0, a1, a2, a3;
-        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                     : "=f"(a0), "=f"(a1), "=f"(a2), "=f"(a3)
-                     : "r"(b_r + ((ci ^ ((ci >> 3) & 3u)) << 4))
-                     : "memory");
-        E[j2][2 * h] = rq::pack2(a0, a1);
-        E[j2][2 * h + 1] = rq::pack2(a2, a3);
+      for (int k = 0; k < 32; ++k) {
+        if ((k & hp) == 0) {
+          const uint64_t a = P[k], b = P[k + hp];
+          P[k] = rq::add2(a, b);
+          P[k + hp] = rq::sub2(a, b);
+        }
       }
     }
 #pragma unroll
-    for (int hb = 1; hb < NJ; hb <<= 1) {                          // strides 1024 (and 2048)
+    for (uint32_t c = 0; c < 16; ++c)
+      sts_pairs((w1 ^ (((c & 7u) ^ (c >> 3)) << 4)) + (c >> 3) * 128u, P[2 * c], P[2 * c + 1]);
+    // (also: every thread of the unit has taken its bytes of the bf16 rows; a lost load ends the loop for all of them)
+    if (!unit_sync_and<T>(unit, ok)) break;
+    if (t == 0 && it + stride < iters) request(it + stride);
 #pragma unroll
-      for (int j2 = 0; j2 < NJ; ++j2) {
-        if ((j2 & hb) == 0) {
+    for (int j = 0; j < 32; ++j) P[j] = lds64((w2 ^ (uint32_t)((((2 * (j & 3)) ^ (j >> 2)) & 7) << 4)) + (uint32_t)(j * 256));
 #pragma unroll
-          for (int i = 0; i < RUN / 2; ++i) {
-            const uint64_t a = E[j2][i], b = E[j2 + hb][i];
-            E[j2][i] = rq::add2(a, b);
-            E[j2 + hb][i] = rq::sub2(a, b);
+    for (int s = 0; s < 5; ++s) {                               // strides 64..1024
+      if (!ROWS || s + 6 < log2k) {
+        const int hp = 1 << s;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+          if ((k & hp) == 0) {
+            const uint64_t a = P[k], b = P[k + hp];
+            P[k] = rq::add2(a, b);
+            P[k + hp] = rq::sub2(a, b);
           }
         }
       }
     }
-    // ---- quantise: run j2 belongs to group (t >> HB) + 32 j2; the NJ lanes t, t^1 (, t^2, t^3) share it
+#pragma unroll
+    for (int j = 0; j < 32; ++j) sts64((w2 ^ (uint32_t)((((2 * (j & 3)) ^ (j >> 2)) & 7) << 4)) + (uint32_t)(j * 256), P[j]);
+    unit_sync<T>(unit);
+    // run j2 starts 2048 elements = 64 lines behind the one before: the same g
 #pragma unroll
     for (int j2 = 0; j2 < NJ; ++j2) {
-      float m = 0.f;
 #pragma unroll
-      for (int i = 0; i < RUN / 2; ++i) {
-        float lo, hi2;
-        rq::unpack2(E[j2][i], lo, hi2);
-        asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(lo), "f"(hi2));
+      for (uint32_t h = 0; h < RUN / 4; ++h) {
+        lds_pairs((r3 ^ (h << 4)) + (uint32_t)(j2 * 8192), P[j2 * (RUN / 2) + 2 * h], P[j2 * (RUN / 2) + 2 * h + 1]);
       }
+    }
+    unit_sync<T>(unit);                                         // (the next pass writes where others read)
+    if constexpr (!ROWS) {
 #pragma unroll
-      for (int d = 1; d < NJ; d <<= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
-      const float c = __uint_as_float(cbits);
-      const uint32_t ef = __float_as_uint(__fmul_rn(m, c)) >> 23;
-      const uint32_t sc = ef > 2u ? ef - 2u : 0u;
-      float r[RUN];
-      if (ef >= 27u && ef <= 250u) {
-        const float c2 = __uint_as_float(cbits + ((127u - sc) << 23));
-        const uint64_t cc = rq::pack2(c2, c2);
+      for (int hb = 1; hb < NJ; hb <<= 1) {                     // strides 2048..
 #pragma unroll
-        for (int i = 0; i < RUN / 2; ++i) rq::unpack2(rq::mul2(E[j2][i], cc), r[2 * i], r[2 * i + 1]);
+        for (int j2 = 0; j2 < NJ; ++j2) {
+          if ((j2 & hb) == 0) {
+#pragma unroll
+            for (int i = 0; i < RUN / 2; ++i) {
+              const uint64_t a = P[j2 * (RUN / 2) + i], b = P[(j2 + hb) * (RUN / 2) + i];
+              P[j2 * (RUN / 2) + i] = rq::add2(a, b);
+              P[(j2 + hb) * (RUN / 2) + i] = rq::sub2(a, b);
+            }
+          }
+        }
+      }
+    }
+    // ---- results: run j2 belongs to group t / G + 64 j2 of the unit
+#pragma unroll
+    for (int j2 = 0; j2 < NJ; ++j2) {
+      const uint64_t* E = P + j2 * (RUN / 2);
+      const int gu = (int)l3 + j2 * 64;
+      const int row = it * rows + (ROWS ? gu >> (log2k - 5) : 0);
+      const int g = ROWS ? gu & ((1 << (log2k - 5)) - 1) : gu;
+      const bool live = row < M;
+      if (MODE == kError) {
+        const float e = run_error<RUN, G>(E, cbits);
+        if (live && t % G == 0) p.mse[((int64_t)row << (log2k - 5)) + g] = e;
+        continue;
+      }
+      uint32_t s, w[RUN >= 8 ? RUN / 8 : 1];
+      if (MODE == kCodes) {
+        s = quantize_run<RUN, G>(E, cbits, w);
+        if (live) {
+          uint8_t* dst = p.codes + ((int64_t)row << (log2k - 1)) + g * 16 + (t % G) * (RUN / 2);
+          if constexpr (RUN == 32) *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+          else if constexpr (RUN == 16) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
+          else if constexpr (RUN == 8) *reinterpret_cast<uint32_t*>(dst) = w[0];
+          else *reinterpret_cast<uint16_t*>(dst) = (uint16_t)w[0];
+        }
       } else {
-        const float p2 = __uint_as_float((254u - sc) << 23);
-        const uint64_t cc = rq::pack2(c, c), pp = rq::pack2(p2, p2);
-#pragma unroll
-        for (int i = 0; i < RUN / 2; ++i) rq::unpack2(rq::mul2(rq::mul2(E[j2][i], cc), pp), r[2 * i], r[2 * i + 1]);
+        const uint32_t ef = __float_as_uint(__fmul_rn(run_amax<RUN, G, false>(E), __uint_as_float(cbits))) >> 23;
+        s = ef > 2u ? ef - 2u : 0u;
       }
-      uint32_t w[RUN / 8];
-#pragma unroll
-      for (int i = 0; i < RUN / 8; ++i)
-        w[i] = rq::pack_e2m1x8(r[8 * i], r[8 * i + 1], r[8 * i + 2], r[8 * i + 3], r[8 * i + 4], r[8 * i + 5], r[8 * i + 6],
-                               r[8 * i + 7]);
-      if (live) {
-        const int g = (t >> HB) + 32 * j2;
-        uint8_t* dst = p.codes + row * (K >> 1) + g * 16 + (t & (NJ - 1)) * (RUN / 2);
-        if (RUN == 8) *reinterpret_cast<uint32_t*>(dst) = w[0];
-        else *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[RUN / 8 - 1]);
-        if ((t & (NJ - 1)) == 0) {
-          if (p.layout == BRO_LAYOUT_GEMM) {
-            const int64_t off = ((row >> 7) * p.scale_kblocks + (g >> 2)) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4 + (g & 3);
-            p.scales[off] = (uint8_t)sc;
+      // scale bytes of 4 consecutive groups -> one 32-bit word (a row has a multiple of 8 groups)
+      s |= __shfl_xor_sync(0xFFFFFFFFu, s, G) << 8;
+      s |= __shfl_xor_sync(0xFFFFFFFFu, s, 2 * G) << 16;
+      if (live && t % (4 * G) == 0) {
+        if (MODE == kCodes && p.layout == BRO_LAYOUT_GEMM) {
+          const int r = row & 127;
+          *reinterpret_cast<uint32_t*>(p.scales + ((int64_t)(row >> 7) * p.scale_kblocks + (g >> 2)) * 512 + (r & 31) * 16 + (r >> 5) * 4) = s;
+        } else {
+          uint8_t* dst = p.scales + ((int64_t)row << (log2k - 5)) + g;
+          if ((reinterpret_cast<uintptr_t>(dst) & 3) == 0) {
+            *reinterpret_cast<uint32_t*>(dst) = s;
           } else {
-            p.scales[row * (K >> 5) + g] = (uint8_t)sc;
+            for (int i = 0; i < 4; ++i) dst[i] = (uint8_t)(s >> (8 * i));
           }
         }
       }
     }
   }
+  // (left before the end only after a lost wait: its copy may still land, wait once more)
+  if (t == 0 && it < iters) mbar_wait(bar, parity ^ 1u, SITE_RQ_DRAIN);
 }
 
-// 3-D view of x for the kernel above: {64 bf16 (128 bytes), K / 64 segments, M rows}, box = whole rows.
+// 3-D view of x for the kernel above: {64 bf16 (128 bytes), K / 64 segments, M rows}, box = whole rows (of at most 256 segments).
 bro_status make_row_map(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx, int box_rows);
+
+template <int LOG2V, int LOG2K = LOG2V>
+inline bro_status launch_wide(const Params& p, int mode, int sm_count, cudaStream_t st) {
+  using S = Shape<LOG2V>;
+  CUtensorMap tmx;
+  const bro_status mrc = make_row_map(&tmx, p.x, p.M, p.K, p.ldx, S::V >> p.log2k);
+  if (mrc != BRO_OK) return mrc;
+  auto go = [&](void (*kernel)(CUtensorMap, Params)) -> bro_status {
+    static DeviceOnce once[3];                                          // (per mode)
+    int per_sm = 1;
+    const bro_status rc = device_once(once[mode], &per_sm, [&](int* n) {
+      if (!cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmemBytes),
+                   "cudaFuncSetAttribute(rotate_quantize_global)"))
+        return BRO_ERR_CUDA;
+      return cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kernel, S::kThreads, S::kSmemBytes),
+                     "occupancy(rotate_quantize_global)")
+                 ? BRO_OK
+                 : BRO_ERR_CUDA;
+    });
+    if (rc != BRO_OK) return rc;
+    const int64_t rows = S::V >> p.log2k, iters = (p.M + rows - 1) / rows, want = (iters + S::kUnits - 1) / S::kUnits;
+    const int64_t cap = (int64_t)sm_count * per_sm;
+    return cuda_ok(launch_kernel(kernel, (unsigned)(want < cap ? want : cap), S::kThreads, S::kSmemBytes, st, 1, tmx, p),
+                   "rotate_quantize_global launch")
+               ? BRO_OK
+               : BRO_ERR_CUDA;
+  };
+  if (mode == kError) return go(rotate_quantize_global_wide_kernel<LOG2V, LOG2K, kError>);
+  if (mode == kBytes) return go(rotate_quantize_global_wide_kernel<LOG2V, LOG2K, kBytes>);
+  return go(rotate_quantize_global_wide_kernel<LOG2V, LOG2K, kCodes>);
+}
 
 inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, const void* signs, void* codes,
                          void* scales, float* mse, int format, bro_layout layout, int64_t scale_kblocks, int sm_count, cudaStream_t st,
@@ -391,39 +541,19 @@ inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, const
   int threads = p.threads_per_row < 256 ? 256 : p.threads_per_row;
   p.rows_per_iter = threads / p.threads_per_row;
   const size_t smem = K > 1024 ? (size_t)p.rows_per_iter * K * sizeof(float) : 0;
-  if (layout == BRO_LAYOUT_GEMM && !mse && !deq && !range_pass && format != rq::kFormatScaleOnly) {
-    // padding rows / groups of the tiled scale buffer must read as 0
-    const size_t bytes = (size_t)((M + 127) / 128) * (size_t)scale_kblocks * 512;
-    if (cudaMemsetAsync(scales, 0, bytes, st) != cudaSuccess) return BRO_ERR_CUDA;
-  }
-  if ((K == 2048 || K == 4096) && !mse && !deq && !range_pass && format != rq::kFormatScaleOnly) {
-    // codes path at these sizes: all stages in registers, two shared-memory transposes
-    const int rows = (int)(128 / (K / 32));
-    const int64_t iters2 = (M + rows - 1) / rows;
-    const size_t smem2 = (size_t)2 * rows * K * sizeof(float) + (size_t)rows * K * 2 + 2048;   // fp32 buffers, bf16 box, barrier, alignment
-    CUtensorMap tmx;
-    const bro_status mrc = make_row_map(&tmx, x, M, K, ldx, rows);
-    if (mrc != BRO_OK) return mrc;
-    auto go2 = [&](auto kernel) -> bro_status {
-      static DeviceOnce once;                                             // (one per instantiation)
-      int per_sm = 1;
-      const bro_status rc = device_once(once, &per_sm, [&](int* n) {
-        if (!cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2),
-                     "cudaFuncSetAttribute(rotate_quantize_global_smem)"))
-          return BRO_ERR_CUDA;
-        return cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kernel, 128, smem2),
-                       "occupancy(rotate_quantize_global_smem)")
-                   ? BRO_OK
-                   : BRO_ERR_CUDA;
-      });
-      if (rc != BRO_OK) return rc;
-      const int64_t cap = (int64_t)sm_count * per_sm;
-      const unsigned grid2 = (unsigned)(iters2 < cap ? iters2 : cap);
-      return cuda_ok(launch_kernel(kernel, grid2, 128u, smem2, st, 1, tmx, p), "rotate_quantize_global_smem launch") ? BRO_OK
-                                                                                                                 : BRO_ERR_CUDA;
-    };
-    if (K == 4096) return signs ? go2(rotate_quantize_global_smem_kernel<12, true>) : go2(rotate_quantize_global_smem_kernel<12, false>);
-    return signs ? go2(rotate_quantize_global_smem_kernel<11, true>) : go2(rotate_quantize_global_smem_kernel<11, false>);
+  // (statistics of few short rows: the shuffle form starts faster, [1000, 1024] 3.05 and 3.34 us, [65536, 1024] 61 and 47)
+  const bool statistic = mse || format == rq::kFormatScaleOnly;
+  if (!deq && !range_pass && (!mse || format == 0) && !(statistic && K <= 1024 && M * K <= ((int64_t)1 << 21))) {
+    const int mode = mse ? kError : (format == rq::kFormatScaleOnly ? kBytes : kCodes);
+    switch (lg) {
+      case 10: return launch_wide<12, 10>(p, mode, sm_count, st);
+      case 11: return launch_wide<12, 11>(p, mode, sm_count, st);
+      case 12: return launch_wide<12>(p, mode, sm_count, st);
+      case 13: return launch_wide<13>(p, mode, sm_count, st);
+      case 14: return launch_wide<14>(p, mode, sm_count, st);
+      case 15: return launch_wide<15>(p, mode, sm_count, st);
+      default: return launch_wide<12, 0>(p, mode, sm_count, st);
+    }
   }
   const int64_t iters = (M + p.rows_per_iter - 1) / p.rows_per_iter;
   const int64_t max_grid = (int64_t)sm_count * (threads <= 512 ? 2 : 1);
