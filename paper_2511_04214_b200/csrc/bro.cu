@@ -461,6 +461,12 @@ bro_status bro_group_scale_bytes(const void* x_bf16, int64_t M, int64_t K, int64
   if (block == 1) {
     // the identity rotation: a sign flip does not change a magnitude, so the signs play no part
     const unsigned grid = bro::stats::grid_for(M * (K / 32), 256, di.sm_count, 8);
+    if (ldx == K || M == 1)
+      return bro::cuda_ok(bro::launch_kernel(bro::stats::group_scale_bytes_identity_flat, grid, 256, 0, st, 1,
+                                             static_cast<const uint16_t*>(x_bf16), M * (K / 32), scales),
+                          "group_scale_bytes launch")
+                 ? BRO_OK
+                 : BRO_ERR_CUDA;
     return bro::cuda_ok(bro::launch_kernel(bro::stats::group_scale_bytes_identity, grid, 256, 0, st, 1,
                                            static_cast<const uint16_t*>(x_bf16), M, K, ldx, scales),
                         "group_scale_bytes launch")
@@ -497,16 +503,17 @@ bro_status bro_outlier_groups(const void* x_bf16, int64_t M, int64_t K, int64_t 
   if (rc != BRO_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   unsigned long long* hist = static_cast<unsigned long long*>(workspace);
-  if (!bro::cuda_ok(cudaMemsetAsync(hist, 0, bro::stats::kWorkspaceBytes, st), "cudaMemsetAsync(histogram)"))
+  const uint16_t* x = static_cast<const uint16_t*>(x_bf16);
+  const unsigned long long n = (unsigned long long)M * (unsigned long long)K;
+  unsigned long long k = (n * (unsigned long long)top_ppm + 999999ull) / 1000000ull;
+  if (k < 1) k = 1;
+  if (!bro::cuda_ok(bro::launch_kernel(bro::stats::outlier_clear, (unsigned)bro::stats::kClearCtas, bro::stats::kScanThreads, 0, st, 1, hist),
+                    "outlier_clear launch"))
     return BRO_ERR_CUDA;
   static bro::DeviceOnce once;
   const int smem = bro::stats::kMagBins * 4;
   rc = bro::device_once(once, nullptr, [&](int*) { return set_smem(bro::stats::outlier_scan, smem); });
   if (rc != BRO_OK) return rc;
-  const uint16_t* x = static_cast<const uint16_t*>(x_bf16);
-  const unsigned long long n = (unsigned long long)M * (unsigned long long)K;
-  unsigned long long k = (n * (unsigned long long)top_ppm + 999999ull) / 1000000ull;
-  if (k < 1) k = 1;
   const unsigned sgrid = bro::stats::grid_for(M * (K / 32), bro::stats::kScanThreads, di.sm_count, 1);
   if (!bro::cuda_ok(bro::launch_kernel(bro::stats::outlier_scan, sgrid, bro::stats::kScanThreads, (size_t)smem, st, 1, x, M, K, ldx,
                                        k, hist, info, mask),
@@ -520,6 +527,11 @@ bro_status bro_outlier_groups(const void* x_bf16, int64_t M, int64_t K, int64_t 
              : BRO_ERR_CUDA;
 }
 
+static bool clear_counts(uint64_t* counts, int n, cudaStream_t st) {
+  return bro::cuda_ok(bro::launch_kernel(bro::stats::clear_counts, 1u, 512u, 0, st, 1, reinterpret_cast<unsigned long long*>(counts), n),
+                      "clear_counts launch");
+}
+
 bro_status bro_scale_histogram(const uint8_t* scales, const uint8_t* mask, int64_t n_groups, uint64_t* hist,
                                void* stream) {
   if (n_groups < 0) return BRO_ERR_SHAPE;
@@ -531,9 +543,7 @@ bro_status bro_scale_histogram(const uint8_t* scales, const uint8_t* mask, int64
   if (rc != BRO_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const bool alone = n_groups > 0 && bro::stats::count_alone(n_groups);
-  if (!alone &&
-      !bro::cuda_ok(cudaMemsetAsync(hist, 0, 2 * 256 * sizeof(uint64_t), st), "cudaMemsetAsync(scale histogram)"))
-    return BRO_ERR_CUDA;
+  if (!alone && !clear_counts(hist, 2 * 256, st)) return BRO_ERR_CUDA;
   if (n_groups == 0) return BRO_OK;
   const unsigned grid = alone ? 1u : bro::stats::grid_for(n_groups, bro::stats::kCountThreads * 16, di.sm_count, 2);
   return bro::cuda_ok(bro::launch_kernel(bro::stats::scale_histogram, grid, bro::stats::kCountThreads, 0, st, 1, scales, mask, n_groups,
@@ -555,9 +565,7 @@ bro_status bro_scale_inflation(const uint8_t* scales_before, const uint8_t* scal
   if (rc != BRO_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const bool alone = n_groups > 0 && bro::stats::count_alone(n_groups);
-  if (!alone &&
-      !bro::cuda_ok(cudaMemsetAsync(counts, 0, 6 * sizeof(uint64_t), st), "cudaMemsetAsync(inflation counts)"))
-    return BRO_ERR_CUDA;
+  if (!alone && !clear_counts(counts, 6, st)) return BRO_ERR_CUDA;
   if (n_groups == 0) return BRO_OK;
   const unsigned grid = alone ? 1u : bro::stats::grid_for(n_groups, bro::stats::kCountThreads * 16, di.sm_count, 2);
   return bro::cuda_ok(bro::launch_kernel(bro::stats::scale_inflation, grid, bro::stats::kCountThreads, 0, st, 1, scales_before, scales_after, mask,

@@ -67,18 +67,58 @@ __device__ __forceinline__ uint32_t group_max_mag(const uint16_t* x, int64_t row
   return m;
 }
 
-// One thread per group.  The byte is max(expfield(amax) - 2, 0) with expfield the 8-bit exponent of
-// amax as fp32 — for a bf16 value that is bits 7..14 of its pattern.
+// The largest magnitude pattern of every group of a run of 32 consecutive groups in memory, by a warp that reads whole lines:
+// lane l holds the 16 bytes 256 j + 8 l .. of the 2 KiB in q[j], a quarter of group 8 j + l / 4.  The four lanes of a quad
+// exchange maxima (both halves of a word at a time) so that lane l is left with group 8 (l mod 4) + l / 4.
+__device__ __forceinline__ uint32_t max_mag8_pairs(uint4 q) {
+  return __vmaxu2(__vmaxu2(q.x & 0x7FFF7FFFu, q.y & 0x7FFF7FFFu), __vmaxu2(q.z & 0x7FFF7FFFu, q.w & 0x7FFF7FFFu));
+}
+__device__ __forceinline__ uint32_t quad_maxima(const uint32_t (&m)[4], int lane) {
+  const bool b0 = (lane & 1) != 0, b1 = (lane & 2) != 0;
+  uint32_t k0 = b0 ? m[1] : m[0], k1 = b0 ? m[3] : m[2];                 // groups j = b0 and b0 + 2
+  k0 = __vmaxu2(k0, __shfl_xor_sync(0xFFFFFFFFu, b0 ? m[0] : m[1], 1));
+  k1 = __vmaxu2(k1, __shfl_xor_sync(0xFFFFFFFFu, b0 ? m[2] : m[3], 1));
+  const uint32_t k = __vmaxu2(b1 ? k1 : k0, __shfl_xor_sync(0xFFFFFFFFu, b1 ? k0 : k1, 2));
+  return max(k & 0xFFFFu, k >> 16);
+}
+__device__ __forceinline__ int quad_group(int lane) { return 8 * (lane & 3) + (lane >> 2); }
+
+// The byte is max(expfield(amax) - 2, 0) with expfield the 8-bit exponent of amax as fp32 — for a bf16 value that is
+// bits 7..14 of its pattern.
+__device__ __forceinline__ uint8_t scale_byte_of(uint32_t mag) {
+  const uint32_t ef = mag >> 7;
+  return (uint8_t)(ef > 2u ? ef - 2u : 0u);
+}
+// One thread per group: rows with a stride.
 __global__ void __launch_bounds__(256) group_scale_bytes_identity(const uint16_t* x, int64_t M, int64_t K, int64_t ldx,
                                                                   uint8_t* scales) {
   griddep_wait();
+  griddep_launch_dependents();
   const int64_t ng = K >> 5, total = M * ng;
   // (divided per group, not walked: the walk's two divisions before the loop and its carry in it cost 0.2 us of a small
   // launch and 24.3 -> 27.2 us at [16384, 4096])
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t row = i / ng, g = i - row * ng;
-    const uint32_t ef = group_max_mag(x, row, ldx, g) >> 7;
-    scales[i] = (uint8_t)(ef > 2u ? ef - 2u : 0u);
+    scales[i] = scale_byte_of(group_max_mag(x, row, ldx, g));
+  }
+}
+// Rows without a stride are one row: 32 groups a warp and pass.
+__global__ void __launch_bounds__(256) group_scale_bytes_identity_flat(const uint16_t* x, int64_t total, uint8_t* scales) {
+  griddep_wait();
+  griddep_launch_dependents();
+  const int lane = threadIdx.x & 31;
+  const int64_t step = (int64_t)gridDim.x * 256;
+  for (int64_t base = (int64_t)blockIdx.x * 256 + (threadIdx.x & ~31u); base < total; base += step) {
+    const uint4* src = reinterpret_cast<const uint4*>(x + base * 32) + lane;
+    uint32_t m[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const bool in = base + 8 * j + (lane >> 2) < total;
+      m[j] = max_mag8_pairs(in ? __ldg(src + 32 * j) : make_uint4(0u, 0u, 0u, 0u));
+    }
+    const uint32_t mag = quad_maxima(m, lane);
+    const int64_t i = base + quad_group(lane);
+    if (i < total) scales[i] = scale_byte_of(mag);
   }
 }
 
@@ -135,12 +175,73 @@ __device__ __forceinline__ bool find_threshold(Count&& count, unsigned long long
   return true;
 }
 
+// The same for counts of 32 bits with one trip to the histogram: a warp holds the 1024 patterns of its segment, the highest with
+// warp 0, and the warp in which the count from above passes k looks into what it holds.  ([300, 4096] 0.6 us less than in two trips.)
+__device__ __forceinline__ bool find_threshold_narrow(const uint32_t* hist, uint32_t k, uint32_t lowest, uint32_t* info) {
+  __shared__ uint32_t segments[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, base = 1024 * (31 - warp);
+  uint4 c[8] = {};                                    // patterns base + 128 j + 4 lane ..
+  uint32_t sum = 0;
+  if (base + 1024 > (int)lowest) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) c[j] = __ldcg(reinterpret_cast<const uint4*>(hist + base + 128 * j) + lane);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sum += c[j].x + c[j].y + c[j].z + c[j].w;
+  }
+  const uint32_t total = __reduce_add_sync(0xFFFFFFFFu, sum);
+  if (lane == 0) segments[warp] = total;
+  __syncthreads();
+  uint32_t above = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? segments[lane] : 0u);      // counted above this segment
+  const bool here = above < k && above + total >= k;
+  if (here) {
+#pragma unroll
+    for (int j = 7; j >= 0; --j) {
+      uint32_t upto = c[j].x + c[j].y + c[j].z + c[j].w;            // -> of this lane and those above it
+      const uint32_t all = __reduce_add_sync(0xFFFFFFFFu, upto);
+      if (above < k && above + all >= k) {
+        const uint32_t v[4] = {c[j].x, c[j].y, c[j].z, c[j].w};
+        const uint32_t mine = upto;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const uint32_t o = __shfl_down_sync(0xFFFFFFFFu, upto, d);
+          if (lane + d < 32) upto += o;
+        }
+        uint32_t count = above + upto - mine;
+#pragma unroll
+        for (int q = 3; q >= 0; --q) {
+          if (count < k && count + v[q] >= k) {
+            info[0] = (uint32_t)(base + 128 * j + 4 * lane + q);
+            info[1] = 0u;
+            info[2] = k;
+            info[3] = 0u;
+          }
+          count += v[q];
+        }
+      }
+      above += all;
+    }
+  }
+  return __syncthreads_or(here) != 0;
+}
+
+// In front of the scan: clears the histogram and the words behind it, and lets the scan start once everything older is complete (a
+// memset in its place stood between the kernel before and the scan without any overlap).
+constexpr int kClearCtas = 8;
+__global__ void __launch_bounds__(kScanThreads) outlier_clear(unsigned long long* hist) {
+  griddep_wait();
+  griddep_launch_dependents();
+  uint4* dst = reinterpret_cast<uint4*>(hist);
+  for (int i = (int)(blockIdx.x * kScanThreads + threadIdx.x); i < (int)(kWorkspaceBytes / 16); i += kClearCtas * kScanThreads)
+    dst[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 // The outliers are the top 0.1 % (top k of n) of the magnitudes, found exactly from a histogram of bf16 patterns; one pass
 // over x.  A shared-memory atomic per value bounded it before (75 us for 67 M values and 20 us for the search in a
 // launch of its own; now 42 us, of which 30 us are the pass, issue-bound, and 12 us merging and search), so only values of
 // at least `lowest` are counted, a pattern that every CTA derives from the same 4096 sampled
 // values such that about 4 k values (and 12 of the sample) lie at or above it: the loop reduces a group to its maximum and
-// touches the histogram for the few groups that reach `lowest`.  The last CTA to merge its histogram searches the
+// touches the histogram for the few groups that reach `lowest`.  Behind outlier_clear, which waited for everything older, it runs up
+// to the merging of the histograms without waiting for the histogram to be cleared.  The last CTA to merge searches the
 // threshold, without a launch of its own.  Should the sample have misled (fewer than k counted), that CTA counts everything
 // by itself: slow, and exact.
 // codes[g] = 0 if the group's maximum is below `lowest`, else group_code(maximum - lowest): see outlier_group_mask.
@@ -155,7 +256,6 @@ __global__ void __launch_bounds__(kScanThreads, 1) outlier_scan(const uint16_t* 
   local[threadIdx.x] = 0u;
   if (threadIdx.x == 0) lowest_s = 0u;
   __syncthreads();
-  griddep_wait();
   const int64_t n = M * K;
   if (n > 16 * kSamples) {
     const unsigned long long want = 4 * ((k * kSamples + n - 1) / n) + 12;      // sampled values at or above `lowest`
@@ -230,6 +330,8 @@ __global__ void __launch_bounds__(kScanThreads, 1) outlier_scan(const uint16_t* 
       }
     }
   }
+  griddep_wait();                                     // the histogram is clear
+  griddep_launch_dependents();
   __syncthreads();
   // Fewer than 2^32 values in all: two 32-bit counts to a 64-bit atomic (no count can carry into its neighbour), half the
   // atomics that all CTAs throw at the same few thousand bins.
@@ -253,7 +355,9 @@ __global__ void __launch_bounds__(kScanThreads, 1) outlier_scan(const uint16_t* 
   auto counted = [&](int b) {
     return wide ? __ldcg(hist + b) : (unsigned long long)__ldcg(reinterpret_cast<const uint32_t*>(hist) + b);
   };
-  if (find_threshold(counted, k, lowest, info, warp_sums)) return;
+  if (wide ? find_threshold(counted, k, lowest, info, warp_sums)
+           : find_threshold_narrow(reinterpret_cast<const uint32_t*>(hist), (uint32_t)k, lowest, info))
+    return;
   // fewer than k at or above `lowest`
   for (int i = (int)threadIdx.x; i < kMagBins; i += kScanThreads) local[i] = 0u;
   __syncthreads();
@@ -278,27 +382,32 @@ __global__ void __launch_bounds__(kScanThreads, 1) outlier_scan(const uint16_t* 
 __global__ void __launch_bounds__(256) outlier_group_mask(const uint16_t* x, int64_t M, int64_t K, int64_t ldx,
                                                           const uint32_t* info, const unsigned long long* hist, uint8_t* mask) {
   griddep_wait();
-  const uint32_t t = info[0], lowest = reinterpret_cast<const uint32_t*>(hist + kMagBins)[kLowestWord];
+  griddep_launch_dependents();
   const int64_t ng = K >> 5, total = M * ng;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, threads = (int64_t)gridDim.x * blockDim.x;
+  const int64_t vec = (reinterpret_cast<uintptr_t>(mask) & 15) == 0 ? total >> 4 : 0;      // 16 groups at a time
+  uint4 v = tid < vec ? reinterpret_cast<uint4*>(mask)[tid] : make_uint4(0u, 0u, 0u, 0u);  // (beside the load of the threshold)
+  const uint32_t t = info[0], lowest = reinterpret_cast<const uint32_t*>(hist + kMagBins)[kLowestWord];
   auto again = [&](int64_t i) { return (uint32_t)(group_max_mag(x, i / ng, ldx, i - i / ng * ng) >= t ? 1 : 0); };
   if (t < lowest) {
     for (int64_t i = tid; i < total; i += threads) mask[i] = (uint8_t)again(i);
     return;
   }
   const uint32_t code = group_code(t - lowest), code4 = code * 0x01010101u;
-  const int64_t vec = (reinterpret_cast<uintptr_t>(mask) & 15) == 0 ? total >> 4 : 0;      // 16 groups at a time
   for (int64_t i = tid; i < vec; i += threads) {
-    const uint4 v = reinterpret_cast<uint4*>(mask)[i];
+    if (i != tid) v = reinterpret_cast<uint4*>(mask)[i];
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    uint32_t r[4];
+    uint32_t r[4], open = 0;                          // one bit a group to be read again
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       r[c] = __vcmpgtu4(w[c], code4) & 0x01010101u;
-      for (uint32_t open = __vcmpeq4(w[c], code4) & 0x01010101u; open; open &= open - 1u) {
-        const int bit = __ffs(open) - 1;
-        r[c] |= again((i << 4) + 4 * c + (bit >> 3)) << bit;
-      }
+      open |= (((__vcmpeq4(w[c], code4) & 0x01010101u) * 0x01020408u) >> 24 & 0xFu) << (4 * c);
+    }
+    for (; open; open &= open - 1u) {                 // (all 16 in one loop: as many trips to memory as the busiest lane has groups)
+      const int bit = __ffs(open) - 1;
+      const uint32_t one = again((i << 4) + bit) << (8 * (bit & 3));
+#pragma unroll
+      for (int c = 0; c < 4; ++c) r[c] |= (bit >> 2) == c ? one : 0u;
     }
     reinterpret_cast<uint4*>(mask)[i] = make_uint4(r[0], r[1], r[2], r[3]);
   }
@@ -307,10 +416,18 @@ __global__ void __launch_bounds__(256) outlier_group_mask(const uint16_t* x, int
 }
 
 // Counts of few groups come from one CTA, which writes them whether or not the output was zeroed (`alone`); more groups
-// add to a zeroed output from the whole grid.  Groups are read 16 at a time where the pointers allow it.
+// add to an output that clear_counts zeroes, from the whole grid.  clear_counts lets the counting kernel start once everything
+// older is complete, so that it counts meanwhile and waits only before it adds; a memset in its place stood between two
+// kernels without any overlap.  Groups are read 16 at a time where the pointers allow it.
 constexpr int kCountThreads = 1024;
 constexpr int64_t kAloneGroups = 65536;
 inline bool count_alone(int64_t n_groups) { return n_groups <= kAloneGroups; }
+
+__global__ void __launch_bounds__(512) clear_counts(unsigned long long* counts, int n) {
+  griddep_wait();
+  griddep_launch_dependents();
+  if ((int)threadIdx.x < n) counts[threadIdx.x] = 0ull;
+}
 
 __device__ __forceinline__ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
@@ -319,7 +436,7 @@ __global__ void __launch_bounds__(kCountThreads) scale_histogram(const uint8_t* 
   __shared__ uint32_t local[512];
   for (int i = threadIdx.x; i < 512; i += kCountThreads) local[i] = 0u;
   __syncthreads();
-  griddep_wait();
+  if (alone) griddep_wait();           // (else the scales and the mask are older than clear_counts, which waited for them)
   const int64_t tid = (int64_t)blockIdx.x * kCountThreads + threadIdx.x, threads = (int64_t)gridDim.x * kCountThreads;
   const int64_t vec = aligned16(scales) && aligned16(mask) ? n >> 4 : 0;
   for (int64_t i = tid; i < vec; i += threads) {
@@ -332,6 +449,8 @@ __global__ void __launch_bounds__(kCountThreads) scale_histogram(const uint8_t* 
     }
   }
   for (int64_t i = (vec << 4) + tid; i < n; i += threads) atomicAdd(&local[(mask[i] ? 256 : 0) + scales[i]], 1u);
+  if (!alone) griddep_wait();
+  griddep_launch_dependents();
   __syncthreads();
   for (int i = threadIdx.x; i < 512; i += kCountThreads) {
     if (alone) hist[i] = local[i];
@@ -344,7 +463,7 @@ __global__ void __launch_bounds__(kCountThreads) scale_inflation(const uint8_t* 
   __shared__ uint32_t local[6];
   if (threadIdx.x < 6) local[threadIdx.x] = 0u;
   __syncthreads();
-  griddep_wait();
+  if (alone) griddep_wait();           // (else: see scale_histogram)
   uint32_t mine[6] = {0, 0, 0, 0, 0, 0};
   const int64_t tid = (int64_t)blockIdx.x * kCountThreads + threadIdx.x, threads = (int64_t)gridDim.x * kCountThreads;
   const int64_t vec = aligned16(before) && aligned16(after) && aligned16(mask) ? n >> 4 : 0;
@@ -373,6 +492,8 @@ __global__ void __launch_bounds__(kCountThreads) scale_inflation(const uint8_t* 
     const uint32_t v = __reduce_add_sync(0xFFFFFFFFu, mine[q]);
     if ((threadIdx.x & 31) == 0 && v) atomicAdd(&local[q], v);
   }
+  if (!alone) griddep_wait();
+  griddep_launch_dependents();
   __syncthreads();
   if (threadIdx.x < 6) {
     if (alone) counts[threadIdx.x] = local[threadIdx.x];
