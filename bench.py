@@ -511,7 +511,15 @@ def gemm_kernel_name(M, K, N, sm_count=148):
     one_wave = (tiles_m == 1 or steps >= 8) if narrow else (M <= 64 and -(-n128 // 2) <= sm_count)
     if one_wave and not (M > 64 and (steps < 2 or (steps < 4 and not 8 <= n128 <= 64))):
         return "gemm_mxfp4_splitk_kernel"
-    pair = K >= 4096 and (-(-M // 256)) * (-(-N // 256)) >= 2 * (sm_count // 2)
+
+    def rounds(units, at_once, half):
+        rem = units % at_once
+        return units // at_once + (0.0 if rem == 0 else half if 2 * rem <= at_once else 1.0)
+
+    single_steps = rounds(tiles_m * -(-N // 256), sm_count, 0.66) * steps
+    pair_steps = rounds(-(-M // 256) * -(-N // 256), sm_count // 2, 0.77) * steps
+    t1, t2, launch = (0.67, 0.47, 1.8) if K % 64 else (0.435, 0.37, 3.0) if K % 256 else (0.41, 0.367, 3.0)
+    pair = M > 128 and pair_steps * t2 + launch < single_steps * t1
     return "gemm_mxfp4_pair_kernel" if pair else "gemm_mxfp4_kernel"
 
 

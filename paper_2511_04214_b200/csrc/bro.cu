@@ -609,6 +609,33 @@ static bro_status check_gemm(const void* acodes, const void* ascales, const void
   return BRO_OK;
 }
 
+// Whether two CTAs per 256 x 256 tile beat one per 128 x 256 tile.  The pair moves a third fewer bytes into shared memory per flop and
+// draws less power for it; its tiles are coarser, its start, hand-over and end cost more.  Compared are the rounds of the grid (a last
+// round of half-width units costs 0.66 and 0.77 of a whole one) times the steps of a tile, in microseconds as measured, for three kinds
+// of rows of codes:
+//   * whole 128-byte lines (K a multiple of 256): 0.41 a step for one CTA, 0.367 for the pair and 3.0 a launch.  Whole layers, half a
+//     second back to back, single -> pair: (8192, 8192, 28672) 875 -> 860 us, (8192, 2048, 8192) 84.7 -> 81.2, (1200, 4096, 28672) 84.3 -> 77.7,
+//     (2500, 14336, 5120) 105.9 -> 103.9; (4096, 14336, 4096) 138.7 both; not taken (4096, 4096, 4096) 44.4 -> 45.1, (2048, 2048, 8192) 25.1 both,
+//     (531, 8192, 14336) 42.9 -> 50.9, (2315, 14336, 7709) 138.8 -> 149.6, (1398, 4096, 16462) 54.4 -> 57.8, (3000, 2048, 2048) 14.4 -> 15.9.
+//   * whole sectors, not lines (multiples of 64): a row of a box lies in two lines, 0.435 and 0.37.  (4096, 7744, 8192) 144.7 -> 133.8,
+//     (512, 13952, 18244) 75.3 -> 70.7, (4713, 3456, 28672) 272 -> 248; not taken (783, 12352, 14336) 91.8 -> 96.2, (543, 4032, 8192) 19.4 -> 20.2.
+//   * an odd multiple of 16 bytes: a row of a box touches five sectors instead of four as well, 0.67 and 0.47, 1.8 a launch.
+//     (2016, 3488, 15387) 87.2 -> 70.8, (1473, 2336, 8841) 30.2 -> 26.4, (3530, 9504, 28672) 649 -> 503, (195, 2848, 14336) 13.0 -> 12.4, the GEMM of
+//     (777, 4384, 6004) 22.9 -> 19.3; not taken (1269, 1056, 4096) 10.8 -> 11.3, (1294, 1696, 1547) 11.1 -> 11.5.
+// At most 128 tokens: the single-CTA kernel loads no more rows of them than there are.
+static bool pair_pays(int64_t M, int64_t N, int64_t K, int sm_count) {
+  if (M <= 128) return false;
+  auto rounds = [](int64_t units, int64_t at_once, double half) {
+    const int64_t rem = units % at_once;
+    return (double)(units / at_once) + (rem == 0 ? 0.0 : (2 * rem <= at_once ? half : 1.0));
+  };
+  const double steps = (double)ceil_div(K, 256);
+  const double single = rounds(ceil_div(M, 128) * ceil_div(N, 256), sm_count, 0.66) * steps;
+  const double pair = rounds(ceil_div(M, 256) * ceil_div(N, 256), sm_count / 2, 0.77) * steps;
+  if (K % 64 != 0) return pair * 0.47 + 1.8 < single * 0.67;
+  return K % 256 != 0 ? pair * 0.37 + 3.0 < single * 0.435 : pair * 0.367 + 3.0 < single * 0.41;
+}
+
 static bro_status gemm_impl(const void* acodes, const void* ascales, const void* wcodes, const void* wscales,
                             int64_t M, int64_t N, int64_t K, void* y, int64_t ldy, bro_out_dtype out_dtype,
                             void* workspace, size_t workspace_bytes, uint32_t flags, void* stream, bool w_static) {
@@ -628,17 +655,14 @@ static bro_status gemm_impl(const void* acodes, const void* ascales, const void*
       return bro::gemms::launch(plan, nullptr, acodes, ascales, wcodes, wscales, M, N, K, y, ldy, (int)out_dtype, di.sm_count,
                                 static_cast<cudaStream_t>(stream), w_static);
   }
-  // Else the two-CTA kernel (256 x 256 tiles, cta_group::2) moves a third fewer bytes into
-  // shared memory per flop and measures 3-7 % faster once a problem has at least two rounds of
-  // 256 x 256 tiles and tiles long enough (K >= 4096) to amortise its costlier tile hand-over; below
-  // that the single-CTA kernel wins (half-width units for the last round, 128-row granularity, cheaper
-  // prologue).  The flags of the *_ex entry point force either.
+  // Else one CTA per 128 x 256 tile, or two per 256 x 256 tile (cta_group::2): see pair_pays.  The flags of the *_ex entry point force
+  // either.
   bool pair = (flags & BRO_FLAG_GEMM_PAIR) != 0;
   if (!(flags & (BRO_FLAG_GEMM_PAIR | BRO_FLAG_GEMM_SINGLE | BRO_FLAG_GEMM_TILE_N128 | BRO_FLAG_GEMM_TILE_N256)))
-    pair = K >= 4096 && ceil_div(M, 256) * ceil_div(N, 256) >= 2 * (int64_t)(di.sm_count / 2);
+    pair = pair_pays(M, N, K, di.sm_count);
   if (pair)
     return bro::gemm2::launch(acodes, ascales, wcodes, wscales, M, N, K, y, ldy, (int)out_dtype, flags, di.sm_count,
-                              static_cast<cudaStream_t>(stream));
+                              static_cast<cudaStream_t>(stream), w_static);
   return bro::gemm::launch(acodes, ascales, wcodes, wscales, M, N, K, y, ldy, (int)out_dtype, workspace,
                            workspace_bytes, flags, di.sm_count, static_cast<cudaStream_t>(stream), w_static);
 }

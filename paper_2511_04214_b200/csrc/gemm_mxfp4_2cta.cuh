@@ -8,6 +8,11 @@
 // halves of W across the pair, so every CTA pulls (128 + 128) x 128 bytes per step for the same
 // flops — 480 flop per byte — with no multicast load anywhere.
 //
+// (What that is worth, and where: pair_pays in bro.cu.)  In the whole-layer calls the weight halves of the first ring are requested
+// before griddepcontrol.wait, as in the single-CTA kernel, and a pair's final unit stages its output in the idle operand stages,
+// a buffer per 64 columns, so that no store has to be waited for: (768, 4384, 6016) 14.0 -> 13.7 us, fp32 output 15.9 -> 15.1,
+// the layer 17.7 -> 16.6; (512, 4128, 14336) 21.5 -> 20.8, 24.1 -> 22.6, 24.7 -> 23.2.
+//
 // Roles in each CTA (192 threads):
 //   warp 0      TMA producer for this CTA's operand halves.  All loads of both CTAs count their
 //               bytes on the LEADER's "full" barrier (cp.async.bulk.tensor ... .cta_group::2).
@@ -56,6 +61,7 @@ struct Params {
   // Work units, as in the single-CTA kernel: units [0, full_units) are whole tiles; when the last round
   // of the grid would be less than half full, its tiles are cut into two 256 x 128 halves each.
   int full_units, total_units;
+  int w_static;             // the weight operand was complete before the previous kernel started
 };
 
 // ---- cluster helpers ---------------------------------------------------------------------------
@@ -171,7 +177,9 @@ gemm_mxfp4_pair_kernel(const __grid_constant__ CUtensorMap tma, const __grid_con
   cluster_sync_all();                       // the partner's barriers exist before anyone signals them
   gemm::tc_fence_after();
   griddep_launch_dependents();
-  griddep_wait();                           // operands come from the kernel before; y may still be read by it
+  // operands come from the kernel before, and y may still be read by it; the weights of a whole-layer call are older
+  const bool early_w = p.w_static != 0 && warp == 0;
+  if (!early_w) griddep_wait();
   const uint32_t tmem_base = __shfl_sync(0xFFFFFFFFu, *tmem_slot_ptr, 0);
   const uint32_t tmem_sfa = tmem_base + kSfaCol;
   const uint32_t tmem_sfb = tmem_base + kSfbCol;
@@ -192,27 +200,50 @@ gemm_mxfp4_pair_kernel(const __grid_constant__ CUtensorMap tma, const __grid_con
       int64_t issued = 0;
       bool ok = true;
       const uint32_t full0 = map_to_cta(bar_full, 0);      // the leader's barriers, as seen from here
-      for (int u = pair; u < p.total_units && ok; u += num_pairs) {
-        int tile, half, bn, tm, tn;
+      auto unit_coords = [&](int u, int& m0, int& n0, int& bn) {
+        int tile, half, tm, tn;
         unit_tile(u, p, tile, half, bn);
         tile_coords(tile, p, tm, tn);
-        const int m0 = tm * 256 + (int)rank * kBM;
-        const int n0 = tn * kBN + half * (kBN / 2);
-        // a half-width unit brings half as many W rows per CTA (through the map with the smaller box)
-        const uint32_t stage_tx = 2u * (uint32_t)(kStageBytes - (bn == kBN ? 0 : kBTileBytes / 2));
-        for (int ks = 0; ks < p.num_k_steps; ++ks) {
+        m0 = tm * 256 + (int)rank * kBM;
+        n0 = tn * kBN + half * (kBN / 2);
+      };
+      // `part`: 1 the weight side, 2 the activation side, 3 both
+      auto issue_step = [&](int m0, int n0, int bn, int ks, int st, int part) {
+        const uint32_t full = full0 + 8 * st;
+        if (part & 1) {
+          // a half-width unit brings half as many W rows per CTA (through the map with the smaller box)
+          if (rank == 0)
+            mbar_arrive_expect_tx_elect(bar_full + 8 * st, 2u * (uint32_t)(kStageBytes - (bn == kBN ? 0 : kBTileBytes / 2)));
+          if (bn == kBN)
+            tma_load_2d_pair(sB + st * kBTileBytes, &tmw, ks * 128, n0 + (int)rank * (kBN / 2), full);
+          else
+            tma_load_2d_pair(sB + st * kBTileBytes, &tmw_half, ks * 128, n0 + (int)rank * (kBN / 4), full);
+          // scale maps are in 32-bit elements: one K step = 1024 bytes = 256 elements per row block
+          tma_load_2d_pair(sSFB + st * kSfbBytes, &tmsfb, ks * 256, n0 >> 7, full);
+        }
+        if (part & 2) {
+          tma_load_2d_pair(sA + st * kATileBytes, &tma, ks * 128, m0, full);
+          tma_load_2d_pair(sSFA + st * kSfaBytes, &tmsfa, ks * 256, m0 >> 7, full);
+        }
+      };
+      int pre = 0;                  // K steps of the first unit whose loads are issued here
+      if (early_w) {
+        int m0, n0, bn;
+        unit_coords(pair, m0, n0, bn);                      // (the grid has no more pairs than units)
+        pre = p.num_k_steps < kStages ? p.num_k_steps : kStages;
+        for (int ks = 0; ks < pre; ++ks) issue_step(m0, n0, bn, ks, ks, 1);   // weights: before the wait
+        griddep_wait();
+        for (int ks = 0; ks < pre; ++ks) issue_step(m0, n0, bn, ks, ks, 2);   // activations: after it
+        issued = pre;
+        if (pre == kStages) phase = 1u; else stage = pre;
+      }
+      for (int u = pair; u < p.total_units && ok; u += num_pairs) {
+        int m0, n0, bn;
+        unit_coords(u, m0, n0, bn);
+        for (int ks = (u == pair ? pre : 0); ks < p.num_k_steps; ++ks) {
           if (issued >= kStages) ok = mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1u, SITE_GEMM_EMPTY);
           if (!ok) break;
-          if (rank == 0) mbar_arrive_expect_tx_elect(bar_full + 8 * stage, stage_tx);
-          const uint32_t full = full0 + 8 * stage;
-          tma_load_2d_pair(sA + stage * kATileBytes, &tma, ks * 128, m0, full);
-          if (bn == kBN)
-            tma_load_2d_pair(sB + stage * kBTileBytes, &tmw, ks * 128, n0 + (int)rank * (kBN / 2), full);
-          else
-            tma_load_2d_pair(sB + stage * kBTileBytes, &tmw_half, ks * 128, n0 + (int)rank * (kBN / 4), full);
-          // scale maps are in 32-bit elements: one K step = 1024 bytes = 256 elements per row block
-          tma_load_2d_pair(sSFA + stage * kSfaBytes, &tmsfa, ks * 256, m0 >> 7, full);
-          tma_load_2d_pair(sSFB + stage * kSfbBytes, &tmsfb, ks * 256, n0 >> 7, full);
+          issue_step(m0, n0, bn, ks, stage, 3);
           ++issued;
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
@@ -253,15 +284,18 @@ gemm_mxfp4_pair_kernel(const __grid_constant__ CUtensorMap tma, const __grid_con
       const uint32_t tmem_acc = tmem_base + buf * kAccStride + ((uint32_t)(q * 32) << 16);
       const int row0 = tm * 256 + (int)rank * kBM + q * 32;
       const int n0 = tn * kBN + half * (kBN / 2);
-      const uint32_t stage_buf = sOut + (uint32_t)q * (32u * 128u);
+      // the final unit of this pair stages every pair of chunks in its own 4 KiB of the (now idle) operand stages
+      const bool last = u + num_pairs >= p.total_units;
+      const uint32_t stage_buf = last ? sA + (uint32_t)q * (OUT_F32 ? 8u * 4096u : 4u * 4096u) : sOut + (uint32_t)q * (32u * 128u);
+      const uint32_t stage_stride = last ? 4096u : 0u;
       auto release_shared = [&] { mbar_arrive_cluster(ovl_free_leader); };
       auto release_all = [&] { mbar_arrive_cluster(acc_free_leader); };
       if (bn == kBN)
         gemm::epilogue_tile<kChunks, true, OUT_F32>(tmem_acc, buf, lane, row0, n0, p.M, p.N, p.y, p.ldy, &tmy, stage_buf,
-                                                    0u, release_shared, release_all);
+                                                    stage_stride, release_shared, release_all);
       else
         gemm::epilogue_tile<kChunks / 2, true, OUT_F32>(tmem_acc, buf, lane, row0, n0, p.M, p.N, p.y, p.ldy, &tmy,
-                                                        stage_buf, 0u, release_shared, release_all);
+                                                        stage_buf, stage_stride, release_shared, release_all);
     }
     // the staging buffer must have been read before this CTA's shared memory goes away; the writes
     // themselves complete with the kernel
@@ -301,8 +335,9 @@ inline int max_resident_pairs(Kern kernel, int sm_count) {
 
 inline bro_status launch(const void* acodes, const void* ascales, const void* wcodes, const void* wscales,
                          int64_t M, int64_t N, int64_t K, void* y, int64_t ldy, int out_dtype, uint32_t flags,
-                         int sm_count, cudaStream_t st) {
+                         int sm_count, cudaStream_t st, bool w_static) {
   Params p;
+  p.w_static = w_static ? 1 : 0;
   p.y = y;
   p.M = M; p.N = N; p.ldy = ldy;
   p.num_k_steps = (int)((K + kBK - 1) / kBK);
