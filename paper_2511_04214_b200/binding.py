@@ -1,4 +1,5 @@
-"""ctypes binding for libbro — argument marshalling only.
+"""Binding for libbro — argument marshalling only: the calls of a layer or a study through ``_call`` (csrc/call.cpp), everything
+else, and what ``_call`` leaves to it, through ctypes.
 
 Every function takes torch CUDA tensors (device memory owned by the caller), passes raw pointers
 and sizes to the C ABI declared in ``include/bro.h`` and raises :class:`BroError` on a non-zero
@@ -8,6 +9,8 @@ if the shared library is missing the import of this module fails.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 
 import torch
@@ -142,7 +145,19 @@ def _load() -> ctypes.CDLL:
     return L
 
 
+def _load_call():
+    path = os.path.join(_HERE, "_call.so")
+    if not os.path.exists(path):
+        raise ImportError(f"{path} is missing: build it with `python -m paper_2511_04214_b200.build`")
+    loader = importlib.machinery.ExtensionFileLoader("_call", path)
+    module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_call", loader, origin=path))
+    loader.exec_module(module)
+    module.bind({name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in module.NAMES})
+    return module
+
+
 lib = _load()
+_call = _load_call()        # its functions return the status, or -1: "not plainly my arguments", and the code below each goes on
 
 
 def status_string(code: int) -> str:
@@ -225,6 +240,10 @@ def alloc_workspace(nbytes: int, device="cuda") -> torch.Tensor:
 
 def rotate_quantize_mxfp4(x: torch.Tensor, block: int, codes: torch.Tensor, scales: torch.Tensor,
                           layout: int = LAYOUT_GEMM, stream=None, flags: int = 0, signs=None) -> None:
+    if not flags:
+        code = _call.rotate_quantize(x, block, codes, scales, layout, signs, stream)
+        if code >= 0:
+            return _check(code, "bro_rotate_quantize_mxfp4" if signs is None else "bro_rotate_quantize_mxfp4_ex")
     assert x.dtype == torch.bfloat16 and x.dim() == 2 and x.stride(1) == 1
     M, K = x.shape
     if flags or signs is not None:
@@ -239,6 +258,9 @@ def rotate_quantize_mxfp4(x: torch.Tensor, block: int, codes: torch.Tensor, scal
 
 def pack_weights(w: torch.Tensor, block: int, wcodes: torch.Tensor, wscales: torch.Tensor,
                  stream=None) -> None:
+    code = _call.pack_weights(w, block, wcodes, wscales, None, stream)
+    if code >= 0:
+        return _check(code, "bro_pack_weights")
     assert w.dtype == torch.bfloat16 and w.dim() == 2 and w.stride(1) == 1
     N, K = w.shape
     _check(lib.bro_pack_weights(_ptr(w), N, K, w.stride(0) if N > 1 else max(w.stride(0), K), block,
@@ -247,6 +269,10 @@ def pack_weights(w: torch.Tensor, block: int, wcodes: torch.Tensor, wscales: tor
 
 def gemm_mxfp4(acodes, ascales, wcodes, wscales, M: int, N: int, K: int, y: torch.Tensor,
                workspace=None, stream=None, flags: int = 0) -> None:
+    if not flags:
+        code = _call.gemm(acodes, ascales, wcodes, wscales, M, N, K, y, workspace, stream)
+        if code >= 0:
+            return _check(code, "bro_gemm_mxfp4")
     out = OUT_BF16 if y.dtype == torch.bfloat16 else OUT_F32
     assert y.dtype in (torch.bfloat16, torch.float32) and y.stride(1) == 1
     wsb = 0 if workspace is None else workspace.numel()
@@ -262,6 +288,10 @@ def gemm_mxfp4(acodes, ascales, wcodes, wscales, M: int, N: int, K: int, y: torc
 
 def linear(x: torch.Tensor, block: int, wcodes, wscales, N: int, y: torch.Tensor,
            workspace: torch.Tensor, stream=None, flags: int = 0, signs=None) -> None:
+    if not flags and signs is None:
+        code = _call.linear(x, block, wcodes, wscales, N, y, workspace, None, stream)
+        if code >= 0:
+            return _check(code, "bro_linear")
     assert x.dtype == torch.bfloat16 and y.dtype == torch.bfloat16
     M, K = x.shape
     if flags:
@@ -325,6 +355,10 @@ def rotate_quantize_mxfp4_rs(x: torch.Tensor, block: int, signs: torch.Tensor, c
 
 
 def pack_weights_rs(w: torch.Tensor, block: int, signs: torch.Tensor, wcodes, wscales, stream=None) -> None:
+    if signs is not None:
+        code = _call.pack_weights(w, block, wcodes, wscales, signs, stream)
+        if code >= 0:
+            return _check(code, "bro_pack_weights_rs")
     assert w.dtype == torch.bfloat16 and signs.dtype == torch.bfloat16 and signs.numel() == w.shape[1]
     N, K = w.shape
     _check(lib.bro_pack_weights_rs(_ptr(w), N, K, _ld(w, K), block, _ptr(signs), _ptr(wcodes),
@@ -333,6 +367,10 @@ def pack_weights_rs(w: torch.Tensor, block: int, signs: torch.Tensor, wcodes, ws
 
 def linear_rs(x: torch.Tensor, block: int, signs: torch.Tensor, wcodes, wscales, N: int, y: torch.Tensor,
               workspace: torch.Tensor, stream=None) -> None:
+    if signs is not None:
+        code = _call.linear(x, block, wcodes, wscales, N, y, workspace, signs, stream)
+        if code >= 0:
+            return _check(code, "bro_linear_rs")
     assert x.dtype == torch.bfloat16 and y.dtype == torch.bfloat16 and signs.dtype == torch.bfloat16
     M, K = x.shape
     _check(lib.bro_linear_rs(_ptr(x), M, K, _ld(x, K), block, _ptr(signs), _ptr(wcodes), _ptr(wscales), N,
@@ -346,6 +384,10 @@ FORMATS = {"mxfp4": 0, "bfp4": 1, "mxint4": 2, "bint4": 3, "int4_row_sym": 4, "i
 def group_quant_error(x: torch.Tensor, block: int, mse: torch.Tensor, signs: torch.Tensor = None,
                       stream=None, fmt: str = "mxfp4") -> None:
     """Per-group quantisation error of the rotated activations: ``mse`` is fp32 [M, K/32]."""
+    if fmt in FORMATS:
+        code = _call.group_quant_error(x, block, mse, signs, FORMATS[fmt], stream)
+        if code >= 0:
+            return _check(code, "bro_group_quant_error_fmt")
     assert x.dtype == torch.bfloat16 and mse.dtype == torch.float32 and mse.is_contiguous()
     M, K = x.shape
     assert mse.shape == (M, K // 32)
@@ -363,6 +405,10 @@ def rotate_fake_quantize(x: torch.Tensor, block: int, deq: torch.Tensor, fmt: st
     x R_block quantised to ``fmt``; block = 1: no rotation, 0: the full dimension.  The per-row formats
     ("int4_row_sym", "int4_row_asym") need ``workspace`` (fake_quantize_workspace_bytes); "none" returns the
     rotated values themselves."""
+    if fmt in FORMATS:
+        code = _call.rotate_fake_quantize(x, block, deq, FORMATS[fmt], signs, workspace, stream)
+        if code >= 0:
+            return _check(code, "bro_rotate_fake_quantize_ws")
     assert x.dtype == torch.bfloat16 and deq.dtype == torch.float32
     M, K = x.shape
     assert deq.shape == (M, K)
@@ -373,6 +419,9 @@ def rotate_fake_quantize(x: torch.Tensor, block: int, deq: torch.Tensor, fmt: st
 
 def group_scale_bytes(x: torch.Tensor, block: int, scales: torch.Tensor, signs: torch.Tensor = None, stream=None) -> None:
     """E8M0 byte of every MX group of x R_block into ``scales`` (uint8 [M, K/32]); block = 1: no rotation."""
+    code = _call.group_scale_bytes(x, block, scales, signs, stream)
+    if code >= 0:
+        return _check(code, "bro_group_scale_bytes")
     assert x.dtype == torch.bfloat16 and scales.dtype == torch.uint8 and scales.is_contiguous()
     M, K = x.shape
     assert scales.shape == (M, K // 32)
@@ -384,6 +433,9 @@ def outlier_groups(x: torch.Tensor, mask: torch.Tensor, info: torch.Tensor, work
                    top_ppm: int = 1000, stream=None) -> None:
     """Groups holding one of the top ``top_ppm`` millionths of |x| -> ``mask`` (uint8 [M, K/32]);
     ``info`` (int32/uint32 [4] on the device) receives the threshold's bf16 pattern and k."""
+    code = _call.outlier_groups(x, mask, info, workspace, top_ppm, stream)
+    if code >= 0:
+        return _check(code, "bro_outlier_groups")
     assert x.dtype == torch.bfloat16 and mask.dtype == torch.uint8 and mask.is_contiguous()
     M, K = x.shape
     assert mask.shape == (M, K // 32) and info.numel() >= 4 and info.element_size() == 4
@@ -397,6 +449,9 @@ def outlier_workspace_bytes() -> int:
 
 def scale_histogram(scales: torch.Tensor, mask: torch.Tensor, hist: torch.Tensor, stream=None) -> None:
     """``hist`` (int64 [2, 256] on the device) <- scale-byte histograms of the regular / outlier groups."""
+    code = _call.scale_histogram(scales, mask, hist, stream)
+    if code >= 0:
+        return _check(code, "bro_scale_histogram")
     assert scales.dtype == torch.uint8 and mask.dtype == torch.uint8 and hist.dtype == torch.int64
     assert scales.is_contiguous() and mask.is_contiguous() and hist.is_contiguous() and hist.numel() == 512
     assert scales.numel() == mask.numel()
@@ -407,6 +462,9 @@ def scale_histogram(scales: torch.Tensor, mask: torch.Tensor, hist: torch.Tensor
 def scale_inflation(before: torch.Tensor, after: torch.Tensor, mask: torch.Tensor, counts: torch.Tensor,
                     stream=None) -> None:
     """``counts`` (int64 [2, 3] on the device) <- per class, groups whose byte went down / stayed / went up."""
+    code = _call.scale_inflation(before, after, mask, counts, stream)
+    if code >= 0:
+        return _check(code, "bro_scale_inflation")
     assert before.dtype == after.dtype == mask.dtype == torch.uint8 and counts.dtype == torch.int64
     assert before.is_contiguous() and after.is_contiguous() and mask.is_contiguous() and counts.numel() == 6
     assert before.numel() == after.numel() == mask.numel()
@@ -437,6 +495,9 @@ def linear_packed(x: torch.Tensor, block: int, weights: PackedWeights, y: torch.
 def swiglu_rotate_quantize_mxfp4(gate: torch.Tensor, up: torch.Tensor, block: int, codes, scales,
                                  layout: int = LAYOUT_GEMM, signs: torch.Tensor = None, stream=None) -> None:
     """rotate_quantize_mxfp4 of h = silu(gate) * up, with h computed inside the kernel."""
+    code = _call.swiglu_rotate_quantize(gate, up, block, codes, scales, layout, signs, stream)
+    if code >= 0:
+        return _check(code, "bro_swiglu_rotate_quantize_mxfp4")
     assert gate.dtype == up.dtype == torch.bfloat16 and gate.shape == up.shape
     assert gate.stride(1) == 1 and up.stride(1) == 1
     M, K = gate.shape
@@ -456,6 +517,9 @@ def swiglu_bf16(gate: torch.Tensor, up: torch.Tensor, h: torch.Tensor, stream=No
 def swiglu_linear(gate: torch.Tensor, up: torch.Tensor, block: int, wcodes, wscales, N: int, y: torch.Tensor,
                   workspace: torch.Tensor, signs: torch.Tensor = None, stream=None) -> None:
     """linear(_rs) on h = silu(gate) * up with the producer fused into rotate+quantize."""
+    code = _call.swiglu_linear(gate, up, block, wcodes, wscales, N, y, workspace, signs, stream)
+    if code >= 0:
+        return _check(code, "bro_swiglu_linear")
     assert gate.dtype == up.dtype == y.dtype == torch.bfloat16 and gate.shape == up.shape
     M, K = gate.shape
     _check(lib.bro_swiglu_linear(_ptr(gate), _ptr(up), M, K, _ld(gate, K), _ld(up, K), block, _ptr(signs), _ptr(wcodes),

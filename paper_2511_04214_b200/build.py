@@ -1,18 +1,22 @@
-"""Build libbro.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Build libbro.so in-tree with nvcc for sm_100a (cross-compiles without a GPU) and the binding's call module with g++."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 SO = os.path.join(HERE, "libbro.so")
 SOURCES = [os.path.join(CSRC, "bro.cu")]
+CALL_SO = os.path.join(HERE, "_call.so")
+CALL_SOURCE = os.path.join(CSRC, "call.cpp")
+HEADER = os.path.join(HERE, "..", "include", "bro.h")
 
 
 def _deps():
-    out = [os.path.join(HERE, "..", "include", "bro.h")]
+    out = [HEADER]
     for name in os.listdir(CSRC):
         if name.endswith((".cu", ".cuh", ".h")):
             out.append(os.path.join(CSRC, name))
@@ -30,11 +34,33 @@ def nvcc_command(verbose: bool = False):
     return cmd
 
 
+def call_command():
+    """The call module reads torch's tensors in place, so it is compiled against the torch that will load it."""
+    import torch
+    from torch.utils import cpp_extension
+    root = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    include = cpp_extension.include_paths() + [sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    return (["g++", "-std=c++17", "-O2", "-fPIC", "-shared", "-fvisibility=hidden", "-w",
+             f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+            + [f"-I{p}" for p in include] + ["-o", CALL_SO, CALL_SOURCE, "-L" + os.path.join(root, "lib")]
+            + ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
+
+
+def _stale(so, deps):
+    return not os.path.exists(so) or os.path.getmtime(so) < max(os.path.getmtime(p) for p in deps)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    newest = max(os.path.getmtime(p) for p in _deps())
-    if not force and os.path.exists(SO) and os.path.getmtime(SO) >= newest:
-        return SO
-    subprocess.run(nvcc_command(verbose), check=True)
+    call = None
+    if force or _stale(CALL_SO, [HEADER, CALL_SOURCE]):
+        call = subprocess.Popen(call_command())
+    try:
+        if force or _stale(SO, _deps()):
+            subprocess.run(nvcc_command(verbose), check=True)
+    finally:
+        if call is not None and call.wait() != 0:
+            raise subprocess.CalledProcessError(call.returncode, call.args)
     return SO
 
 
