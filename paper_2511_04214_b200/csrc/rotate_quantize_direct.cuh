@@ -38,7 +38,8 @@ struct Params {
   int rows_padded;              // rows the task grid covers (a multiple of 128 for the tensor-core layout)
   int groups_padded;            // groups per row it covers (scale padding included)
   int chunks_per_row;           // ceil(groups_padded / 32)
-  int total_tasks;              // rows_padded * chunks_per_row; one task = one warp, 32 groups of a row
+  int total_tasks;              // rows_padded (spread: M) * chunks_per_row; one task = one warp, 32 groups of a row
+  int spread;                   // see first_task
   const uint16_t* up;           // the gated kernel: the second operand of h = silu(x) * up, [M, K] with row stride ldu
   int64_t ldu;
   float* mse;                   // STATS kernels: [M, K/32] per-group quantisation error instead of codes/scales
@@ -161,6 +162,22 @@ __device__ __forceinline__ uint4 swiglu_bf16x8_table(uint4 g, uint4 u, uint32_t 
   return make_uint4(h[0], h[1], h[2], h[3]);
 }
 
+// A warp's first task.  Neighbouring tasks go to one CTA, 16 KiB of x in a row, which the memory likes: dealt out one to each CTA,
+// [16384, 4096] takes 29.8 us, not 28.9.  But where at least half of the rows only pad the tiled scales to 128 (up to 64 rows), the
+// real ones are then all in the first few CTAs; `spread` deals them out, and the padding is not quantised but cleared: [1, 14336]
+// 3.0 -> 2.4 us, [16, 4096] 2.4 -> 2.1, block 128 3.5 -> 2.5 and 2.7 -> 2.4; gated [1, 14336] 4.8 -> 4.2, [16, 4096] 3.5 -> 3.2.
+__device__ __forceinline__ int first_task(const Params& p, int warp) {
+  return p.spread ? warp * (int)gridDim.x + (int)blockIdx.x : (int)blockIdx.x * kWarps + warp;
+}
+
+// `spread` (one block of 128 rows): zero scales for the rows that pad, whole lines of the tiled layout by each warp
+__device__ __forceinline__ void clear_padding(const Params& p) {
+  for (int64_t i = blockIdx.x * kThreads + threadIdx.x; i < (p.scale_kblocks << 7); i += gridDim.x * kThreads) {
+    const int slot = (int)(i & 127), row = ((slot & 3) << 5) | (slot >> 2);
+    if (row >= p.M) reinterpret_cast<uint32_t*>(p.scales)[i] = 0u;
+  }
+}
+
 // Rotate and quantise the 32 groups of one task, a lane's 64 bytes in cur (odd lanes of blocks of 64 / 128: halves
 // exchanged, see kSplit), and store codes and scale bytes (STATS: the statistic).
 template <int LOG2B, bool STATS>
@@ -168,10 +185,10 @@ __device__ __forceinline__ void finish_task(const Params& p, const uint4 (&cur)[
   constexpr bool kSplit = LOG2B >= 6 && !STATS;
   constexpr uint32_t cbits = rq::norm_bits<LOG2B>();
   const int ng = (int)(p.K >> 5);
+  const int g = chunk * 32 + lane;
   uint64_t P[16];
 #pragma unroll
   for (int j = 0; j < 4; ++j) rq::unpack_stage1(cur[j], P + 4 * j);
-  const int g = chunk * 32 + lane;
   const bool live = row < p.M && g < ng;
   if constexpr (kSplit) {
     rq::fwht32_stages_2_to_8(P);
@@ -264,7 +281,7 @@ rotate_quantize_direct_kernel(const Params p) {
   griddep_launch_dependents();
 
   // task -> (row, chunk); advanced incrementally (no division in the loop)
-  int task = (int)blockIdx.x * kWarps + (int)(threadIdx.x >> 5);
+  int task = first_task(p, (int)(threadIdx.x >> 5));
   int row = task / p.chunks_per_row, chunk = task - row * p.chunks_per_row;
   const int step_row = num_warps / p.chunks_per_row, step_chunk = num_warps - step_row * p.chunks_per_row;
 
@@ -291,6 +308,7 @@ rotate_quantize_direct_kernel(const Params p) {
 
   uint4 cur[4], nxt[4];
   if (task < p.total_tasks) load(row, chunk, cur);
+  if (!STATS && p.spread) clear_padding(p);       // (while the loads are on their way)
   while (task < p.total_tasks) {
     // the next task of this warp: issue its loads now, use them in the next iteration
     const int ntask = task + num_warps;
@@ -353,9 +371,10 @@ rotate_quantize_gated_kernel(const __grid_constant__ CUtensorMap tmx, const __gr
   __syncthreads();
   griddep_wait();               // x may be written, codes/scales still read, by the kernel before
   griddep_launch_dependents();  // (only now: see the direct form)
+  if (p.spread) clear_padding(p);
 
   const int num_warps = (int)gridDim.x * kWarps;
-  int task = (int)blockIdx.x * kWarps + warp;
+  int task = first_task(p, warp);
   int row = task / p.chunks_per_row, chunk = task - row * p.chunks_per_row;
   const int step_row = num_warps / p.chunks_per_row, step_chunk = num_warps - step_row * p.chunks_per_row;
   auto advance = [&](int& t, int& r, int& c) {
@@ -435,7 +454,7 @@ inline bro_status launch_one(Params& p, int sm_count, cudaStream_t st) {
                : BRO_ERR_CUDA;
   });
   if (rc != BRO_OK) return rc;
-  const int64_t want = ((int64_t)p.total_tasks + kWarps - 1) / kWarps;
+  const int64_t want = ((int64_t)p.rows_padded * p.chunks_per_row + kWarps - 1) / kWarps;
   const int64_t cap = (int64_t)sm_count * blocks_per_sm;
   const unsigned grid = (unsigned)(want < cap ? want : cap);
   return cuda_ok(launch_kernel(kernel, grid, kThreads, 0, st, 1, p), "rotate_quantize_direct launch") ? BRO_OK
@@ -462,7 +481,7 @@ inline bro_status launch_gated(Params& p, int sm_count, cudaStream_t st) {
   if (rc != BRO_OK) return rc;
   rc = make_group_map(&tmu, p.up, p.M, p.K, p.ldu);
   if (rc != BRO_OK) return rc;
-  const int64_t want = ((int64_t)p.total_tasks + kWarps - 1) / kWarps, cap = (int64_t)sm_count * blocks_per_sm;
+  const int64_t want = ((int64_t)p.rows_padded * p.chunks_per_row + kWarps - 1) / kWarps, cap = (int64_t)sm_count * blocks_per_sm;
   return cuda_ok(launch_kernel(kernel, (unsigned)(want < cap ? want : cap), kThreads, R::kSmemBytes, st, 1, tmx, tmu, p),
                  "rotate_quantize_gated launch")
              ? BRO_OK
@@ -515,7 +534,8 @@ inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, int l
   p.rows_padded = (int)(layout == BRO_LAYOUT_GEMM ? (M + 127) / 128 * 128 : M);
   p.groups_padded = (int)(layout == BRO_LAYOUT_GEMM ? scale_kblocks * 4 : K / 32);
   p.chunks_per_row = (p.groups_padded + 31) / 32;
-  p.total_tasks = p.rows_padded * p.chunks_per_row;
+  p.spread = p.rows_padded >= 2 * M ? 1 : 0;
+  p.total_tasks = (p.spread ? (int)M : p.rows_padded) * p.chunks_per_row;
   return up ? launch_any<false, true>(p, log2b, sm_count, st) : launch_any<false>(p, log2b, sm_count, st);
 }
 
@@ -539,6 +559,7 @@ inline bro_status launch_stats(const void* x, int64_t M, int64_t K, int64_t ldx,
   p.groups_padded = (int)(K / 32);
   p.chunks_per_row = (p.groups_padded + 31) / 32;
   p.total_tasks = p.rows_padded * p.chunks_per_row;
+  p.spread = 0;
   return launch_any<true>(p, log2b, sm_count, st);
 }
 
