@@ -116,7 +116,7 @@ __device__ __forceinline__ void unpack_to(uint64_t v, float* a, float* b) {
 // magnitudes, 2^-25 up to below 128, for both signs.  Below 2^-25 the sigmoid above is exactly 1/2, from 128 on exactly
 // 1 or 0 (an infinity included; a NaN gate stays NaN in the product), as in the first and the last entries: the index
 // clamps.  The arithmetic bounded the kernel, a gather of one word a value (about 3 bank conflicts deep) is a third of it.
-// Fused kernel, block 32, [16384, 4096]: IEEE division 121.8 us, sigmoid2 for every value 96.3 us, table 63.5 us;
+// Fused kernel, block 32, [16384, 4096]: IEEE division 121.8 us, sigmoid2 for every value 96.3 us, table 63.5 us (before the ring);
 // [16, 14336]: 5.6, 4.5 and 4.3 us.
 constexpr uint32_t kSigmoidLow = (127 - 25) << 7, kSigmoidEntries = 32 << 7;       // per sign
 __device__ __forceinline__ void fill_sigmoid_table(float* table, int thread, int threads) {
@@ -144,15 +144,23 @@ __device__ __forceinline__ float lds_f32(uint32_t addr) {
   asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
   return v;
 }
+// Two gates of one word less the table's low end: a half within the table has its bits 14..12 clear, one outside does not
+// (less than the low end wraps: 0xCD00 and up, with the sign 0x4D00 and up; a borrow goes with a wrap below it).
+__device__ __forceinline__ uint32_t sigmoid_offsets(uint32_t gates) { return gates - kSigmoidLow * 0x10001u; }
+constexpr uint32_t kSigmoidOutside = 0x70007000u;
+// A task whose gates all lie inside (2^-25 up to 128: all but the odd one, unless they are exact zeros) needs no clamps.  A table of
+// silu(g) would save the products too, but then a gate outside costs 40 % and not 5 %: [4096, 14336] 44.7 : 68.5 us.
+// INSIDE: every gate lies within the table (or the value has no use: the reads stay inside it all the same).
+template <bool INSIDE>
 __device__ __forceinline__ uint4 swiglu_bf16x8_table(uint4 g, uint4 u, uint32_t table) {
   const uint32_t gw[4] = {g.x, g.y, g.z, g.w}, uw[4] = {u.x, u.y, u.z, u.w};
   constexpr uint32_t low = kSigmoidLow * 0x10001u, high = (kSigmoidLow + kSigmoidEntries - 1u) * 0x10001u;
   uint32_t h[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const uint32_t mag = __vminu2(__vmaxu2(gw[k] & 0x7FFF7FFFu, low), high) - low;
+    const uint32_t mag = INSIDE ? sigmoid_offsets(gw[k]) & 0x0FFF0FFFu : __vminu2(__vmaxu2(gw[k] & 0x7FFF7FFFu, low), high) - low;
     const uint32_t at = mag | ((gw[k] >> 3) & 0x10001000u);          // entry 4096 and up: negative gates
-    const float s0 = lds_f32(table + ((at << 2) & 0x7FFCu)), s1 = lds_f32(table + ((at >> 14) & 0x7FFCu));
+    const float s0 = lds_f32(table + ((at << 2) & 0x7FFCu)), s1 = lds_f32(table + (at >> 14));
     const uint64_t gg = rq::pack2(__uint_as_float(gw[k] << 16), __uint_as_float(gw[k] & 0xFFFF0000u));
     const uint64_t up = rq::pack2(__uint_as_float(uw[k] << 16), __uint_as_float(uw[k] & 0xFFFF0000u));
     float lo, hi;
@@ -329,11 +337,15 @@ rotate_quantize_direct_kernel(const Params p) {
 // The same tasks on h = silu(gate) * up (see sigmoid2).  A warp's 2 x 2 KiB arrive by TMA in a ring of its own in shared memory
 // (one box of 32 groups of a row each, 64-byte swizzle, a barrier per stage, nothing shared with other warps).  What bounds this
 // kernel is the L1 data path, the table's gathers above all: a warp-wide 16-byte global load whose lanes are 64 bytes apart
-// takes 16 passes of it, eight of them a task, the same read of the swizzled ring 4.  [16384, 4096], block 32: loads into
+// takes 16 passes of it, eight of them a task, the same read of the swizzled ring 4; then issue.  [16384, 4096], block 32: loads into
 // registers 63.5 us, ring 54.5; [512, 8192] 6.8 -> 6.2.  (Without a producer the ring is slower, 28 -> 34 us: the plain
 // kernel is bound by issue, and requesting and waiting cost a quarter of its instructions.  128-byte segments: no difference.)
+// With one stage three CTAs fit an SM, 24 warps instead of 16 to hide the chain of a task, and the next boxes still land while the
+// warp rotates; with the short form of the table (only here: twice the code costs small calls 0.3 us) [4096, 14336] 49.3 -> 45.3 us,
+// block 128 57.2 -> 54.5.  (One CTA of 24 warps with two stages: block 32 57 us.)
+template <int STAGES>
 struct Ring {
-  static constexpr int kStages = 2;
+  static constexpr int kStages = STAGES;
   static constexpr int kBoxBytes = 2048;
   static constexpr int kStageBytes = 2 * kBoxBytes;                        // gate and up
   static constexpr int kTableAt = kWarps * kStages * kStageBytes;
@@ -350,10 +362,10 @@ __device__ __forceinline__ void tma_load_3d_elect(uint32_t dst, const CUtensorMa
       : "memory");
 }
 
-template <int LOG2B, bool SIGNS>
-__global__ void __launch_bounds__(kThreads, 2)
+template <int LOG2B, bool SIGNS, int STAGES>
+__global__ void __launch_bounds__(kThreads, 4 - STAGES)
 rotate_quantize_gated_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmu, const Params p) {
-  using R = Ring;
+  using R = Ring<STAGES>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int lane = threadIdx.x & 31, warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);
@@ -407,10 +419,23 @@ rotate_quantize_gated_kernel(const __grid_constant__ CUtensorMap tmx, const __gr
     if (loads(row, chunk)) {
       if (!mbar_wait_warp(bars + 8 * stage, phase, SITE_RQ_FULL)) break;
       const uint32_t src = ring + (uint32_t)(stage * R::kStageBytes) + (uint32_t)lane * 64u;
+      auto at = [&](uint32_t j) { return src + (((j ^ hswz) ^ swz) << 4); };
+      bool inside = false;
+      if constexpr (STAGES == 1) {
+        uint32_t outside = 0u;
 #pragma unroll
-      for (uint32_t j = 0; j < 4; ++j) {                                  // (zeros beyond K: silu(0) * 0 = 0)
-        const uint32_t at = src + (((j ^ hswz) ^ swz) << 4);
-        cur[j] = swiglu_bf16x8_table(lds128(at), lds128(at + R::kBoxBytes), table);
+        for (uint32_t j = 0; j < 4; ++j) {
+          cur[j] = lds128(at(j));
+          outside |= sigmoid_offsets(cur[j].x) | sigmoid_offsets(cur[j].y) | sigmoid_offsets(cur[j].z) | sigmoid_offsets(cur[j].w);
+        }
+        inside = __all_sync(0xFFFFFFFFu, (outside & kSigmoidOutside) == 0u || chunk * 32 + lane >= ng);
+      }
+      if (inside) {                                                       // (beyond K: a finite entry * 0 * 0 = 0)
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) cur[j] = swiglu_bf16x8_table<true>(cur[j], lds128(at(j) + R::kBoxBytes), table);
+      } else {
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) cur[j] = swiglu_bf16x8_table<false>(lds128(at(j)), lds128(at(j) + R::kBoxBytes), table);
       }
       __syncwarp();
       in_flight += request(stage) ? 0 : -1;
@@ -461,10 +486,10 @@ inline bro_status launch_one(Params& p, int sm_count, cudaStream_t st) {
                                                                                                        : BRO_ERR_CUDA;
 }
 
-template <int LOG2B, bool SIGNS>
+template <int LOG2B, bool SIGNS, int STAGES>
 inline bro_status launch_gated(Params& p, int sm_count, cudaStream_t st) {
-  using R = Ring;
-  auto kernel = rotate_quantize_gated_kernel<LOG2B, SIGNS>;
+  using R = Ring<STAGES>;
+  auto kernel = rotate_quantize_gated_kernel<LOG2B, SIGNS, STAGES>;
   static DeviceOnce once;            // (one per template instantiation)
   int blocks_per_sm = 1;
   bro_status rc = device_once(once, &blocks_per_sm, [&](int* n) {
@@ -490,7 +515,13 @@ inline bro_status launch_gated(Params& p, int sm_count, cudaStream_t st) {
 
 template <bool SIGNS, bool STATS, bool GATED, int LOG2B>
 inline bro_status launch_of(Params& p, int sm_count, cudaStream_t st) {
-  if constexpr (GATED) return launch_gated<LOG2B, SIGNS>(p, sm_count, st);
+  if constexpr (GATED) {
+    // A ring of two stages a warp and two CTAs an SM, or one stage and three (see Ring).  Up to 2^24 elements the two stages are faster:
+    // [512, 8192] 7.1 : 8.4 us, [2048, 4096] 10.4 : 10.9, [2048, 8192] 16.5 : 16.2 (gates outside the table: 16.4 : 17.0),
+    // [1544, 11008] 17.7 : 17.2, [4096, 14336] 47.8 : 45.3, block 128 56.0 : 54.5.
+    return p.M * p.K <= (int64_t)1 << 24 ? launch_gated<LOG2B, SIGNS, 2>(p, sm_count, st)
+                                         : launch_gated<LOG2B, SIGNS, 1>(p, sm_count, st);
+  }
   else return launch_one<LOG2B, SIGNS, STATS>(p, sm_count, st);
 }
 template <bool SIGNS, bool STATS, bool GATED>

@@ -149,3 +149,29 @@ def test_fused_with_row_strides_of_any_multiple_of_8(bro, block, M, K):
     codes.check(); scales.check()
     assert np.array_equal(to_canonical(scales.numpy(), M, K), rs)
     assert np.array_equal(codes.numpy().reshape(M, K // 2), rc)
+
+
+@pytest.mark.parametrize("M,K,block", [(4099, 4128, 32), (4099, 4224, 128), (131, 131072, 64)])
+def test_fused_table_without_clamps_at_large_sizes(bro, M, K, block):
+    """More than 2^24 elements: tasks whose gates all lie within the table take it unclamped, the others do not.  Rows of
+    in-range gates, rows of every pattern and rows of zeros in turn, K ragged in the last task of a row: codes and scales of the
+    two-step path."""
+    gen = torch.Generator(device="cuda").manual_seed(M + K)
+    pats = torch.arange(-32768, 32768, dtype=torch.int32, device="cuda").to(torch.int16).view(torch.bfloat16)
+    g = torch.randn(M, K, device="cuda", generator=gen).to(torch.bfloat16)
+    every = torch.arange(M, device="cuda") % 3 == 1
+    g[every] = pats.repeat(-(-int(every.sum()) * K // 65536))[:int(every.sum()) * K].view(-1, K)
+    g[5::7] = 0.0
+    u = torch.randn(M, K, device="cuda", generator=gen).to(torch.bfloat16)
+    h = torch.empty_like(g)
+    bro.swiglu_bf16(g, u, h)
+    out = []
+    for fused in (True, False):
+        c, s = bro.alloc_codes(M, K), bro.alloc_scales(M, K, bro.LAYOUT_GEMM)
+        if fused:
+            bro.swiglu_rotate_quantize_mxfp4(g, u, block, c, s, bro.LAYOUT_GEMM)
+        else:
+            bro.rotate_quantize_mxfp4(h, block, c, s, bro.LAYOUT_GEMM)
+        out.append((c, s))
+    assert bro.last_device_status() == 0
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
