@@ -8,9 +8,9 @@
 // What differs is how the bytes travel.  The 32 lanes of a warp take 32 consecutive groups of one
 // row (2 KiB of contiguous bf16), each lane loading its 64 bytes with four 16-byte loads straight
 // into registers, and the loads of the warp's NEXT task are issued before the current one is
-// computed.  Nothing goes through shared memory: in the TMA-ring form the shared-memory port carries
-// every byte twice (TMA write, then the consumers' loads) and all consumer warps wake on the same
-// barrier, which together cost about a third of its run time on a [16384, 4096] tensor; here more
+// computed.  Nothing goes through shared memory: in a CTA-wide TMA ring the shared-memory port carried
+// every byte twice (TMA write, then the consumers' loads) and all consumer warps woke on the same
+// barrier, which together cost about a third of the run time on a [16384, 4096] tensor; here more
 // warps are resident and they drift apart, so loads, arithmetic and stores of different warps
 // overlap.  Blocks of 64 / 128 channels pair lanes l ^ 1 (and l ^ 2) for their last one / two stages,
 // each lane exchanging half of its values (rq::cross_lane_split); the per-group error kernels keep the
@@ -458,7 +458,7 @@ rotate_quantize_gated_kernel(const __grid_constant__ CUtensorMap tmx, const __gr
   }
 }
 
-// Rows x padded groups must fit 31 bits of task index; larger problems use the TMA-ring kernel.
+// Rows x padded groups must fit 31 bits of task index; larger problems use the wide kernel.
 inline bool supports(int64_t M, int64_t K, bro_layout layout, int64_t scale_kblocks) {
   const int64_t rows = layout == BRO_LAYOUT_GEMM ? (M + 127) / 128 * 128 : M;
   const int64_t groups = layout == BRO_LAYOUT_GEMM ? scale_kblocks * 4 : K / 32;
