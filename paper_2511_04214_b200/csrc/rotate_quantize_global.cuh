@@ -191,13 +191,16 @@ __device__ __forceinline__ void sts_pairs(uint32_t addr, uint64_t a, uint64_t b)
   asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(addr), "l"(a), "l"(b) : "memory");
 }
 
-// All threads of a unit; the result is true if it was true in each of them.
+// All threads of a unit; the result is true if it was true in each of them.  (The barriers are .aligned: every thread of a warp has to
+// be there, and behind a wait, or the request of one thread, nothing promises that the warp is whole again.)
 template <int T>
 __device__ __forceinline__ bool unit_sync_and(int unit, bool ok) {
+  __syncwarp();
   return gemm::named_barrier_and(unit + 1, T, ok);
 }
 template <int T>
 __device__ __forceinline__ void unit_sync(int unit) {
+  __syncwarp();
   gemm::named_barrier_sync(unit + 1, T);
 }
 
