@@ -250,9 +250,13 @@ bro_status launch_rotate_quantize(const void* x, int64_t M, int64_t K, int64_t l
   const bool can_wide = wide_takes(B, K) && !up;
   bool wide = can_wide && (B == 32 ? elements >= (int64_t)1 << (layer ? 24 : 20) && elements <= (int64_t)1 << 25
                                    : elements > (int64_t)1 << (layer ? 22 : 19));
-  const bool can_direct = bro::rqd::supports(M, K, layout, gemm_scale_kblocks(K));
-  if (flags & BRO_FLAG_RQ_TMA_RING) wide = can_wide;
-  else if (flags & BRO_FLAG_RQ_DIRECT) wide = can_wide && !can_direct;
+  // From 2^30 rows the register-streaming kernel's tasks number as many as it can count: the wide kernel then takes what it can, and
+  // a plain block of 32 over rows of 32 channels, the only other call of that length, is counted to the last task.
+  const int64_t tasks = bro::rqd::tasks(M, K, layout, gemm_scale_kblocks(K));
+  const bool can_direct = tasks < bro::rqd::kMaxTasks || (tasks == bro::rqd::kMaxTasks && B == 32 && !up);
+  if (tasks >= bro::rqd::kMaxTasks) wide = can_wide;
+  else if (flags & BRO_FLAG_RQ_TMA_RING) wide = can_wide;
+  else if (flags & BRO_FLAG_RQ_DIRECT) wide = false;
   if (wide)
     return bro::rqw::launch(x, M, K, ldx, log2_of(B), signs, codes, scales, nullptr, layout, gemm_scale_kblocks(K), di.sm_count, st);
   if (!can_direct) return BRO_ERR_UNSUPPORTED;

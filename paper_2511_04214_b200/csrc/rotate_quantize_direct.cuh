@@ -458,11 +458,15 @@ rotate_quantize_gated_kernel(const __grid_constant__ CUtensorMap tmx, const __gr
   }
 }
 
-// Rows x padded groups must fit 31 bits of task index; larger problems use the wide kernel.
-inline bool supports(int64_t M, int64_t K, bro_layout layout, int64_t scale_kblocks) {
+// Tasks of a call.  Their index is an int that runs on by up to a grid's warps, so 2^30 tasks fit it.
+constexpr int64_t kMaxTasks = (int64_t)1 << 30;
+inline int64_t tasks(int64_t M, int64_t K, bro_layout layout, int64_t scale_kblocks) {
   const int64_t rows = layout == BRO_LAYOUT_GEMM ? (M + 127) / 128 * 128 : M;
   const int64_t groups = layout == BRO_LAYOUT_GEMM ? scale_kblocks * 4 : K / 32;
-  return rows * ((groups + 31) / 32) < ((int64_t)1 << 30);
+  return rows * ((groups + 31) / 32);
+}
+inline bool supports(int64_t M, int64_t K, bro_layout layout, int64_t scale_kblocks) {
+  return tasks(M, K, layout, scale_kblocks) < kMaxTasks;
 }
 
 // x as a 3-D tensor {32 bf16 (one group), K / 32 groups, M rows}, box = 32 groups of a row, 64-byte swizzle.

@@ -85,3 +85,35 @@ def test_gemm_output_beyond_8_gib(bro, kernel):
     yv = y.view(reps, PERIOD, N)
     for r in range(1, reps):
         assert torch.equal(yv[r], yv[0]), f"rows of repeat {r} differ from the first period"
+
+
+@pytest.mark.parametrize("K,layout", [(32, 0), (32, 1), (64, 0)])
+def test_the_most_rows_that_a_call_takes(bro, K, layout):
+    """2^30 rows of one or two groups: as many tasks as the register-streaming kernel counts.  Rows repeat as above."""
+    M = 1 << 30
+    torch.cuda.empty_cache()
+    if free_bytes() < M * (2 * K + K // 2) + bro.scales_bytes(M, K, layout) + (4 << 30):
+        pytest.skip("needs most of the device's memory")
+    tile = synth.activations(PERIOD, K, seed=34)
+    rc, rs = oracle.rotate_quantize_mxfp4(synth.bf16_bits(tile), 32)
+    td = tile.cuda()
+    x = torch.empty(M, K, dtype=torch.bfloat16, device="cuda")
+    reps, rest = divmod(M, PERIOD)
+    x[:reps * PERIOD].view(reps, PERIOD, K).copy_(td.expand(reps, PERIOD, K))
+    x[reps * PERIOD:].copy_(td[:rest])
+    codes, scales = bro.alloc_codes(M, K), bro.alloc_scales(M, K, layout)
+    bro.rotate_quantize_mxfp4(x, 32, codes, scales, layout)
+    assert bro.last_device_status() == 0
+    # row r of every block of 128 of the tiled layout stands at its word (r % 32) * 4 + r / 32, the groups of the row in its bytes
+    if layout == 1:
+        words = torch.arange(128, device="cuda")
+        scales = scales.view(M // 128, -1, 128, 4)[:, 0]
+        scales = scales[:, (words % 32) * 4 + words // 32].reshape(M, 4)[:, :K // 32]
+    exp_c, exp_s = torch.from_numpy(rc).cuda(), torch.from_numpy(rs).cuda()
+    c, s = codes.view(M, K // 2), scales.reshape(M, K // 32)
+    for first in range(0, reps, 8192):
+        n = min(8192, reps - first)
+        a, b = first * PERIOD, (first + n) * PERIOD
+        assert torch.equal(c[a:b].view(n, PERIOD, K // 2), exp_c.expand(n, PERIOD, K // 2)), first
+        assert torch.equal(s[a:b].view(n, PERIOD, K // 32), exp_s.expand(n, PERIOD, K // 32)), first
+    assert torch.equal(c[reps * PERIOD:], exp_c[:rest]) and torch.equal(s[reps * PERIOD:], exp_s[:rest])
