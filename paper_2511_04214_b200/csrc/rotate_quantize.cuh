@@ -19,6 +19,17 @@
 namespace bro {
 namespace rq {
 
+// Zero tiled scales for the rows that pad the last block of 128, by all threads of a grid; whole lines by each warp.
+__device__ __forceinline__ void clear_padding(void* scales, int64_t M, int64_t kblocks, int64_t thread, int64_t threads) {
+  const int rest = (int)(M & 127);
+  if (rest == 0) return;
+  uint32_t* block = reinterpret_cast<uint32_t*>(scales) + (M >> 7) * kblocks * 128;
+  for (int64_t i = thread; i < kblocks * 128; i += threads) {
+    const int slot = (int)(i & 127), row = ((slot & 3) << 5) | (slot >> 2);
+    if (row >= rest) block[i] = 0u;
+  }
+}
+
 // x diag(s): flip the bf16 sign bits of a 16-byte chunk of x where the sign vector is negative.
 // One three-input logic operation per 32-bit word (x ^ (s & 0x80008000)); exact.
 __device__ __forceinline__ uint4 apply_signs(uint4 q, uint4 sg) {

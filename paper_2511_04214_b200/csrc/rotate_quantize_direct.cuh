@@ -38,8 +38,8 @@ struct Params {
   int rows_padded;              // rows the task grid covers (a multiple of 128 for the tensor-core layout)
   int groups_padded;            // groups per row it covers (scale padding included)
   int chunks_per_row;           // ceil(groups_padded / 32)
+  int spread;                   // most rows only pad: see first_task
   int total_tasks;              // rows_padded (spread: M) * chunks_per_row; one task = one warp, 32 groups of a row
-  int spread;                   // see first_task
   const uint16_t* up;           // the gated kernel: the second operand of h = silu(x) * up, [M, K] with row stride ldu
   int64_t ldu;
   float* mse;                   // STATS kernels: [M, K/32] per-group quantisation error instead of codes/scales
@@ -174,16 +174,14 @@ __device__ __forceinline__ uint4 swiglu_bf16x8_table(uint4 g, uint4 u, uint32_t 
 // [16384, 4096] takes 29.8 us, not 28.9.  But where at least half of the rows only pad the tiled scales to 128 (up to 64 rows), the
 // real ones are then all in the first few CTAs; `spread` deals them out, and the padding is not quantised but cleared: [1, 14336]
 // 3.0 -> 2.4 us, [16, 4096] 2.4 -> 2.1, block 128 3.5 -> 2.5 and 2.7 -> 2.4; gated [1, 14336] 4.8 -> 4.2, [16, 4096] 3.5 -> 3.2.
-__device__ __forceinline__ int first_task(const Params& p, int warp) {
-  return p.spread ? warp * (int)gridDim.x + (int)blockIdx.x : (int)blockIdx.x * kWarps + warp;
+// (Without a producer in a kernel of its own: chosen at run time it cost the kernel for everything else, which stands at its 80
+// registers, up to 16 bytes of spills.)
+__device__ __forceinline__ int first_task(bool spread, int warp) {
+  return spread ? warp * (int)gridDim.x + (int)blockIdx.x : (int)blockIdx.x * kWarps + warp;
 }
 
-// `spread` (one block of 128 rows): zero scales for the rows that pad, whole lines of the tiled layout by each warp
 __device__ __forceinline__ void clear_padding(const Params& p) {
-  for (int64_t i = blockIdx.x * kThreads + threadIdx.x; i < (p.scale_kblocks << 7); i += gridDim.x * kThreads) {
-    const int slot = (int)(i & 127), row = ((slot & 3) << 5) | (slot >> 2);
-    if (row >= p.M) reinterpret_cast<uint32_t*>(p.scales)[i] = 0u;
-  }
+  rq::clear_padding(p.scales, p.M, p.scale_kblocks, blockIdx.x * kThreads + threadIdx.x, gridDim.x * kThreads);
 }
 
 // Rotate and quantise the 32 groups of one task, a lane's 64 bytes in cur (odd lanes of blocks of 64 / 128: halves
@@ -277,7 +275,7 @@ __device__ __forceinline__ void finish_task(const Params& p, const uint4 (&cur)[
 
 // STATS: nothing is quantised to memory; the kernel writes the per-group quantisation error
 // (rq::group_error) — the analysis behind the paper's regular-block / outlier-block comparison.
-template <int LOG2B, bool SIGNS, bool STATS>
+template <int LOG2B, bool SIGNS, bool STATS, bool SPREAD>
 __global__ void __launch_bounds__(kThreads, 3)
 rotate_quantize_direct_kernel(const Params p) {
   const int lane = threadIdx.x & 31;
@@ -289,7 +287,7 @@ rotate_quantize_direct_kernel(const Params p) {
   griddep_launch_dependents();
 
   // task -> (row, chunk); advanced incrementally (no division in the loop)
-  int task = first_task(p, (int)(threadIdx.x >> 5));
+  int task = first_task(SPREAD, (int)(threadIdx.x >> 5));
   int row = task / p.chunks_per_row, chunk = task - row * p.chunks_per_row;
   const int step_row = num_warps / p.chunks_per_row, step_chunk = num_warps - step_row * p.chunks_per_row;
 
@@ -316,7 +314,7 @@ rotate_quantize_direct_kernel(const Params p) {
 
   uint4 cur[4], nxt[4];
   if (task < p.total_tasks) load(row, chunk, cur);
-  if (!STATS && p.spread) clear_padding(p);       // (while the loads are on their way)
+  if (SPREAD) clear_padding(p);                   // (while the loads are on their way)
   while (task < p.total_tasks) {
     // the next task of this warp: issue its loads now, use them in the next iteration
     const int ntask = task + num_warps;
@@ -386,7 +384,7 @@ rotate_quantize_gated_kernel(const __grid_constant__ CUtensorMap tmx, const __gr
   if (p.spread) clear_padding(p);
 
   const int num_warps = (int)gridDim.x * kWarps;
-  int task = first_task(p, warp);
+  int task = first_task(p.spread != 0, warp);
   int row = task / p.chunks_per_row, chunk = task - row * p.chunks_per_row;
   const int step_row = num_warps / p.chunks_per_row, step_chunk = num_warps - step_row * p.chunks_per_row;
   auto advance = [&](int& t, int& r, int& c) {
@@ -472,9 +470,9 @@ inline bool supports(int64_t M, int64_t K, bro_layout layout, int64_t scale_kblo
 // x as a 3-D tensor {32 bf16 (one group), K / 32 groups, M rows}, box = 32 groups of a row, 64-byte swizzle.
 bro_status make_group_map(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx);
 
-template <int LOG2B, bool SIGNS, bool STATS>
+template <int LOG2B, bool SIGNS, bool STATS, bool SPREAD>
 inline bro_status launch_one(Params& p, int sm_count, cudaStream_t st) {
-  auto kernel = rotate_quantize_direct_kernel<LOG2B, SIGNS, STATS>;
+  auto kernel = rotate_quantize_direct_kernel<LOG2B, SIGNS, STATS, SPREAD>;
   static DeviceOnce once;            // (one per template instantiation)
   int blocks_per_sm = 1;
   const bro_status rc = device_once(once, &blocks_per_sm, [&](int* n) {
@@ -526,7 +524,8 @@ inline bro_status launch_of(Params& p, int sm_count, cudaStream_t st) {
     return p.M * p.K <= (int64_t)1 << 24 ? launch_gated<LOG2B, SIGNS, 2>(p, sm_count, st)
                                          : launch_gated<LOG2B, SIGNS, 1>(p, sm_count, st);
   }
-  else return launch_one<LOG2B, SIGNS, STATS>(p, sm_count, st);
+  else if constexpr (STATS) return launch_one<LOG2B, SIGNS, true, false>(p, sm_count, st);
+  else return p.spread ? launch_one<LOG2B, SIGNS, false, true>(p, sm_count, st) : launch_one<LOG2B, SIGNS, false, false>(p, sm_count, st);
 }
 template <bool SIGNS, bool STATS, bool GATED>
 inline bro_status launch_size(Params& p, int log2b, int sm_count, cudaStream_t st) {
@@ -569,7 +568,8 @@ inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, int l
   p.rows_padded = (int)(layout == BRO_LAYOUT_GEMM ? (M + 127) / 128 * 128 : M);
   p.groups_padded = (int)(layout == BRO_LAYOUT_GEMM ? scale_kblocks * 4 : K / 32);
   p.chunks_per_row = (p.groups_padded + 31) / 32;
-  p.spread = p.rows_padded >= 2 * M ? 1 : 0;
+  // (with signs, which each load waits for, one or two short rows are clear sooner as padding: block 16 of [1, 1056] 1.5 : 1.6 us)
+  p.spread = p.rows_padded >= 2 * M && !(signs && !up && M <= 2 && p.chunks_per_row <= 2) ? 1 : 0;
   p.total_tasks = (p.spread ? (int)M : p.rows_padded) * p.chunks_per_row;
   return up ? launch_any<false, true>(p, log2b, sm_count, st) : launch_any<false>(p, log2b, sm_count, st);
 }

@@ -1,4 +1,6 @@
 """Helpers shared by the GPU parity tests (not a test module)."""
+import ctypes
+
 import numpy as np
 import torch
 
@@ -48,3 +50,39 @@ class Guarded:
 
 def x_from_bits(bits: np.ndarray) -> torch.Tensor:
     return synth.bits_to_bf16(bits).cuda()
+
+
+class _KernelNode(ctypes.Structure):
+    """CUDA_KERNEL_NODE_PARAMS of the driver API."""
+    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3), ("block", ctypes.c_uint * 3), ("smem", ctypes.c_uint),
+                ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p), ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+
+def kernels_of(f, attribute=None):
+    """Names (as the compiler writes them) of the kernels that f() launches, from a captured call; with the number of an attribute
+    (CUfunction_attribute), pairs of the name and its value."""
+    f()                                    # (a first launch sets the kernel up, which a capture does not take)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        f()
+    cuda, raw, n = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(0)
+    assert cuda.cuGraphGetNodes(raw, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert cuda.cuGraphGetNodes(raw, nodes, ctypes.byref(n)) == 0
+    names = []
+    for node in nodes:
+        kind, params, name = ctypes.c_int(-1), _KernelNode(), ctypes.c_char_p()
+        assert cuda.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        if kind.value != 0:                # CU_GRAPH_NODE_TYPE_KERNEL
+            continue
+        assert cuda.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(params)) == 0
+        func = ctypes.c_void_p(params.func)
+        if not params.func:
+            assert cuda.cuKernelGetFunction(ctypes.byref(func), ctypes.c_void_p(params.kern)) == 0
+        assert cuda.cuFuncGetName(ctypes.byref(name), func) == 0
+        value = ctypes.c_int(0)
+        if attribute is not None:
+            assert cuda.cuFuncGetAttribute(ctypes.byref(value), ctypes.c_int(attribute), func) == 0
+        names.append(name.value.decode() if attribute is None else (name.value.decode(), value.value))
+    return names
