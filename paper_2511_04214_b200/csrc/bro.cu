@@ -900,7 +900,8 @@ bro_status bro_linear_static(const void* x_bf16, int64_t M, int64_t K, int64_t l
   unsigned char* acodes = base;
   unsigned char* ascales = acodes + codes_sz;
   unsigned char* gws = ascales + scales_sz;
-  bro_status rc = bro_rotate_quantize_mxfp4(x_bf16, M, K, ldx, block, acodes, ascales, BRO_LAYOUT_GEMM, stream);
+  bro_status rc = launch_rotate_quantize(x_bf16, M, K, ldx, block, nullptr, acodes, ascales, BRO_LAYOUT_GEMM, 0u,
+                                         static_cast<cudaStream_t>(stream), nullptr, 0, true);
   if (rc != BRO_OK) return rc;
   // (as in bro_linear: the packed weights are older than the kernel just enqueued, so the GEMM may
   // fetch its first weight tiles before that kernel has finished)

@@ -13,6 +13,19 @@ def bro():
     return binding
 
 
+@pytest.mark.parametrize("M,K,N,block", [(2048, 2048, 1024, 32), (1000, 2048, 2048, 64), (1500, 4096, 1000, 128)])
+def test_the_layer_without_a_workspace_launches_what_the_layer_does(bro, M, K, N, block):
+    """In front of a GEMM the line between the rotate+quantise kernels lies elsewhere than alone, whoever provides the buffers."""
+    x = torch.randn(M, K, device="cuda").to(torch.bfloat16)
+    wc, ws = bro.alloc_codes(N, K), bro.alloc_scales(N, K, bro.LAYOUT_GEMM)
+    bro.pack_weights(torch.randn(N, K, device="cuda").to(torch.bfloat16), block, wc, ws)
+    work = bro.alloc_workspace(bro.linear_workspace_bytes(M, N, K))
+    y = torch.empty(M, N, dtype=torch.bfloat16, device="cuda")
+    layer = kernels_of(lambda: bro.linear(x, block, wc, ws, N, y, work))
+    assert len(layer) == 2
+    assert kernels_of(lambda: bro.linear_static(x, block, wc, ws, N, y)) == layer
+
+
 @pytest.mark.parametrize("block", [16, 32, 64, 128])
 def test_plain_blocks_stay_in_registers(bro, block):
     """The register-streaming kernel stands at the registers that three CTAs an SM leave it; what only a few tokens need is not in the
