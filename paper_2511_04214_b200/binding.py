@@ -15,6 +15,8 @@ import os
 
 import torch
 
+from .build import call_tag
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _SO = os.path.join(_HERE, "libbro.so")
 
@@ -145,13 +147,15 @@ def _load() -> ctypes.CDLL:
     return L
 
 
-def _load_call():
-    path = os.path.join(_HERE, "_call.so")
+def _load_call(path=os.path.join(_HERE, "_call.so")):
     if not os.path.exists(path):
         raise ImportError(f"{path} is missing: build it with `python -m paper_2511_04214_b200.build`")
     loader = importlib.machinery.ExtensionFileLoader("_call", path)
     module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_call", loader, origin=path))
     loader.exec_module(module)
+    if getattr(module, "TAG", None) != call_tag():
+        raise ImportError(f"{path} was built as '{getattr(module, 'TAG', None)}', this is '{call_tag()}': build it again with "
+                          "`python -m paper_2511_04214_b200.build`")
     module.bind({name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in module.NAMES})
     return module
 

@@ -34,15 +34,21 @@ def nvcc_command(verbose: bool = False):
     return cmd
 
 
+def call_tag() -> str:
+    """What the call module is good for: it reads torch's tensors in place, so only the torch, the C++ ABI and the Python that it was
+    compiled against may load it."""
+    import torch
+    return f"call module for torch {torch.__version__}, C++11 ABI {int(torch._C._GLIBCXX_USE_CXX11_ABI)}, {sysconfig.get_config_var('SOABI')}"
+
+
 def call_command():
-    """The call module reads torch's tensors in place, so it is compiled against the torch that will load it."""
     import torch
     from torch.utils import cpp_extension
     root = os.path.dirname(torch.__file__)
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     include = cpp_extension.include_paths() + [sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
     return (["g++", "-std=c++17", "-O2", "-fPIC", "-shared", "-fvisibility=hidden", "-w",
-             f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+             f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DBRO_CALL_TAG="{call_tag()}"']
             + [f"-I{p}" for p in include] + ["-o", CALL_SO, CALL_SOURCE, "-L" + os.path.join(root, "lib")]
             + ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
 
@@ -51,9 +57,16 @@ def _stale(so, deps):
     return not os.path.exists(so) or os.path.getmtime(so) < max(os.path.getmtime(p) for p in deps)
 
 
+def _call_stale():
+    if _stale(CALL_SO, [HEADER, CALL_SOURCE]):
+        return True
+    with open(CALL_SO, "rb") as f:
+        return call_tag().encode() + b"\0" not in f.read()
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     call = None
-    if force or _stale(CALL_SO, [HEADER, CALL_SOURCE]):
+    if force or _call_stale():
         call = subprocess.Popen(call_command())
     try:
         if force or _stale(SO, _deps()):

@@ -359,5 +359,6 @@ PyMODINIT_FUNC PyInit__call() {
   BRO_CALLS(BRO_NAME)
 #undef BRO_NAME
   PyModule_AddObject(m, "NAMES", names);
+  PyModule_AddStringConstant(m, "TAG", BRO_CALL_TAG);      // the torch, the ABI and the Python of the build, which the binding compares
   return m;
 }
