@@ -175,21 +175,6 @@ __device__ __forceinline__ constexpr uint32_t make_idesc() {
          ((uint32_t)(kBM >> 4) << 24);
 }
 
-
-// Barrier over `nthreads` threads that also ANDs a predicate, so that all of them take the same
-// branch afterwards (used to leave the tile loop together after a lost wait).
-__device__ __forceinline__ bool named_barrier_and(int id, int nthreads, bool pred) {
-  uint32_t out;
-  asm volatile(
-      "{ .reg .pred p, q; setp.ne.u32 q, %3, 0; bar.red.and.pred p, %1, %2, q; selp.u32 %0, 1, 0, p; }"
-      : "=r"(out)
-      : "r"(id), "r"(nthreads), "r"((uint32_t)pred)
-      : "memory");
-  return out != 0;
-}
-__device__ __forceinline__ void named_barrier_sync(int id, int nthreads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
 // TMA store shared -> global of one box; out-of-range parts of the box are clipped.
 // Forms for a converged warp.  The fp32 epilogue elects the lane per instruction, the bf16 one names it by a flag (`issue`,
 // not zero in that lane): electing made launches that the bf16 epilogue bounds slower, flag -> elected (512, 256, 28672)

@@ -145,9 +145,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rotate_quantize_global_kernel(
 //   phase 2   element bits 0, 6..10   : 32 pairs of channels 64 apart
 //   phase 3   element bits 11..       : NJ runs of 64 / NJ consecutive channels, NJ = V / 2048
 // Stage order is ascending stride with one fp32 rounding per add / subtract, so the result is that of the shuffle form
-// bit for bit.  A unit of V = max(K, 4096) elements (several rows where K < 4096, and then the stages of stride K and more
-// are left out) is worked on by V / 64 threads of their own, which meet at a named barrier; no barrier spans the CTA.
-// Between the phases the unit passes through ONE shared-memory buffer of fp32: phase 2 writes back where it read.  128-byte
+// bit for bit.  A CTA of V / 64 threads works on V = max(K, 4096) elements at a time (several rows where K < 4096, and then the stages
+// of stride K and more are left out).
+// Between the phases they pass through ONE shared-memory buffer of fp32: phase 2 writes back where it read.  128-byte
 // lines of 32 values, 16-byte piece q of line L at q ^ g(L), g(L) = (L ^ (L >> 3)) & 7; all accesses are free of bank
 // conflicts: 16 bytes a thread and threads 2 lines apart (phase 1) or one line or less apart (phase 3), 8 bytes a
 // thread and a warp on two lines (phase 2).
@@ -155,25 +155,24 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rotate_quantize_global_kernel(
 // instruction issue.  64 values a thread rather than 32: the strided side of both transposes moves 8 bytes an instruction instead of
 // 4, its five stages are all packed, and from K = 4096 down a thread ends with whole MX groups (no shuffle for their maximum).
 // [16384, 4096] codes 66.5 -> 52.7 us, scale bytes 98 -> 49, error 113 -> 55; K = 2048 60 -> 52, 1024 71 -> 51, 8192 124 -> 61, 16384 152 -> 78,
-// 32768 (one CTA an SM) 174 -> 105 us for as many elements; [300, 4096] 5.5 -> 4.1.
+// 32768 (one CTA an SM) 174 -> 105 us for as many elements; [300, 4096] 5.5 -> 4.1.  (With two such pieces a CTA, which met at barriers of
+// their own, 52.7 us where it is 52.1 now, [700, 2048] 3.3 and 3.0: the smaller CTAs fill the SMs more evenly.)
 // The bf16 rows arrive by TMA (128-byte segments, 128-byte swizzle: a thread's 64 channels are a segment), requested for the
-// unit's NEXT pass as soon as its threads have taken the current one.
+// NEXT pass as soon as all threads have taken the current one.
 enum Mode { kCodes = 0, kBytes = 1, kError = 2 };
 
 template <int LOG2V>
 struct Shape {
   static constexpr int V = 1 << LOG2V;
-  static constexpr int T = V / 64;                          // threads of a unit
-  static constexpr int kThreads = T < 128 ? 128 : T;
-  static constexpr int kUnits = kThreads / T;
+  static constexpr int T = V / 64;                          // threads of a CTA
   static constexpr int NJ = V / 2048;                       // runs of a thread in phase 3
   static constexpr int RUN = 64 / NJ;
   static constexpr int G = 32 / RUN;                        // lanes that share an MX group
   static constexpr int kRawBytes = V * 2;
   static constexpr int kBufBytes = V * 4;
-  static constexpr int kBarAt = kUnits * (kRawBytes + kBufBytes);
+  static constexpr int kBarAt = kRawBytes + kBufBytes;
   static constexpr int kSmemBytes = kBarAt + 128 + 1024 /*alignment*/;
-  static constexpr int kMinBlocks = kThreads == 128 ? 4 : (kThreads == 256 ? 2 : 1);
+  static constexpr int kMinBlocks = 512 / T;
 };
 
 __device__ __forceinline__ uint64_t lds64(uint32_t addr) {
@@ -189,19 +188,6 @@ __device__ __forceinline__ void lds_pairs(uint32_t addr, uint64_t& a, uint64_t& 
 }
 __device__ __forceinline__ void sts_pairs(uint32_t addr, uint64_t a, uint64_t b) {
   asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(addr), "l"(a), "l"(b) : "memory");
-}
-
-// All threads of a unit; the result is true if it was true in each of them.  (The barriers are .aligned: every thread of a warp has to
-// be there, and behind a wait, or the request of one thread, nothing promises that the warp is whole again.)
-template <int T>
-__device__ __forceinline__ bool unit_sync_and(int unit, bool ok) {
-  __syncwarp();
-  return gemm::named_barrier_and(unit + 1, T, ok);
-}
-template <int T>
-__device__ __forceinline__ void unit_sync(int unit) {
-  __syncwarp();
-  gemm::named_barrier_sync(unit + 1, T);
 }
 
 // Maximum of the magnitudes of a group whose values lie in G neighbouring lanes, RUN of them in E; NaN-preserving on demand.
@@ -292,27 +278,25 @@ __device__ __forceinline__ float run_error(const uint64_t* E, uint32_t cbits) {
   return __fmul_rn(__fmul_rn(__fmul_rn(sum, 0.03125f), pe), pe);
 }
 
-// K = 2^LOG2K; 0: p.log2k.  K < V: units of several rows.
+// K = 2^LOG2K; 0: p.log2k.  K < V: several rows at a time.
 template <int LOG2V, int LOG2K, int MODE>
-__global__ void __launch_bounds__(Shape<LOG2V>::kThreads, Shape<LOG2V>::kMinBlocks)
+__global__ void __launch_bounds__(Shape<LOG2V>::T, Shape<LOG2V>::kMinBlocks)
 rotate_quantize_global_wide_kernel(const __grid_constant__ CUtensorMap tmx, const Params p) {
   using S = Shape<LOG2V>;
   constexpr int V = S::V, T = S::T, NJ = S::NJ, RUN = S::RUN, G = S::G;
-  extern __shared__ uint8_t smem_raw[];      // [units: bf16 | units: fp32 | barriers], 1 KiB aligned
-  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const int unit = (int)threadIdx.x / T, t = (int)threadIdx.x % T;
-  const uint32_t raw = base + (uint32_t)(unit * S::kRawBytes), buf = base + (uint32_t)(S::kUnits * S::kRawBytes + unit * S::kBufBytes);
-  const uint32_t bar = base + (uint32_t)(S::kBarAt + 8 * unit);
+  extern __shared__ uint8_t smem_raw[];      // [bf16 | fp32 | barrier], 1 KiB aligned
+  const uint32_t raw = (smem_u32(smem_raw) + 1023u) & ~1023u, buf = raw + (uint32_t)S::kRawBytes, bar = raw + (uint32_t)S::kBarAt;
+  const int t = (int)threadIdx.x;
   constexpr bool ROWS = LOG2K != LOG2V;
   const int log2k = LOG2K == 0 ? p.log2k : LOG2K;
   const int segs = 1 << (log2k - 6);          // 128-byte segments of a row
-  const int rows = V >> log2k;                // rows of a unit
+  const int rows = V >> log2k;                // at a time
   const uint32_t cbits = (log2k % 2 == 0) ? (uint32_t)(127 - log2k / 2) << 23 : 0x3FB504F3u - ((uint32_t)((log2k + 1) / 2) << 23);
   if (t == 0) {
     mbar_init(bar, 1);
     mbar_fence_init();
     fence_proxy_async_smem();
-    if (unit == 0) tma_prefetch_desc(&tmx);
+    tma_prefetch_desc(&tmx);
   }
   __syncthreads();
   griddep_wait();               // x may be written, the outputs still read, by the kernel before
@@ -324,27 +308,35 @@ rotate_quantize_global_wide_kernel(const __grid_constant__ CUtensorMap tmx, cons
     for (int b = 0; b < V / 64 / kBoxSegs; ++b)
       tma_load_3d(raw + (uint32_t)(b * kBoxSegs * 128), &tmx, 0, b * kBoxSegs, it * rows, bar);
   };
-  const int M = (int)p.M, iters = (M + rows - 1) / rows, stride = (int)gridDim.x * S::kUnits;      // (M is at most 2^30)
-  int it = (int)blockIdx.x * S::kUnits + unit;
+  const int M = (int)p.M, iters = (M + rows - 1) / rows, stride = (int)gridDim.x;      // (M is at most 2^30)
+  int it = (int)blockIdx.x;
   if (t == 0 && it < iters) request(it);
+  if (MODE == kCodes && p.layout == BRO_LAYOUT_GEMM)
+    rq::clear_padding(p.scales, p.M, p.scale_kblocks, (int64_t)blockIdx.x * T + t, (int64_t)gridDim.x * T);
   // A thread's 64 channels are the same in every pass, so the signs are two registers: bits 31 - k and 15 - k of sg[h] are those of
-  // the two channels of word 16 h + k.
+  // the two channels of word 16 h + k.  A warp reads the signs of its 2048 channels in whole lines and deals them out as bits
+  // through its own part of the (still idle) buffer, a byte to 8 channels; every thread reading its own 128 bytes was
+  // 32 lines an instruction, and 1.8 us where the whole chip starts at once: [700, 4096] 6.9 -> 5.7 us, [64, 2048] 3.1 -> 2.6.
   uint32_t sg[2] = {0u, 0u};
   if (p.signs) {
-    const uint4* sp = reinterpret_cast<const uint4*>(p.signs) + (t & (segs - 1)) * 8;
+    const int lane = t & 31;
+    const uint32_t mine = buf + (uint32_t)(t >> 5) * 8192u;
+    uint4 q[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      q[j] = __ldg(reinterpret_cast<const uint4*>(p.signs) + (((t & ~31) + 4 * j + (lane >> 3)) & (segs - 1)) * 8 + (lane & 7));
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      const uint4 q = __ldg(sp + j);
-      const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-      for (int c = 0; c < 4; ++c) sg[j >> 2] |= (w[c] & 0x80008000u) >> ((4 * j + c) & 15);
+      const uint32_t m = (q[j].x & 0x80008000u) | (q[j].y & 0x80008000u) >> 1 | (q[j].z & 0x80008000u) >> 2 | (q[j].w & 0x80008000u) >> 3;
+      asm volatile("st.shared.u8 [%0], %1;" ::"r"(mine + (uint32_t)(32 * j + lane)), "r"((m >> 24 & 0xF0u) | (m >> 12 & 0xFu)) : "memory");
     }
-  }
-  if (MODE == kCodes && p.layout == BRO_LAYOUT_GEMM) {        // the rows that pad the scale buffer to 128 read as zero
-    const int pad = (int)((128 - (p.M & 127)) & 127), words = pad << (log2k - 7);
-    for (int i = (int)(blockIdx.x * S::kThreads + threadIdx.x); i < words; i += (int)gridDim.x * S::kThreads) {
-      const int r = (int)(p.M & 127) + (i >> (log2k - 7)), kb = i & ((1 << (log2k - 7)) - 1);
-      *reinterpret_cast<uint32_t*>(p.scales + ((p.M >> 7) * p.scale_kblocks + kb) * 512 + (r & 31) * 16 + (r >> 5) * 4) = 0u;
+    __syncwarp();
+    const uint64_t bytes = lds64(mine + 8u * (uint32_t)lane);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {              // (channels 8 i ..: the odd ones in the upper half of the byte)
+      const uint32_t b = (uint32_t)(bytes >> (8 * i)) & 0xFFu;
+      sg[i >> 2] |= ((b >> 4) << 28 | (b & 0xFu) << 12) >> (4 * (i & 3));
     }
   }
 
@@ -388,8 +380,8 @@ rotate_quantize_global_wide_kernel(const __grid_constant__ CUtensorMap tmx, cons
 #pragma unroll
     for (uint32_t c = 0; c < 16; ++c)
       sts_pairs((w1 ^ (((c & 7u) ^ (c >> 3)) << 4)) + (c >> 3) * 128u, P[2 * c], P[2 * c + 1]);
-    // (also: every thread of the unit has taken its bytes of the bf16 rows; a lost load ends the loop for all of them)
-    if (!unit_sync_and<T>(unit, ok)) break;
+    // (also: every thread has taken its bytes of the bf16 rows; a lost load ends the loop for all of them)
+    if (!__syncthreads_and(ok)) break;
     if (t == 0 && it + stride < iters) request(it + stride);
 #pragma unroll
     for (int j = 0; j < 32; ++j) P[j] = lds64((w2 ^ (uint32_t)((((2 * (j & 3)) ^ (j >> 2)) & 7) << 4)) + (uint32_t)(j * 256));
@@ -409,7 +401,7 @@ rotate_quantize_global_wide_kernel(const __grid_constant__ CUtensorMap tmx, cons
     }
 #pragma unroll
     for (int j = 0; j < 32; ++j) sts64((w2 ^ (uint32_t)((((2 * (j & 3)) ^ (j >> 2)) & 7) << 4)) + (uint32_t)(j * 256), P[j]);
-    unit_sync<T>(unit);
+    __syncthreads();
     // run j2 starts 2048 elements = 64 lines behind the one before: the same g
 #pragma unroll
     for (int j2 = 0; j2 < NJ; ++j2) {
@@ -418,7 +410,7 @@ rotate_quantize_global_wide_kernel(const __grid_constant__ CUtensorMap tmx, cons
         lds_pairs((r3 ^ (h << 4)) + (uint32_t)(j2 * 8192), P[j2 * (RUN / 2) + 2 * h], P[j2 * (RUN / 2) + 2 * h + 1]);
       }
     }
-    unit_sync<T>(unit);                                         // (the next pass writes where others read)
+    __syncthreads();                                            // (the next pass writes where others read)
     if constexpr (!ROWS) {
 #pragma unroll
       for (int hb = 1; hb < NJ; hb <<= 1) {                     // strides 2048..
@@ -435,7 +427,7 @@ rotate_quantize_global_wide_kernel(const __grid_constant__ CUtensorMap tmx, cons
         }
       }
     }
-    // ---- results: run j2 belongs to group t / G + 64 j2 of the unit
+    // ---- results: run j2 belongs to group t / G + 64 j2 of the V / 32
 #pragma unroll
     for (int j2 = 0; j2 < NJ; ++j2) {
       const uint64_t* E = P + j2 * (RUN / 2);
@@ -487,6 +479,17 @@ rotate_quantize_global_wide_kernel(const __grid_constant__ CUtensorMap tmx, cons
 // 3-D view of x for the kernel above: {64 bf16 (128 bytes), K / 64 segments, M rows}, box = whole rows (of at most 256 segments).
 bro_status make_row_map(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx, int box_rows);
 
+// CTAs for `passes` over the rows; with few of them as many as it takes to clear the tiled scales' padding at two words a thread (one CTA
+// for one row cleared it all by itself: [1, 32768] 27.0 -> 8.6 us, [1, 8192] 7.1 -> 3.0).
+inline unsigned grid_for(int64_t passes, const Params& p, int mode, int threads, int64_t cap) {
+  int64_t want = passes;
+  if (mode == kCodes && p.layout == BRO_LAYOUT_GEMM && (p.M & 127) != 0) {
+    const int64_t clearing = (p.scale_kblocks * 128 + 2 * threads - 1) / (2 * threads);
+    if (want < clearing) want = clearing;
+  }
+  return (unsigned)(want < cap ? want : cap);
+}
+
 template <int LOG2V, int LOG2K = LOG2V>
 inline bro_status launch_wide(const Params& p, int mode, int sm_count, cudaStream_t st) {
   using S = Shape<LOG2V>;
@@ -500,15 +503,15 @@ inline bro_status launch_wide(const Params& p, int mode, int sm_count, cudaStrea
       if (!cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmemBytes),
                    "cudaFuncSetAttribute(rotate_quantize_global)"))
         return BRO_ERR_CUDA;
-      return cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kernel, S::kThreads, S::kSmemBytes),
+      return cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kernel, S::T, S::kSmemBytes),
                      "occupancy(rotate_quantize_global)")
                  ? BRO_OK
                  : BRO_ERR_CUDA;
     });
     if (rc != BRO_OK) return rc;
-    const int64_t rows = S::V >> p.log2k, iters = (p.M + rows - 1) / rows, want = (iters + S::kUnits - 1) / S::kUnits;
-    const int64_t cap = (int64_t)sm_count * per_sm;
-    return cuda_ok(launch_kernel(kernel, (unsigned)(want < cap ? want : cap), S::kThreads, S::kSmemBytes, st, 1, tmx, p),
+    const int64_t rows = S::V >> p.log2k;
+    return cuda_ok(launch_kernel(kernel, grid_for((p.M + rows - 1) / rows, p, mode, S::T, (int64_t)sm_count * per_sm), S::T,
+                                 S::kSmemBytes, st, 1, tmx, p),
                    "rotate_quantize_global launch")
                ? BRO_OK
                : BRO_ERR_CUDA;

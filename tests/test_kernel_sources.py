@@ -12,16 +12,11 @@ def code_lines(name):
     return [line for line in lines if line]
 
 
-def test_warps_are_whole_at_every_named_barrier():
-    """A named barrier is an .aligned instruction: undefined unless all lanes of a warp execute it together, which nothing promises
-    behind a lane's own wait or branch.  So each call of the helpers stands right behind a __syncwarp()."""
-    calls = 0
+def test_no_barrier_by_hand():
+    """bar.sync and its kin are .aligned instructions: undefined unless all lanes of a warp execute them together, which nothing
+    promises behind a lane's own wait or branch.  The threads of a block meet at __syncthreads(), before which the compiler joins
+    them."""
     for name in sorted(os.listdir(CSRC)):
-        if not name.endswith((".cu", ".cuh")):
-            continue
-        lines = code_lines(name)
-        for before, line in zip(lines, lines[1:]):
-            if re.search(r"\bnamed_barrier_(and|sync)\(", line) and "__device__" not in line:
-                calls += 1
-                assert before == "__syncwarp();", (name, line)
-    assert calls > 0
+        if name.endswith((".cu", ".cuh")):
+            for line in code_lines(name):
+                assert not re.search(r"\bbar(rier)?\.(cta\.)?(sync|red|arrive)\b", line), (name, line)
