@@ -2,10 +2,11 @@
 // Sec. 5.2) fused with MXFP4 quantisation.  K = 2^p, 32 <= K <= 32768.
 //
 // Same arithmetic contract as the block kernel: butterflies with ascending stride in fp32, one
-// multiply by fp32(1/sqrt(K)), then per-32 quantisation.  Two kernels:
+// multiply by fp32(1/sqrt(K)), then per-32 quantisation.  Three kernels:
 //   rotate_quantize_global_wide_kernel   codes, scale bytes, MXFP4 error: every stage in registers, two transposes through shared
 //                                        memory
-//   rotate_quantize_global_kernel        everything else (simulated quantisation, the error in the other formats, the statistics of few
+//   rotate_quantize_global_few_kernel    codes of few rows, K = 2048 and 4096: the same with twice the threads
+//   rotate_quantize_global_kernel        everything else (simulated quantisation, the error in the other formats, codes and statistics of
 //                                        short rows): a thread owns one MX group; strides 1..16 in registers, 32..512 between
 //                                        lanes (one shuffle per element per stage), >= 1024 between warps through shared memory.
 // The global rotation costs log2(K) stages instead of 5; it is expected to run below the HBM
@@ -39,7 +40,8 @@ struct Params {
   int range_pass;
 };
 
-template <int kMaxThreads>
+// CODES: codes and scales (short rows); else what p asks for.
+template <int kMaxThreads, bool CODES>
 __global__ void __launch_bounds__(kMaxThreads, 1) rotate_quantize_global_kernel(const Params p) {
   extern __shared__ float xch[];   // [rows_per_iter][K] fp32, only used when K > 1024
   const int T = p.threads_per_row;
@@ -52,6 +54,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rotate_quantize_global_kernel(
   // (only now: a dependent that starts early may then rely on everything older than this kernel)
   griddep_launch_dependents();
   // a thread always works on the same 32 channels, so its slice of the sign vector is loaded once
+  if (CODES && p.layout == BRO_LAYOUT_GEMM)
+    rq::clear_padding(p.scales, p.M, p.scale_kblocks, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
   uint4 sg[4] = {};
   if (p.signs) {
     const uint4* sp = reinterpret_cast<const uint4*>(p.signs + (int64_t)gi * 32);
@@ -101,6 +105,16 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rotate_quantize_global_kernel(
         P[2 * c] = rq::pack2(__fmaf_rn(a0, sgn, o.x), __fmaf_rn(a1, sgn, o.y));
         P[2 * c + 1] = rq::pack2(__fmaf_rn(a2, sgn, o.z), __fmaf_rn(a3, sgn, o.w));
       }
+    }
+    if constexpr (CODES) {
+      uint32_t w[4];
+      const uint32_t sbyte = rq::quantize_group(P, cbits, w);
+      if (live) {
+        *reinterpret_cast<uint4*>(p.codes + row * (p.K >> 1) + (int64_t)gi * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+        p.scales[p.layout == BRO_LAYOUT_GEMM ? ((row >> 7) * p.scale_kblocks + (gi >> 2)) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4 + (gi & 3)
+                                             : row * (p.K >> 5) + gi] = (uint8_t)sbyte;
+      }
+      continue;
     }
     if (p.format == rq::kFormatScaleOnly && !p.deq && !p.range_pass) {   // analysis mode (uniform over the grid): scale byte only
       const uint32_t sbyte = rq::group_scale_byte(P, cbits);
@@ -476,7 +490,126 @@ rotate_quantize_global_wide_kernel(const __grid_constant__ CUtensorMap tmx, cons
   if (t == 0 && it < iters) mbar_wait(bar, parity ^ 1u, SITE_RQ_DRAIN);
 }
 
-// 3-D view of x for the kernel above: {64 bf16 (128 bytes), K / 64 segments, M rows}, box = whole rows (of at most 256 segments).
+// ---- codes of few rows, K = 2048 and 4096 ----
+// The same three phases with 32 values a thread, so twice the threads for a row, one value instead of a pair in phase 2 (element bits
+// 5..9, 32 channels 32 apart) and two buffers, a barrier a transpose: what few rows are bound by is the chain of one pass.
+// 64 values a thread : 32, [64, 2048] 2.24 : 1.98 us, with signs 2.60 : 2.10, [64, 4096] with signs 2.67 : 2.34.
+template <int LOG2K, bool SIGNS>
+__global__ void __launch_bounds__(128, 5) rotate_quantize_global_few_kernel(const __grid_constant__ CUtensorMap tmx, const Params p) {
+  static_assert(LOG2K == 11 || LOG2K == 12, "K = 2048 or 4096");
+  constexpr int K = 1 << LOG2K, T = K / 32, ROWS = 128 / T;    // threads of a row; rows at a time
+  constexpr int NJ = K / 1024, RUN = 32 / NJ;                 // phase 3: runs of a thread, consecutive values of a run
+  extern __shared__ uint8_t smem_raw[];                        // [bf16 rows | barrier | two fp32 buffers], 1 KiB aligned
+  const uint32_t raw = (smem_u32(smem_raw) + 1023u) & ~1023u, bar = raw + ROWS * K * 2;
+  constexpr uint32_t cbits = rq::norm_bits<LOG2K>();
+  const int t = threadIdx.x % T, rs = threadIdx.x / T;         // thread within the row, row of the pass
+  const uint32_t bufa = bar + 1024u + (uint32_t)(rs * K * 4), bufb = bufa + ROWS * K * 4;
+  const int M = (int)p.M, iters = (M + ROWS - 1) / ROWS;
+  if (threadIdx.x == 0) {
+    mbar_init(bar, 1);
+    mbar_fence_init();
+    fence_proxy_async_smem();
+    tma_prefetch_desc(&tmx);
+  }
+  __syncthreads();
+  griddep_wait();               // x may be written, the outputs still read, by the kernel before
+  griddep_launch_dependents();
+  auto request = [&](int it) {
+    mbar_arrive_expect_tx(bar, ROWS * K * 2);
+    tma_load_3d(raw, &tmx, 0, 0, it * ROWS, bar);
+  };
+  int it = (int)blockIdx.x;
+  if (threadIdx.x == 0 && it < iters) request(it);
+  uint4 sg[4] = {};
+  if (SIGNS) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) sg[j] = __ldg(reinterpret_cast<const uint4*>(p.signs) + t * 4 + j);
+  }
+  if (p.layout == BRO_LAYOUT_GEMM)
+    rq::clear_padding(p.scales, p.M, p.scale_kblocks, (int64_t)blockIdx.x * 128 + threadIdx.x, (int64_t)gridDim.x * 128);
+  // the thread's 64 bytes: segment t / 2 of its row, pieces 4 (t & 1) + j, swizzled with the segment
+  const uint32_t seg = (uint32_t)(rs * (K / 64) + (t >> 1)), raw_mine = raw + seg * 128u;
+  // pieces of 16 bytes: transpose 1 swizzled with the line, transpose 2 with its bits 0..1
+  const uint32_t lane = (uint32_t)t & 31u, column = (uint32_t)(t >> 5) * 4096u + (lane & 3u) * 4u;
+  uint32_t parity = 0;
+  for (; it < iters; it += (int)gridDim.x) {
+    const bool ok = mbar_wait(bar, parity, SITE_RQ_FULL);
+    parity ^= 1u;
+    uint64_t P[16];
+#pragma unroll
+    for (uint32_t j = 0; j < 4; ++j) {
+      const uint4 q = lds128(raw_mine + (((((uint32_t)t & 1u) * 4u + j) ^ (seg & 7u)) << 4));
+      rq::unpack_stage1(SIGNS ? rq::apply_signs(q, sg[j]) : q, P + 4 * j);
+    }
+    rq::fwht32_stages_2_to_16(P);
+#pragma unroll
+    for (uint32_t c = 0; c < 8; ++c) sts_pairs(bufa + (uint32_t)t * 128u + ((c ^ ((uint32_t)t & 7u)) << 4), P[2 * c], P[2 * c + 1]);
+    // (also: every thread has taken its bytes of the bf16 rows; a lost load ends the loop for all of them)
+    if (!__syncthreads_and(ok)) break;
+    if (threadIdx.x == 0 && it + (int)gridDim.x < iters) request(it + (int)gridDim.x);
+    float v[32];
+#pragma unroll
+    for (uint32_t j = 0; j < 32; ++j)
+      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[j]) : "r"(bufa + column + (((lane >> 2) ^ (j & 7u)) << 4) + j * 128u) : "memory");
+    // strides 32..256 on pairs (v[k], v[k + 16]), 512 inside them
+#pragma unroll
+    for (int k = 0; k < 16; ++k) P[k] = rq::pack2(v[k], v[k + 16]);
+    rq::fwht32_stages_2_to_16(P);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      float a, b;
+      rq::unpack2(P[k], a, b);
+      v[k] = __fadd_rn(a, b);
+      v[k + 16] = __fsub_rn(a, b);
+    }
+#pragma unroll
+    for (uint32_t j = 0; j < 32; ++j)
+      asm volatile("st.shared.f32 [%0], %1;" ::"r"(bufb + column + (((lane >> 2) ^ (j & 3u)) << 4) + j * 128u), "f"(v[j]) : "memory");
+    __syncthreads();
+    // runs of RUN consecutive values, 1024 apart
+#pragma unroll
+    for (int j2 = 0; j2 < NJ; ++j2) {
+#pragma unroll
+      for (int h = 0; h < RUN / 4; ++h) {
+        const uint32_t piece = (uint32_t)(j2 * 256 + t * (RUN / 4) + h);
+        lds_pairs(bufb + ((piece ^ ((piece >> 3) & 3u)) << 4), P[j2 * (RUN / 2) + 2 * h], P[j2 * (RUN / 2) + 2 * h + 1]);
+      }
+    }
+#pragma unroll
+    for (int hb = 1; hb < NJ; hb <<= 1) {                       // strides 1024..
+#pragma unroll
+      for (int j2 = 0; j2 < NJ; ++j2) {
+        if ((j2 & hb) == 0) {
+#pragma unroll
+          for (int i = 0; i < RUN / 2; ++i) {
+            const uint64_t a = P[j2 * (RUN / 2) + i], b = P[(j2 + hb) * (RUN / 2) + i];
+            P[j2 * (RUN / 2) + i] = rq::add2(a, b);
+            P[(j2 + hb) * (RUN / 2) + i] = rq::sub2(a, b);
+          }
+        }
+      }
+    }
+    const int row = it * ROWS + rs;
+#pragma unroll
+    for (int j2 = 0; j2 < NJ; ++j2) {                           // run j2 belongs to group t / NJ + 32 j2
+      const int g = t / NJ + 32 * j2;
+      uint32_t w[RUN / 8];
+      const uint32_t s = quantize_run<RUN, NJ>(P + j2 * (RUN / 2), cbits, w);
+      if (row < M) {
+        uint8_t* dst = p.codes + (int64_t)row * (K / 2) + g * 16 + (t % NJ) * (RUN / 2);
+        if constexpr (RUN == 16) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
+        else *reinterpret_cast<uint32_t*>(dst) = w[0];
+        if (t % NJ == 0)
+          p.scales[p.layout == BRO_LAYOUT_GEMM ? ((row >> 7) * p.scale_kblocks + (g >> 2)) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4 + (g & 3)
+                                               : (int64_t)row * (K / 32) + g] = (uint8_t)s;
+      }
+    }
+  }
+  // (left before the end only after a lost wait: its copy may still land, wait once more)
+  if (threadIdx.x == 0 && it < iters) mbar_wait(bar, parity ^ 1u, SITE_RQ_DRAIN);
+}
+
+// 3-D view of x for the kernels above: {64 bf16 (128 bytes), K / 64 segments, M rows}, box = whole rows (of at most 256 segments).
 bro_status make_row_map(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx, int box_rows);
 
 // CTAs for `passes` over the rows; with few of them as many as it takes to clear the tiled scales' padding at two words a thread (one CTA
@@ -521,6 +654,29 @@ inline bro_status launch_wide(const Params& p, int mode, int sm_count, cudaStrea
   return go(rotate_quantize_global_wide_kernel<LOG2V, LOG2K, kCodes>);
 }
 
+template <int LOG2K, bool SIGNS>
+inline bro_status launch_few(const Params& p, int sm_count, cudaStream_t st) {
+  constexpr int K = 1 << LOG2K, ROWS = 4096 / K, kSmem = ROWS * K * 2 + 2048 + 2 * ROWS * K * 4;
+  CUtensorMap tmx;
+  const bro_status mrc = make_row_map(&tmx, p.x, p.M, p.K, p.ldx, ROWS);
+  if (mrc != BRO_OK) return mrc;
+  auto kernel = rotate_quantize_global_few_kernel<LOG2K, SIGNS>;
+  static DeviceOnce once;            // (one per template instantiation)
+  int per_sm = 1;
+  const bro_status rc = device_once(once, &per_sm, [&](int* n) {
+    return cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem),
+                   "cudaFuncSetAttribute(rotate_quantize_global_few)") &&
+                   cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kernel, 128, kSmem), "occupancy(rotate_quantize_global_few)")
+               ? BRO_OK
+               : BRO_ERR_CUDA;
+  });
+  if (rc != BRO_OK) return rc;
+  return cuda_ok(launch_kernel(kernel, grid_for((p.M + ROWS - 1) / ROWS, p, kCodes, 128, (int64_t)sm_count * per_sm), 128, kSmem, st, 1, tmx, p),
+                 "rotate_quantize_global launch")
+             ? BRO_OK
+             : BRO_ERR_CUDA;
+}
+
 inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, const void* signs, void* codes,
                          void* scales, float* mse, int format, bro_layout layout, int64_t scale_kblocks, int sm_count, cudaStream_t st,
                          float* deq = nullptr, int64_t ldd = 0, uint32_t* rowstats = nullptr, bool range_pass = false) {
@@ -547,14 +703,29 @@ inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, const
   int threads = p.threads_per_row < 256 ? 256 : p.threads_per_row;
   p.rows_per_iter = threads / p.threads_per_row;
   const size_t smem = K > 1024 ? (size_t)p.rows_per_iter * K * sizeof(float) : 0;
-  // (statistics of few short rows: the shuffle form starts faster, [1000, 1024] 3.05 and 3.34 us, [65536, 1024] 61 and 47)
-  const bool statistic = mse || format == rq::kFormatScaleOnly;
-  if (!deq && !range_pass && (!mse || format == 0) && !(statistic && K <= 1024 && M * K <= ((int64_t)1 << 21))) {
-    const int mode = mse ? kError : (format == rq::kFormatScaleOnly ? kBytes : kCodes);
+  const int mode = mse ? kError : (format == rq::kFormatScaleOnly ? kBytes : kCodes);
+  const int64_t elements = M * K;
+  // Short rows need few shuffles, and the shuffle form starts faster.  Shuffles : transposes, K = 256 codes [300, 256] 2.25 : 2.40 us,
+  // [65536, 256] 15.2 : 15.7, [262144, 256] 56.5 : 50.7, bytes [65536, 256] 13.7 : 14.9; K = 512 codes [2048, 512] 2.47 : 2.74, [16384, 512]
+  // 10.5 : 9.9, bytes [8192, 512] 5.5 : 5.8, [16384, 512] 9.7 : 9.5; K = 1024 codes [300, 1024] 2.53 : 2.28, bytes [1000, 1024] 3.05 : 3.34,
+  // [4096, 1024] 6.0 : 5.3; error from K = 256 on [16384, 256] 6.3 : 6.0, [8192, 512] 6.8 : 6.1.
+  int64_t shuffles = 0;
+  if (mode == kError) shuffles = K <= 1024 ? (int64_t)1 << 21 : 0;
+  else if (K == 256) shuffles = (int64_t)1 << 24;
+  else if (K == 512) shuffles = (int64_t)1 << (mode == kCodes ? 20 : 22);
+  else if (K == 1024) shuffles = mode == kCodes ? 0 : (int64_t)1 << 21;
+  if (!deq && !range_pass && (!mse || format == 0) && elements > shuffles) {
+    // Few rows: one CTA an SM of that kernel (K = 4096) or up to 2.5 (K = 2048).  [700, 2048] 2.82 : 3.01 us, [1000, 2048] 3.7 : 3.3;
+    // [129, 4096] with signs 2.42 : 2.73, [160, 4096] 2.55 : 2.45.
+    const bool few = mode == kCodes && (K == 2048 ? M <= 5 * sm_count : M <= sm_count);
     switch (lg) {
       case 10: return launch_wide<12, 10>(p, mode, sm_count, st);
-      case 11: return launch_wide<12, 11>(p, mode, sm_count, st);
-      case 12: return launch_wide<12>(p, mode, sm_count, st);
+      case 11:
+        if (few) return signs ? launch_few<11, true>(p, sm_count, st) : launch_few<11, false>(p, sm_count, st);
+        return launch_wide<12, 11>(p, mode, sm_count, st);
+      case 12:
+        if (few) return signs ? launch_few<12, true>(p, sm_count, st) : launch_few<12, false>(p, sm_count, st);
+        return launch_wide<12>(p, mode, sm_count, st);
       case 13: return launch_wide<13>(p, mode, sm_count, st);
       case 14: return launch_wide<14>(p, mode, sm_count, st);
       case 15: return launch_wide<15>(p, mode, sm_count, st);
@@ -563,19 +734,20 @@ inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, const
   }
   const int64_t iters = (M + p.rows_per_iter - 1) / p.rows_per_iter;
   const int64_t max_grid = (int64_t)sm_count * (threads <= 512 ? 2 : 1);
-  const int grid = (int)(iters < max_grid ? iters : max_grid);
+  const unsigned grid = grid_for(iters, p, deq || range_pass ? kBytes : mode, threads, max_grid);
   auto go = [&](auto kernel) -> bro_status {
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return BRO_ERR_CUDA;
-    return cuda_ok(launch_kernel(kernel, (unsigned)grid, (unsigned)threads, smem, st, 1, p),
+    return cuda_ok(launch_kernel(kernel, grid, (unsigned)threads, smem, st, 1, p),
                    "rotate_quantize_global launch")
                ? BRO_OK
                : BRO_ERR_CUDA;
   };
-  if (threads <= 256) return go(rotate_quantize_global_kernel<256>);
-  if (threads <= 512) return go(rotate_quantize_global_kernel<512>);
-  return go(rotate_quantize_global_kernel<1024>);
+  if (mode == kCodes && !deq && !range_pass) return go(rotate_quantize_global_kernel<256, true>);        // (K = 256 and 512)
+  if (threads <= 256) return go(rotate_quantize_global_kernel<256, false>);
+  if (threads <= 512) return go(rotate_quantize_global_kernel<512, false>);
+  return go(rotate_quantize_global_kernel<1024, false>);
 }
 
 }  // namespace rqg
