@@ -202,6 +202,27 @@ __global__ void __launch_bounds__(256) swiglu_kernel(const uint16_t* gate, const
 // ---- rotate + quantise ---------------------------------------------------------------------------
 inline bool wide_takes(int64_t B, int64_t K) { return B >= 32 && B <= 128 && K % 64 == 0; }
 
+// Whether the wide kernel (a lane owns 64 channels) beats the register-streaming one, both by what a call comes to on this chip: the wide
+// one's tasks of 16 rows x 128 channels in whole rounds of eight-warp CTAs, one an SM (its warps do one or two tasks, and a round begun is a
+// round taken), against the other's tasks of up to 32 groups of a row, half as many values and, with K not a multiple of 1024, idle
+// lanes.  Over 2452 forms (K 192 to 28672, 2^17 to 2^26 elements, both layouts, with and without signs) the choice is on average within 0.3 %
+// of the better of the two for blocks of 64, 0.1 % for 128 and 0.4 % for 32.  Direct : wide, block 128 canonical [64, 14336] 2.20 : 2.47 us, [300, 4096] 2.73 : 2.40, [16384, 4096] 37.2 : 30.8; block 64 [1000, 1024]
+// 2.05 : 2.24, [1000, 1088] 3.15 : 2.34; block 32 [100, 65536] 5.28 : 6.52, [4096, 1088] 5.94 : 4.12.
+bool wide_pays(int64_t B, int64_t M, int64_t K, bro_layout layout, bool signs, int sm_count) {
+  if (!wide_takes(B, K)) return false;
+  const int64_t kblocks = layout == BRO_LAYOUT_GEMM ? gemm_scale_kblocks(K) : ceil_div(K, 128);
+  const int64_t rows16 = layout == BRO_LAYOUT_GEMM ? ceil_div(M, 128) * 8 : ceil_div(M, 16);
+  const int64_t round = 8 * (int64_t)sm_count, wide = rows16 * kblocks, rounds = ceil_div(wide, round);
+  int64_t direct = bro::rqd::tasks(M, K, layout, gemm_scale_kblocks(K));
+  if (layout == BRO_LAYOUT_GEMM && M <= 64) direct = direct / 128 * M;        // (the padding is cleared, not quantised)
+  if (B > 32 || signs) return rounds * round <= direct;
+  // A plain block of 32 has no exchange to save: one round, the lanes saved, or the sizes in between those where the caches help and those
+  // where the memory bounds both.  [1500, 4096] 5.1 : 6.1, [4096, 4096] 8.8 : 9.4, [8192, 4096] 15.5 : 14.7, [14336, 4096] 25.2 : 25.8.
+  if (rounds == 1) return 11 * round <= 10 * direct;
+  if (204 * wide <= 100 * direct) return rounds * round <= direct;
+  return M * K >= (int64_t)3 << 23 && M * K <= (int64_t)1 << 25;
+}
+
 // Arguments of a rotate+quantize launch; BRO_OK with M == 0 means that there is nothing to do.
 // (up != nullptr: x is the gate of the fused producer, the rotated tensor is silu(x) * up)
 bro_status check_rotate_quantize(const void* x, int64_t M, int64_t K, int64_t ldx, int block, const void* signs,
@@ -239,17 +260,15 @@ bro_status launch_rotate_quantize(const void* x, int64_t M, int64_t K, int64_t l
     return bro::rqg::launch(x, M, K, ldx, signs, codes, scales, nullptr, 0, layout, gemm_scale_kblocks(K), di.sm_count, st);
   }
 
-  // The wide kernel (a lane owns 64 channels) for blocks of 64 and 128 beyond 2^19 elements ([300, 4096], block 128, 3.5 -> 3.0 us,
-  // [16384, 4096] 37.2 -> 30.8, block 64 33.3 -> 29.4; [128, 4096] 2.6 -> 2.9) and for block 32 from 2^20 to 2^25 ([2048, 2048]
-  // 4.0 -> 3.7, [8192, 4096] 16.4 -> 15.0; [128, 4096] even, [14336, 4096] 26.0 -> 26.5).  In front of a GEMM (`layer`) it has to
-  // save more, since its shared memory keeps the GEMM's CTAs from starting under its tail: beyond 2^22 elements and from 2^24
-  // (whole layers, block 64: (1500, 5120, 2500) 19.9 -> 18.8, (2048, 2048, 8192) 21.1 -> 21.5, block 32: (4096, 4096, 4096) 38.0 -> 37.3,
-  // (2048, 2048, 8192) 20.6 -> 21.4).  Else, and where K is not a multiple of 64, below the MX group and with the fused producer, the
-  // register-streaming kernel.  The flags of the *_ex entry point override the choice.
+  // In front of a GEMM (`layer`) the wide kernel has to save more, since its shared memory keeps the GEMM's CTAs from starting under its
+  // tail: beyond 2^22 elements, block 32 from 2^24 (whole layers, block 64: (1500, 5120, 2500) 19.9 -> 18.8, (2048, 2048, 8192) 21.1 -> 21.5,
+  // block 32: (4096, 4096, 4096) 38.0 -> 37.3, (2048, 2048, 8192) 20.6 -> 21.4).  Where K is not a multiple of 64, below the MX group and
+  // with the fused producer, the register-streaming kernel.  The flags of the *_ex entry point override the choice.
   const int64_t elements = M * K;
   const bool can_wide = wide_takes(B, K) && !up;
-  bool wide = can_wide && (B == 32 ? elements >= (int64_t)1 << (layer ? 24 : 20) && elements <= (int64_t)1 << 25
-                                   : elements > (int64_t)1 << (layer ? 22 : 19));
+  bool wide = can_wide && (!layer   ? wide_pays(B, M, K, layout, signs != nullptr, di.sm_count)
+                           : B == 32 ? elements >= (int64_t)1 << 24 && elements <= (int64_t)1 << 25
+                                     : elements > (int64_t)1 << 22);
   // From 2^30 rows the register-streaming kernel's tasks number as many as it can count: the wide kernel then takes what it can, and
   // a plain block of 32 over rows of 32 channels, the only other call of that length, is counted to the last task.
   const int64_t tasks = bro::rqd::tasks(M, K, layout, gemm_scale_kblocks(K));
@@ -387,9 +406,9 @@ bro_status bro_group_quant_error_fmt(const void* x_bf16, int64_t M, int64_t K, i
     return bro::fq::launch(x_bf16, M, K, ldx, (int)B, signs_bf16, (int)format, nullptr, 0, mse, nullptr, di.sm_count, st);
   if (B > 128)
     return bro::rqg::launch(x_bf16, M, K, ldx, signs_bf16, nullptr, nullptr, mse, (int)format, BRO_LAYOUT_CANONICAL, 0, di.sm_count, st);
-  // (MXFP4, wide kernel: block 128 of [16384, 4096] 42.9 -> 35.4 us, block 64 36.2 -> 31.6, block 32 32.0 -> 29.3; [128, 4096] 2.6 -> 3.0,
-  // block 32 of [4096, 4096] 9.8 -> 10.1)
-  if (format == BRO_FMT_MXFP4 && wide_takes(B, K) && M * K > (B == 32 ? ((int64_t)1 << 25) - 1 : (int64_t)1 << 19))
+  // (MXFP4, wide kernel: block 128 of [16384, 4096] 42.9 -> 35.4 us, block 64 36.2 -> 31.6, block 32 32.0 -> 29.3, but [4096, 4096] 9.8 -> 10.1)
+  if (format == BRO_FMT_MXFP4 && (B == 32 ? wide_takes(B, K) && M * K >= (int64_t)1 << 25
+                                          : wide_pays(B, M, K, BRO_LAYOUT_CANONICAL, signs_bf16 != nullptr, di.sm_count)))
     return bro::rqw::launch(x_bf16, M, K, ldx, log2_of(B), signs_bf16, nullptr, nullptr, mse, BRO_LAYOUT_CANONICAL, 0, di.sm_count, st);
   if (!bro::rqd::supports(M, K, BRO_LAYOUT_CANONICAL, 0)) return BRO_ERR_UNSUPPORTED;
   return bro::rqd::launch_stats(x_bf16, M, K, ldx, B == 32 ? 5 : (B == 64 ? 6 : 7), signs_bf16, (int)format, mse, nullptr, di.sm_count, st);
@@ -482,8 +501,8 @@ bro_status bro_group_scale_bytes(const void* x_bf16, int64_t M, int64_t K, int64
   if (B > 128)
     return bro::rqg::launch(x_bf16, M, K, ldx, signs_bf16, nullptr, scales, nullptr, bro::rq::kFormatScaleOnly,
                             BRO_LAYOUT_CANONICAL, 0, di.sm_count, st);
-  // (wide kernel: block 128 of [16384, 4096] 38.1 -> 25.9 us, block 64 30.3 -> 24.3; block 32 23.6 -> 24.2, [128, 4096] 2.4 -> 2.5)
-  if (B > 32 && wide_takes(B, K) && M * K > (int64_t)1 << 19)
+  // (wide kernel: block 128 of [16384, 4096] 38.1 -> 25.9 us, block 64 30.3 -> 24.3; block 32 23.6 -> 24.2)
+  if (B > 32 && wide_pays(B, M, K, BRO_LAYOUT_CANONICAL, signs_bf16 != nullptr, di.sm_count))
     return bro::rqw::launch(x_bf16, M, K, ldx, log2_of(B), signs_bf16, nullptr, scales, nullptr, BRO_LAYOUT_CANONICAL, 0, di.sm_count, st);
   if (!bro::rqd::supports(M, K, BRO_LAYOUT_CANONICAL, 0)) return BRO_ERR_UNSUPPORTED;
   return bro::rqd::launch_stats(x_bf16, M, K, ldx, B == 32 ? 5 : (B == 64 ? 6 : 7), signs_bf16,

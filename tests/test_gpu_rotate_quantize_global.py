@@ -1,5 +1,5 @@
-"""GPU parity of the full-dimension rotation, units of every size, in all three outputs — codes, scale bytes, MXFP4 error — against
-the CPU oracle."""
+"""GPU parity of the full-dimension rotation of few rows, every row length, in all three outputs — codes, scale bytes, MXFP4 error —
+against the CPU oracle.  (Which kernel computes which at which size, and those that only many rows reach: test_gpu_large_forms.py.)"""
 import pytest
 
 from paper_2511_04214_b200 import synth
@@ -18,7 +18,7 @@ def bro():
                                  (1, 8192), (130, 8192), (3, 16384), (2, 32768)])
 @pytest.mark.parametrize("signs", [False, True])
 def test_full_dimension_units(bro, M, K, signs):
-    """Every size of unit: several rows (the last ones missing), one row in a warp, in several warps; rows with gaps."""
+    """Several rows at a time (the last ones missing), one row in a warp, in several warps; rows with gaps."""
     x = synth.activations(M, K, seed=M + K)
     s = synth.rotation_signs(K, seed=3) if signs else None
     all_outputs(bro, x, device_copy(x, 8 if signs else 0), 0, s, 0)

@@ -1,5 +1,7 @@
 """GPU parity of the rotate+quantise kernel whose lanes own 64 channels (blocks 32, 64, 128, K a multiple of 64) where its tiles and
-stores can go wrong, in all three outputs — codes, scale bytes, MXFP4 error — against the CPU oracle."""
+stores can go wrong — codes and their scale bytes, by the flag that asks for it — and of the statistics of the same small tensors,
+which the register-streaming kernel computes at these sizes, against the CPU oracle.  (The statistics of large tensors, which
+the first kernel computes, are in test_gpu_large_forms.py.)"""
 import numpy as np
 import pytest
 import torch
