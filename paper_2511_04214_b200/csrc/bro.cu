@@ -484,7 +484,9 @@ bro_status bro_group_scale_bytes(const void* x_bf16, int64_t M, int64_t K, int64
   if (block == 1) {
     // the identity rotation: a sign flip does not change a magnitude, so the signs play no part
     const unsigned grid = bro::stats::grid_for(M * (K / 32), 256, di.sm_count, 8);
-    if (ldx == K || M == 1)
+    // (whole lines pay once x no longer comes from L2: [16384, 4096] 24.3 -> 22.4 us, [4096, 4096] 7.3 -> 6.8, but [4096, 1088] 3.05 -> 3.6,
+    // [1000, 1024] 1.6 -> 1.7)
+    if ((ldx == K || M == 1) && M * K >= (int64_t)1 << 24)
       return bro::cuda_ok(bro::launch_kernel(bro::stats::group_scale_bytes_identity_flat, grid, 256, 0, st, 1,
                                              static_cast<const uint16_t*>(x_bf16), M * (K / 32), scales),
                           "group_scale_bytes launch")

@@ -12,9 +12,10 @@ def bro():
     return binding
 
 
-@pytest.mark.parametrize("M,K", [(1, 32), (1, 992), (3, 64), (7, 1056), (33, 4096), (1000, 3008), (5000, 32)])
+@pytest.mark.parametrize("M,K", [(1, 32), (1, 992), (3, 64), (7, 1056), (33, 4096), (1000, 3008), (5000, 32), (16385, 1024), (5590, 3008),
+                                 (1, 16777216 + 32), (524289, 32)])
 def test_scale_bytes_without_a_rotation(bro, M, K):
-    """Last warps with one to 32 groups, rows that end inside a warp's 32."""
+    """Last warps with one to 32 groups, rows that end inside a warp's 32 (read as one row from 2^24 elements)."""
     gen = torch.Generator().manual_seed(M + K)
     x = (torch.randn(M, K, generator=gen) * torch.exp2(torch.randint(-130, 120, (M, K // 32, 1), generator=gen).float()).expand(
         M, K // 32, 32).reshape(M, K)).to(torch.bfloat16)
