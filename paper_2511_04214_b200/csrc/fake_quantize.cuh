@@ -404,9 +404,18 @@ __global__ void __launch_bounds__(kThreads, 2) fake_quantize_kernel(const Params
     float neglo = 0.f, hi = 0.f;
     if (whole_rows || (MODE == kStatistics && !p.mse && !p.scale_bytes)) {     // the range of this chunk
       group_range(P, cbits, neglo, hi);
-      // (all 32 lanes hold groups of the same row; dead lanes hold zeros.  Non-negative floats order like their bits.)
-      neglo = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(neglo)));
-      hi = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(hi)));
+      // All 32 lanes hold groups of the same row; dead lanes hold zeros.  Non-negative floats order like their bits.  (In the pass over long
+      // rows, which does little else, shuffles: [4096, 14336] block 128 117 us with the reduction, 112 with them.)
+      if constexpr (MODE == kStatistics) {
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) {
+          neglo = fmaxf(neglo, __shfl_xor_sync(0xFFFFFFFFu, neglo, d));
+          hi = fmaxf(hi, __shfl_xor_sync(0xFFFFFFFFu, hi, d));
+        }
+      } else {
+        neglo = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(neglo)));
+        hi = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(hi)));
+      }
     }
     if (whole_rows) {
       if (lane == 0) ranges[round & 1][warp] = make_float2(neglo, hi);
