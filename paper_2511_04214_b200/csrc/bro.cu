@@ -532,6 +532,7 @@ bro_status bro_outlier_groups(const void* x_bf16, int64_t M, int64_t K, int64_t 
   const unsigned long long n = (unsigned long long)M * (unsigned long long)K;
   unsigned long long k = (n * (unsigned long long)top_ppm + 999999ull) / 1000000ull;
   if (k < 1) k = 1;
+  // (outlier_scan relies on outlier_clear directly in front of it: see griddep_wait)
   if (!bro::cuda_ok(bro::launch_kernel(bro::stats::outlier_clear, (unsigned)bro::stats::kClearCtas, bro::stats::kScanThreads, 0, st, 1, hist),
                     "outlier_clear launch"))
     return BRO_ERR_CUDA;
@@ -552,6 +553,7 @@ bro_status bro_outlier_groups(const void* x_bf16, int64_t M, int64_t K, int64_t 
              : BRO_ERR_CUDA;
 }
 
+// (the counting kernels rely on this one directly in front of them: see griddep_wait)
 static bool clear_counts(uint64_t* counts, int n, cudaStream_t st) {
   return bro::cuda_ok(bro::launch_kernel(bro::stats::clear_counts, 1u, 512u, 0, st, 1, reinterpret_cast<unsigned long long*>(counts), n),
                       "clear_counts launch");

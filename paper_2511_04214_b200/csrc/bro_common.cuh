@@ -80,7 +80,7 @@ __device__ unsigned int g_device_status = 0u;
 constexpr uint64_t kWaitBudgetNs = 2000ull * 1000ull * 1000ull;
 
 enum WaitSite : unsigned {
-  SITE_RQ_FULL = 1, SITE_RQ_EMPTY = 2, SITE_RQ_DRAIN = 3,
+  SITE_RQ_FULL = 1, /* 2: a kernel that is gone */ SITE_RQ_DRAIN = 3,
   SITE_GEMM_FULL = 4, SITE_GEMM_EMPTY = 5, SITE_GEMM_ACC_FULL = 6, SITE_GEMM_ACC_EMPTY = 7,
   SITE_GEMM_DRAIN = 8, SITE_GEMM_TMEM = 9, SITE_SELF_TEST = 10
 };
@@ -145,30 +145,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigne
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* m) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
 }
-// 2-D tiled load global -> shared, completion counted in bytes on `bar`.  x is the innermost
-// coordinate (elements of the map's data type); x * element size must be a multiple of 16 bytes.
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* m, int x, int y,
-                                            uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
-// 3-D tiled load (x innermost; the same alignment rule for x).
+// 3-D tiled load global -> shared, completion counted in bytes on `bar`.  x is the innermost coordinate (elements of the map's data
+// type); x * element size must be a multiple of 16 bytes.
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* m, int x, int y, int z, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
       " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(z), "r"(bar)
-      : "memory");
-}
-// 1-D bulk copy global -> shared (both addresses 16-byte aligned, size a multiple of 16).
-__device__ __forceinline__ void bulk_load_1d(uint32_t dst, const void* src, uint32_t bytes,
-                                             uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar)
       : "memory");
 }
 
@@ -177,10 +160,14 @@ __device__ __forceinline__ void bulk_load_1d(uint32_t dst, const void* src, uint
 // so the next kernel in the stream may be scheduled while this one still runs: its CTAs start on
 // SMs as they become free and run their prologue (barrier set-up, TMEM allocation, descriptor
 // prefetch) early.  griddep_wait() blocks until all earlier grids in the stream have completed
-// and their writes are visible; every thread calls it before its first access to global memory, with two
-// exceptions, both of the weights in the GEMMs: inside the whole-layer calls, where the weights are older than the kernel
-// in front (whose own wait precedes its launch_dependents), the first weight tiles are loaded before it, and the
-// one-kernel layer, which has no such kernel in front, only draws them into L2.
+// and their writes are visible; every thread calls it before its first access to global memory, with these exceptions:
+//   * the weights in the GEMMs.  Inside the whole-layer calls they are older than the kernel in front, whose own wait precedes its
+//     launch_dependents, and the first weight tiles are loaded before the wait; the one-kernel layer, which has no such kernel in
+//     front, only draws them into L2.
+//   * the statistics that add to counts: outlier_scan (reads x, writes the mask), scale_histogram and scale_inflation (read the scale
+//     bytes and the mask).  The kernel that clears their counts stands directly in front of them, and its wait precedes its
+//     launch_dependents, so whatever is older than it is complete when they start; they wait for the clearing before they add.
+// Where one of these is launched, no kernel that signals before its own wait may come between it and the one in front.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -206,6 +193,15 @@ __device__ __forceinline__ void tma_load_2d_elect(uint32_t dst, const CUtensorMa
       "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
+__device__ __forceinline__ void tma_load_3d_elect(uint32_t dst, const CUtensorMap* m, int x, int y, int z, uint32_t bar) {
+  asm volatile(
+      "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
+      "@q cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4}], [%5]; }" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(z), "r"(bar)
+      : "memory");
+}
+// (both addresses 16-byte aligned, size a multiple of 16 bytes)
 __device__ __forceinline__ void bulk_load_1d_elect(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile(
       "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"

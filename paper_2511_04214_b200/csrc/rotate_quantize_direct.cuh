@@ -351,15 +351,6 @@ struct Ring {
   static constexpr int kSmemBytes = kBarAt + kWarps * kStages * 8 + 1024 /*alignment*/;
 };
 
-__device__ __forceinline__ void tma_load_3d_elect(uint32_t dst, const CUtensorMap* m, int x, int y, int z, uint32_t bar) {
-  asm volatile(
-      "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
-      "@q cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4}], [%5]; }" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(z), "r"(bar)
-      : "memory");
-}
-
 template <int LOG2B, bool SIGNS, int STAGES>
 __global__ void __launch_bounds__(kThreads, 4 - STAGES)
 rotate_quantize_gated_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmu, const Params p) {

@@ -48,15 +48,6 @@ struct Params {
   int wide_stores;              // codes start on 32 bytes
 };
 
-__device__ __forceinline__ void tma_load_3d_elect(uint32_t dst, const CUtensorMap* m, int x, int y, int z, uint32_t bar) {
-  asm volatile(
-      "{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t"
-      "@q cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4}], [%5]; }" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(z), "r"(bar)
-      : "memory");
-}
-
 __device__ __forceinline__ void stg256(void* dst, const uint32_t (&a)[4], const uint32_t (&b)[4]) {
   asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst), "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]),
                "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3])
@@ -191,6 +182,7 @@ __device__ __forceinline__ void error_two(const uint64_t (&P)[32], uint32_t cbit
 template <int LOG2B, bool SIGNS, int MODE>
 __global__ void __launch_bounds__(kThreads, 2) rotate_quantize_wide_kernel(const __grid_constant__ CUtensorMap tmx, const Params p) {
   static_assert(LOG2B >= 5 && LOG2B <= 7, "blocks of 32, 64, 128");
+  static_assert(LOG2B > 5 || MODE != kBytes, "scale bytes: blocks of 64 and 128");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int lane = threadIdx.x & 31, warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);
@@ -300,14 +292,7 @@ __global__ void __launch_bounds__(kThreads, 2) rotate_quantize_wide_kernel(const
     }
     uint32_t wx[4] = {}, wy[4] = {}, sx, sy;
     if constexpr (LOG2B == 5) {
-      if constexpr (MODE == kBytes) {
-        float ma, mb;
-        amax_two<false>(P, ma, mb);
-        sx = byte_of(exp_field(ma, cbits));
-        sy = byte_of(exp_field(mb, cbits));
-      } else {
-        quantize_two(P, cbits, wx, sx, wy, sy);
-      }
+      quantize_two(P, cbits, wx, sx, wy, sy);
     } else if constexpr (MODE == kBytes) {
       sx = rq::group_scale_byte(X, cbits);
       sy = rq::group_scale_byte(Y, cbits);
@@ -397,7 +382,9 @@ inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, int l
     constexpr int MODE = decltype(mode)::value;
     if (log2b == 6) return signs ? launch_one<6, true, MODE>(tmx, p, sm_count, st) : launch_one<6, false, MODE>(tmx, p, sm_count, st);
     if (log2b == 7) return signs ? launch_one<7, true, MODE>(tmx, p, sm_count, st) : launch_one<7, false, MODE>(tmx, p, sm_count, st);
-    return signs ? launch_one<5, true, MODE>(tmx, p, sm_count, st) : launch_one<5, false, MODE>(tmx, p, sm_count, st);
+    // (scale bytes of blocks of 32: the register-streaming kernel is the faster one)
+    if constexpr (MODE == kBytes) return BRO_ERR_UNSUPPORTED;
+    else return signs ? launch_one<5, true, MODE>(tmx, p, sm_count, st) : launch_one<5, false, MODE>(tmx, p, sm_count, st);
   };
   if (mse) return size(std::integral_constant<int, kError>());
   if (!codes) return size(std::integral_constant<int, kBytes>());

@@ -42,8 +42,11 @@ struct GroupWalk {
 
 // max of the 15-bit magnitude patterns of 8 bf16 values (finite non-negative floats order like integers), both halves of
 // a word at a time
+__device__ __forceinline__ uint32_t max_mag8_pairs(uint4 q) {
+  return __vmaxu2(__vmaxu2(q.x & 0x7FFF7FFFu, q.y & 0x7FFF7FFFu), __vmaxu2(q.z & 0x7FFF7FFFu, q.w & 0x7FFF7FFFu));
+}
 __device__ __forceinline__ uint32_t max_mag8(uint4 q) {
-  const uint32_t m = __vmaxu2(__vmaxu2(q.x & 0x7FFF7FFFu, q.y & 0x7FFF7FFFu), __vmaxu2(q.z & 0x7FFF7FFFu, q.w & 0x7FFF7FFFu));
+  const uint32_t m = max_mag8_pairs(q);
   return max(m & 0xFFFFu, m >> 16);
 }
 
@@ -70,9 +73,6 @@ __device__ __forceinline__ uint32_t group_max_mag(const uint16_t* x, int64_t row
 // The largest magnitude pattern of every group of a run of 32 consecutive groups in memory, by a warp that reads whole lines:
 // lane l holds the 16 bytes 256 j + 8 l .. of the 2 KiB in q[j], a quarter of group 8 j + l / 4.  The four lanes of a quad
 // exchange maxima (both halves of a word at a time) so that lane l is left with group 8 (l mod 4) + l / 4.
-__device__ __forceinline__ uint32_t max_mag8_pairs(uint4 q) {
-  return __vmaxu2(__vmaxu2(q.x & 0x7FFF7FFFu, q.y & 0x7FFF7FFFu), __vmaxu2(q.z & 0x7FFF7FFFu, q.w & 0x7FFF7FFFu));
-}
 __device__ __forceinline__ uint32_t quad_maxima(const uint32_t (&m)[4], int lane) {
   const bool b0 = (lane & 1) != 0, b1 = (lane & 2) != 0;
   uint32_t k0 = b0 ? m[1] : m[0], k1 = b0 ? m[3] : m[2];                 // groups j = b0 and b0 + 2
