@@ -180,8 +180,12 @@ __device__ __forceinline__ int first_task(bool spread, int warp) {
   return spread ? warp * (int)gridDim.x + (int)blockIdx.x : (int)blockIdx.x * kWarps + warp;
 }
 
+// `spread` (one block of 128 rows): zero scales for the rows that pad, whole lines of the tiled layout by each warp
 __device__ __forceinline__ void clear_padding(const Params& p) {
-  rq::clear_padding(p.scales, p.M, p.scale_kblocks, blockIdx.x * kThreads + threadIdx.x, gridDim.x * kThreads);
+  for (int64_t i = blockIdx.x * kThreads + threadIdx.x; i < (p.scale_kblocks << 7); i += gridDim.x * kThreads) {
+    const int slot = (int)(i & 127), row = ((slot & 3) << 5) | (slot >> 2);
+    if (row >= p.M) reinterpret_cast<uint32_t*>(p.scales)[i] = 0u;
+  }
 }
 
 // Rotate and quantise the 32 groups of one task, a lane's 64 bytes in cur (odd lanes of blocks of 64 / 128: halves
