@@ -509,12 +509,13 @@ inline bro_status best_split(int64_t tiles, int num_k_steps, int sm_count, Cost&
 // K = 256, N = 8192 4.85 -> 5.1; but K = 512, N = 1000 4.0 -> 3.6 and K = 768, N = 8192 4.5 -> 4.0; 4 steps gain throughout
 // (K = 1024, N = 16384 5.9 -> 5.3, N = 64 3.9 -> 3.7).
 //
-// fused = true asks for a plan that quantises inside the GEMM.  It saves the other kernel (2 us on the device, 3 us of
-// the host's time to launch it) and costs the tasks of the quantising warps, of which about half the time that the
-// weights take from HBM hides; what is left may cost up to 2.9 us.  Whole layer in a graph, two kernels -> fused:
-// (1, 8192, 28672) 24.3 -> 22.6 us, (3, 1024, 1024) 4.2 -> 3.3, (16, 2048, 2048) 5.1 -> 3.9, (16, 4096, 4096) 6.8 -> 5.6,
-// (16, 8192, 28672) and (24, 5120, 5120) even, (64, 2048, 2048) 6.0 -> 6.4 and (16, 14336, 4096) 10.5 -> 11.9; called
-// one by one, where the host binds, (64, 2048, 2048) 9.0 -> 6.9.  Beyond the line (32, 8192, 28672) 24.8 -> 29.5.
+// fused = true asks for a plan that quantises inside the GEMM.  It saves the other kernel and costs the tasks of the quantising warps,
+// of which about half the time that the weights take from HBM hides; what is left may cost up to 2.9 us.  Whole layer, two kernels ->
+// fused, in a graph and called one by one: (1, 8192, 28672) 23.4 -> 21.0 and 23.0 -> 22.1 us, (3, 1024, 1024) 4.4 -> 3.4 and 4.9 -> 3.8,
+// (16, 2048, 2048) 4.9 -> 3.9 and 5.7 -> 4.4, (16, 4096, 4096) 5.5 -> 5.4 and 5.9 -> 5.4, (16, 8192, 28672) 23.8 -> 22.9 and 23.6 -> 24.2.  The
+// line was drawn when the second kernel cost the host 3 us and quantising few tokens took longer, and by now it lies too high:
+// (28, 4096, 4096) 5.9 -> 6.6 and 6.3 -> 6.5, (64, 2048, 2048) 6.0 -> 6.4 and 6.1 -> 6.8, (48, 1536, 4096) 5.4 -> 6.2 and 5.5 -> 6.2,
+// (24, 5120, 5120) 7.0 -> 8.5 and 6.6 -> 7.7, (16, 14336, 4096) 8.0 -> 10.1 and 8.2 -> 10.1.  Beyond it (32, 8192, 28672) 24.8 -> 29.5.
 // With few K steps the line is lower, 1.25 us and 0.2 us a step: there the persistent kernel is quick, and no layer may be
 // slower in a graph than with it: (64, 512, 4096) persistent 5.1, two kernels 4.4, fused 5.4 us, (48, 1024, 8192) 6.3, 5.3
 // and 6.5, but (48, 1536, 4096) 6.6, 5.4 and 6.2.  More than 64 tokens are two tasks a warp and step and 128 columns:

@@ -27,8 +27,8 @@ def test_traffic_is_null_when_the_kernels_changed(monkeypatch):
 def test_kernel_label_follows_the_dispatch_rule():
     assert bench.gemm_kernel_name(128, 8192, 28672) == "gemm_mxfp4_kernel"           # one tile row
     assert bench.gemm_kernel_name(1024, 8192, 28672) == "gemm_mxfp4_pair_kernel"
-    assert bench.gemm_kernel_name(2048, 2048, 8192) == "gemm_mxfp4_kernel"           # K < 4096
-    assert bench.gemm_kernel_name(4096, 4096, 1024) == "gemm_mxfp4_kernel"           # fewer than two rounds of pairs
+    assert bench.gemm_kernel_name(2048, 2048, 8192) == "gemm_mxfp4_kernel"           # 3.66 rounds of 8 steps, 3.77 of the pair's
+    assert bench.gemm_kernel_name(4096, 4096, 1024) == "gemm_mxfp4_kernel"           # one round either way
     assert bench.gemm_kernel_name(16, 8192, 28672) == "gemm_mxfp4_splitk_kernel"     # one wave of 256-row tiles of W
     assert bench.gemm_kernel_name(512, 2048, 2048) == "gemm_mxfp4_splitk_kernel"     # four token tiles, 8 K steps
     assert bench.gemm_kernel_name(512, 1024, 2048) == "gemm_mxfp4_kernel"            # 4 K steps
