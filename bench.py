@@ -65,7 +65,7 @@ def select_shapes(args):
 # output that does not fit the 126 MB L2, so written bytes do reach DRAM).  The traffic of this kernel grows
 # in proportion to M for a fixed weight matrix (the packed weights are re-read once per raster band of 8
 # tile rows of 256, the output is written once), so the figure for the whole record is the captured one scaled by
-# the rows processed.  "cfg3" holds the one shape captured with `--set full -k regex:gemm_mxfp4 -s 3 -c 2`
+# the rows processed.  "cfg3" holds the one shape captured with the same metrics
 # under `--workload cfg3 --shape-index 1`, "cfg4" the block-32 kernel captured with `-k
 # regex:rotate_quantize_direct -s 6 -c 2` under `--workload cfg4 --only-block --block 32`.
 # The figures belong to one exact version of the kernels: every entry names the kernel source files it was
@@ -75,12 +75,12 @@ def select_shapes(args):
 GEMM_SOURCES = ("bro_common.cuh", "gemm_mxfp4.cuh", "gemm_mxfp4_2cta.cuh")
 RQ_SOURCES = ("bro_common.cuh", "rotate_quantize.cuh", "rotate_quantize_direct.cuh")
 NCU_TRAFFIC = {
-    "cfg5": {"sources": GEMM_SOURCES, "digest": "096c61cb1b9865ca985e775b0d340c5efb1060c2d39547c30f96dd9d3d65fab1",
-             "per_row_of": (8192, 8192, 28672), "bytes": 535339776 + 441953536},
-    "cfg3": {"sources": GEMM_SOURCES, "digest": "096c61cb1b9865ca985e775b0d340c5efb1060c2d39547c30f96dd9d3d65fab1",
-             "shapes": {(4096, 4096, 14336): 68345088 + 69353728}},
-    "cfg4": {"sources": RQ_SOURCES, "digest": "aa6e030cc76b05e3c4883ecbdfdbfc516261469c9425d0325a4fb2e97853c75c",
-             "shapes": {(16384, 4096, 32): 134233600 + 19132928}},
+    "cfg5": {"sources": GEMM_SOURCES, "digest": "49ab7565188e8384a2fdbe5579fa86605abe9616f2fc8fe10a7b56b94f267506",
+             "per_row_of": (8192, 8192, 28672), "bytes": 535290112 + 440916992},
+    "cfg3": {"sources": GEMM_SOURCES, "digest": "49ab7565188e8384a2fdbe5579fa86605abe9616f2fc8fe10a7b56b94f267506",
+             "shapes": {(4096, 4096, 14336): 67853312 + 69395456}},
+    "cfg4": {"sources": RQ_SOURCES, "digest": "896c8adff1339690e1c145cc5a6f8f8c8444fcd6356b68930d84461b0011690c",
+             "shapes": {(16384, 4096, 32): 134233088 + 18386944}},
 }
 
 
