@@ -111,13 +111,21 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
                "r"(bytes)
                : "memory");
 }
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
-  asm volatile(
-      "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
+  if constexpr (CLUSTER)
+    asm volatile(
+        "{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+  else
+    asm volatile(
+        "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
   return ok != 0;
 }
 __device__ __forceinline__ uint64_t global_timer_ns() {
@@ -128,14 +136,15 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
 // Bounded wait.  Returns false (after recording the site) if the phase has not completed within
 // `budget_ns`.  The first probe costs nothing extra; the timer is read once per 32 failed probes
 // (each failed try_wait already suspends the thread for a hardware-defined interval).
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned site,
                                           uint64_t budget_ns = kWaitBudgetNs) {
-  if (mbar_try_wait(bar, parity)) return true;
+  if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
   const uint64_t t0 = global_timer_ns();
   do {
 #pragma unroll 1
     for (int i = 0; i < 32; ++i)
-      if (mbar_try_wait(bar, parity)) return true;
+      if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
   } while (global_timer_ns() - t0 <= budget_ns);
   report_timeout(site);
   return false;
@@ -212,6 +221,11 @@ __device__ __forceinline__ void bulk_load_1d_elect(uint32_t dst, const void* src
 // Bounded wait executed by a whole converged warp; the result is the same in every lane.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, unsigned site) {
   const bool ok = mbar_wait(bar, parity, site);
+  return __all_sync(0xFFFFFFFFu, ok);
+}
+// The same for a barrier on which CTAs of the cluster count what they write here (and so with an acquire of the cluster's scope).
+__device__ __forceinline__ bool mbar_wait_warp_cluster(uint32_t bar, uint32_t parity, unsigned site) {
+  const bool ok = mbar_wait<true>(bar, parity, site);
   return __all_sync(0xFFFFFFFFu, ok);
 }
 

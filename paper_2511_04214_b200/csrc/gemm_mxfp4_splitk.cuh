@@ -10,13 +10,16 @@
 //     and sends its fp32 partial sums to the CTAs that own the tokens (distributed shared memory); a token's
 //     owner adds the parts in rank order, converts and stores.  No workspace, no atomics, fixed order.
 //   * FUSED (the whole-layer calls with at most 64 tokens, see plan()): there is no rotate+quantize kernel in front.
-//     Sixteen warps, eight of them those of the epilogue, rotate and quantise the [tokens, 256] slice of x of every K
+//     8 or 16 warps, eight of them those of the epilogue, rotate and quantise the [tokens, 256] slice of x of every K
 //     step straight into the stage (a lane owns one MX group, the arithmetic is that of the stand-alone kernel, bit for
 //     bit) and arrive on its barrier beside the weight bytes.  Every CTA repeats the work on its K range, hidden behind the weights; the
 //     first tile of columns also leaves codes and scales in the caller's workspace, as the stand-alone kernel would.
 //   * otherwise, with W packed before the previous kernel in the stream started (the whole-layer calls), the whole ring of
 //     weight tiles is requested before griddepcontrol.wait, under the rotate+quantize kernel.
-// Warps: 0 TMA producer, 1 TMEM owner and MMA issuer, 2..9 epilogue (FUSED: 2..17 quantise).  Every mbarrier wait is bounded, and all
+// A launch is a chain, and so is a decoding step of many.  FUSED lets the next kernel in (launch_dependents) once the last load has been
+// requested; where that one's CTAs fit beside these, they have set up when these end.  At the start instead, they compete for the loads:
+// (16, 4096, 4096) 5.1 -> 6.3 us, (1, 8192, 28672) 21.3 -> 21.8.  Without a quantiser the next kernel is a small one, let in at the start.
+// Warps: 0 TMA producer, 1 TMEM owner and MMA issuer, 2.. epilogue (FUSED: quantise before).  Every mbarrier wait is bounded, and all
 // threads of a cluster reach both cluster barriers whatever happened before.
 #pragma once
 
@@ -28,17 +31,18 @@ namespace bro {
 namespace gemms {
 
 constexpr int kEpilogueWarps = 8;                // two per TMEM lane quadrant
-constexpr int kQuantWarps = 16;                  // FUSED: the epilogue warps and as many more rotate and quantise
-constexpr int kThreads = (2 + kEpilogueWarps) * 32, kThreadsFused = (2 + kQuantWarps) * 32;
+constexpr int threads_of(int quant_warps) { return (2 + (quant_warps > kEpilogueWarps ? quant_warps : kEpilogueWarps)) * 32; }
 constexpr int kRowsW = 128;                      // rows of W per MMA
 constexpr int kMaxTokens = 128;                  // tokens per tile
-constexpr int kMaxTokensFused = 4 * kQuantWarps; // FUSED: a warp quantises 4 tokens of a K step
+constexpr int kCountedTokens = 32;               // of a tile whose parts are exchanged by counted stores (see the epilogue)
+constexpr int kMaxTokensFused = 64;              // FUSED: a warp task of a K step, 4 tokens, for each of at most 16 warps
 constexpr int kWTileBytes = kRowsW * 128;        // 16 KiB: one 256-element K step of 128 rows
 constexpr int kScaleBytes = 1024;                // its scales: 2 blocks of 512 B
 constexpr int kMaxStages = 11;
 constexpr int kMaxSplit = 8;                     // portable cluster size
 constexpr int kMaxSmem = 227 * 1024;
 constexpr int kFixedSmem = 1024 /*align*/ + 256 /*barriers*/;
+static_assert(8 * (2 * kMaxStages + 2) + 4 <= 256, "barriers and the TMEM address");
 constexpr int kScaleCols = 32;                   // TMEM columns kept for scales: W 2 x 8, tokens 2 x 4
 constexpr int kTmemCols = 256;                   // accumulators below them: 128 tokens, or 2 row blocks of at most 64
 static_assert(kMaxTokens + kScaleCols <= kTmemCols && 2 * 64 + kScaleCols <= kTmemCols, "accumulators and scales share the columns");
@@ -55,8 +59,8 @@ struct Params {
   int split;                // CTAs of a cluster, K parts of a tile
   int groups;               // split > 1: groups of 4 tokens that each CTA of a cluster owns
   int groups_magic;         // ceil(65536 / groups): i / groups == (i * groups_magic) >> 16 for i < 32
-  int stages, stage_bytes;
-  int a_box_bytes;          // bytes one activation box brings (rows beyond M up to the next power of two)
+  int stages;
+  int tok_bytes;            // token codes of a stage: what one box brings (rows beyond M up to the next power of two; FUSED: all columns)
   int tmem_cols;            // kTmemCols
   int out_f32;
   int w_static;             // the weight operand was complete before the previous kernel started
@@ -69,13 +73,20 @@ struct Params {
   int groups_k;             // K / 32
   int log2b;                // rotation size 2^1 .. 2^7
   uint32_t cbits;           // fp32 bits of 2^(-log2b / 2)
-  int token_quads;          // ceil(M / 4): warp tasks per K step
+  int log2_quads;           // groups of 4 tokens, rounded up to a power of two: warp tasks per K step
 };
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void st_cluster_128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+// 16 bytes into the shared memory of a CTA of the cluster, counted on a barrier of that CTA.
+__device__ __forceinline__ void st_async_128(uint32_t addr, uint32_t bar, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%2, %3, %4, %5}, [%1];" ::"r"(addr), "r"(bar), "r"(a),
+               "r"(b), "r"(c), "r"(d)
+               : "memory");
 }
 __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
@@ -85,6 +96,8 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "r"(taddr)
       : "memory");
 }
+
+__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) { asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
 
 // One token's value of the row of W (column n of y) that this lane holds.
 __device__ __forceinline__ void store_f32(void* y, int64_t at, uint32_t v) { static_cast<uint32_t*>(y)[at] = v; }
@@ -104,12 +117,12 @@ __device__ __forceinline__ void l2_prefetch_2d_elect(const CUtensorMap* m, int x
       : "memory");
 }
 
-// Rotation of size 2^log2b (a run-time value) and quantisation of one MX group per lane; groups of a block sit in
-// neighbouring lanes.  Same operations in the same order as the stand-alone kernel's.
-__device__ __forceinline__ uint32_t rotate_quantize_lane(const uint4 (&v)[4], int log2b, uint32_t cbits, int lane, uint32_t (&w)[4]) {
-  uint64_t P[16];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) rq::unpack_stage1(v[j], P + 4 * j);
+// Rotation of size 2^LOG2B (0: log2b_run) and quantisation of one MX group per lane; groups of a block sit in neighbouring lanes.  Same
+// operations in the same order as the stand-alone kernel's.
+template <int LOG2B>
+__device__ __forceinline__ uint32_t rotate_quantize_lane(uint64_t (&P)[16], int log2b_run, uint32_t cbits_run, int lane, uint32_t (&w)[4]) {
+  const int log2b = LOG2B ? LOG2B : log2b_run;
+  const uint32_t cbits = LOG2B ? rq::norm_bits<LOG2B>() : cbits_run;
 #pragma unroll
   for (int s = 0; s < 4; ++s) {
     if (log2b >= s + 2) {
@@ -129,20 +142,22 @@ __device__ __forceinline__ uint32_t rotate_quantize_lane(const uint4 (&v)[4], in
   return rq::quantize_group(P, cbits, w);
 }
 
-template <int ROW_BLOCKS, bool FUSED>
-__global__ void __launch_bounds__(FUSED ? kThreadsFused : kThreads, 1)
+template <int ROW_BLOCKS, int QUANT_WARPS>
+__global__ void __launch_bounds__(threads_of(QUANT_WARPS), QUANT_WARPS == 8 ? 2 : 1)
 gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_constant__ CUtensorMap tmw, const Params p) {
+  constexpr bool FUSED = QUANT_WARPS > 0;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  // stage: W tiles | token tile | W scales | token scales; behind the ring (split > 1) the parts received, the barriers
-  constexpr uint32_t w_bytes = (uint32_t)ROW_BLOCKS * kWTileBytes;
-  const uint32_t off_sfw = w_bytes + (uint32_t)p.tokens * 128u;
-  const uint32_t off_sfa = off_sfw + (uint32_t)ROW_BLOCKS * kScaleBytes;
-  const uint32_t parts = smem_base + (uint32_t)(p.stages * p.stage_bytes);     // [source rank][group][row][4 tokens] fp32
+  // stages of W tiles and W scales; token codes of all stages; token scales of all stages; (split > 1) the parts received; the barriers
+  constexpr uint32_t w_bytes = (uint32_t)ROW_BLOCKS * kWTileBytes, w_stage = w_bytes + (uint32_t)ROW_BLOCKS * kScaleBytes;
+  const uint32_t tok = smem_base + (uint32_t)p.stages * w_stage;
+  const uint32_t sfa = tok + (uint32_t)(p.stages * p.tok_bytes);
+  const uint32_t parts = sfa + (uint32_t)p.stages * kScaleBytes;               // [source rank][group][row][4 tokens] fp32
   const uint32_t bar_full = parts + (p.split > 1 ? (uint32_t)(p.split * p.groups) * (kRowsW * 16u) : 0u);   // [kMaxStages]
   const uint32_t bar_empty = bar_full + 8 * kMaxStages;                        // [kMaxStages]
   const uint32_t bar_acc = bar_empty + 8 * kMaxStages;
-  const uint32_t tmem_slot = bar_acc + 8;
+  const uint32_t bar_parts = bar_acc + 8;     // the parts sent to this CTA
+  const uint32_t tmem_slot = bar_parts + 8;
   uint32_t* tmem_slot_ptr = reinterpret_cast<uint32_t*>(smem_raw + (tmem_slot - smem_u32(smem_raw)));
 
   const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);
@@ -153,28 +168,34 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
   const int k_each = p.num_k_steps / p.split, k_more = p.num_k_steps - k_each * p.split;
   const int k_first = rank * k_each + min(rank, k_more), k_count = k_each + (rank < k_more ? 1 : 0);
 
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < p.stages; ++s) {
-      mbar_init(bar_full + 8 * s, FUSED ? 1u + kQuantWarps : 1u);
-      mbar_init(bar_empty + 8 * s, 1);
+  const int live = (int)(p.M - m0 < p.tokens ? p.M - m0 : p.tokens);       // tokens of this tile that exist
+
+  if (warp == 0) {
+    if (lane < p.stages) {
+      mbar_init(bar_full + 8 * lane, FUSED ? 1u + (1u << p.log2_quads) : 1u);
+      mbar_init(bar_empty + 8 * lane, 1);
+    } else if (lane == kMaxStages) {
+      mbar_init(bar_acc, 1);
+      mbar_init(bar_parts, 1);
     }
-    mbar_init(bar_acc, 1);
     mbar_fence_init();
     fence_proxy_async_smem();
-  }
-  if (warp == 1) {
+    if (lane == kMaxStages && p.split > 1) {  // 16 bytes a row, group of 4 tokens and source
+      const int mine = min(max((live + 3) / 4 - rank * p.groups, 0), p.groups);
+      mbar_arrive_expect_tx(bar_parts, (uint32_t)(mine * p.split) * (kRowsW * 16u));
+    }
+  } else if (warp == 1) {
     gemm::tmem_alloc(tmem_slot, (uint32_t)p.tmem_cols);
     gemm::tmem_relinquish();
-  }
-  if (threadIdx.x == 0) {
-    tma_prefetch_desc(&tma);
+  } else if (warp == 2 && lane == 0) {
+    if (!FUSED) tma_prefetch_desc(&tma);
     tma_prefetch_desc(&tmw);
   }
   gemm::tc_fence_before();
   __syncthreads();
   gemm::tc_fence_after();
   if (p.split > 1) cluster_arrive();          // (waited for before the first write to another CTA)
-  griddep_launch_dependents();
+  if (!FUSED) griddep_launch_dependents();
   const bool early_w = (FUSED || p.w_static != 0) && warp == 0;
   if (!early_w) griddep_wait();
   const uint32_t tmem_base = __shfl_sync(0xFFFFFFFFu, *tmem_slot_ptr, 0);
@@ -187,18 +208,18 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
     const int blocks = ROW_BLOCKS == 2 && (int64_t)n0 + kRowsW < p.N ? 2 : 1;
     // `part`: 1 the weight side, 2 the token side, 3 both
     auto issue_step = [&](int i, int st, int part) {
-      const uint32_t full = bar_full + 8 * st, base = smem_base + (uint32_t)(st * p.stage_bytes);
+      const uint32_t full = bar_full + 8 * st, base = smem_base + (uint32_t)st * w_stage;
       const int ks = k_first + i;
       if (part & 1) {
-        mbar_arrive_expect_tx_elect(full, w_bytes + (uint32_t)blocks * kScaleBytes + (FUSED ? 0u : (uint32_t)p.a_box_bytes + kScaleBytes));
+        mbar_arrive_expect_tx_elect(full, w_bytes + (uint32_t)blocks * kScaleBytes + (FUSED ? 0u : (uint32_t)p.tok_bytes + kScaleBytes));
         tma_load_2d_elect(base, &tmw, ks * 128, n0, full);                               // (rows beyond N arrive as zeros)
         const uint8_t* src = p.wscales + ((int64_t)(n0 / kRowsW) * p.kblocks + 2 * ks) * 512;
-        bulk_load_1d_elect(base + off_sfw, src, kScaleBytes, full);
-        if (blocks == 2) bulk_load_1d_elect(base + off_sfw + kScaleBytes, src + p.kblocks * 512, kScaleBytes, full);
+        bulk_load_1d_elect(base + w_bytes, src, kScaleBytes, full);
+        if (blocks == 2) bulk_load_1d_elect(base + w_bytes + kScaleBytes, src + p.kblocks * 512, kScaleBytes, full);
       }
       if (!FUSED && (part & 2)) {
-        tma_load_2d_elect(base + w_bytes, &tma, ks * 128, m0, full);
-        bulk_load_1d_elect(base + off_sfa, p.ascales + ((int64_t)tm * p.kblocks + 2 * ks) * 512, kScaleBytes, full);
+        tma_load_2d_elect(tok + (uint32_t)(st * p.tok_bytes), &tma, ks * 128, m0, full);
+        bulk_load_1d_elect(sfa + (uint32_t)st * kScaleBytes, p.ascales + ((int64_t)tm * p.kblocks + 2 * ks) * 512, kScaleBytes, full);
       }
     };
     int i = 0;
@@ -222,6 +243,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
       issue_step(i, stage, 3);
       if (++stage == p.stages) { stage = 0; phase ^= 1u; }
     }
+    if (FUSED) griddep_launch_dependents();
     if (!ok) {
       // do not leave while copies may still land: wait (bounded) for the last load armed on every stage
       for (int j = i > p.stages ? i - p.stages : 0; j < i; ++j)
@@ -237,9 +259,9 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
     for (int i = 0; i < k_count; ++i) {
       if (!mbar_wait_warp(bar_full + 8 * stage, phase, SITE_GEMM_FULL)) break;
       gemm::tc_fence_after();
-      const uint32_t base = smem_base + (uint32_t)(stage * p.stage_bytes);
-      const uint32_t w_lo = gemm::desc_lo_sw128(base), a_lo = gemm::desc_lo_sw128(base + w_bytes);
-      const uint32_t sfw_lo = gemm::desc_lo_sf(base + off_sfw), sfa_lo = gemm::desc_lo_sf(base + off_sfa);
+      const uint32_t base = smem_base + (uint32_t)stage * w_stage;
+      const uint32_t w_lo = gemm::desc_lo_sw128(base), a_lo = gemm::desc_lo_sw128(tok + (uint32_t)(stage * p.tok_bytes));
+      const uint32_t sfw_lo = gemm::desc_lo_sf(base + w_bytes), sfa_lo = gemm::desc_lo_sf(sfa + (uint32_t)stage * kScaleBytes);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {       // the two 128-element halves of the step own separate scale columns
         gemm::tc_cp_sf<1>(tmem_sfa + 4 * h, sfa_lo + 32u * h, gemm::kDescHiSf);
@@ -266,79 +288,74 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
   // ------------------------------ epilogue ------------------------------
   // A lane holds one row of W (column of y) and its tokens: a warp's store of one token is 64 (fp32: 128)
   // contiguous bytes.  Two warps per TMEM lane quadrant share the row blocks or the chunks of 16 tokens.
-  const int live = (int)(p.M - m0 < p.tokens ? p.M - m0 : p.tokens);       // tokens of this tile that exist
   const int q = warp & 3, half = (warp - 2) >> 2;
   const uint32_t tmem_acc = tmem_base + ((uint32_t)(q * 32) << 16);
   bool ok = true;
   if (FUSED && warp >= 2) {
     // ------------------------------ rotate + quantise x ------------------------------
-    // One warp task: 4 tokens x the 8 groups of a K step, one group per lane; task t goes to warp t mod 16.  (At most 64
-    // tokens, so a warp has one task of a step or none; the loop below takes any number, and as a straight block it
-    // measured slower, (64, 2048, 2048) 6.45 -> 6.55 us.)
-    const int in_quad = lane >> 3, g = lane & 7;
-    auto load = [&](int step, int quad, uint4 (&v)[4]) {
-      const int token = quad * 4 + in_quad, group = (k_first + step) * 8 + g;
-      const bool in = token < live && group < p.groups_k;
-      const uint4* src = reinterpret_cast<const uint4*>(p.x + (int64_t)(in ? token : 0) * p.ldx + (int64_t)(in ? group : 0) * 32);
+    // One warp task: 4 tokens x the 8 groups of a K step, one group per lane.  The groups of 4 tokens, as many as the next power of two, go
+    // to as many warps, and where these are fewer the steps are dealt out too: a warp has the same tokens throughout, so that rows and
+    // addresses are computed once.  The default rotation has code of its own: with the size a value of the run throughout, a task took
+    // 520 instructions instead of 330, and (64, 2048, 2048) 6.7 us instead of 6.3.  (Half a group a lane, and all of it in the 56 registers
+    // that would let two CTAs of 16 such warps share an SM: 7.6 to 8.1 us.)
+    const int w = warp - 2, every = QUANT_WARPS >> p.log2_quads, first = w >> p.log2_quads;
+    const int g = lane & 7, row = (w & ((1 << p.log2_quads) - 1)) * 4 + (lane >> 3);
+    const uint32_t tok_at = tok + (uint32_t)(row * 128) + (uint32_t)((g ^ (row & 7)) << 4);
+    const uint32_t sf_at = (uint32_t)((g >> 2) * 512 + (row & 31) * 16 + (row >> 5) * 4);
+    const int64_t x_at = (int64_t)k_first * 256 + g * 32;
+    uint4 cur[4];
+    auto load = [&](int step) {
+      cur[0] = cur[1] = cur[2] = cur[3] = make_uint4(0u, 0u, 0u, 0u);               // padding quantises to zeros
+      if (row < live && (k_first + step) * 8 + g < p.groups_k) {
+        const uint4* src = reinterpret_cast<const uint4*>(p.x + (int64_t)row * p.ldx + x_at + step * 256);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = in ? __ldg(src + j) : make_uint4(0u, 0u, 0u, 0u);     // padding quantises to zeros
-      if (p.signs && in) {
-        const uint4* sp = reinterpret_cast<const uint4*>(p.signs + (int64_t)group * 32);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) v[j] = rq::apply_signs(v[j], __ldg(sp + j));
+        for (int j = 0; j < 4; ++j) cur[j] = __ldg(src + j);
       }
     };
-    auto advance = [&](int& step, int& quad) {
-      quad += kQuantWarps;
-      while (quad >= p.token_quads) { quad -= p.token_quads; ++step; }
-    };
-    int step = 0, quad = warp - 2 - kQuantWarps;      // this warp's next task
-    advance(step, quad);
-    uint4 cur[4];
-    if (step < k_count) load(step, quad, cur);
-    // Every warp arrives for every step, with or without a task in it: a warp that skipped steps could find the ring two
-    // rounds away from what it saw last, and a parity tells a phase from its neighbours only.
+    if (first < k_count) load(first);
     int stage = 0;
-    uint32_t phase = 1u;                                 // (parity of the phase before the first: passes at once)
+    uint32_t phase = 1u;                                 // (parity of the phase before the first)
     for (int i = 0; i < k_count; ++i) {
-      const uint32_t base = smem_base + (uint32_t)(stage * p.stage_bytes);
-      bool waited = false;
-      do {
-        const bool has = step == i;
-        const int row = quad * 4 + in_quad;
-        uint32_t w[4], sb = 0u;
-        if (has) {
-          sb = rotate_quantize_lane(cur, p.log2b, p.cbits, lane, w);
-          advance(step, quad);
-          if (step < k_count) load(step, quad, cur);     // in flight while this task's stage is waited for and written
-          // scale bytes of 4 consecutive groups -> one 32-bit word in the lane with g % 4 == 0
-          sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 1) << 8;
-          sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 2) << 16;
+      // Every warp waits for every step of a stage used again, its own or not: a warp that skipped some could find the ring two rounds
+      // away from what it saw last, and a parity tells a phase from its neighbours only.
+      if (i >= p.stages) {
+        ok = mbar_wait_warp(bar_empty + 8 * stage, phase, SITE_GEMM_EMPTY);
+        if (!ok) break;
+      }
+      if ((i & (every - 1)) == first) {
+        const int group = (k_first + i) * 8 + g;
+        if (p.signs && group < p.groups_k) {
+          const uint4* sp = reinterpret_cast<const uint4*>(p.signs + (int64_t)group * 32);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) cur[j] = rq::apply_signs(cur[j], __ldg(sp + j));
         }
-        if (!waited) ok = mbar_wait_warp(bar_empty + 8 * stage, phase, SITE_GEMM_EMPTY);
-        waited = true;
-        if (!has || !ok) break;
-        const uint32_t sf_at = (uint32_t)((g >> 2) * 512 + (row & 31) * 16 + (row >> 5) * 4);
-        gemm::sts128(base + w_bytes + (uint32_t)row * 128u + (uint32_t)((g ^ (row & 7)) << 4), w[0], w[1], w[2], w[3]);
-        if ((g & 3) == 0) asm volatile("st.shared.b32 [%0], %1;" ::"r"(base + off_sfa + sf_at), "r"(sb) : "memory");
+        uint64_t P[16];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) rq::unpack_stage1(cur[j], P + 4 * j);
+        if (i + every < k_count) load(i + every);             // (in flight while this task is computed)
+        uint32_t c[4];
+        uint32_t sb = p.log2b == 5 ? rotate_quantize_lane<5>(P, 5, 0u, lane, c) : rotate_quantize_lane<0>(P, p.log2b, p.cbits, lane, c);
+        // scale bytes of 4 consecutive groups -> one 32-bit word in the lane with lane % 4 == 0
+        sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 1) << 8;
+        sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 2) << 16;
+        gemm::sts128(tok_at + (uint32_t)(stage * p.tok_bytes), c[0], c[1], c[2], c[3]);
+        if ((lane & 3) == 0) sts32(sfa + (uint32_t)stage * kScaleBytes + sf_at, sb);
         if (tn == 0) {
-          const int group = (k_first + i) * 8 + g;
           if (row < live && group < p.groups_k)
-            *reinterpret_cast<uint4*>(p.codes + ((int64_t)row * p.groups_k + group) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-          if ((g & 3) == 0) *reinterpret_cast<uint32_t*>(p.scales + (int64_t)(k_first + i) * 1024 + sf_at) = sb;
+            *reinterpret_cast<uint4*>(p.codes + ((int64_t)row * p.groups_k + group) * 16) = make_uint4(c[0], c[1], c[2], c[3]);
+          if ((lane & 3) == 0) *reinterpret_cast<uint32_t*>(p.scales + (int64_t)(k_first + i) * 1024 + sf_at) = sb;
         }
-      } while (step == i);
-      if (!ok) break;
-      fence_proxy_async_smem();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar_full + 8 * stage);
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_full + 8 * stage);
+      }
       if (++stage == p.stages) { stage = 0; phase ^= 1u; }
     }
     if (tn == 0) {                            // the rows that pad the scale buffer to 128 read as zero
-      const int first = p.token_quads * 4;
-      for (int j = (int)threadIdx.x - 64; j < k_count * 2 * kRowsW; j += kQuantWarps * 32) {
+      const int pad_from = 4 << p.log2_quads;
+      for (int j = (int)threadIdx.x - 64; j < k_count * 2 * kRowsW; j += QUANT_WARPS * 32) {
         const int row = j & (kRowsW - 1);
-        if (row >= first)
+        if (row >= pad_from)
           *reinterpret_cast<uint32_t*>(p.scales + ((int64_t)k_first * 2 + j / kRowsW) * 512 + (row & 31) * 16 + (row >> 5) * 4) = 0u;
       }
     }
@@ -378,9 +395,12 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
       }
     }
   } else {
-    // (16-byte stores straight into the owners' shared memory; staged locally and sent as bulk copies, 128 tokens took
-    // 2 us longer)
-    cluster_wait();                           // every CTA of the cluster runs
+    // Straight into the owners' shared memory.  Up to 32 tokens the stores are counted on a barrier of the owner (st.async): a barrier of the
+    // cluster, whose release waits for every store of every CTA, takes 0.4 us more, (16, 4096, 4096) 5.0 : 5.5 us, (8, 1024, 1024) 3.4 : 3.6.
+    // More are more stores than one barrier counts in that time: (64, 4096, 4096) 7.9 : 7.6, (64, 14336, 4096) 11.2 : 11.0.  (Staged locally
+    // and sent as bulk copies, 128 tokens took 2 us longer.)
+    const bool counted = p.tokens <= kCountedTokens;
+    cluster_wait();                           // every CTA of the cluster runs, its barriers are ready
     if (epilogue && ok) {
       for (int c = half * 16; c < live; c += 32) {
         uint32_t r[16];
@@ -390,15 +410,22 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
         for (int g = 0; g < 4; ++g) {
           const int gi = (c >> 2) + g;
           const int owner = (gi * p.groups_magic) >> 16, slot = gi - owner * p.groups;
-          if (4 * gi < live)
-            st_cluster_128(gemm2::map_to_cta(parts + (uint32_t)(((rank * p.groups + slot) * kRowsW + q * 32 + lane) * 16), (uint32_t)owner),
-                           r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
+          if (4 * gi < live) {
+            const uint32_t to = gemm2::map_to_cta(parts + (uint32_t)(((rank * p.groups + slot) * kRowsW + q * 32 + lane) * 16), (uint32_t)owner);
+            if (counted) st_async_128(to, gemm2::map_to_cta(bar_parts, (uint32_t)owner), r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
+            else st_cluster_128(to, r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
+          }
         }
       }
     }
     __syncwarp();
-    cluster_arrive();
-    cluster_wait();                           // all parts have arrived; nobody writes here any more
+    if (counted) {
+      cluster_arrive_relaxed();               // this warp sends nothing any more
+      if (epilogue) ok = mbar_wait_warp_cluster(bar_parts, 0u, SITE_GEMM_ACC_FULL) && ok;
+    } else {
+      cluster_arrive();
+      cluster_wait();                         // all parts have arrived; nobody writes here any more
+    }
     if (epilogue && ok) {
       const int row = q * 32 + lane;
       const int64_t n = (int64_t)n0 + row;
@@ -418,6 +445,8 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
         if (n < p.N) store4((int64_t)(m0 + token) * p.ldy + n, v, live - token);
       }
     }
+    __syncwarp();
+    if (counted) cluster_wait();              // nobody writes into this CTA's shared memory any more
   }
   gemm::tc_fence_before();
   __syncthreads();
@@ -428,8 +457,8 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
 inline bro_status resident_clusters(int split, int sm_count, int* out) {
   static DeviceOnce attr, once[kMaxSplit + 1];
   bro_status rc = device_once(attr, nullptr, [&](int*) {
-    for (auto kernel : {gemm_mxfp4_splitk_kernel<1, false>, gemm_mxfp4_splitk_kernel<2, false>, gemm_mxfp4_splitk_kernel<1, true>,
-                        gemm_mxfp4_splitk_kernel<2, true>})
+    for (auto kernel : {gemm_mxfp4_splitk_kernel<1, 0>, gemm_mxfp4_splitk_kernel<2, 0>, gemm_mxfp4_splitk_kernel<1, 8>,
+                        gemm_mxfp4_splitk_kernel<2, 8>, gemm_mxfp4_splitk_kernel<1, 16>, gemm_mxfp4_splitk_kernel<2, 16>})
       if (!cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem),
                    "cudaFuncSetAttribute(gemm split-K)"))
         return BRO_ERR_CUDA;
@@ -441,7 +470,7 @@ inline bro_status resident_clusters(int split, int sm_count, int* out) {
   rc = device_once(once[split], &plus_one, [&](int* n) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(sm_count / split * split), 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.blockDim = dim3((unsigned)threads_of(0), 1, 1);
     cfg.dynamicSmemBytes = kMaxSmem;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -450,7 +479,7 @@ inline bro_status resident_clusters(int split, int sm_count, int* out) {
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (!cuda_ok(cudaOccupancyMaxActiveClusters(n, gemm_mxfp4_splitk_kernel<1, false>, &cfg), "occupancy(gemm split-K)"))
+    if (!cuda_ok(cudaOccupancyMaxActiveClusters(n, gemm_mxfp4_splitk_kernel<1, 0>, &cfg), "occupancy(gemm split-K)"))
       return BRO_ERR_CUDA;
     ++*n;
     return BRO_OK;
@@ -474,7 +503,7 @@ struct Plan {
 // warp tasks (4 tokens of one K step each) of the quantising warps.
 inline int64_t step_ns(int tokens) { return 90 + tokens; }
 inline int64_t exchange_ns(int tokens) { return tokens <= 64 ? 100 + 18 * tokens : 4500; }
-inline int64_t quantise_ns(int64_t tasks) { return 300 + 72 * tasks; }
+inline int64_t quantise_ns(int64_t tasks) { return 300 + 76 * tasks; }
 
 // K parts of a tile: among the cluster sizes whose clusters are all resident at once, the one of least cost.
 template <typename Cost>
@@ -511,11 +540,11 @@ inline bro_status best_split(int64_t tiles, int num_k_steps, int sm_count, Cost&
 //
 // fused = true asks for a plan that quantises inside the GEMM.  It saves the other kernel and costs the tasks of the quantising warps,
 // of which about half the time that the weights take from HBM hides; what is left may cost up to 2.9 us.  Whole layer, two kernels ->
-// fused, in a graph and called one by one: (1, 8192, 28672) 23.4 -> 21.0 and 23.0 -> 22.1 us, (3, 1024, 1024) 4.4 -> 3.4 and 4.9 -> 3.8,
-// (16, 2048, 2048) 4.9 -> 3.9 and 5.7 -> 4.4, (16, 4096, 4096) 5.5 -> 5.4 and 5.9 -> 5.4, (16, 8192, 28672) 23.8 -> 22.9 and 23.6 -> 24.2.  The
-// line was drawn when the second kernel cost the host 3 us and quantising few tokens took longer, and by now it lies too high:
-// (28, 4096, 4096) 5.9 -> 6.6 and 6.3 -> 6.5, (64, 2048, 2048) 6.0 -> 6.4 and 6.1 -> 6.8, (48, 1536, 4096) 5.4 -> 6.2 and 5.5 -> 6.2,
-// (24, 5120, 5120) 7.0 -> 8.5 and 6.6 -> 7.7, (16, 14336, 4096) 8.0 -> 10.1 and 8.2 -> 10.1.  Beyond it (32, 8192, 28672) 24.8 -> 29.5.
+// fused, in a graph: (1, 8192, 28672) 23.5 -> 21.0 us, (4, 1024, 1024) 4.4 -> 3.0, (16, 2048, 2048) 5.1 -> 3.7, (16, 4096, 4096)
+// 5.8 -> 4.8, (24, 4096, 4096) 6.1 -> 6.0, (64, 2048, 2048) 6.0 both (called one by one 6.6 -> 6.3), (16, 8192, 28672) 24.1 -> 23.5; not taken
+// (32, 8192, 28672) 24.1 -> 25.9, (24, 5120, 6144) 8.6 -> 8.9, (16, 5120, 14336) 10.2 -> 11.6.  Over 690 layers of 1 to 64 tokens, K 1024 to
+// 14336, N 1024 to 28672, the choice is on average within 0.6 % of the better of the two; single ones lose up to 14 %, (16, 5120, 19000)
+// 13.7 : 12.1, (8, 11008, 11008) 14.7 : 15.2, (48, 2048, 4096) 6.0 : 6.5.
 // With few K steps the line is lower, 1.25 us and 0.2 us a step: there the persistent kernel is quick, and no layer may be
 // slower in a graph than with it: (64, 512, 4096) persistent 5.1, two kernels 4.4, fused 5.4 us, (48, 1024, 8192) 6.3, 5.3
 // and 6.5, but (48, 1536, 4096) 6.6, 5.4 and 6.2.  More than 64 tokens are two tasks a warp and step and 128 columns:
@@ -583,23 +612,24 @@ inline bro_status launch(const Plan& pl, const Source* src, const void* acodes, 
   // stage held, finite fp4 codes under zero-padded scales, and feed columns that are never stored
   int a_rows = p.tokens;
   while (a_rows > 8 && a_rows / 2 >= M) a_rows /= 2;
-  p.a_box_bytes = a_rows * 128;
+  p.tok_bytes = (src ? p.tokens : a_rows) * 128;
   const int tile_groups = (int)((M < p.tokens ? M : p.tokens) + 3) / 4;
   p.groups = (tile_groups + p.split - 1) / p.split;
   p.groups_magic = (65536 + p.groups - 1) / p.groups;
-  p.stage_bytes = pl.row_blocks * (kWTileBytes + kScaleBytes) + p.tokens * 128 + kScaleBytes;
+  const int stage_bytes = pl.row_blocks * (kWTileBytes + kScaleBytes) + p.tok_bytes + kScaleBytes;
   const int parts = p.split > 1 ? p.split * p.groups * kRowsW * 16 : 0;
   const int steps = (p.num_k_steps + p.split - 1) / p.split;
-  p.stages = (kMaxSmem - kFixedSmem - parts) / p.stage_bytes;
+  p.stages = (kMaxSmem - kFixedSmem - parts) / stage_bytes;
   if (p.stages > kMaxStages) p.stages = kMaxStages;
   if (p.stages > steps) p.stages = steps;
   // At least a third of an SM, so that no third CTA of 256 TMEM columns can be resident and wait for columns that
   // CTAs of waiting clusters hold.
-  int smem = kFixedSmem + parts + p.stages * p.stage_bytes;
+  int smem = kFixedSmem + parts + p.stages * stage_bytes;
   if (smem < kMaxSmem / 3 + 1024) smem = kMaxSmem / 3 + 1024;
   p.tmem_cols = kTmemCols;       // (read by the kernel as a parameter: as a constant there, (64, 2048, 2048) took 6.6 us, not 6.45)
   p.groups_k = (int)(K / 32);
-  p.token_quads = (int)((M + 3) / 4);
+  p.log2_quads = 0;
+  while ((4 << p.log2_quads) < M) ++p.log2_quads;
   p.x = nullptr;
   p.ldx = 0;
   p.signs = nullptr;
@@ -615,7 +645,7 @@ inline bro_status launch(const Plan& pl, const Source* src, const void* acodes, 
     p.codes = static_cast<uint8_t*>(const_cast<void*>(acodes));
     p.scales = static_cast<uint8_t*>(const_cast<void*>(ascales));
     p.log2b = src->log2b;
-    p.cbits = (src->log2b % 2 == 0) ? (uint32_t)(127 - src->log2b / 2) << 23 : 0x3FB504F3u - ((uint32_t)((src->log2b + 1) / 2) << 23);
+    p.cbits = rq::norm_bits_of(src->log2b);
   } else {
     rc = gemm::make_codes_map(&tma, acodes, M, K, a_rows);
     if (rc != BRO_OK) return rc;
@@ -627,9 +657,16 @@ inline bro_status launch(const Plan& pl, const Source* src, const void* acodes, 
   rc = resident_clusters(p.split, sm_count, &fit);      // (also the opt-in to large shared memory)
   if (rc != BRO_OK) return rc;
   const unsigned grid = (unsigned)(pl.tiles_m * pl.tiles_n * p.split);
-  auto kernel = src ? (pl.row_blocks == 2 ? gemm_mxfp4_splitk_kernel<2, true> : gemm_mxfp4_splitk_kernel<1, true>)
-                    : (pl.row_blocks == 2 ? gemm_mxfp4_splitk_kernel<2, false> : gemm_mxfp4_splitk_kernel<1, false>);
-  return cuda_ok(launch_kernel(kernel, grid, src ? kThreadsFused : kThreads, (size_t)smem, st, (unsigned)p.split, tma, tmw, p),
+  // With few warp tasks in all (4 tokens of a K step each) eight warps quantise: their CTA is small enough for the next layer's to stand beside it
+  // before it ends, where shared memory allows.  16 -> 8 warps, (16, 4096, 4096) 5.4 -> 5.0 us, (16, 2048, 4096) 4.7 -> 4.0, (1, 8192, 28672)
+  // 21.5 -> 21.2; more tasks need the 16: (16, 4096, 8192), 32 tasks, 6.7 : 7.2, (16, 14336, 4096) 9.5 : 11.3; tiles of 256 rows stream
+  // twice the weights beside them, (16, 3072, 19000), 48 tasks, 9.1 -> 8.8, (16, 5120, 19000), 80, 12.1 : 12.8.
+  int quant_warps = 0;
+  if (src) quant_warps = p.log2_quads == 0 || (p.log2_quads <= 3 && (steps << p.log2_quads) <= (pl.row_blocks == 1 ? 24 : 48)) ? 8 : 16;
+  auto kernel = quant_warps == 8    ? (pl.row_blocks == 2 ? gemm_mxfp4_splitk_kernel<2, 8> : gemm_mxfp4_splitk_kernel<1, 8>)
+                : quant_warps == 16 ? (pl.row_blocks == 2 ? gemm_mxfp4_splitk_kernel<2, 16> : gemm_mxfp4_splitk_kernel<1, 16>)
+                                    : (pl.row_blocks == 2 ? gemm_mxfp4_splitk_kernel<2, 0> : gemm_mxfp4_splitk_kernel<1, 0>);
+  return cuda_ok(launch_kernel(kernel, grid, (unsigned)threads_of(quant_warps), (size_t)smem, st, (unsigned)p.split, tma, tmw, p),
                  "gemm_mxfp4 split-K launch")
              ? BRO_OK
              : BRO_ERR_CUDA;

@@ -63,6 +63,11 @@ __device__ __forceinline__ constexpr uint32_t norm_bits() {
                           : 0x3FB504F3u - ((uint32_t)((LOG2B + 1) / 2) << 23);
 }
 
+// the same for a run-time log2b
+__host__ __device__ inline uint32_t norm_bits_of(int log2b) {
+  return (log2b % 2 == 0) ? (uint32_t)(127 - log2b / 2) << 23 : 0x3FB504F3u - ((uint32_t)((log2b + 1) / 2) << 23);
+}
+
 // ---- packed fp32x2 arithmetic (sm_100): one issue slot for two IEEE round-to-nearest results.
 // A group's 32 values live in 16 register pairs; pair k holds elements (2k, 2k+1).
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
@@ -223,6 +228,38 @@ __device__ __forceinline__ uint32_t encode_pairs8(const uint64_t (&P)[8], float 
     w[j] = pack_e2m1x8(r[8 * j], r[8 * j + 1], r[8 * j + 2], r[8 * j + 3], r[8 * j + 4], r[8 * j + 5],
                        r[8 * j + 6], r[8 * j + 7]);
   return s;
+}
+
+// A group in four neighbouring lanes, 8 values each: the lane's 8 codes, and the group's scale byte in every lane (same arithmetic as
+// quantize_group).
+__device__ __forceinline__ uint32_t encode_pairs4(const uint64_t (&P)[4], uint32_t cbits, uint32_t& scale) {
+  float v[8];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) unpack2(P[k], v[2 * k], v[2 * k + 1]);
+  float m = 0.f, m2 = 0.f;
+  asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(v[0]), "f"(v[1]));
+  asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m2) : "f"(v[2]), "f"(v[3]));
+  asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(v[4]), "f"(v[5]));
+  asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m2) : "f"(v[6]), "f"(v[7]));
+  m = fmaxf(m, m2);
+  m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 1));
+  m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, 2));
+  const float c = __uint_as_float(cbits);
+  const uint32_t ef = __float_as_uint(__fmul_rn(m, c)) >> 23;
+  const uint32_t s = ef > 2u ? ef - 2u : 0u;
+  scale = s;
+  if (ef >= 27u && ef <= 250u) {
+    const float c2 = __uint_as_float(cbits + ((127u - s) << 23));
+    const uint64_t cc = pack2(c2, c2);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) unpack2(mul2(P[k], cc), v[2 * k], v[2 * k + 1]);
+  } else {
+    const float p2 = __uint_as_float((254u - s) << 23);
+    const uint64_t cc = pack2(c, c), pp = pack2(p2, p2);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) unpack2(mul2(mul2(P[k], cc), pp), v[2 * k], v[2 * k + 1]);
+  }
+  return pack_e2m1x8(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]);
 }
 
 // The cross-lane stages of a 64- or 128-channel block on the registers described above, then the

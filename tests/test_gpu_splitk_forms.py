@@ -1,0 +1,47 @@
+"""The forms of the split-K kernel that its plan chooses between by tokens and tasks: parts exchanged by counted stores or over a barrier of
+the cluster, eight or sixteen quantising warps.  The outputs against the persistent kernel on the operands that the layer leaves in its
+workspace, and those against the rotate+quantise kernel bit for bit."""
+import pytest
+import torch
+
+from gpu_util import kernels_of
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M,K,N,warps", [
+    (1, 14336, 256, 8),        # one group of 4 tokens: a warp each step, eight parts of seven steps
+    (4, 8192, 19000, 8),       # the same over tiles of 256 rows, a ring used again
+    (5, 4096, 4096, 8),        # a second group with one token
+    (16, 4096, 4096, 8),
+    (16, 2048, 11008, 16),     # 32 tasks, one part
+    (17, 2048, 2048, 8),       # five groups on eight warps
+    (32, 1024, 2048, 8),       # the last tokens that are counted
+    (33, 1024, 2048, 16),      # the first that are not
+    (33, 1056, 1000, 16),      # and a half-empty last step
+    (64, 2048, 2048, 16),
+])
+def test_one_kernel_layer(M, K, N, warps):
+    from paper_2511_04214_b200 import binding as bro
+    gen = torch.Generator(device="cuda").manual_seed(M * K + N)
+    x = torch.randn(M, K, generator=gen, device="cuda").to(torch.bfloat16)
+    wc, ws = bro.alloc_codes(N, K), bro.alloc_scales(N, K, bro.LAYOUT_GEMM)
+    bro.pack_weights((torch.randn(N, K, generator=gen, device="cuda") * 0.02).to(torch.bfloat16), 32, wc, ws)
+    work = bro.alloc_workspace(bro.linear_workspace_bytes(M, N, K))
+    y = torch.empty(M, (N + 7) // 8 * 8, dtype=torch.bfloat16, device="cuda")[:, :N]
+    layer = lambda: bro.linear(x, 32, wc, ws, N, y, work)  # noqa: E731
+    (name,) = kernels_of(layer)
+    assert f"gemm_mxfp4_splitk_kernelILi{2 if N > 148 * 128 else 1}ELi{warps}E" in name
+    work.fill_(0x5A), y.fill_(float("nan"))
+    for _ in range(3):
+        layer()                                            # (right behind one another: a CTA may start beside the one before it)
+    assert bro.last_device_status() == 0
+    ac, asc = bro.alloc_codes(M, K), bro.alloc_scales(M, K, bro.LAYOUT_GEMM)
+    bro.rotate_quantize_mxfp4(x, 32, ac, asc)
+    at = (ac.numel() + 1023) // 1024 * 1024
+    assert torch.equal(work[:ac.numel()], ac.flatten()) and torch.equal(work[at:at + asc.numel()], asc)
+    ref = torch.empty_like(y)
+    bro.gemm_mxfp4(ac, asc, wc, ws, M, N, K, ref, flags=bro.FLAG_GEMM_SINGLE)
+    # the same sums in another order, then one rounding to bf16: at most one ulp, 2^-8 of the row's largest magnitude
+    top = ref.float().abs().amax(1, keepdim=True)
+    assert ((y.float() - ref.float()).abs() <= top * 2.0 ** -8).all()
