@@ -11,6 +11,7 @@
 #include "rotate_quantize_global.cuh"
 #include "rotate_quantize_direct.cuh"
 #include "rotate_quantize_wide.cuh"
+#include "rotate_quantize_few.cuh"
 #include "gemm_mxfp4.cuh"
 #include "gemm_mxfp4_2cta.cuh"
 #include "gemm_mxfp4_splitk.cuh"
@@ -259,6 +260,15 @@ bro_status launch_rotate_quantize(const void* x, int64_t M, int64_t K, int64_t l
   if (B > 128) {
     return bro::rqg::launch(x, M, K, ldx, signs, codes, scales, nullptr, 0, layout, gemm_scale_kblocks(K), di.sm_count, st);
   }
+
+  // One block of tiled scales and no more tasks than the warps that one CTA an SM gives: the kernel of a quarter group a lane, with the
+  // producer always, without it from 65 rows on (below, the register-streaming kernel in its spread form takes 1.3 us and this one 1.5).
+  // [16, 14336] gated 3.4 -> 2.1 us, [64, 4096] 2.4 -> 2.1, [100, 4384] 2.5 -> 2.3; plain [80, 2048] 1.82 -> 1.65, [128, 4384] 1.9 -> 1.7.
+  // In front of a GEMM its registers would keep that one's CTAs out, (104, 2048, 11584) 6.65 -> 7.2, which a plain rotation does not outweigh.
+  // Beyond, warps take several tasks in turn: gated [128, 8192] 3.2 : 3.4 us, plain [100, 8192] 2.1 : 2.4.
+  if (layout == BRO_LAYOUT_GEMM && M <= bro::rqf::kMaxRows && (up || (M > 64 && !layer)) && !(flags & (BRO_FLAG_RQ_TMA_RING | BRO_FLAG_RQ_DIRECT)) &&
+      M * ceil_div(K, 256) <= (int64_t)di.sm_count * bro::rqf::kWarps)
+    return bro::rqf::launch(x, M, K, ldx, log2_of(B), signs, codes, scales, di.sm_count, st, up, ldu);
 
   // In front of a GEMM (`layer`) the wide kernel has to save more, since its shared memory keeps the GEMM's CTAs from starting under its
   // tail: beyond 2^22 elements, block 32 from 2^24 (whole layers, block 64: (1500, 5120, 2500) 19.9 -> 18.8, (2048, 2048, 8192) 21.1 -> 21.5,
@@ -825,7 +835,7 @@ bro_status bro_swiglu_linear(const void* gate_bf16, const void* up_bf16, int64_t
   uint8_t* ascales = acodes + align_up(bro_codes_bytes(M, K), 1024);
   uint8_t* gws = ascales + align_up(bro_scales_bytes(M, K, BRO_LAYOUT_GEMM), 1024);
   bro_status rc = launch_rotate_quantize(gate_bf16, M, K, ldg, block, signs_bf16, acodes, ascales, BRO_LAYOUT_GEMM, 0u,
-                                         static_cast<cudaStream_t>(stream), up_bf16, ldu);
+                              static_cast<cudaStream_t>(stream), up_bf16, ldu);
   if (rc != BRO_OK) return rc;
   return gemm_impl(acodes, ascales, wcodes, wscales, M, N, K, y_bf16, ldy, BRO_OUT_BF16, gws,
                    bro_gemm_workspace_bytes(M, N, K), 0u, stream, true);

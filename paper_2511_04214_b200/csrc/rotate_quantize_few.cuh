@@ -1,0 +1,132 @@
+// Kernel 1 for few tokens (at most one block of 128 rows of the tiled scales): rotation + MXFP4 quantisation with or without the fused
+// producer h = silu(gate) * up (paper Sec. 4.3 Eq. 1, Sec. 4.1, Sec. 6), as it stands in front of a GEMM that is one pass over the weights.
+//
+// Such a call is a chain of latencies: the kernel before ends, x arrives, is rotated and stored, the GEMM begins.  So a LANE has 8
+// consecutive channels and a warp one K step of a row (256 channels): one 16-byte load a lane, three stages in registers, the others and
+// the group's maximum across lanes, a third of the instructions in a row that a whole group in a lane takes.  The sigmoid is computed:
+// a table in shared memory (the gated kernel for more tokens) has to be filled first and, with its ring, keeps the CTA from
+// starting before the GEMM in front has ended; here nothing is held in shared memory, and with 16 warps no more than two CTAs fit an SM
+// that happens to be empty early (of 8 warps, up to eight did, and the last of them ended 1 us after the others).
+// [16, 14336] gated 3.62 -> 2.15 us, with its GEMM (N = 4096) 11.3 -> 9.1; what is left is the start, a load, the chain and a store.
+#pragma once
+
+#include "bro_common.cuh"
+#include "rotate_quantize.cuh"
+#include "rotate_quantize_direct.cuh"
+
+namespace bro {
+namespace rqf {
+
+constexpr int kThreads = 512, kWarps = kThreads / 32;
+constexpr int kMaxRows = 128;
+
+struct Params {
+  const uint16_t* x;
+  const uint16_t* up;                     // the fused producer's second operand (GATED)
+  int64_t ldx, ldu;
+  int M, K, ksteps;                       // ceil(K / 256)
+  const uint16_t* signs;                  // [K] bf16 +-1 or nullptr
+  uint8_t* codes;                         // [M, K / 2]
+  uint8_t* scales;                        // tiled, one block of 128 rows
+  int log2b;                              // rotation size 2^1 .. 2^7
+  uint32_t cbits;                         // fp32 bits of 2^(-log2b / 2)
+};
+
+// Rotation of size 2^LOG2B (0: log2b_run) and quantisation of a quarter of an MX group per lane, 8 values, from the stage of stride 2 on.
+template <int LOG2B>
+__device__ __forceinline__ uint32_t rotate_quantize_quarter(uint64_t (&P)[4], int log2b_run, uint32_t cbits_run, int lane, uint32_t& scale) {
+  const int log2b = LOG2B ? LOG2B : log2b_run;
+  // stages of stride 2 and 4 in registers, 8 .. 64 across lanes: low lane a + b, high lane a - b, one rounding each
+#pragma unroll
+  for (int st = 0; st < 2; ++st) {
+    if (log2b >= st + 2) {
+      const int hp = 1 << st;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if ((k & hp) == 0) {
+          const uint64_t a = P[k], b = P[k + hp];
+          P[k] = rq::add2(a, b);
+          P[k + hp] = rq::sub2(a, b);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int st = 0; st < 4; ++st) {
+    if (log2b >= st + 4) {
+      const float sgn = (lane >> st) & 1 ? -1.f : 1.f;
+      const uint64_t sgn2 = rq::pack2(sgn, sgn);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) P[k] = rq::fma2(P[k], sgn2, rq::shfl_xor2(P[k], 1 << st));
+    }
+  }
+  return rq::encode_pairs4(P, LOG2B ? rq::norm_bits<LOG2B>() : cbits_run, scale);
+}
+
+template <bool GATED>
+__global__ void __launch_bounds__(kThreads)
+rotate_quantize_few_kernel(const Params p) {
+  const int lane = threadIdx.x & 31;
+  griddep_wait();               // x may be written, codes/scales still read, by the kernel before
+  griddep_launch_dependents();  // (only now: a dependent that starts early may then rely on everything older than this kernel)
+
+  const int tasks = p.M * p.ksteps, stride = (int)gridDim.x * kWarps;
+  int task = (int)(threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x;       // (neighbouring tasks on different SMs)
+  int row = task / p.ksteps, ks = task - row * p.ksteps;
+  const int step_row = stride / p.ksteps, step_k = stride - step_row * p.ksteps;
+  uint4 v, u, s;
+  auto load = [&](int r, int k) {
+    const int c = k * 256 + lane * 8;
+    v = u = s = make_uint4(0u, 0u, 0u, 0u);                                    // padding quantises to zeros
+    if (c < p.K) {
+      v = __ldg(reinterpret_cast<const uint4*>(p.x + r * p.ldx + c));
+      if (GATED) u = __ldg(reinterpret_cast<const uint4*>(p.up + r * p.ldu + c));
+      if (p.signs) s = __ldg(reinterpret_cast<const uint4*>(p.signs + c));
+    }
+  };
+  if (task < tasks) load(row, ks);
+  rq::clear_padding(p.scales, p.M, 2 * p.ksteps, (int64_t)blockIdx.x * kThreads + threadIdx.x, (int64_t)gridDim.x * kThreads);
+  while (task < tasks) {
+    uint64_t P[4];
+    rq::unpack_stage1(rq::apply_signs(GATED ? rqd::swiglu_bf16x8(v, u) : v, s), P);
+    const int row_now = row, ks_now = ks;
+    task += stride;
+    row += step_row;
+    ks += step_k;
+    if (ks >= p.ksteps) { ks -= p.ksteps; ++row; }
+    if (task < tasks) load(row, ks);                                           // (in flight while this task is computed)
+    uint32_t sb;
+    const uint32_t word = p.log2b == 5 ? rotate_quantize_quarter<5>(P, 5, 0u, lane, sb) : rotate_quantize_quarter<0>(P, p.log2b, p.cbits, lane, sb);
+    const int c = ks_now * 256 + lane * 8;
+    if (c < p.K) *reinterpret_cast<uint32_t*>(p.codes + (int64_t)row_now * (p.K >> 1) + (c >> 1)) = word;
+    // scale bytes of 4 consecutive groups, 4 lanes each -> one 32-bit word
+    sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 4) << 8;
+    sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 8) << 16;
+    if ((lane & 15) == 0)
+      *reinterpret_cast<uint32_t*>(p.scales + (ks_now * 2 + (lane >> 4)) * 512 + (row_now & 31) * 16 + (row_now >> 5) * 4) = sb;
+  }
+}
+
+inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, int log2b, const void* signs, void* codes, void* scales,
+                         int sm_count, cudaStream_t st, const void* up, int64_t ldu) {
+  Params p;
+  p.x = static_cast<const uint16_t*>(x);
+  p.up = static_cast<const uint16_t*>(up);
+  p.ldx = ldx;
+  p.ldu = ldu;
+  p.M = (int)M;
+  p.K = (int)K;
+  p.ksteps = (int)((K + 255) / 256);
+  p.signs = static_cast<const uint16_t*>(signs);
+  p.codes = static_cast<uint8_t*>(codes);
+  p.scales = static_cast<uint8_t*>(scales);
+  p.log2b = log2b;
+  p.cbits = rq::norm_bits_of(log2b);
+  return cuda_ok(launch_kernel(up ? rotate_quantize_few_kernel<true> : rotate_quantize_few_kernel<false>, (unsigned)sm_count, kThreads, 0, st, 1, p),
+                 "rotate_quantize_few launch")
+             ? BRO_OK
+             : BRO_ERR_CUDA;
+}
+
+}  // namespace rqf
+}  // namespace bro
