@@ -108,15 +108,27 @@ __device__ __forceinline__ uint64_t shfl_xor2(uint64_t v, int lane_mask) {
   return r;
 }
 
+// The two values of a word, lo and hi -> lo + hi and lo - hi.  The sum of a bf16 and an fp32 is one instruction (exact operands, one
+// rounding), so the low value needs no unpacking: 16 instructions of a group's 300 less, [16384, 4096] block 32 28.7 -> 28.1 us (at the power cap
+// 31.1 -> 30.2), block 128 30.6 -> 29.9, the full dimension 50.8 -> 50.0, the gated producer [4096, 14336] 45.8 -> 44.8.
+__device__ __forceinline__ void stage1(uint32_t word, float& sum, float& diff) {
+  const float hi = __uint_as_float(word & 0xFFFF0000u);
+  asm("{ .reg .b16 l, h; mov.b32 {l, h}, %2;\n\t"
+      "add.rn.f32.bf16 %0, l, %3;\n\t"
+      "sub.rn.f32.bf16 %1, l, %3; }"
+      : "=f"(sum), "=f"(diff)
+      : "r"(word), "f"(hi));
+}
+
 // 8 bf16 (one 16-byte chunk) -> 4 pairs, fused with butterfly stage h = 1, which pairs the two
 // halves of one 32-bit word: (lo, hi) -> (lo + hi, lo - hi).
 __device__ __forceinline__ void unpack_stage1(const uint4& q, uint64_t* P) {
   const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const float lo = __uint_as_float(w[k] << 16);
-    const float hi = __uint_as_float(w[k] & 0xFFFF0000u);
-    P[k] = pack2(__fadd_rn(lo, hi), __fsub_rn(lo, hi));
+    float sum, diff;
+    stage1(w[k], sum, diff);
+    P[k] = pack2(sum, diff);
   }
 }
 

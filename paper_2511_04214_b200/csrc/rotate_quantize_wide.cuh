@@ -70,15 +70,16 @@ __device__ __forceinline__ void stages_2_to_16(uint64_t (&P)[32]) {
 }
 
 // ---- block 32: the two groups of a lane side by side in the halves of packed registers, P[e] = (A_e, B_e) ----
-// Every stage is then packed arithmetic, the first too, and so are the multiplies by the two groups' scales.
+// Every stage but the first (see rq::stage1) is then packed arithmetic, and so are the multiplies by the two groups' scales.
 __device__ __forceinline__ void unpack_stage1_two(const uint4& a, const uint4& b, uint64_t* P) {
   const uint32_t wa[4] = {a.x, a.y, a.z, a.w}, wb[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const uint64_t lo = rq::pack2(__uint_as_float(wa[k] << 16), __uint_as_float(wb[k] << 16));
-    const uint64_t hi = rq::pack2(__uint_as_float(wa[k] & 0xFFFF0000u), __uint_as_float(wb[k] & 0xFFFF0000u));
-    P[2 * k] = rq::add2(lo, hi);
-    P[2 * k + 1] = rq::sub2(lo, hi);
+    float sa, da, sb, db;
+    rq::stage1(wa[k], sa, da);
+    rq::stage1(wb[k], sb, db);
+    P[2 * k] = rq::pack2(sa, sb);
+    P[2 * k + 1] = rq::pack2(da, db);
   }
 }
 __device__ __forceinline__ void stages_2_to_16_two(uint64_t (&P)[32]) {
