@@ -161,6 +161,24 @@ bro_status bro::rqg::make_row_map(CUtensorMap* map, const void* x, int64_t M, in
   return make_map_3d(map, x, M, K, ldx, 64, (uint32_t)(K / 64 < 256 ? K / 64 : 256), (uint32_t)box_rows, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
+// The even or the odd 128-byte segments of whole rows, with the 128-byte swizzle.
+bro_status bro::rqg::make_parity_map(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx, int box_rows) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn) {
+    snprintf(bro::g_last_cuda_error, sizeof(bro::g_last_cuda_error), "cuTensorMapEncodeTiled unavailable");
+    return BRO_ERR_CUDA;
+  }
+  cuuint64_t dims[4] = {64, 2, (cuuint64_t)(K / 128), (cuuint64_t)M};
+  cuuint64_t strides[3] = {128, 256, (cuuint64_t)ldx * 2};
+  cuuint32_t box[4] = {64, 1, (cuuint32_t)(K / 128), (cuuint32_t)box_rows};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS)
+    snprintf(bro::g_last_cuda_error, sizeof(bro::g_last_cuda_error), "cuTensorMapEncodeTiled (4-D): CUresult %d", (int)r);
+  return r == CUDA_SUCCESS ? BRO_OK : BRO_ERR_CUDA;
+}
+
 // 16 rows x 128 channels: 128-byte segments, two a row, with the 128-byte swizzle.
 bro_status bro::rqw::make_tile_map(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx) {
   return make_map_3d(map, x, M, K, ldx, 64, 2, kRows, CU_TENSOR_MAP_SWIZZLE_128B);

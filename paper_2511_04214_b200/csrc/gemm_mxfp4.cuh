@@ -211,10 +211,6 @@ template <int N>
 __device__ __forceinline__ void bulk_wait_read_elect() {
   asm volatile("{ .reg .pred q; elect.sync _|q, 0xffffffff;\n\t@q cp.async.bulk.wait_group.read %0; }" ::"n"(N) : "memory");
 }
-__device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-
 __device__ __forceinline__ uint32_t lds32(uint32_t addr) {
   uint32_t v;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");

@@ -97,8 +97,6 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "memory");
 }
 
-__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) { asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
-
 // One token's value of the row of W (column n of y) that this lane holds.
 __device__ __forceinline__ void store_f32(void* y, int64_t at, uint32_t v) { static_cast<uint32_t*>(y)[at] = v; }
 __device__ __forceinline__ void store_bf16_pair(void* y, int64_t at, int64_t ldy, uint32_t v0, uint32_t v1, bool second) {
@@ -338,7 +336,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
         // scale bytes of 4 consecutive groups -> one 32-bit word in the lane with lane % 4 == 0
         sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 1) << 8;
         sb |= __shfl_xor_sync(0xFFFFFFFFu, sb, 2) << 16;
-        gemm::sts128(tok_at + (uint32_t)(stage * p.tok_bytes), c[0], c[1], c[2], c[3]);
+        sts128(tok_at + (uint32_t)(stage * p.tok_bytes), c[0], c[1], c[2], c[3]);
         if ((lane & 3) == 0) sts32(sfa + (uint32_t)stage * kScaleBytes + sf_at, sb);
         if (tn == 0) {
           if (row < live && group < p.groups_k)

@@ -55,6 +55,18 @@ __device__ __forceinline__ uint32_t pack_e2m1x8(float r0, float r1, float r2, fl
   return w;
 }
 
+// the same for 4 values, in the low 16 bits (and once more in the high ones)
+__device__ __forceinline__ uint32_t pack_e2m1x4(float r0, float r1, float r2, float r3) {
+  uint32_t w;
+  asm("{ .reg .b8 b0, b1;\n\t"
+      "cvt.rn.satfinite.e2m1x2.f32 b0, %2, %1;\n\t"
+      "cvt.rn.satfinite.e2m1x2.f32 b1, %4, %3;\n\t"
+      "mov.b32 %0, {b0, b1, b0, b1}; }"
+      : "=r"(w)
+      : "f"(r0), "f"(r1), "f"(r2), "f"(r3));
+  return w;
+}
+
 // c = fp32 nearest 1/sqrt(2^LOG2B)
 template <int LOG2B>
 __device__ __forceinline__ constexpr uint32_t norm_bits() {

@@ -609,6 +609,192 @@ __global__ void __launch_bounds__(128, 5) rotate_quantize_global_few_kernel(cons
   if (threadIdx.x == 0 && it < iters) mbar_wait(bar, parity ^ 1u, SITE_RQ_DRAIN);
 }
 
+// ---- a warp for 4096 channels: codes and scale bytes of K = 1024, 2048 (four and two rows at a time) and 4096 ------------------------
+// The kernel of 64 values a thread passes a row through shared memory twice, since a thread that quantises needs whole runs, and meets at
+// barriers for it; its bound is those bytes.  Here a lane has 128 values and, after one pass, C = 4, 8 or 16 consecutive channels of every 128:
+// seven stages on its 128 consecutive channels, the rest between the 128s of a row, whose lanes exchange them.  The maximum of a group is then
+// spread over 32 / C lanes, which share the search for it: each is left with the maxima of four groups, finds their scales and gives them
+// back through shared memory.  Nothing is shared between warps: each has its rows (TMA, the even and the odd 128-byte segments
+// apart, so that the lanes read without conflicts) and its 16 KiB of exchange, and there is no barrier.  Two warps on each of an SM's four
+// schedulers, for the registers (a ninth leaves one of them with three: 62 us); bound by the latencies that two warps do not hide (issue 54 %).
+// Codes go out as they are, 64 bytes of a row a store: collected in shared memory first, K = 4096 took 47.3 us, not 44.5 (K = 2048 44.7, not 45.4).
+constexpr int kRowWarps = 8;
+constexpr int kRowWarpBytes = 8192 + 16384, kRowWarpSmem = kRowWarps * kRowWarpBytes + kRowWarps * 8 + 1024;
+template <int LOG2K, int MODE>
+__global__ void __launch_bounds__(kRowWarps * 32, 1) rotate_quantize_global_warp_kernel(const __grid_constant__ CUtensorMap tmx, const Params p) {
+  constexpr int K = 1 << LOG2K, LR = K / 128, ROWS = 32 / LR;      // lanes of a row, rows of a warp
+  constexpr int C = 128 / LR, GL = 32 / C;                         // channels of a lane in every 128, lanes of a group
+  static_assert(LOG2K >= 10 && LOG2K <= 12, "K = 1024, 2048, 4096");
+  extern __shared__ uint8_t smem_raw[];
+  const int lane = threadIdx.x & 31, warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);
+  const uint32_t raw = ((smem_u32(smem_raw) + 1023u) & ~1023u) + (uint32_t)(warp * kRowWarpBytes), xch = raw + 8192u;
+  const uint32_t bar = ((smem_u32(smem_raw) + 1023u) & ~1023u) + (uint32_t)(kRowWarps * kRowWarpBytes + warp * 8);
+  constexpr uint32_t cbits = rq::norm_bits<LOG2K>();
+  const int rs = lane / LR, L = lane % LR;                         // row of the warp's, lane of the row
+  if (lane == 0) {
+    mbar_init(bar, 1);
+    mbar_fence_init();
+    fence_proxy_async_smem();
+    tma_prefetch_desc(&tmx);
+  }
+  __syncwarp();
+  griddep_wait();               // x may be written, the outputs still read, by the kernel before
+  griddep_launch_dependents();
+  const int64_t tasks = (p.M + ROWS - 1) / ROWS, step = (int64_t)gridDim.x * kRowWarps;
+  int64_t task = (int64_t)warp * gridDim.x + blockIdx.x;
+  auto request = [&](int64_t t) {                                  // (rows beyond M arrive as zeros)
+    mbar_arrive_expect_tx_elect(bar, 8192u);
+    tma_load_4d_elect(raw, &tmx, 0, 0, 0, (int)(t * ROWS), bar);
+    tma_load_4d_elect(raw + 4096u, &tmx, 0, 1, 0, (int)(t * ROWS), bar);
+  };
+  if (task < tasks) request(task);
+  if (MODE == kCodes && p.layout == BRO_LAYOUT_GEMM)
+    rq::clear_padding(p.scales, p.M, p.scale_kblocks, (int64_t)blockIdx.x * (kRowWarps * 32) + threadIdx.x, (int64_t)gridDim.x * (kRowWarps * 32));
+
+  // exchange: line of 512 bytes a lane, its piece i of 16 bytes at i ^ (i / 8) ^ (line mod 8): no conflicts either way
+  const uint32_t mine = xch + (uint32_t)lane * 512u, from = xch + (uint32_t)(rs * LR) * 512u;
+  auto piece_at = [](uint32_t i) { return (i ^ (i >> 3)) << 4; };
+  const int o = L / GL, g = L % GL;                                // group of the 128, lane of the group
+  const uint32_t pick1 = (o & 1) ? 0x3715u : 0x6240u, pick2 = (o & 2) ? 0x3276u : 0x5410u;
+  uint32_t parity = 0;
+  bool ok = true;
+  for (; task < tasks; task += step) {
+    ok = mbar_wait_warp(bar, parity, SITE_RQ_FULL);
+    if (!ok) break;
+    parity ^= 1u;
+    uint64_t P[64];
+#pragma unroll
+    for (uint32_t j = 0; j < 16; ++j) {
+      rq::unpack_stage1(lds128(raw + (j >> 3) * 4096u + (uint32_t)lane * 128u + (((j & 7u) ^ ((uint32_t)lane & 7u)) << 4)), P + 4 * j);
+    }
+    __syncwarp();                                                  // (everyone has read the rows and, before, the exchange)
+    if (task + step < tasks) request(task + step);
+#pragma unroll
+    for (int h = 1; h < 64; h <<= 1) {                             // strides 2 .. 64
+#pragma unroll
+      for (int k = 0; k < 64; ++k) {
+        if ((k & h) == 0) {
+          const uint64_t a = P[k], b = P[k + h];
+          P[k] = rq::add2(a, b);
+          P[k + h] = rq::sub2(a, b);
+        }
+      }
+    }
+#pragma unroll
+    for (uint32_t i = 0; i < 32; ++i) sts_pairs(mine + (piece_at(i) ^ (((uint32_t)lane & 7u) << 4)), P[2 * i], P[2 * i + 1]);
+    __syncwarp();
+#pragma unroll
+    for (uint32_t j = 0; j < LR; ++j) {
+#pragma unroll
+      for (uint32_t q = 0; q < C / 4; ++q)
+        lds_pairs(from + j * 512u + (piece_at((uint32_t)(C / 4) * L + q) ^ ((j & 7u) << 4)), P[j * (C / 2) + 2 * q], P[j * (C / 2) + 2 * q + 1]);
+    }
+#pragma unroll
+    for (int h = 1; h < LR; h <<= 1) {                             // strides 128 .. K / 2
+#pragma unroll
+      for (int j = 0; j < LR; ++j) {
+        if ((j & h) == 0) {
+#pragma unroll
+          for (int i = 0; i < C / 2; ++i) {
+            const uint64_t a = P[j * (C / 2) + i], b = P[(j + h) * (C / 2) + i];
+            P[j * (C / 2) + i] = rq::add2(a, b);
+            P[(j + h) * (C / 2) + i] = rq::sub2(a, b);
+          }
+        }
+      }
+    }
+    // maxima: of the lane's C values of every 128, then over the group's lanes, which share the 128s among them: four are left to each
+    float m[LR];
+#pragma unroll
+    for (int j = 0; j < LR; ++j) {
+      m[j] = 0.f;
+#pragma unroll
+      for (int i = 0; i < C / 2; ++i) {
+        float a, b;
+        rq::unpack2(P[j * (C / 2) + i], a, b);
+        asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m[j]) : "f"(a), "f"(b));
+      }
+    }
+#pragma unroll
+    for (int d = GL / 2; d > 0; d >>= 1) {
+      const bool up = (lane & d) != 0;
+#pragma unroll
+      for (int k = 0; k < 4 * d; ++k) {
+        const float keep = up ? m[k + 4 * d] : m[k], send = up ? m[k] : m[k + 4 * d];
+        m[k] = fmaxf(keep, __shfl_xor_sync(0xFFFFFFFFu, send, d));
+      }
+    }
+    // this lane's groups: o of the 128s 4 g .. 4 g + 3
+    uint32_t bytes = 0, ef[4];
+    bool usual = true;                                             // c * 2^-E is a normal fp32 (see rq::quantize_group)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      ef[k] = __float_as_uint(__fmul_rn(m[k], __uint_as_float(cbits))) >> 23;
+      usual = usual && ef[k] >= 27u && ef[k] <= 250u;
+      bytes |= (ef[k] > 2u ? ef[k] - 2u : 0u) << (8 * k);
+    }
+    const int64_t row0 = task * ROWS;
+    if constexpr (MODE == kCodes) {
+      usual = __all_sync(0xFFFFFFFFu, usual);
+      uint32_t f[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t s = (bytes >> (8 * k)) & 0xFFu;
+        f[k] = usual ? cbits + ((127u - s) << 23) : (254u - s) << 23;
+      }
+      __syncwarp();                                                  // (everyone has read the exchange)
+      sts128(xch + (uint32_t)lane * 16u, f[0], f[1], f[2], f[3]);
+      __syncwarp();
+      uint8_t* const codes_at = p.codes + (row0 + rs) * (K / 2) + L * (C / 2);
+      const bool live = row0 + rs < p.M;
+      if (!usual) {                                                // (two roundings then, as everywhere)
+        const uint64_t cc = rq::pack2(__uint_as_float(cbits), __uint_as_float(cbits));
+#pragma unroll
+        for (int k = 0; k < 64; ++k) P[k] = rq::mul2(P[k], cc);
+      }
+#pragma unroll
+      for (int jj = 0; jj < LR / 4; ++jj) {
+        const uint4 scale = lds128(xch + (uint32_t)(lane - g + jj) * 16u);
+        const uint32_t sc[4] = {scale.x, scale.y, scale.z, scale.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int j = 4 * jj + k;
+          const uint64_t ff = rq::pack2(__uint_as_float(sc[k]), __uint_as_float(sc[k]));
+          float r[C];
+#pragma unroll
+          for (int i = 0; i < C / 2; ++i) rq::unpack2(rq::mul2(P[j * (C / 2) + i], ff), r[2 * i], r[2 * i + 1]);
+          if constexpr (C == 4) {
+            if (live) *reinterpret_cast<uint16_t*>(codes_at + j * 64) = (uint16_t)rq::pack_e2m1x4(r[0], r[1], r[2], r[3]);
+          } else if constexpr (C == 8) {
+            if (live) *reinterpret_cast<uint32_t*>(codes_at + j * 64) = rq::pack_e2m1x8(r[0], r[1], r[2], r[3], r[4], r[5], r[6], r[7]);
+          } else {
+            if (live)
+              *reinterpret_cast<uint2*>(codes_at + j * 64) = make_uint2(rq::pack_e2m1x8(r[0], r[1], r[2], r[3], r[4], r[5], r[6], r[7]),
+                                                                        rq::pack_e2m1x8(r[8], r[9], r[10], r[11], r[12], r[13], r[14], r[15]));
+          }
+        }
+      }
+    }
+    // scale bytes: lane (o, g) has those of group o of four 128s; it gets all four groups' of the 128 number 4 g + o
+    const uint32_t w1 = __byte_perm(bytes, __shfl_xor_sync(0xFFFFFFFFu, bytes, GL), pick1);
+    const uint32_t w2 = __byte_perm(w1, __shfl_xor_sync(0xFFFFFFFFu, w1, 2 * GL), pick2);
+    const int64_t row = row0 + rs;
+    const int j = 4 * g + o;
+    if (row < p.M) {
+      uint8_t* dst = p.scales + (MODE == kCodes && p.layout == BRO_LAYOUT_GEMM
+                                     ? ((row >> 7) * p.scale_kblocks + j) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4
+                                     : row * (K / 32) + 4 * j);
+      if (MODE == kCodes || (reinterpret_cast<uintptr_t>(dst) & 3) == 0) {
+        *reinterpret_cast<uint32_t*>(dst) = w2;
+      } else {
+        for (int i = 0; i < 4; ++i) dst[i] = (uint8_t)(w2 >> (8 * i));
+      }
+    }
+  }
+  // (left before the end only after a lost wait: its copies may still land, wait once more)
+  if (!ok) mbar_wait_warp(bar, parity, SITE_RQ_DRAIN);
+}
+
 // 3-D view of x for the kernels above: {64 bf16 (128 bytes), K / 64 segments, M rows}, box = whole rows (of at most 256 segments).
 bro_status make_row_map(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx, int box_rows);
 
@@ -621,6 +807,29 @@ inline unsigned grid_for(int64_t passes, const Params& p, int mode, int threads,
     if (want < clearing) want = clearing;
   }
   return (unsigned)(want < cap ? want : cap);
+}
+
+// 4-D view of x: {64 bf16 (128 bytes), even or odd segment, K / 128, M rows}, box = the even or the odd segments of `box_rows` rows.
+bro_status make_parity_map(CUtensorMap* map, const void* x, int64_t M, int64_t K, int64_t ldx, int box_rows);
+
+template <int LOG2K>
+inline bro_status launch_warp(const Params& p, int mode, int sm_count, cudaStream_t st) {
+  constexpr int K = 1 << LOG2K, ROWS = 4096 / K;
+  CUtensorMap tmx;
+  const bro_status mrc = make_parity_map(&tmx, p.x, p.M, p.K, p.ldx, ROWS);
+  if (mrc != BRO_OK) return mrc;
+  auto kernel = mode == kBytes ? rotate_quantize_global_warp_kernel<LOG2K, kBytes> : rotate_quantize_global_warp_kernel<LOG2K, kCodes>;
+  static DeviceOnce once[2];         // (per mode)
+  const bro_status rc = device_once(once[mode == kBytes ? 1 : 0], nullptr, [&](int*) {
+    return cuda_ok(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowWarpSmem), "cudaFuncSetAttribute(rotate_quantize_global_warp)")
+               ? BRO_OK
+               : BRO_ERR_CUDA;
+  });
+  if (rc != BRO_OK) return rc;
+  return cuda_ok(launch_kernel(kernel, grid_for((p.M + ROWS - 1) / ROWS, p, mode, kRowWarps * 32, sm_count), kRowWarps * 32, kRowWarpSmem, st, 1, tmx, p),
+                 "rotate_quantize_global launch")
+             ? BRO_OK
+             : BRO_ERR_CUDA;
 }
 
 template <int LOG2V, int LOG2K = LOG2V>
@@ -718,6 +927,17 @@ inline bro_status launch(const void* x, int64_t M, int64_t K, int64_t ldx, const
     // Few rows: one CTA an SM of that kernel (K = 4096) or up to 2.5 (K = 2048).  [700, 2048] 2.82 : 3.01 us, [1000, 2048] 3.7 : 3.3;
     // [129, 4096] with signs 2.42 : 2.73, [160, 4096] 2.55 : 2.45.
     const bool few = mode == kCodes && (K == 2048 ? M <= 5 * sm_count : M <= sm_count);
+    // Rows for every SM: a warp for 4096 channels.  It has one round to lose at the end, eight times an SM's 4096 channels, and starts later.
+    // 64 values a thread : warp, codes [1448, 1024] 3.0 : 3.15 us, [2896, 1024] 4.8 : 4.2, [65536, 1024] 49.3 : 41.4, [1024, 2048] 3.3 : 3.6,
+    // [1448, 2048] 4.9 : 4.55, [2896, 2048] 7.4 : 7.7, [32768, 2048] 50.0 : 45.4, [512, 4096] 3.3 : 3.4, [724, 4096] 4.95 : 4.5, [2048, 4096] 9.7 : 9.5,
+    // [16384, 4096] 50.5 : 44.5; scale bytes [2896, 1024] 4.3 : 3.6, [1448, 2048] 4.4 : 3.65, [65536, 1024] 45.3 : 35.0, [16384, 4096] 47.4 : 37.9
+    // (these gain a little from 2^20.5 on, [724, 2048] 2.86 : 2.77; one line for both).
+    // With signs, whose bits each lane has to gather first, 4 us more.
+    if (!signs && lg >= 10 && lg <= 12 && mode != kError && elements >= (int64_t)5 << 19) {
+      if (lg == 10) return launch_warp<10>(p, mode, sm_count, st);
+      if (lg == 11) return launch_warp<11>(p, mode, sm_count, st);
+      return launch_warp<12>(p, mode, sm_count, st);
+    }
     switch (lg) {
       case 10: return launch_wide<12, 10>(p, mode, sm_count, st);
       case 11:

@@ -1,0 +1,60 @@
+"""GPU parity of the full-dimension rotation by a warp for 4096 channels (K = 1024, 2048, 4096, many rows): codes bit for bit and scale
+bytes against the CPU oracle, at the rows where it begins, with rows left over from a warp's, rows with a stride, rows of zeros and of values at
+the ends of the exponent range, which take the general form of the scaling."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from gpu_util import Guarded, kernels_of
+from paper_2511_04214_b200 import synth
+from test_gpu_rotate_quantize_decode import tiled
+
+pytestmark = pytest.mark.gpu
+KERNEL = "rotate_quantize_global_warp_kernel"
+
+
+def rows_of(M, K, stride):
+    x = synth.activations(M, K, seed=M + K)
+    x[1] = 0
+    x[2, :40] = 0
+    x[M - 1] *= 2.0 ** -120
+    x[M // 2] *= 2.0 ** 110
+    d = torch.zeros(M, stride, dtype=torch.bfloat16, device="cuda")[:, :K]
+    d.copy_(x)
+    return synth.bf16_bits(x), d
+
+
+@pytest.mark.parametrize("M,K,pad", [(2561, 1024, 0), (2563, 1024, 8), (1281, 2048, 8), (1282, 2048, 0), (641, 4096, 16), (2500, 4096, 0)])
+@pytest.mark.parametrize("layout", [0, 1])
+def test_codes(M, K, pad, layout):
+    from paper_2511_04214_b200 import binding as bro
+    bits, x = rows_of(M, K, K + pad)
+    rc, rs = oracle.rotate_quantize_mxfp4(bits, K)
+    codes, scales = Guarded(bro.codes_bytes(M, K)), Guarded(bro.scales_bytes(M, K, layout))
+    call = lambda: bro.rotate_quantize_mxfp4(x, 0, codes.view, scales.view, layout)  # noqa: E731
+    (name,) = kernels_of(call)
+    assert KERNEL in name
+    codes.view.fill_(0xA5), scales.view.fill_(0xA5)
+    call()
+    assert bro.last_device_status() == 0
+    codes.check(), scales.check()
+    assert np.array_equal(codes.numpy().reshape(M, K // 2), rc)
+    assert np.array_equal(scales.numpy(), tiled(rs) if layout else rs.reshape(-1))
+
+
+@pytest.mark.parametrize("M,K,shift", [(2561, 1024, 1), (1281, 2048, 0), (1283, 2048, 2), (641, 4096, 0), (642, 4096, 3)])
+def test_scale_bytes(M, K, shift):
+    from paper_2511_04214_b200 import binding as bro
+    bits, x = rows_of(M, K, K)
+    out = Guarded(M * K // 32 + 4)
+    call = lambda: bro.group_scale_bytes(x, 0, out.view[shift:shift + M * K // 32].view(M, K // 32))  # noqa: E731
+    (name,) = kernels_of(call)
+    assert KERNEL in name
+    out.view.fill_(0xA5)
+    call()
+    assert bro.last_device_status() == 0
+    out.check()
+    got = out.numpy()
+    assert np.array_equal(got[shift:shift + M * K // 32].reshape(M, K // 32), oracle.rotate_quantize_mxfp4(bits, K)[1])
+    assert (got[:shift] == 0xA5).all() and (got[shift + M * K // 32:] == 0xA5).all()
