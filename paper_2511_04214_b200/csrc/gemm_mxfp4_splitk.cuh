@@ -16,9 +16,11 @@
 //     first tile of columns also leaves codes and scales in the caller's workspace, as the stand-alone kernel would.
 //   * otherwise, with W packed before the previous kernel in the stream started (the whole-layer calls), the whole ring of
 //     weight tiles is requested before griddepcontrol.wait, under the rotate+quantize kernel.
-// A launch is a chain, and so is a decoding step of many.  FUSED lets the next kernel in (launch_dependents) once the last load has been
-// requested; where that one's CTAs fit beside these, they have set up when these end.  At the start instead, they compete for the loads:
-// (16, 4096, 4096) 5.1 -> 6.3 us, (1, 8192, 28672) 21.3 -> 21.8.  Without a quantiser the next kernel is a small one, let in at the start.
+// A launch is a chain, and so is a decoding step of many.  FUSED lets the next kernel in (launch_dependents) once its own wait has returned, and with
+// eight quantising warps, where that one's CTAs fit beside these and have set up when these end, behind its last load: earlier, what comes
+// in draws on the same memory, (1, 8192, 28672) 21.2 -> 22.0 us, four layers of 2 tokens, 3072 wide, 24.4 -> 26.4, and before the wait the kernel
+// after the next takes its place, (16, 4096, 4096) 5.1 -> 6.3.  With sixteen nothing fits, and behind the last load is late: four layers
+// of 16 tokens 36.6 -> 37.5.  Without a quantiser the next kernel is a small one, let in at the start.
 // Warps: 0 TMA producer, 1 TMEM owner and MMA issuer, 2.. epilogue (FUSED: quantise before).  Every mbarrier wait is bounded, and all
 // threads of a cluster reach both cluster barriers whatever happened before.
 #pragma once
@@ -144,6 +146,7 @@ template <int ROW_BLOCKS, int QUANT_WARPS>
 __global__ void __launch_bounds__(threads_of(QUANT_WARPS), QUANT_WARPS == 8 ? 2 : 1)
 gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_constant__ CUtensorMap tmw, const Params p) {
   constexpr bool FUSED = QUANT_WARPS > 0;
+  constexpr bool kLetInLate = QUANT_WARPS == 8;      // (see the top of the file)
   extern __shared__ uint8_t smem_raw[];
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   // stages of W tiles and W scales; token codes of all stages; token scales of all stages; (split > 1) the parts received; the barriers
@@ -225,6 +228,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
       // the weights may be what the kernel before is still writing: before the wait they are only drawn into L2
       for (int s = 0; s < min(k_count, p.stages); ++s) l2_prefetch_2d_elect(&tmw, (k_first + s) * 128, n0);
       griddep_wait();
+      if (!kLetInLate) griddep_launch_dependents();
     } else if (early_w) {
       const int pre = min(k_count, p.stages);
       for (int s = 0; s < pre; ++s) issue_step(s, s, 1);       // weights: before the wait
@@ -241,7 +245,7 @@ gemm_mxfp4_splitk_kernel(const __grid_constant__ CUtensorMap tma, const __grid_c
       issue_step(i, stage, 3);
       if (++stage == p.stages) { stage = 0; phase ^= 1u; }
     }
-    if (FUSED) griddep_launch_dependents();
+    if (FUSED && kLetInLate) griddep_launch_dependents();
     if (!ok) {
       // do not leave while copies may still land: wait (bounded) for the last load armed on every stage
       for (int j = i > p.stages ? i - p.stages : 0; j < i; ++j)
