@@ -75,12 +75,12 @@ def select_shapes(args):
 GEMM_SOURCES = ("bro_common.cuh", "gemm_mxfp4.cuh", "gemm_mxfp4_2cta.cuh")
 RQ_SOURCES = ("bro_common.cuh", "rotate_quantize.cuh", "rotate_quantize_direct.cuh")
 NCU_TRAFFIC = {
-    "cfg5": {"sources": GEMM_SOURCES, "digest": "49ab7565188e8384a2fdbe5579fa86605abe9616f2fc8fe10a7b56b94f267506",
-             "per_row_of": (8192, 8192, 28672), "bytes": 535290112 + 440916992},
-    "cfg3": {"sources": GEMM_SOURCES, "digest": "49ab7565188e8384a2fdbe5579fa86605abe9616f2fc8fe10a7b56b94f267506",
-             "shapes": {(4096, 4096, 14336): 67853312 + 69395456}},
-    "cfg4": {"sources": RQ_SOURCES, "digest": "896c8adff1339690e1c145cc5a6f8f8c8444fcd6356b68930d84461b0011690c",
-             "shapes": {(16384, 4096, 32): 134233088 + 18386944}},
+    "cfg5": {"sources": GEMM_SOURCES, "digest": "aafd488bb74d75d704d3aa29a36cd5397b50cd07622a07d1432b018c186f4ea4",
+             "per_row_of": (8192, 8192, 28672), "bytes": 535109376 + 440277504},
+    "cfg3": {"sources": GEMM_SOURCES, "digest": "aafd488bb74d75d704d3aa29a36cd5397b50cd07622a07d1432b018c186f4ea4",
+             "shapes": {(4096, 4096, 14336): 68069888 + 68973312}},
+    "cfg4": {"sources": RQ_SOURCES, "digest": "ada0edf9e536ea39d6e8104bc5ebf363780ecf0d7b9927f5c0c08aaf888074d5",
+             "shapes": {(16384, 4096, 32): 134228224 + 18085632}},
 }
 
 

@@ -616,7 +616,7 @@ __global__ void __launch_bounds__(128, 5) rotate_quantize_global_few_kernel(cons
 // spread over 32 / C lanes, which share the search for it: each is left with the maxima of four groups, finds their scales and gives them
 // back through shared memory.  Nothing is shared between warps: each has its rows (TMA, the even and the odd 128-byte segments
 // apart, so that the lanes read without conflicts) and its 16 KiB of exchange, and there is no barrier.  Two warps on each of an SM's four
-// schedulers, for the registers (a ninth leaves one of them with three: 62 us); bound by the latencies that two warps do not hide (issue 54 %).
+// schedulers, for the registers (a ninth leaves one of them with three: 62 us); bound by the latencies that two warps do not hide (issue 57 %, L1 data path 61 %).
 // Codes go out as they are, 64 bytes of a row a store: collected in shared memory first, K = 4096 took 47.3 us, not 44.5 (K = 2048 44.7, not 45.4).
 constexpr int kRowWarps = 8;
 constexpr int kRowWarpBytes = 8192 + 16384, kRowWarpSmem = kRowWarps * kRowWarpBytes + kRowWarps * 8 + 1024;
