@@ -236,7 +236,8 @@ __global__ void __launch_bounds__(kScanThreads) outlier_clear(unsigned long long
 
 // The outliers are the top 0.1 % (top k of n) of the magnitudes, found exactly from a histogram of bf16 patterns; one pass
 // over x.  A shared-memory atomic per value bounded it before (75 us for 67 M values and 20 us for the search in a
-// launch of its own; now 42 us, of which 30 us are the pass, issue-bound, and 12 us merging and search), so only values of
+// launch of its own; now 36 us with the mask, of which 22 us are the pass, 134 MB at 0.93 of the copy bandwidth, and the rest a chain
+// that [300, 4096], 14 us, has too: clear, sample, merge, search, mask; a warp that reads whole lines gives 35.9 as well), so only values of
 // at least `lowest` are counted, a pattern that every CTA derives from the same 4096 sampled
 // values such that about 4 k values (and 12 of the sample) lie at or above it: the loop reduces a group to its maximum and
 // touches the histogram for the few groups that reach `lowest`.  Behind outlier_clear, which waited for everything older, it runs up
